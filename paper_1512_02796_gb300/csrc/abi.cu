@@ -166,6 +166,13 @@ uint64_t next_op_stamp() {
     return counter.fetch_add(1, std::memory_order_relaxed) + 1;
 }
 
+ElemScratch elem_scratch(qpat_mesh_s* M, cudaStream_t s, cudaError_t* err) {
+    ElemScratch w;
+    w.tet = M->ws.get<double2>("el.tet", size_t(M->el.E), s, err);
+    w.edge = M->ws.get<double2>("el.edge", size_t(M->el.NE), s, err);
+    return w;
+}
+
 // Operator state of one K(kappa, mu) or M_delta(kt, mt), library order.
 int prepare_K(qpat_mesh_s* M, const double* kap_l, const double* mu_l, OpState& st, cudaStream_t s,
               const char* tag) {
@@ -184,13 +191,13 @@ int prepare_K(qpat_mesh_s* M, const double* kap_l, const double* mu_l, OpState& 
     st.v64[0] = M->ws.get<double>(t + ".v64", M->d.sell_entries, s, &e);
     st.v32[0] = M->ws.get<float>(t + ".v32", M->d.sell_entries, s, &e);
     st.gbound = M->ws.get<double>(t + ".gb", 1, s, &e);
+    const ElemScratch scratch = elem_scratch(M, s, &e);
     if (e != cudaSuccess) return cuda_fail(e, "workspace");
     if ((e = launch_cast_d2f(N, kap_l, st.c1_32, s)) != cudaSuccess) return cuda_fail(e, "cast");
     if ((e = launch_cast_d2f(N, mu_l, st.c2_32, s)) != cudaSuccess) return cuda_fail(e, "cast");
-    if ((e = launch_assemble_K(M->d, kap_l, mu_l, st.v64[0], st.inv64, st.inv32, s, st.gbound)) != cudaSuccess)
+    if ((e = launch_assemble_K(M->d, M->el, scratch, kap_l, mu_l, st.v64[0], st.v32[0], st.inv64, st.inv32, s,
+                               st.gbound)) != cudaSuccess)
         return cuda_fail(e, "assemble_K");
-    if ((e = launch_cast_vals(M->d.sell_entries, st.v64[0], st.v32[0], s)) != cudaSuccess)
-        return cuda_fail(e, "cast");
     return QPAT_OK;
 }
 
@@ -216,11 +223,12 @@ int prepare_prior(qpat_mesh_s* M, const double* kt_l, const double* mt_l, double
     st.v64[0] = M->ws.get<double>("opP.v64a", M->dp.sell_entries, s, &e);
     st.v64[1] = M->ws.get<double>("opP.v64b", M->dp.sell_entries, s, &e);
     st.gbound = M->ws.get<double>("opP.gb", 1, s, &e);
+    const ElemScratch scratch = elem_scratch(M, s, &e);
     if (e != cudaSuccess) return cuda_fail(e, "workspace");
     if ((e = launch_cast_d2f(N, kt_l, st.c1_32, s)) != cudaSuccess) return cuda_fail(e, "cast");
     if ((e = launch_cast_d2f(N, mt_l, st.c2_32, s)) != cudaSuccess) return cuda_fail(e, "cast");
-    if ((e = launch_assemble_prior(M->dp, kt_l, mt_l, st.inv_T2, kind, q, b_over_a, delta, st.v64[0], st.v64[1],
-                                   st.inv64, st.inv32, s, st.gbound)) != cudaSuccess)
+    if ((e = launch_assemble_prior(M->dp, M->el, scratch, kt_l, mt_l, st.inv_T2, kind, q, b_over_a, delta, st.v64[0],
+                                   st.v64[1], st.inv64, st.inv32, s, st.gbound)) != cudaSuccess)
         return cuda_fail(e, "assemble_prior");
     return QPAT_OK;
 }
@@ -717,6 +725,8 @@ int qpat_mesh_host_info(const double* xyz, int64_t N, const int32_t* tets, int64
         info8[8] = nfull;
         info8[9] = nsub;
     }
+    msg = check_element_plan(h, build_element_plan(h));
+    if (!msg.empty()) return fail(QPAT_EINVAL, "host check: " + msg);
     if (faces) std::memcpy(faces, h.faces_caller.data(), sizeof(int32_t) * 3 * h.F);
     if (perm) std::memcpy(perm, h.perm.data(), sizeof(int32_t) * h.N);
     // every tet must be listed once per distinct patch owning one of its

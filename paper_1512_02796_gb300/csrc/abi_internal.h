@@ -88,6 +88,7 @@ struct qpat_mesh_s {
     qpat::HostMesh h;
     qpat::MeshDev d{};
     qpat::MeshDev dp{};  // d with the stiffness-only pattern of the prior operators (psell)
+    qpat::ElemDev el{};  // element plan and geometry
     std::vector<void*> dev_allocs;
     int device = 0;
     cudaStream_t stream = nullptr;   // used by the host-pointer entry points
@@ -111,6 +112,8 @@ int cuda_fail(cudaError_t e, const char* where);
 int round_rhs(int K);
 
 int upload_mesh(qpat_mesh_s* M);
+// scratch of the element kernels (element.cu), in the mesh's workspace
+ElemScratch elem_scratch(qpat_mesh_s* M, cudaStream_t s, cudaError_t* err);
 int prepare_K(qpat_mesh_s* M, const double* kap_l, const double* mu_l, OpState& st, cudaStream_t s,
               const char* tag = "opK");
 int prepare_prior(qpat_mesh_s* M, const double* kt_l, const double* mt_l, double T, int kind, double q,

@@ -22,6 +22,7 @@ struct qpat_batch_s {
         double *kl = nullptr, *ml = nullptr, *vals = nullptr, *inv = nullptr;     // library layout
         double *f = nullptr, *x = nullptr, *r = nullptr, *p0 = nullptr, *p1 = nullptr, *q = nullptr;
         double *partials = nullptr, *ctl = nullptr;
+        qpat::ElemScratch scratch;                 // of this problem's assembly
         double *z = nullptr, *gb = nullptr;  // patch-local Chebyshev preconditioner
     };
     int device = 0;
@@ -68,8 +69,8 @@ int batch_sequence(qpat_batch_s* B, cudaStream_t s) {
         if ((e = launch_to_lib<double, double>(m, 1, 1, P.kappa, P.kl, s)) != cudaSuccess ||
             (e = launch_to_lib<double, double>(m, 1, 1, P.mu, P.ml, s)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: to_lib");
-        if ((e = launch_assemble_K(m, P.kl, P.ml, P.vals, P.inv, nullptr, s, B->poly_deg > 0 ? P.gb : nullptr)) !=
-            cudaSuccess)
+        if ((e = launch_assemble_K(m, P.mesh->el, P.scratch, P.kl, P.ml, P.vals, nullptr, P.inv, nullptr, s,
+                                   B->poly_deg > 0 ? P.gb : nullptr)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: assemble");
         if ((e = cudaMemsetAsync(P.f, 0, sizeof(double) * N * B->R, s)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: memset");
@@ -124,6 +125,10 @@ int qpat_batch_create(int nprob, const qpat_mesh_t* meshes, const int* K, const 
             (rc = batch_alloc(B, &P.p1, N * R)) || (rc = batch_alloc(B, &P.q, N * R)) ||
             (rc = batch_alloc(B, &P.partials, pcg_partials_doubles())) || (rc = batch_alloc(B, &P.ctl, 64)))
             break;
+        double *tq = nullptr, *ev = nullptr;
+        if ((rc = batch_alloc(B, &tq, 2 * size_t(P.mesh->el.E))) || (rc = batch_alloc(B, &ev, 2 * size_t(P.mesh->el.NE))))
+            break;
+        P.scratch = {reinterpret_cast<double2*>(tq), reinterpret_cast<double2*>(ev)};
         if (B->poly_deg > 0 && ((rc = batch_alloc(B, &P.z, N * R)) || (rc = batch_alloc(B, &P.gb, 1)))) break;
         PcgBatchProblem q;
         q.m = P.mesh->d;

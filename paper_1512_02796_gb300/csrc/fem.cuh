@@ -56,17 +56,6 @@ __host__ __device__ inline T prior_weight(int kind, T g2, T inv_T2, T q) {
     return e == T(0) ? T(1) : pow(g2 + T(1) / inv_T2, e);
 }
 
-// Slot of local column c in library row g of the sliced-ELLPACK pattern.
-__device__ __forceinline__ int64_t sell_slot(const MeshDev& m, int g, int c) {
-    const int64_t base = m.sell_ptr[g >> 5];
-    const int lane = g & 31, len = m.sell_len[g];
-    for (int k = 0; k < len; ++k) {
-        const int64_t idx = (base + k) * 32 + lane;
-        if (m.sell_col[idx] == c) return idx;
-    }
-    return -1;
-}
-
 // Rows [ob, ob + nown) of an assembled operator applied to staged input
 // xin (touched x R, node-major), R right-hand sides; result written by
 // `emit(i, r, value)` with i the owned local row.

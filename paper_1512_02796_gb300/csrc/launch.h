@@ -5,6 +5,7 @@
 
 #include <vector>
 
+#include "element.h"
 #include "fem.cuh"
 #include "qpat_internal.h"
 
@@ -26,25 +27,31 @@ cudaError_t launch_invdiag_K(const MeshDev& m, const double* kappa, const double
 cudaError_t launch_invdiag_prior(const MeshDev& m, const double* u1, const double* u2, double inv_T2, int kind,
                                  double q, double scale1, double delta, double* inv64, float* inv32,
                                  cudaStream_t s);
+// ---------------------------------------------------------------- element.cu
 // Assembly of K (FP64 values in the sliced-ELLPACK pattern; val must hold
 // m.sell_entries) and of the two prior blocks with delta on the diagonal;
-// both also write the inverse diagonal (FP64 and, if not null, FP32).
+// both also write the inverse diagonal (FP64 and, if not null, FP32), K its
+// FP32 values too if val32 is not null.
 // gbound (optional, one double): receives max over rows and value sets of
 // sum_j |a_ij| / a_ii, a Gershgorin bound of the spectrum of D^-1 A (and of
 // D^-1 A_pp for every principal block A_pp).
-cudaError_t launch_assemble_K(const MeshDev& m, const double* kappa, const double* mu, double* val, double* inv64,
-                              float* inv32, cudaStream_t s, double* gbound = nullptr);
-cudaError_t launch_assemble_prior(const MeshDev& m, const double* u1, const double* u2, double inv_T2, int kind,
-                                  double q, double scale1, double delta, double* val0, double* val1, double* inv64,
-                                  float* inv32, cudaStream_t s, double* gbound = nullptr);
-cudaError_t launch_cast_vals(int64_t n, const double* in, float* out, cudaStream_t s);
+cudaError_t launch_assemble_K(const MeshDev& m, const ElemDev& el, const ElemScratch& w, const double* kappa,
+                              const double* mu, double* val, float* val32, double* inv64, float* inv32, cudaStream_t s,
+                              double* gbound = nullptr);
+cudaError_t launch_assemble_prior(const MeshDev& m, const ElemDev& el, const ElemScratch& w, const double* u1,
+                                  const double* u2, double inv_T2, int kind, double q, double scale1, double delta,
+                                  double* val0, double* val1, double* inv64, float* inv32, cudaStream_t s,
+                                  double* gbound = nullptr);
+// y = -(S(c1) + M(c2)) x for R right-hand sides, N x R node-major, without the Robin term (c1, c2 of any sign)
+cudaError_t launch_rhs_jv(const MeshDev& m, const ElemDev& el, const ElemScratch& w, int R, const double* c1,
+                          const double* c2, const double* x, double* y, cudaStream_t s);
+// y (N x 2) = [ sum_k G1^T z_k ; sum_k G2 z_k ] for N x R phi and z (see element.cu); node: N doubles of scratch
+cudaError_t launch_vjp_accum(const MeshDev& m, const ElemDev& el, const ElemScratch& w, double* node, int R,
+                             const double* phi, const double* z, double* y, cudaStream_t s);
 // y = A x with an assembled operator (NV = 1: one value set for R RHS; NV = 2: the prior, R = 2)
 template <typename T>
 cudaError_t launch_apply_csr(const MeshDev& m, int NV, int R, const T* v0, const T* v1, const T* x, T* y,
                              cudaStream_t s);
-// y (N x 2) = [ -sum_k G1-transpose-type term ; -sum_k M(phi_k) z_k ] (see kernels.cu)
-template <typename T>
-cudaError_t launch_vjp_accum(const MeshDev& m, int K, const T* phi, const T* z, T* y, cudaStream_t s);
 // f (N x R node-major, library order, column k < K) += 2 Phi_F |F| / 3 at the
 // vertices of every face (flux: K x F canonical order); f must be zeroed.
 cudaError_t launch_load(const MeshDev& m, int K, int R, const double* flux, double* f, cudaStream_t s);

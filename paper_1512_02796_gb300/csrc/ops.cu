@@ -60,18 +60,21 @@ __global__ void k_unpack2(int64_t N, int R, const double* in, double* a, double*
 }
 
 template <typename T>
-int up(qpat_mesh_s* M, const std::vector<T>& v, const T** dst) {
+int room(qpat_mesh_s* M, size_t count, const T** dst) {
     void* p = nullptr;
-    size_t bytes = std::max<size_t>(v.size() * sizeof(T), 16);
-    cudaError_t e = cudaMalloc(&p, bytes);
+    cudaError_t e = cudaMalloc(&p, std::max<size_t>(count * sizeof(T), 16));
     if (e != cudaSuccess) return cuda_fail(e, "qpat_mesh: cudaMalloc");
     M->dev_allocs.push_back(p);
-    if (!v.empty()) {
-        e = cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_fail(e, "qpat_mesh: cudaMemcpy");
-    }
     *dst = static_cast<const T*>(p);
     return QPAT_OK;
+}
+
+template <typename T>
+int up(qpat_mesh_s* M, const std::vector<T>& v, const T** dst) {
+    const int rc = room(M, v.size(), dst);
+    if (rc != QPAT_OK || v.empty()) return rc;
+    const cudaError_t e = cudaMemcpy(const_cast<T*>(*dst), v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? QPAT_OK : cuda_fail(e, "qpat_mesh: cudaMemcpy");
 }
 
 }  // namespace
@@ -138,6 +141,32 @@ int upload_mesh(qpat_mesh_s* M) {
         return rc;
     dp.sell_entries = int64_t(h.psell_col.size());
     dp.sell_wmax = h.psell_wmax;
+    {
+        const ElementPlan plan = build_element_plan(h);
+        ElemDev& el = M->el;
+        el.E = h.E;
+        el.NE = plan.NE;
+        const int32_t *tet = nullptr, *edge = nullptr;
+        const double *re = nullptr, *rn = nullptr;
+        if ((rc = up(M, plan.tet, &tet)) || (rc = up(M, plan.node_ptr, &el.node_ptr)) ||
+            (rc = up(M, plan.node_tet, &el.node_tet)) || (rc = up(M, plan.ent_edge, &el.ent_edge)) ||
+            (rc = up(M, plan.ent_col, &el.ent_col)) || (rc = up(M, plan.pent_edge, &el.pent_edge)) ||
+            (rc = up(M, plan.edge, &edge)) || (rc = up(M, plan.tet_edge, &el.tet_edge)) ||
+            (rc = up(M, plan.edge_ptr, &el.edge_ptr)) || (rc = up(M, plan.edge_tet, &el.edge_tet)) ||
+            (rc = up(M, plan.in_prior, &el.in_prior)))
+            return rc;
+        el.tet = reinterpret_cast<const int4*>(tet);
+        el.edge = reinterpret_cast<const int2*>(edge);
+        if ((rc = up(M, plan.edge_vr, &re)) || (rc = up(M, plan.node_vr, &rn))) return rc;
+        el.edge_vr = reinterpret_cast<double2*>(const_cast<double*>(re));
+        el.node_vr = reinterpret_cast<double2*>(const_cast<double*>(rn));
+        const double *gs = nullptr, *gv = nullptr;
+        if ((rc = room(M, size_t(6 * el.E), &gs)) || (rc = room(M, size_t(el.E), &gv))) return rc;
+        el.s = const_cast<double*>(gs);
+        el.vm = const_cast<double*>(gv);
+        if ((e = launch_element_geometry(d, el, nullptr)) != cudaSuccess || (e = cudaStreamSynchronize(nullptr)) != cudaSuccess)
+            return cuda_fail(e, "qpat_mesh: element geometry");
+    }
     if ((e = cudaStreamCreateWithFlags(&M->stream, cudaStreamNonBlocking)) != cudaSuccess)
         return cuda_fail(e, "qpat_mesh: stream");
     if ((e = cudaMallocHost(&M->host_scratch, 256 * sizeof(double))) != cudaSuccess)
@@ -207,11 +236,12 @@ int jvp_lib(qpat_mesh_s* M, const SolveOpts& so, LinState& L, const double* s1, 
     double* b = M->ws.get<double>("jv.b", N, s, &e);
     double* rhs = M->ws.get<double>("jv.rhs", N * R, s, &e);
     double* x = M->ws.get<double>("jv.x", N * R, s, &e);
+    const ElemScratch scratch = elem_scratch(M, s, &e);
     if (e != cudaSuccess) return cuda_fail(e, "workspace");
     k_mul_launch(N, L.kap, s1, a, s);
     k_mul_launch(N, L.mu, s2, b, s);
     // rhs = G1 diag(kappa) s1 + G2 diag(mu) s2 = -(S(kappa o s1) + M(mu o s2)) phi
-    if ((e = launch_apply_K<double>(M->d, R, a, b, 0, -1.0, L.phi, rhs, s)) != cudaSuccess)
+    if ((e = launch_rhs_jv(M->d, M->el, scratch, R, a, b, L.phi, rhs, s)) != cudaSuccess)
         return cuda_fail(e, "jv rhs");
     int rc = solve(M, L.opK, so, R, rhs, x, s);
     if (rc != QPAT_OK) return rc;
@@ -228,6 +258,8 @@ int vjp_lib(qpat_mesh_s* M, const SolveOpts& so, LinState& L, const double* t, d
     double* rhs = M->ws.get<double>("jt.rhs", N * R, s, &e);
     double* z = M->ws.get<double>("jt.z", N * R, s, &e);
     double* y = M->ws.get<double>("jt.y", N * 2, s, &e);
+    double* dn = M->ws.get<double>("jt.dn", N, s, &e);
+    const ElemScratch scratch = elem_scratch(M, s, &e);
     if (e != cudaSuccess) return cuda_fail(e, "workspace");
     if (L.w)
         k_mul_launch(N * R, L.w, t, tw, s);
@@ -236,7 +268,7 @@ int vjp_lib(qpat_mesh_s* M, const SolveOpts& so, LinState& L, const double* t, d
     k_rowscale_launch(N, R, L.mu, tw, rhs, s);
     int rc = solve(M, L.opK, so, R, rhs, z, s);
     if (rc != QPAT_OK) return rc;
-    if ((e = launch_vjp_accum<double>(M->d, R, L.phi, z, y, s)) != cudaSuccess) return cuda_fail(e, "vjp accum");
+    if ((e = launch_vjp_accum(M->d, M->el, scratch, dn, R, L.phi, z, y, s)) != cudaSuccess) return cuda_fail(e, "vjp accum");
     k_jt_out_launch(N, R, L.kap, L.mu, y, L.phi, tw, o1, o2, s);
     return QPAT_OK;
 }
@@ -516,6 +548,8 @@ int qpat_jvp_vjp_pair_dev(qpat_mesh_t M, const qpat_params* prm, const double* k
     double* oj = M->ws.get<double>("pair.oj", N * R, s, &e);
     double* o1 = M->ws.get<double>("pair.o1", N, s, &e);
     double* o2 = M->ws.get<double>("pair.o2", N, s, &e);
+    double* dn = M->ws.get<double>("pair.dn", N, s, &e);
+    const ElemScratch scratch = elem_scratch(M, s, &e);
     if (e != cudaSuccess) return cuda_fail(e, "workspace");
     if ((e = launch_to_lib<double, double>(M->d, 1, 1, sv, s1, s)) != cudaSuccess ||
         (e = launch_to_lib<double, double>(M->d, 1, 1, sv + N, s2, s)) != cudaSuccess ||
@@ -524,7 +558,7 @@ int qpat_jvp_vjp_pair_dev(qpat_mesh_t M, const qpat_params* prm, const double* k
     // J s right-hand sides
     k_mul_launch(N, L.kap, s1, a, s);
     k_mul_launch(N, L.mu, s2, b, s);
-    if ((e = launch_apply_K<double>(M->d, R, a, b, 0, -1.0, L.phi, rj, s)) != cudaSuccess)
+    if ((e = launch_rhs_jv(M->d, M->el, scratch, R, a, b, L.phi, rj, s)) != cudaSuccess)
         return cuda_fail(e, "jv rhs");
     // J^T w right-hand sides
     if (L.w)
@@ -539,7 +573,7 @@ int qpat_jvp_vjp_pair_dev(qpat_mesh_t M, const qpat_params* prm, const double* k
     qpat::note_launch(1);
     k_unpack2<<<grid_n(N * 2 * R), 256, 0, s>>>(N, R, x2, xj, z);
     k_jv_out_launch(N, R, L.mu, b, xj, L.phi, L.w, oj, s);
-    if ((e = launch_vjp_accum<double>(M->d, R, L.phi, z, y, s)) != cudaSuccess) return cuda_fail(e, "vjp accum");
+    if ((e = launch_vjp_accum(M->d, M->el, scratch, dn, R, L.phi, z, y, s)) != cudaSuccess) return cuda_fail(e, "vjp accum");
     k_jt_out_launch(N, R, L.kap, L.mu, y, L.phi, tw, o1, o2, s);
     if ((e = launch_from_lib<double, double>(M->d, K, R, oj, out_jv, s)) != cudaSuccess ||
         (e = launch_from_lib<double, double>(M->d, 1, 1, o1, out_vjp, s)) != cudaSuccess ||
