@@ -642,9 +642,10 @@ def kernel_table(d, prm, precision: int, acc, sm_mhz: float, nsm: int, hbm_peak:
 
 def mg_kernel_table(d, prm, acc, sm_mhz: float, nsm: int, hbm_peak: float, step_ms_total: float):
     """The multigrid-preconditioned solves of a timed region: per solve kind
-    the whole CG solve (events around it) and its dominant kernel, the fine-
-    level Chebyshev smoothing step (events around each launch), with that
-    kernel's algorithmic work per launch:
+    the whole CG solve (events around it) and the fine level's smoothing
+    product (events around each launch) with its algorithmic work per launch:
+    at degree 1 the residual kernel (below), at higher degrees the Chebyshev
+    smoothing step:
       flops  2 nnz R + 6 N R   (the SpMV of b - A x, then d = c_d d + c_r D^-1 res, x += d)
       bytes  (s + 4) nnz nv + 2 N + 5 s R N + s N nv   (values and column ids, row lengths,
              b, x_in, d read, d and x_out written, D^-1)
@@ -665,6 +666,16 @@ def mg_kernel_table(d, prm, acc, sm_mhz: float, nsm: int, hbm_peak: float, step_
                   "bytes_per_launch": (2 * 8 + 4.0) * mesh.prior_entries + 2.0 * N + 5.0 * 8 * 2 * N + 16.0 * N,
                   "arith": "fp64"},
     }
+    if getattr(prm, "mg_degree", None) == 1:
+        # the degree-1 cycle: the fine level's residual after the pre-smoothing step, b - (A diag(wd)) b, on the
+        # stiffness-only pattern (flops 2 nnz R + N R; bytes (s nv + 4) nnz + 2 N + 2 s R N)
+        nnz = float(mesh.prior_entries)
+        for k, Rk, nv, sk in (("pair", R, 1, s), ("prior", 2, 2, 8)):
+            t = "float" if sk == 4 else "double"
+            kern[k].update(kernel=f"k_level<{t}, {Rk}, {nv}, 0, 1, 1> (fine-level residual after the pre-smoothing step of "
+                                  f"the multigrid V-cycle, {Rk} RHS)",
+                           flops_per_launch=2.0 * nnz * Rk + N * Rk,
+                           bytes_per_launch=(sk * nv + 4.0) * nnz + 2.0 * N + 2.0 * sk * Rk * N)
     f64_peak = fp64_peak_tflops(sm_mhz, nsm)
     for k, v in kern.items():
         v.update(acc[k])

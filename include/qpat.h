@@ -133,10 +133,13 @@ typedef struct {
                               1 = conjugate gradients with one V-cycle of
                               smoothed-aggregation algebraic multigrid per
                               iteration (Vanek, Mandel, Brezina 1996: aggregates
-                              of the matrix graph, P = (I - 4/(3 hi) D^-1 A) P_tent,
+                              of 8 nodes of the stiffness graph, P_tent smoothed
+                              by one damped Jacobi step that keeps the constants,
                               Galerkin coarse operators P^T A P, Chebyshev
                               smoothing in D^-1 A, an exact dense solve on the
-                              coarsest level of <= 128 rows), all in FP64; the K
+                              coarsest level of <= 128 rows; the cycle of K works
+                              on K with its couplings outside the stiffness
+                              pattern lumped on the diagonal), all in FP64; the K
                               solves then run FP64 iterates whatever `precision`
                               says;
                               2 = as 1 with the V-cycle of the K solves in FP32
@@ -153,7 +156,7 @@ typedef struct {
                               and degree 1 was the fastest measured) */
     double mg_ratio;       /* the smoothing polynomial targets [hi / mg_ratio, hi] of
                               the spectrum of D^-1 A, hi its Gershgorin bound
-                              (> 1; 0 = 30) */
+                              times a margin of 1.13 (> 1; 0 = 30) */
 } qpat_params;
 
 /* Report of qpat_reconstruct (Algorithm 1). */
@@ -212,8 +215,8 @@ int qpat_mesh_host_info(const double* xyz, int64_t N, const int32_t* tets, int64
                         int patch_nodes, int64_t* info8, int32_t* faces, int32_t* perm);
 
 /* Host-only check (needs no GPU) of the multigrid hierarchy that
- * qpat_params.multigrid builds for the K pattern (prior = 0) or the prior's
- * pattern (prior = 1) of the mesh qpat_mesh_ex would prepare: builds the
+ * qpat_params.multigrid builds for K (prior = 0) or M_delta (prior = 1), one
+ * and the same, on the mesh qpat_mesh_ex would prepare: builds the
  * aggregates, the level patterns and the index plans of the device set-up
  * and verifies every invariant the device relies on (P rows, R = P^T, the
  * slots of A P and P^T A P, symmetric coarse patterns, a coarsest level of
@@ -237,16 +240,17 @@ int qpat_mesh_reset_stats(qpat_mesh_t mesh);
  * -1 for a NULL mesh.  Not in the paper (diagnostics). */
 int64_t qpat_mesh_rhs_iterations(qpat_mesh_t mesh);
 
-/* Rows of every level of the multigrid hierarchy built for the K pattern
- * (prior = 0) or the prior's pattern (prior = 1), finest first, into rows
+/* Rows of every level of the multigrid hierarchy of the K solves
+ * (prior = 0) or the M_delta solves (prior = 1), finest first, into rows
  * (up to max_levels); returns the number of levels (0 before the first
  * multigrid solve of that kind).  Not in the paper (diagnostics). */
 int qpat_mesh_multigrid_levels(qpat_mesh_t mesh, int prior, int64_t* rows, int max_levels);
 
 /* With timing on (qpat_mesh_set_timing): the summed device time (ms) and
- * the count of the fine-level Chebyshev smoothing launches of the multigrid
- * cycles since the last reset (the cycle's dominant kernel; each launch
- * bracketed by CUDA events on its stream).  Not in the paper (diagnostics). */
+ * the count of the fine level's smoothing products in the multigrid cycles
+ * since the last reset (mg_degree 1: the residual after the pre-smoothing
+ * step; higher degrees: the Chebyshev smoothing steps; each launch bracketed
+ * by CUDA events on its stream).  Not in the paper (diagnostics). */
 int qpat_mesh_multigrid_fine_time(qpat_mesh_t mesh, double* ms, int64_t* launches);
 
 /* When on, every PCG launch is bracketed by CUDA events recorded on the

@@ -563,7 +563,12 @@ cudaError_t allow_smem(const void* func, size_t smem) {
     }
     return smem <= it->second ? cudaSuccess : cudaErrorInvalidValue;
 }
-void note_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+static thread_local int64_t t_launches = 0;
+void note_launch(int n) {
+    g_launches.fetch_add(n, std::memory_order_relaxed);
+    t_launches += n;
+}
+int64_t thread_launches() { return t_launches; }
 }  // namespace qpat
 
 extern "C" {
@@ -624,7 +629,9 @@ int qpat_multigrid_host_info(const double* xyz, int64_t N, const int32_t* tets, 
     HostMesh h;
     std::string msg = build_host_mesh(xyz, N, tets, E, patch_nodes, 0, h);
     if (!msg.empty()) return fail(QPAT_EINVAL, msg);
-    const AmgPlan plan = amg_build_plan(amg_fine_pattern(h, prior ? 1 : 0));
+    (void)prior;  // one hierarchy pattern serves K and M_delta
+    const SellPattern fine = amg_fine_pattern(h);
+    const AmgPlan plan = amg_build_plan(fine, amg_fine_graph(h, fine));
     msg = amg_check_plan(plan);
     if (!msg.empty()) return fail(QPAT_EINVAL, "multigrid plan: " + msg);
     const int L = int(plan.levels.size());

@@ -28,10 +28,10 @@ struct SellDev {
     int64_t n = 0;
     const int64_t* ptr = nullptr;
     const int32_t* col = nullptr;
-    const uint16_t* len = nullptr;
+    const uint16_t* len = nullptr;  // nullptr (row-major only): ptr[i + 1] - ptr[i]
     int64_t entries = 0;
     int maxlen = 0;
-    int rowmajor = 0;  // layout (see SellPattern); row-major rows are applied by 8 lanes each
+    int rowmajor = 0;  // layout (see SellPattern)
 };
 
 struct LevelDev {
@@ -55,11 +55,35 @@ struct LevelDev {
 
 namespace {
 
+__device__ __forceinline__ int row_len(const SellDev& S, int64_t i) {
+    return S.len ? int(S.len[i]) : int(S.ptr[i + 1] - S.ptr[i]);
+}
+
 __device__ __forceinline__ int64_t spos(const SellDev& S, int64_t row, int k) {
     return S.rowmajor ? S.ptr[row] + k : (S.ptr[row >> 5] + k) * 32 + (row & 31);
 }
 
 // ---------------------------------------------------------------- set-up kernels
+
+// The fine operator of K's cycle: the entries of K in the prior's pattern (a
+// subset of each row, in the same order), the others added to the diagonal.
+__global__ void __launch_bounds__(256) k_lump(SellDev K, const int* ent_edge, const uint8_t* in_prior, SellDev F,
+                                              const int32_t* diag, const double* val, double* out) {
+    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (i >= K.n) return;
+    const int L = K.len[i];
+    double lump = 0.0;
+    int k2 = 0;
+    for (int k = 0; k < L; ++k) {
+        const int64_t at = spos(K, i, k);
+        const int e = ent_edge[at];
+        if (e < 0 || in_prior[e])
+            out[spos(F, i, k2++)] = val[at];
+        else
+            lump += val[at];
+    }
+    out[spos(F, i, diag[i])] += lump;
+}
 
 // Inverse diagonal (n x NV, interleaved) and the Gershgorin bound
 // max_i sum_j |a_ij| / a_ii of D^-1 A per value set (hi must start at 0; the
@@ -95,23 +119,66 @@ __global__ void __launch_bounds__(256) k_dinv_hi(SellDev A, const int32_t* diag,
     }
 }
 
-// P = (I - omega D^-1 A) P_tent, omega = 4 / (3 hi): row i of P from row i of A.
+// Upper end of the smoothing interval: the Gershgorin bound with a margin.
+// A single step (degree 1) multiplies the top of the spectrum by
+// 1 - 2 / (1 + 1 / ratio) = -0.94 without it, so error there (the checkerboard
+// of a structured grid, which reaches the bound) would hardly decay; with 1.13
+// it is -0.71 and the 128^3 solves take half the iterations.
+constexpr double kSmoothMargin = 1.13;
+
+// Weighted inverse diagonal of the degree-1 smoother, wd = D^-1 / theta, and the scaled operator A diag(wd), so that
+// one gather forms b - A (wd b).
 template <int NV>
-__global__ void k_prolong(SellDev A, SellDev P, const uint16_t* a2p, const uint16_t* pself, const double* v0,
-                          const double* v1, const double* dinv, const double* hi, double* p0, double* p1) {
+__global__ void __launch_bounds__(256) k_weights(int64_t n, const double* dinv, const double* hi, double ratio,
+                                                 double* wd) {
+    __shared__ double w[NV];
+    if (threadIdx.x < NV) {
+        const double h = kSmoothMargin * hi[threadIdx.x];
+        w[threadIdx.x] = 1.0 / (0.5 * (h + h / ratio));
+    }
+    __syncthreads();
+    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (i < n * NV) wd[i] = w[i % NV] * dinv[i];
+}
+template <int NV>
+__global__ void __launch_bounds__(256) k_scaled(int64_t entries, const int32_t* col, const double* wd, const double* v0,
+                                                const double* v1, double* s0, double* s1) {
+    const int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (e >= entries) return;
+    const int64_t j = col[e];
+    s0[e] = v0[e] * wd[j * NV];
+    if (NV == 2) s1[e] = v1[e] * wd[j * NV + 1];
+}
+
+// Row i of P: 1 - omega on the row's own aggregate and omega shared out over
+// the aggregates of its graph neighbours by their couplings -a_ij (only
+// negative ones count).  For a row that sums to 0 this is one damped Jacobi
+// step on P_tent; for every row it keeps the constants exactly, which is what
+// the 1 / delta mode of M_delta needs.  omega: amg.h.
+template <int NV>
+__global__ void __launch_bounds__(256) k_prolong(SellDev A, SellDev P, const int32_t* diag, const uint16_t* a2p,
+                                                 const uint16_t* pself, const double* v0, const double* v1, double* p0,
+                                                 double* p1) {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i >= A.n) return;
-    const int L = A.len[i], LP = P.len[i];
+    const int L = A.len[i], LP = P.len[i], dk = diag[i];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const double* val = v == 0 ? v0 : v1;
         double* pv = v == 0 ? p0 : p1;
-        const double w = (4.0 / 3.0) / hi[v] * dinv[i * NV + v];
-        for (int k = 0; k < LP; ++k) pv[spos(P, i, k)] = 0.0;
-        pv[spos(P, i, pself[i])] = 1.0;
+        double sum = 0.0;
         for (int k = 0; k < L; ++k) {
             const int64_t at = spos(A, i, k);
-            pv[spos(P, i, a2p[at])] -= w * val[at];
+            if (k != dk && a2p[at] != kAmgDropped) sum += fmax(-val[at], 0.0);
+        }
+        for (int k = 0; k < LP; ++k) pv[spos(P, i, k)] = 0.0;
+        const bool any = sum > 0.0;
+        pv[spos(P, i, pself[i])] = any ? 1.0 - kAmgOmega : 1.0;
+        if (!any) continue;
+        const double w = kAmgOmega / sum;
+        for (int k = 0; k < L; ++k) {
+            const int64_t at = spos(A, i, k);
+            if (k != dk && a2p[at] != kAmgDropped) pv[spos(P, i, a2p[at])] += w * fmax(-val[at], 0.0);
         }
     }
 }
@@ -121,12 +188,13 @@ __global__ void k_prolong(SellDev A, SellDev P, const uint16_t* a2p, const uint1
 // of A are taken one after the other and the 8 lanes add a_ij P[j, :] into
 // the row's shared accumulator; the columns of one P row differ, so no two
 // lanes meet on a slot and every value is summed in the same order on every
-// run.
+// run.  Also writes P2 = P - wd (A P), the prolongation followed by the
+// degree-1 smoother's step, in the pattern of A P (wd: nullptr = not wanted).
 constexpr int kApLanes = 8;
 template <int NV>
-__global__ void k_ap(SellDev A, SellDev P, const int64_t* ap_ptr, const int64_t* ap_sptr, const uint16_t* ap_slot,
-                     int64_t ap_nnz, int ap_maxlen, const double* v0, const double* v1, const double* p0,
-                     const double* p1, double* ap) {
+__global__ void k_ap(SellDev A, SellDev P, const int32_t* diag, const int64_t* ap_ptr, const int64_t* ap_sptr,
+                     const uint16_t* ap_slot, int64_t ap_nnz, int ap_maxlen, const double* v0, const double* v1,
+                     const double* p0, const double* p1, const double* wd, double* ap, double* p2) {
     extern __shared__ double acc_all[];
     const int grp = threadIdx.x / kApLanes, sub = threadIdx.x % kApLanes;
     const int64_t task = blockIdx.x * int64_t(blockDim.x / kApLanes) + grp;
@@ -136,12 +204,11 @@ __global__ void k_ap(SellDev A, SellDev P, const int64_t* ap_ptr, const int64_t*
     double* acc = acc_all + int64_t(grp) * ap_maxlen;
     const double* val = v == 0 ? v0 : v1;
     const double* pv = v == 0 ? p0 : p1;
-    double* out = ap + v * ap_nnz;
     const int64_t b = valid ? ap_ptr[i] : 0, cnt = valid ? ap_ptr[i + 1] - b : 0;
     for (int64_t t = sub; t < cnt; t += kApLanes) acc[t] = 0.0;
     __syncwarp();
-    int64_t o = valid ? ap_sptr[i] : 0;
-    const int L = valid ? A.len[i] : 0;
+    int64_t o = valid ? ap_sptr[i] : 0, own = 0;
+    const int L = valid ? A.len[i] : 0, dk = valid ? diag[i] : 0;
     // the longest row of the warp sets the step count, so that every lane reaches each __syncwarp
     int Lw = L;
 #pragma unroll
@@ -152,12 +219,24 @@ __global__ void k_ap(SellDev A, SellDev P, const int64_t* ap_ptr, const int64_t*
             const int64_t j = A.col[at];
             const double a = val[at];
             const int LPj = P.len[j];
+            if (k == dk) own = o;
             for (int kk = sub; kk < LPj; kk += kApLanes) acc[ap_slot[o + kk]] += a * pv[spos(P, j, kk)];
             o += LPj;
         }
         __syncwarp();
     }
-    for (int64_t t = sub; t < cnt; t += kApLanes) out[b + t] = acc[t];
+    double* out = ap + v * ap_nnz + b;
+    for (int64_t t = sub; t < cnt; t += kApLanes) out[t] = acc[t];
+    if (wd) {
+        const double w = valid ? wd[i * NV + v] : 0.0;
+        for (int64_t t = sub; t < cnt; t += kApLanes) acc[t] *= -w;
+        __syncwarp();
+        const int LP = valid ? P.len[i] : 0;
+        for (int kk = sub; kk < LP; kk += kApLanes) acc[ap_slot[own + kk]] += pv[spos(P, i, kk)];
+        __syncwarp();
+        double* out2 = p2 + v * ap_nnz + b;
+        for (int64_t t = sub; t < cnt; t += kApLanes) out2[t] = acc[t];
+    }
 }
 
 // R = P^T values gathered from P (padding 0).
@@ -252,7 +331,7 @@ namespace {
 
 // ---------------------------------------------------------------- solve kernels
 
-constexpr int kRedMaxGrid = 1024;  // blocks of the reducing vector kernels
+constexpr int kRedMaxGrid = 152 * 8;  // blocks of the reducing kernels
 
 template <typename T, int R>
 __device__ __forceinline__ void ldR(const T* p, T* v) {
@@ -307,7 +386,7 @@ __device__ __forceinline__ void row_apply(const SellDev& A, const T* v0, const T
                                           bool valid, T* acc) {
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = T(0);
-    const int L = valid ? A.len[i] : 0;
+    const int L = valid ? row_len(A, i) : 0;
     const int64_t base = !valid ? 0 : A.rowmajor ? A.ptr[i] : A.ptr[i >> 5] * 32 + (i & 31);
     const int64_t stride = A.rowmajor ? 1 : 32;
     for (int k = sub; k < L; k += G) {
@@ -352,7 +431,7 @@ __global__ void __launch_bounds__(256) k_spmv(SellDev A, const T* v0, const T* v
     stR<T, R>(y + i * R, acc);
 }
 
-// Chebyshev smoothing step k (of a polynomial in D^-1 A on [hi / ratio, hi]):
+// Chebyshev smoothing step k (of a polynomial in D^-1 A on [hi / ratio, hi], hi with its margin):
 //   res = b - A x_in  (FIRST: x_in = 0, res = b),
 //   d = c_d d + c_r D^-1 res,  x_out = x_in + d,
 // with the coefficients of the three-term recurrence (Saad, Iterative
@@ -374,7 +453,7 @@ __global__ void __launch_bounds__(256) k_cheb(SellDev A, const T* v0, const T* v
     T cd[NV], cr[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        const double h = hi[v], lo = h / ratio;
+        const double h = kSmoothMargin * hi[v], lo = h / ratio;
         const double theta = 0.5 * (h + lo), delta = 0.5 * (h - lo), sigma = theta / delta;
         double rho_prev = 1.0 / sigma, rho = rho_prev;
         for (int j = 1; j <= k; ++j) {
@@ -413,7 +492,7 @@ __global__ void __launch_bounds__(256) k_cheb(SellDev A, const T* v0, const T* v
 // x = A^-1 b on the coarsest level (dense inverse, n <= kAmgCoarsest).
 template <typename T, int R, int NV>
 __global__ void k_dense_apply(int n, const T* inv, const T* b, T* x) {
-    for (int t = threadIdx.x; t < n * R; t += blockDim.x) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * R; t += gridDim.x * blockDim.x) {
         const int i = t / R, r = t % R;
         const T* row = inv + int64_t(NV == 2 ? r : 0) * n * n + int64_t(i) * n;
         T s = T(0);
@@ -448,9 +527,162 @@ __device__ __forceinline__ void block_partials(double* v, double* part) {
 
 // Total of quantity q over G block partials (a full warp calls it; every lane gets it).
 __device__ __forceinline__ double total_of(const double* part, int G, int Q, int q) {
-    double s = 0.0;
-    for (int g = threadIdx.x & 31; g < G; g += 32) s += part[int64_t(g) * Q + q];
-    return warp_sum(s);
+    double s[4] = {0.0, 0.0, 0.0, 0.0};  // four loads in flight
+    const int lane = threadIdx.x & 31;
+    for (int g = lane; g < G; g += 128)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (g + 32 * u < G) s[u] += __ldcg(part + int64_t(g + 32 * u) * Q + q);
+    return warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+}
+
+// Grid totals of the block partials by the block that finishes last (the
+// counter wraps back to 0): true in that block only, tot[q] then holds the
+// totals, summed in the same order whichever block it is.
+template <int Q>
+__device__ __forceinline__ bool last_block_totals(const double* part, unsigned* count, double* tot) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(count, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    for (int q = threadIdx.x >> 5; q < Q; q += int(blockDim.x >> 5)) {
+        const double t = total_of(part, gridDim.x, Q, q);
+        if ((threadIdx.x & 31) == 0) tot[q] = t;
+    }
+    __syncthreads();
+    return true;
+}
+
+// ---- rows with several lanes: lanes x C right-hand sides (16-byte accesses) x G groups that share a row's entries
+// (G may span the warps of a block).  The group's sums are combined by an xor tree, then over the warps in order.
+template <typename T, int R>
+constexpr int kLaneRhs = R == 1 ? 1 : sizeof(T) == 8 ? 2 : R % 4 == 0 ? 4 : 2;
+
+template <typename T, int R, int NV>
+__device__ __forceinline__ void row_part(const SellDev& A, const T* v0, const T* v1, const T* x, int64_t i, int c0, int g,
+                                         int G, bool valid, T* acc) {
+    constexpr int C = kLaneRhs<T, R>, U = 4;  // U entries in flight
+#pragma unroll
+    for (int r = 0; r < C; ++r) acc[r] = T(0);
+    const int L = valid ? row_len(A, i) : 0;
+    const int64_t base = !valid ? 0 : A.rowmajor ? A.ptr[i] : A.ptr[i >> 5] * 32 + (i & 31);
+    const int64_t stride = A.rowmajor ? 1 : 32;
+    for (int k0 = g; k0 < L; k0 += U * G) {
+        T a0[U], a1[U], xv[U][C];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int k = k0 + u * G;
+            const int64_t at = base + int64_t(k < L ? k : k0) * stride;
+            a0[u] = k < L ? __ldg(v0 + at) : T(0);
+            if (NV == 2) a1[u] = k < L ? __ldg(v1 + at) : T(0);
+            ldR<T, C>(x + int64_t(__ldg(A.col + at)) * R + c0, xv[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k0 + u * G >= L) break;
+            if constexpr (NV == 1) {
+#pragma unroll
+                for (int r = 0; r < C; ++r) acc[r] = fma(a0[u], xv[u][r], acc[r]);
+            } else {
+                acc[0] = fma(a0[u], xv[u][0], acc[0]);
+                acc[1] = fma(a1[u], xv[u][1], acc[1]);
+            }
+        }
+    }
+}
+
+// Threads of a block over rows: LPR lanes of one row's right-hand sides, GW
+// entry groups in a warp, W warps per row.  rows() per block.
+template <typename T, int R, int GW, int W>
+struct RowMap {
+    static constexpr int C = kLaneRhs<T, R>, LPR = R / C, PER = LPR * GW, RPB = W > 1 ? 8 / W : 256 / PER;
+    static_assert(PER <= 32 && (W == 1 || PER == 32), "a row's lanes fill whole warps when it spans several");
+    int lane, warp, c0, g, slot;  // slot: row within the block
+    __device__ RowMap() {
+        lane = threadIdx.x & 31;
+        warp = threadIdx.x >> 5;
+        c0 = (lane % LPR) * C;
+        g = (lane % PER) / LPR + (W > 1 ? (warp % W) * GW : 0);
+        slot = W > 1 ? warp / W : threadIdx.x / PER;
+    }
+    // sums the groups of the row; valid in lanes with g == 0
+    __device__ void combine(T* acc) const {
+        if constexpr (GW > 1) {
+#pragma unroll
+            for (int r = 0; r < C; ++r)
+#pragma unroll
+                for (int o = PER / 2; o >= LPR; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+        }
+        if constexpr (W > 1) {
+            __shared__ T part[8][R];
+            if (lane < LPR)
+#pragma unroll
+                for (int r = 0; r < C; ++r) part[warp][c0 + r] = acc[r];
+            __syncthreads();
+            if (g == 0)
+                for (int w = 1; w < W; ++w)
+#pragma unroll
+                    for (int r = 0; r < C; ++r) acc[r] += part[warp + w][c0 + r];
+            __syncthreads();
+        }
+    }
+    // block totals of NQ quantities per right-hand side (acc[q * C + r] in the lanes with g == 0; 0 elsewhere)
+    template <int NQ>
+    __device__ void block_totals(const double* acc, double* part) const {
+        __shared__ double red[8][NQ * R];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int r = 0; r < C; ++r) {
+                double v = acc[q * C + r];
+#pragma unroll
+                for (int o = 16; o >= LPR; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane < LPR) red[warp][q * R + c0 + r] = v;
+            }
+        __syncthreads();
+        if (threadIdx.x < NQ * R) {
+            double t = 0.0;
+            for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+            part[int64_t(blockIdx.x) * NQ * R + threadIdx.x] = t;
+        }
+    }
+};
+
+// Degree-1 cycle on one level (b the level's right-hand side, wd the weighted inverse diagonal, see k_weights):
+//   MODE 0: y = b - (A diag(wd)) b           (residual after the pre-smoothing step from zero)
+//   MODE 1: y = R x                          (restriction)
+//   MODE 2: y = P2 e + wd (b + res)          (prolongation, correction and post-smoothing step: with x = wd b + P e,
+//                                             x + wd (b - A x) = wd (b + res) + (P - wd A P) e)
+// Three kernels a level; the smoothed iterate itself is never stored.  FP64: bound by FP64 issue (A, P and P2 rows
+// hold 7, 4 and 10 entries on a Kuhn mesh, 21 multiply-adds a node and right-hand side).
+template <typename T, int R, int NV, int MODE, int GW, int W>
+__global__ void __launch_bounds__(256) k_level(SellDev A, const T* __restrict__ v0, const T* __restrict__ v1,
+                                               const T* __restrict__ x, const T* __restrict__ wd,
+                                               const T* __restrict__ b, const T* __restrict__ res, T* __restrict__ y) {
+    const RowMap<T, R, GW, W> m;
+    constexpr int C = RowMap<T, R, GW, W>::C;
+    const int64_t i = blockIdx.x * int64_t(m.RPB) + m.slot;
+    T acc[C];
+    row_part<T, R, NV>(A, v0, v1, x, i, m.c0, m.g, GW * W, i < A.n, acc);
+    m.combine(acc);
+    if (i >= A.n || m.g != 0) return;
+    const int64_t o = i * R + m.c0;
+    if constexpr (MODE == 0) {
+        T bv[C];
+        ldR<T, C>(b + o, bv);
+#pragma unroll
+        for (int r = 0; r < C; ++r) acc[r] = bv[r] - acc[r];
+    } else if constexpr (MODE == 2) {
+        T bv[C], rv[C];
+        ldR<T, C>(b + o, bv);
+        ldR<T, C>(res + o, rv);
+#pragma unroll
+        for (int r = 0; r < C; ++r) acc[r] = fma(wd[i * NV + (NV == 2 ? m.c0 + r : 0)], bv[r] + rv[r], acc[r]);
+    }
+    stR<T, C>(y + o, acc);
 }
 
 // ---- conjugate gradients (FP64), R right-hand sides; ctl[0] status, ctl[1] RHS still running
@@ -524,31 +756,36 @@ __global__ void k_cg_start(const double* part, int G, double* bb, int* ctl) {
     }
 }
 
-// q = A p and partials of p.q
-template <int R, int NV>
-__global__ void __launch_bounds__(256) k_cg_apply(SellDev A, const double* v0, const double* v1, const double* p,
-                                                  double* q, double* part) {
-    double acc[R];
+// q = A p, p.q; the last block forms alpha = r.z / p.q on the running right-hand sides (0 on the others)
+template <int R, int NV, int GW>
+__global__ void __launch_bounds__(256) k_cg_apply(SellDev A, const double* __restrict__ v0, const double* __restrict__ v1,
+                                                  const double* __restrict__ p, double* __restrict__ q, double* part,
+                                                  unsigned* count, const double* rz, double* alpha, int* ctl) {
+    const RowMap<double, R, GW, 1> m;
+    constexpr int C = RowMap<double, R, GW, 1>::C;
+    __shared__ double tot[R];
+    double dot[C];
 #pragma unroll
-    for (int t = 0; t < R; ++t) acc[t] = 0.0;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < A.n; i += int64_t(gridDim.x) * blockDim.x) {
-        double qv[R], pv[R];
-        row_apply<double, R, NV, 1>(A, v0, v1, p, i, 0, true, qv);
-        ldR<double, R>(p + i * R, pv);
+    for (int r = 0; r < C; ++r) dot[r] = 0.0;
+    for (int64_t i0 = int64_t(blockIdx.x) * m.RPB; i0 < A.n; i0 += int64_t(gridDim.x) * m.RPB) {
+        const int64_t i = i0 + m.slot;
+        double acc[C];
+        row_part<double, R, NV>(A, v0, v1, p, i, m.c0, m.g, GW, i < A.n, acc);
+        m.combine(acc);
+        if (i < A.n && m.g == 0) {
+            double pv[C];
+            ldR<double, C>(p + i * R + m.c0, pv);
 #pragma unroll
-        for (int t = 0; t < R; ++t) acc[t] = fma(pv[t], qv[t], acc[t]);
-        stR<double, R>(q + i * R, qv);
+            for (int r = 0; r < C; ++r) dot[r] = fma(pv[r], acc[r], dot[r]);
+            stR<double, C>(q + i * R + m.c0, acc);
+        }
     }
-    block_partials<R>(acc, part);
-}
-
-// alpha = r.z / p.q on the running right-hand sides (0 on the others)
-template <int R>
-__global__ void k_cg_alpha(const double* part, int G, const double* rz, double* alpha, int* ctl) {
-    const int* active = ctl + kCtlActive;
-    const int r = threadIdx.x >> 5;
-    const double pq = total_of(part, G, R, r);
-    if ((threadIdx.x & 31) == 0) {
+    m.template block_totals<1>(dot, part);
+    if (!last_block_totals<R>(part, count, tot)) return;
+    if (threadIdx.x < R) {
+        const int* active = ctl + kCtlActive;
+        const int r = threadIdx.x;
+        const double pq = tot[r];
         double a = 0.0;
         if (active[r]) {
             if (!(pq > 0.0) || !isfinite(pq) || !isfinite(rz[r]))
@@ -560,75 +797,149 @@ __global__ void k_cg_alpha(const double* part, int G, const double* rz, double* 
     }
 }
 
-// x += alpha p, r -= alpha q, partials of r.r
-// The vector passes of the CG give each node's R values to R / C threads
-// of C right-hand sides each (C = 8 for R = 16): fewer live registers per
-// thread, more loads in flight for these memory-bound passes.
-template <int R>
-constexpr int kChunk = R > 8 ? 8 : R;
-
-// Block totals of per-thread partials over C right-hand sides when thread t
-// holds chunk t % (R / C): an xor tree over the lanes of the same chunk,
-// then the warps in order; part[blockIdx * R * NQ + q * R + r] for the NQ
-// quantities of acc (acc[q * C + j] belongs to right-hand side chunk * C + j).
-template <int R, int NQ>
-__device__ __forceinline__ void chunk_partials(const double* acc, double* part) {
-    constexpr int C = kChunk<R>, NCH = R / C;
-    __shared__ double red[8][NQ * R];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q)
-#pragma unroll
-        for (int j = 0; j < C; ++j) {
-            double v = acc[q * C + j];
-#pragma unroll
-            for (int o = 16; o >= NCH; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane < NCH) red[warp][q * R + lane * C + j] = v;
-        }
+// beta = r.z / (r.z)_old from the totals of r.z; FLEX: z.(r - r_old) / (r.z)_old with r - r_old = -alpha q (the form
+// that tolerates a preconditioner that varies slightly between applications), tot[R ..] = q.z.  0 before the first
+// direction (ctl[3], cleared here).  rz <- r.z.  By the threads of one block.
+template <int R, bool FLEX>
+__device__ __forceinline__ void cg_beta(const double* tot, double* rz, const double* alpha, double* beta, int* ctl) {
+    const int first = ctl[3];
+    if (threadIdx.x < R) {
+        const int* active = ctl + kCtlActive;
+        const int r = threadIdx.x;
+        const double t = tot[r];
+        double b = 0.0;
+        if (!first && active[r]) b = (FLEX ? -alpha[r] * tot[R + r] : t) / rz[r];
+        if (active[r] && (!isfinite(t) || !(t > 0.0))) atomicExch(ctl, int(QPAT_EBREAKDOWN));
+        beta[r] = b;
+        rz[r] = t;
+    }
     __syncthreads();
-    if (threadIdx.x < NQ * R) {
-        double t = 0.0;
-        for (int w = 0; w < int(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
-        part[int64_t(blockIdx.x) * NQ * R + threadIdx.x] = t;
+    if (threadIdx.x == 0) ctl[3] = 0;
+}
+
+// The fine level's MODE 2 of k_level with z in FP64, the dots r.z (FLEX, the FP32 cycle: and q.z) and, in the last
+// block, beta.
+template <typename T, int R, int NV, int GW>
+__global__ void __launch_bounds__(256) k_top(SellDev P2, const T* __restrict__ v0, const T* __restrict__ v1,
+                                             const T* __restrict__ e, const T* __restrict__ wd, const T* __restrict__ b,
+                                             const T* __restrict__ res, const double* __restrict__ rr,
+                                             const double* __restrict__ q, double* __restrict__ z, double* part,
+                                             unsigned* count, double* rz, const double* alpha, double* beta, int* ctl) {
+    constexpr bool FLEX = !std::is_same<T, double>::value;
+    constexpr int NQ = FLEX ? 2 : 1;
+    const RowMap<T, R, GW, 1> m;
+    constexpr int C = RowMap<T, R, GW, 1>::C;
+    __shared__ double tot[NQ * R];
+    double dot[NQ * C];
+#pragma unroll
+    for (int r = 0; r < NQ * C; ++r) dot[r] = 0.0;
+    for (int64_t i0 = int64_t(blockIdx.x) * m.RPB; i0 < P2.n; i0 += int64_t(gridDim.x) * m.RPB) {
+        const int64_t i = i0 + m.slot;
+        T acc[C];
+        row_part<T, R, NV>(P2, v0, v1, e, i, m.c0, m.g, GW, i < P2.n, acc);
+        m.combine(acc);
+        if (i < P2.n && m.g == 0) {
+            const int64_t o = i * R + m.c0;
+            T bv[C], rv[C];
+            ldR<T, C>(b + o, bv);
+            ldR<T, C>(res + o, rv);
+            double zv[C], rd[C];
+#pragma unroll
+            for (int r = 0; r < C; ++r) {
+                zv[r] = double(fma(wd[i * NV + (NV == 2 ? m.c0 + r : 0)], bv[r] + rv[r], acc[r]));
+                if constexpr (!FLEX) rd[r] = bv[r];
+            }
+            if constexpr (FLEX) ldR<double, C>(rr + o, rd);
+#pragma unroll
+            for (int r = 0; r < C; ++r) dot[r] = fma(rd[r], zv[r], dot[r]);
+            if constexpr (FLEX) {
+                ldR<double, C>(q + o, rd);
+#pragma unroll
+                for (int r = 0; r < C; ++r) dot[C + r] = fma(rd[r], zv[r], dot[C + r]);
+            }
+            stR<double, C>(z + o, zv);
+        }
+    }
+    m.template block_totals<NQ>(dot, part);
+    if (last_block_totals<NQ * R>(part, count, tot)) cg_beta<R, FLEX>(tot, rz, alpha, beta, ctl);
+}
+
+// The vector passes: thread per two right-hand sides of a node (16-byte accesses; the same right-hand sides in every
+// step of the grid).  Bound by HBM.
+template <int R>
+using FlatMap = RowMap<double, R, 1, 1>;
+#define FOR_FLAT(n, R)                                                                                  \
+    for (int64_t o = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) * C; o < (n) * (R);               \
+         o += int64_t(gridDim.x) * blockDim.x * C)
+
+// r.z (FLEX: and q.z) and, in the last block, beta, where no fused kernel has formed them
+template <int R, bool FLEX>
+__global__ void __launch_bounds__(256) k_cg_dots(int64_t n, const double* __restrict__ r, const double* __restrict__ z,
+                                                 const double* __restrict__ qv, double* part, unsigned* count, double* rz,
+                                                 const double* alpha, double* beta, int* ctl) {
+    constexpr int C = FlatMap<R>::C, NQ = FLEX ? 2 : 1;
+    const FlatMap<R> m;
+    __shared__ double tot[NQ * R];
+    double dot[NQ * C];
+#pragma unroll
+    for (int t = 0; t < NQ * C; ++t) dot[t] = 0.0;
+    FOR_FLAT(n, R) {
+        double a[C], zv[C];
+        ldR<double, C>(r + o, a);
+        ldR<double, C>(z + o, zv);
+#pragma unroll
+        for (int t = 0; t < C; ++t) dot[t] = fma(a[t], zv[t], dot[t]);
+        if constexpr (FLEX) {
+            ldR<double, C>(qv + o, a);
+#pragma unroll
+            for (int t = 0; t < C; ++t) dot[C + t] = fma(a[t], zv[t], dot[C + t]);
+        }
+    }
+    m.template block_totals<NQ>(dot, part);
+    if (last_block_totals<NQ * R>(part, count, tot)) cg_beta<R, FLEX>(tot, rz, alpha, beta, ctl);
+}
+
+// p = z + beta p
+template <int R>
+__global__ void __launch_bounds__(256) k_cg_dir(int64_t n, const double* beta, const double* __restrict__ z,
+                                                double* __restrict__ p) {
+    constexpr int C = FlatMap<R>::C;
+    const FlatMap<R> m;
+    double be[C];
+#pragma unroll
+    for (int t = 0; t < C; ++t) be[t] = beta[m.c0 + t];
+    FOR_FLAT(n, R) {
+        double zv[C], pv[C];
+        ldR<double, C>(z + o, zv);
+        ldR<double, C>(p + o, pv);
+#pragma unroll
+        for (int t = 0; t < C; ++t) pv[t] = fma(be[t], pv[t], zv[t]);
+        stR<double, C>(p + o, pv);
     }
 }
 
-// The next cycle's first fine-level smoothing step (from x = 0: x = d =
-// c_r D^-1 b with b = r, c_r = 1 / theta as in k_cheb), taken in the CG
-// update on the residual it has just written instead of by a separate pass
-// over r; for the FP32 cycle also the FP32 copy of r.  The same operations
-// in the same order as k_cheb's first step, so the results do not change.
-template <typename T, int NV>
-struct PreStep {
-    const T* dinv = nullptr;      // fine level, n x NV
-    const double* hi = nullptr;   // Gershgorin bounds of the fine level, per value set
-    double ratio = 30.0;
-    T* x = nullptr;               // the cycle's first fine-level buffer (x = d after the step)
-    T* d = nullptr;               // null when no later pre-smoothing step reads d (degree 1)
-    float* b32 = nullptr;         // FP32 cycle: the fine level's right-hand side
-};
-
-template <int R, int NV, typename T>
-__global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alpha, const double* p, const double* q,
-                                                   double* x, double* r, double* part, PreStep<T, NV> pre) {
-    constexpr int C = kChunk<R>, NCH = R / C;
-    const int c0 = int(threadIdx.x % NCH) * C;
-    double al[C], acc[C];
+// x += alpha p, r -= alpha q (b32: and the FP32 copy of r), r.r.  The last
+// block checks: a right-hand side stops once |r| <= rtol |b|; one more
+// iteration is done.  Inside a graph (use_graph) it also sets the loop's
+// condition: go on while some right-hand side runs, the status is clean and
+// the cap is not reached (reaching it with a running right-hand side is
+// QPAT_ENOCONV).
+template <int R>
+__global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alpha, const double* __restrict__ p,
+                                                   const double* __restrict__ q, double* __restrict__ x,
+                                                   double* __restrict__ r, float* __restrict__ b32, double* part,
+                                                   unsigned* count, const double* bb, const double* rtol2, double* rr,
+                                                   int* ctl, cudaGraphConditionalHandle cond, int use_graph) {
+    constexpr int C = FlatMap<R>::C;
+    const FlatMap<R> m;
+    __shared__ double tot[R];
+    double al[C], dot[C];
 #pragma unroll
     for (int t = 0; t < C; ++t) {
-        al[t] = alpha[c0 + t];
-        acc[t] = 0.0;
+        al[t] = alpha[m.c0 + t];
+        dot[t] = 0.0;
     }
-    T cr[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const double h = pre.hi[v], lo = h / pre.ratio;
-        cr[v] = T(1.0 / (0.5 * (h + lo)));
-    }
-    for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < n * NCH;
-         g += int64_t(gridDim.x) * blockDim.x) {
-        const int64_t node = g / NCH;
-        const int64_t o = node * R + c0;
+    FOR_FLAT(n, R) {
         double pv[C], qv[C], xv[C], rv[C];
         ldR<double, C>(p + o, pv);
         ldR<double, C>(q + o, qv);
@@ -638,118 +949,31 @@ __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alph
         for (int t = 0; t < C; ++t) {
             xv[t] = fma(al[t], pv[t], xv[t]);
             rv[t] = fma(-al[t], qv[t], rv[t]);
-            acc[t] = fma(rv[t], rv[t], acc[t]);
+            dot[t] = fma(rv[t], rv[t], dot[t]);
         }
         stR<double, C>(x + o, xv);
         stR<double, C>(r + o, rv);
-        T rc[C], up[C];
+        if (b32)
 #pragma unroll
-        for (int t = 0; t < C; ++t) {
-            const int v = NV == 2 ? c0 + t : 0;
-            rc[t] = T(rv[t]);
-            const T upd = cr[v] * pre.dinv[node * NV + v] * rc[t];
-            up[t] = T(0) + upd;
-        }
-        if constexpr (std::is_same<T, float>::value) stR<float, C>(pre.b32 + o, rc);
-        if (pre.d) stR<T, C>(pre.d + o, up);
-        stR<T, C>(pre.x + o, up);
+            for (int t = 0; t < C; ++t) b32[o + t] = float(rv[t]);
     }
-    chunk_partials<R, 1>(acc, part);
-}
-
-// a right-hand side stops once |r| <= rtol |b|; one more iteration is done.
-// Inside a graph (use_graph) the kernel also sets the loop's condition: go
-// on while some right-hand side runs, the status is clean and the cap is not
-// reached (reaching it with a running right-hand side is QPAT_ENOCONV).
-template <int R>
-__global__ void k_cg_check(const double* part, int G, const double* bb, const double* rtol2, double* rr, int* ctl,
-                           cudaGraphConditionalHandle cond, int use_graph) {
+    m.template block_totals<1>(dot, part);
+    if (!last_block_totals<R>(part, count, tot)) return;
     int* active = ctl + kCtlActive;
-    const int r = threadIdx.x >> 5;
-    const double t = total_of(part, G, R, r);
-    if ((threadIdx.x & 31) == 0) {
-        rr[r] = t;
+    if (threadIdx.x < R) {
+        const double t = tot[threadIdx.x];
+        rr[threadIdx.x] = t;
         if (!isfinite(t)) atomicExch(ctl, int(QPAT_EBREAKDOWN));
-        if (active[r] && t <= *rtol2 * bb[r]) active[r] = 0;
+        if (active[threadIdx.x] && t <= *rtol2 * bb[threadIdx.x]) active[threadIdx.x] = 0;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         int c = 0;
-        for (int q = 0; q < R; ++q) c += active[q];
+        for (int k = 0; k < R; ++k) c += active[k];
         ctl[1] = c;
         const int it = ++ctl[2];
         if (c > 0 && it >= ctl[4] && ctl[0] == QPAT_OK) ctl[0] = QPAT_ENOCONV;
         if (use_graph) cudaGraphSetConditional(cond, (c > 0 && ctl[0] == QPAT_OK) ? 1u : 0u);
-    }
-}
-
-// partials of r.z (and, FLEX, of r.z_old)
-template <int R, bool FLEX>
-__global__ void __launch_bounds__(256) k_cg_dots(int64_t n, const double* r, const double* z, const double* zo,
-                                                 double* part) {
-    constexpr int C = kChunk<R>, NCH = R / C, NQ = FLEX ? 2 : 1;
-    const int c0 = int(threadIdx.x % NCH) * C;
-    double acc[NQ * C];
-#pragma unroll
-    for (int t = 0; t < NQ * C; ++t) acc[t] = 0.0;
-    for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < n * NCH;
-         g += int64_t(gridDim.x) * blockDim.x) {
-        const int64_t o = (g / NCH) * R + c0;
-        double rv[C], zv[C];
-        ldR<double, C>(r + o, rv);
-        ldR<double, C>(z + o, zv);
-#pragma unroll
-        for (int t = 0; t < C; ++t) acc[t] = fma(rv[t], zv[t], acc[t]);
-        if constexpr (FLEX) {
-            ldR<double, C>(zo + o, zv);
-#pragma unroll
-            for (int t = 0; t < C; ++t) acc[C + t] = fma(rv[t], zv[t], acc[C + t]);
-        }
-    }
-    chunk_partials<R, NQ>(acc, part);
-}
-
-// beta = r.z / (r.z)_old (FLEX: (r.z - r.z_old) / (r.z)_old, the form that
-// tolerates a preconditioner that varies slightly between applications);
-// 0 before the first direction (ctl[3], cleared here).  rz <- r.z.
-template <int R, bool FLEX>
-__global__ void k_cg_beta(const double* part, int G, double* rz, double* beta, int* ctl) {
-    constexpr int Q = FLEX ? 2 * R : R;
-    const int* active = ctl + kCtlActive;
-    const int first = ctl[3];
-    const int r = threadIdx.x >> 5;
-    const double t = total_of(part, G, Q, r);
-    const double to = FLEX ? total_of(part, G, Q, R + r) : 0.0;
-    if ((threadIdx.x & 31) == 0) {
-        double b = 0.0;
-        if (!first && active[r]) b = (t - to) / rz[r];
-        if (active[r] && (!isfinite(t) || !(t > 0.0))) atomicExch(ctl, int(QPAT_EBREAKDOWN));
-        beta[r] = b;
-        rz[r] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) ctl[3] = 0;
-}
-
-// p = z + beta p (FLEX: and z_old = z for the next beta)
-template <int R, bool FLEX>
-__global__ void __launch_bounds__(256) k_cg_dir(int64_t n, const double* beta, const double* z, double* p,
-                                                double* zo) {
-    constexpr int C = kChunk<R>, NCH = R / C;
-    const int c0 = int(threadIdx.x % NCH) * C;
-    double be[C];
-#pragma unroll
-    for (int t = 0; t < C; ++t) be[t] = beta[c0 + t];
-    for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < n * NCH;
-         g += int64_t(gridDim.x) * blockDim.x) {
-        const int64_t o = (g / NCH) * R + c0;
-        double zv[C], pv[C];
-        ldR<double, C>(z + o, zv);
-        ldR<double, C>(p + o, pv);
-#pragma unroll
-        for (int t = 0; t < C; ++t) pv[t] = fma(be[t], pv[t], zv[t]);
-        stR<double, C>(p + o, pv);
-        if constexpr (FLEX) stR<double, C>(zo + o, zv);
     }
 }
 
@@ -768,8 +992,10 @@ __global__ void k_f2d_vec(int64_t n, const float* in, double* out) {
 
 struct AmgHierDev {
     bool tried = false;
+    bool used[2] = {false, false};  // a K (M_delta) solve has run on it
     std::string error;
     std::vector<LevelDev> lv;
+    SellDev K;                      // the full pattern of K (the products of its CG)
     std::vector<void*> allocs;
 };
 
@@ -777,12 +1003,14 @@ struct AmgValues {
     uint64_t stamp = 0;
     bool valid = false;
     bool has32 = false;
-    std::vector<std::array<double*, 2>> A, P, R;  // A[0] unused (the operator's own values)
-    std::vector<double*> AP, dinv;
+    double ratio = 0.0;     // mg_ratio of S, wd and P2
+    std::vector<std::array<double*, 2>> A, P, R;  // A[0]: K taken into the fine pattern (M_delta: its own values)
+    std::vector<std::array<double*, 2>> S, P2;    // degree-1 cycle: A diag(wd), P - wd A P
+    std::vector<double*> AP, dinv, wd;
     double* hi = nullptr;   // 2 per level
     double* inv = nullptr;  // coarsest inverse, NV x n x n
-    std::vector<std::array<float*, 2>> A32, P32, R32;  // A32[0]: FP32 copy of the operator
-    std::vector<float*> dinv32;
+    std::vector<std::array<float*, 2>> A32, P32, R32, S32, P232;
+    std::vector<float*> dinv32, wd32;
     float* inv32 = nullptr;
     std::vector<void*> allocs;
 };
@@ -793,9 +1021,10 @@ struct AmgVecs {
 };
 
 struct AmgCg {
-    double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *zo = nullptr, *part = nullptr;
+    double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *part = nullptr;
     double *bb = nullptr, *rz = nullptr, *alpha = nullptr, *beta = nullptr, *rr = nullptr, *rtol2 = nullptr;
     int* ctl = nullptr;  // control words (see k_cg_start)
+    unsigned* count = nullptr;  // blocks that have finished (see last_block_totals)
     std::vector<void*> allocs;
 };
 
@@ -809,9 +1038,9 @@ struct AmgGraph {
 };
 
 struct AmgState {
-    AmgHierDev hier[2];  // 0: the K pattern, 1: the prior's stiffness-only pattern
+    AmgHierDev hier;     // on the prior's pattern, for K and M_delta
     std::map<const void*, AmgValues> vals;
-    std::map<std::pair<int, int>, AmgVecs> vecs;  // (pattern * 64 + R, FP32 V-cycle)
+    std::map<std::pair<int, int>, AmgVecs> vecs;  // (R, FP32 V-cycle)
     std::map<int, AmgCg> cg;                       // R
     std::map<std::string, AmgGraph> graphs;
     cudaStream_t capture = nullptr;                // a non-default stream to capture on
@@ -848,11 +1077,24 @@ SellDev upload_sell(std::vector<void*>& list, const SellPattern& S, cudaError_t&
     return d;
 }
 
+// Grid of a kernel that strides over its work: every resident block of the
+// device (a grid between one and two waves would leave half of it idle at the
+// end), at most `most`.
+template <typename K>
+int full_grid(K kernel, int most) {
+    int dev = 0, nsm = 0, per = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 256, 0) != cudaSuccess || nsm * per < 1)
+        return most;
+    return std::min(most, nsm * per);
+}
+
 inline int blocks_of(int64_t n, int per = 256) { return int(std::max<int64_t>(1, (n + per - 1) / per)); }
 
-int build_hier(qpat_mesh_s* M, int prior, AmgHierDev& H) {
+int build_hier(qpat_mesh_s* M, AmgHierDev& H) {
     H.tried = true;
-    const AmgPlan plan = amg_build_plan(amg_fine_pattern(M->h, prior));
+    const SellPattern fine = amg_fine_pattern(M->h);
+    const AmgPlan plan = amg_build_plan(fine, amg_fine_graph(M->h, fine));
     if (!plan.error.empty()) {
         H.error = plan.error;
         return fail(QPAT_EINVAL, plan.error);
@@ -881,6 +1123,13 @@ int build_hier(qpat_mesh_s* M, int prior, AmgHierDev& H) {
         }
         H.lv.push_back(d);
     }
+    const std::vector<uint16_t> len(M->h.sell_len.begin(), M->h.sell_len.end());
+    H.K.n = M->h.N;
+    H.K.ptr = M->d.sell_ptr;
+    H.K.col = M->el.ent_col;
+    H.K.len = upload(H.allocs, len, e);
+    H.K.entries = M->d.sell_entries;
+    H.K.maxlen = M->d.sell_wmax;
     if (e != cudaSuccess) {
         H.error = std::string("multigrid upload: ") + cudaGetErrorString(e);
         return cuda_fail(e, "multigrid upload");
@@ -889,22 +1138,33 @@ int build_hier(qpat_mesh_s* M, int prior, AmgHierDev& H) {
 }
 
 template <int NV>
-cudaError_t numeric_levels(const AmgHierDev& H, const OpState& st, AmgValues& V, cudaStream_t s) {
+cudaError_t numeric_levels(const qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V, bool fast,
+                           double ratio, cudaStream_t s) {
     const int L = int(H.lv.size());
     cudaError_t e = cudaMemsetAsync(V.hi, 0, sizeof(double) * 2 * L, s);
     if (e != cudaSuccess) return e;
+    if (NV == 1) {
+        note_launch(1);
+        k_lump<<<blocks_of(H.K.n), 256, 0, s>>>(H.K, M->el.ent_edge, M->el.in_prior, H.lv[0].A, H.lv[0].diag, st.v64[0],
+                                                V.A[0][0]);
+    }
     for (int l = 0; l < L; ++l) {
         const LevelDev& d = H.lv[size_t(l)];
-        const double* a0 = l == 0 ? st.v64[0] : V.A[size_t(l)][0];
-        const double* a1 = l == 0 ? st.v64[1] : V.A[size_t(l)][1];
+                const double *a0 = V.A[size_t(l)][0], *a1 = V.A[size_t(l)][1];
+        double* hi = V.hi + 2 * l;
         note_launch(1);
-        k_dinv_hi<NV><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, d.diag, a0, a1, V.dinv[size_t(l)], V.hi + 2 * l);
+        k_dinv_hi<NV><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, d.diag, a0, a1, V.dinv[size_t(l)], hi);
         if (l + 1 == L) break;
         const auto& Pv = V.P[size_t(l)];
         const auto& Rv = V.R[size_t(l)];
+        if (fast) {
+            note_launch(2);
+            k_weights<NV><<<blocks_of(d.A.n * NV), 256, 0, s>>>(d.A.n, V.dinv[size_t(l)], hi, ratio, V.wd[size_t(l)]);
+            k_scaled<NV><<<blocks_of(d.A.entries), 256, 0, s>>>(d.A.entries, d.A.col, V.wd[size_t(l)], a0, a1,
+                                                                V.S[size_t(l)][0], V.S[size_t(l)][1]);
+        }
         note_launch(4);
-        k_prolong<NV><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, d.P, d.a2p, d.pself, a0, a1, V.dinv[size_t(l)],
-                                                        V.hi + 2 * l, Pv[0], Pv[1]);
+        k_prolong<NV><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, d.P, d.diag, d.a2p, d.pself, a0, a1, Pv[0], Pv[1]);
         k_rvals<NV><<<blocks_of(d.R.entries), 256, 0, s>>>(d.R.entries, d.r_src, Pv[0], Pv[1], Rv[0], Rv[1]);
         {
             int wpb = 8;  // warps per block, kApLanes lanes per row
@@ -913,8 +1173,8 @@ cudaError_t numeric_levels(const AmgHierDev& H, const OpState& st, AmgValues& V,
             const size_t smem = size_t(wpb * rpw) * size_t(d.ap_maxlen) * sizeof(double);
             if ((e = allow_smem(reinterpret_cast<const void*>(&k_ap<NV>), smem)) != cudaSuccess) return e;
             k_ap<NV><<<blocks_of(d.A.n * NV, wpb * rpw), 32 * wpb, smem, s>>>(
-                d.A, d.P, d.ap_ptr, d.ap_sptr, d.ap_slot, d.ap_nnz, d.ap_maxlen, a0, a1, Pv[0], Pv[1],
-                V.AP[size_t(l)]);
+                d.A, d.P, d.diag, d.ap_ptr, d.ap_sptr, d.ap_slot, d.ap_nnz, d.ap_maxlen, a0, a1, Pv[0], Pv[1],
+                fast ? V.wd[size_t(l)] : nullptr, V.AP[size_t(l)], fast ? V.P2[size_t(l)][0] : nullptr);
         }
         const LevelDev& c = H.lv[size_t(l + 1)];
         int wpb = 8;
@@ -930,8 +1190,7 @@ cudaError_t numeric_levels(const AmgHierDev& H, const OpState& st, AmgValues& V,
     const int n = int(c.A.n);
     const size_t smem = size_t(n) * size_t(n + 1) * sizeof(double);
     if ((e = allow_smem(reinterpret_cast<const void*>(&k_dense_inv<NV>), smem)) != cudaSuccess) return e;
-    const double* a0 = L == 1 ? st.v64[0] : V.A[size_t(L - 1)][0];
-    const double* a1 = L == 1 ? st.v64[1] : V.A[size_t(L - 1)][1];
+    const double *a0 = V.A[size_t(L - 1)][0], *a1 = V.A[size_t(L - 1)][1];
     note_launch(1);
     k_dense_inv<NV><<<NV, 256, smem, s>>>(c.A, a0, a1, V.inv);
     return cudaGetLastError();
@@ -944,21 +1203,25 @@ cudaError_t cast_to_f32(const double* in, float* out, int64_t n, cudaStream_t s)
 }
 
 // Values of the hierarchy for the operator st (allocated once per operator
-// buffer, recomputed when st was prepared again).
-int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V, bool need32, cudaStream_t s) {
+// buffer, recomputed when st was prepared again or the cycle's form changed).
+// fast: the degree-1 cycle's S, wd and P2 too.
+int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V, bool fast, double ratio, bool need32,
+            cudaStream_t s) {
     const int L = int(H.lv.size());
     const int NV = st.nv;
     cudaError_t e = cudaSuccess;
+    auto set = [&](auto& list) { list.assign(size_t(L), {nullptr, nullptr}); };
     if (V.A.empty()) {
-        V.A.assign(size_t(L), {nullptr, nullptr});
-        V.P.assign(size_t(L), {nullptr, nullptr});
-        V.R.assign(size_t(L), {nullptr, nullptr});
+        set(V.A);
+        set(V.P);
+        set(V.R);
         V.AP.assign(size_t(L), nullptr);
         V.dinv.assign(size_t(L), nullptr);
         for (int l = 0; l < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
             for (int v = 0; v < NV; ++v) {
-                if (l > 0) V.A[size_t(l)][size_t(v)] = dalloc<double>(V.allocs, size_t(d.A.entries), e);
+                V.A[size_t(l)][size_t(v)] =
+                    l == 0 && NV == 2 ? st.v64[v] : dalloc<double>(V.allocs, size_t(d.A.entries), e);
                 if (l + 1 < L) {
                     V.P[size_t(l)][size_t(v)] = dalloc<double>(V.allocs, size_t(d.P.entries), e);
                     V.R[size_t(l)][size_t(v)] = dalloc<double>(V.allocs, size_t(d.R.entries), e);
@@ -971,17 +1234,35 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         const int64_t nco = H.lv.back().A.n;
         V.inv = dalloc<double>(V.allocs, size_t(NV * nco * nco), e);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
-        // P and A P padding entries are never written: keep them 0
-        for (int l = 0; l + 1 < L; ++l)
-            for (int v = 0; v < NV; ++v)
-                if ((e = cudaMemsetAsync(V.P[size_t(l)][size_t(v)], 0, sizeof(double) * H.lv[size_t(l)].P.entries, s)) !=
-                    cudaSuccess)
-                    return cuda_fail(e, "multigrid memset");
+        // padding entries are never written: keep them 0
+        for (int l = 0; l < L && e == cudaSuccess; ++l)
+            for (int v = 0; v < NV && e == cudaSuccess; ++v) {
+                const LevelDev& d = H.lv[size_t(l)];
+                if (l + 1 < L) e = cudaMemsetAsync(V.P[size_t(l)][size_t(v)], 0, sizeof(double) * d.P.entries, s);
+                if (e == cudaSuccess && !(l == 0 && NV == 2))
+                    e = cudaMemsetAsync(V.A[size_t(l)][size_t(v)], 0, sizeof(double) * d.A.entries, s);
+            }
+        if (e != cudaSuccess) return cuda_fail(e, "multigrid memset");
+    }
+    if (NV == 2) V.A[0] = {st.v64[0], st.v64[1]};
+    if (fast && V.S.empty()) {
+        set(V.S);
+        set(V.P2);
+        V.wd.assign(size_t(L), nullptr);
+        for (int l = 0; l + 1 < L; ++l) {
+            const LevelDev& d = H.lv[size_t(l)];
+            for (int v = 0; v < NV; ++v) V.S[size_t(l)][size_t(v)] = dalloc<double>(V.allocs, size_t(d.A.entries), e);
+            double* p2 = dalloc<double>(V.allocs, size_t(d.ap_nnz) * NV, e);
+            V.P2[size_t(l)] = {p2, NV == 2 ? p2 + d.ap_nnz : nullptr};
+            V.wd[size_t(l)] = dalloc<double>(V.allocs, size_t(d.A.n) * NV, e);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
+        V.valid = false;
     }
     if (need32 && !V.has32) {
-        V.A32.assign(size_t(L), {nullptr, nullptr});
-        V.P32.assign(size_t(L), {nullptr, nullptr});
-        V.R32.assign(size_t(L), {nullptr, nullptr});
+        set(V.A32);
+        set(V.P32);
+        set(V.R32);
         V.dinv32.assign(size_t(L), nullptr);
         for (int l = 0; l < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
@@ -1000,27 +1281,51 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         V.has32 = true;
         V.valid = false;
     }
-    if (V.valid && V.stamp == st.stamp) return QPAT_OK;
-    e = NV == 1 ? numeric_levels<1>(H, st, V, s) : numeric_levels<2>(H, st, V, s);
+    if (fast && V.has32 && V.S32.empty()) {
+        set(V.S32);
+        set(V.P232);
+        V.wd32.assign(size_t(L), nullptr);
+        for (int l = 0; l + 1 < L; ++l) {
+            const LevelDev& d = H.lv[size_t(l)];
+            for (int v = 0; v < NV; ++v) {
+                V.S32[size_t(l)][size_t(v)] = dalloc<float>(V.allocs, size_t(d.A.entries), e);
+                V.P232[size_t(l)][size_t(v)] = dalloc<float>(V.allocs, size_t(d.ap_nnz), e);
+            }
+            V.wd32[size_t(l)] = dalloc<float>(V.allocs, size_t(d.A.n) * NV, e);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
+        V.valid = false;
+    }
+    if (V.valid && V.stamp == st.stamp && (!fast || V.ratio == ratio)) return QPAT_OK;
+    const bool scaled = !V.S.empty();  // once allocated kept up to date
+    if (fast || V.ratio == 0.0) V.ratio = ratio;
+    e = NV == 1 ? numeric_levels<1>(M, H, st, V, scaled, V.ratio, s) : numeric_levels<2>(M, H, st, V, scaled, V.ratio, s);
     if (e != cudaSuccess) return cuda_fail(e, "multigrid set-up");
     if (V.has32) {
-        for (int l = 0; l < L && e == cudaSuccess; ++l) {
+        auto cast = [&](const double* in, float* out, int64_t n) {
+            if (e == cudaSuccess && out) e = cast_to_f32(in, out, n, s);
+        };
+        for (int l = 0; l < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
-            for (int v = 0; v < NV && e == cudaSuccess; ++v) {
-                const double* a = l == 0 ? st.v64[v] : V.A[size_t(l)][size_t(v)];
-                e = cast_to_f32(a, V.A32[size_t(l)][size_t(v)], d.A.entries, s);
-                if (e == cudaSuccess && l + 1 < L) e = cast_to_f32(V.P[size_t(l)][size_t(v)], V.P32[size_t(l)][size_t(v)], d.P.entries, s);
-                if (e == cudaSuccess && l + 1 < L) e = cast_to_f32(V.R[size_t(l)][size_t(v)], V.R32[size_t(l)][size_t(v)], d.R.entries, s);
+            for (int v = 0; v < NV; ++v) {
+                const size_t i = size_t(l), j = size_t(v);
+                cast(V.A[i][j], V.A32[i][j], d.A.entries);
+                cast(V.P[i][j], V.P32[i][j], d.P.entries);
+                cast(V.R[i][j], V.R32[i][j], d.R.entries);
+                if (!V.S32.empty()) {
+                    cast(V.S[i][j], V.S32[i][j], d.A.entries);
+                    cast(V.P2[i][j], V.P232[i][j], d.ap_nnz);
+                }
             }
-            if (e == cudaSuccess) e = cast_to_f32(V.dinv[size_t(l)], V.dinv32[size_t(l)], d.A.n * NV, s);
+            cast(V.dinv[size_t(l)], V.dinv32[size_t(l)], d.A.n * NV);
+            if (!V.wd32.empty()) cast(V.wd[size_t(l)], V.wd32[size_t(l)], d.A.n * NV);
         }
         const int64_t nco = H.lv.back().A.n;
-        if (e == cudaSuccess) e = cast_to_f32(V.inv, V.inv32, NV * nco * nco, s);
+        cast(V.inv, V.inv32, NV * nco * nco);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid set-up");
     }
     V.stamp = st.stamp;
     V.valid = true;
-    (void)M;
     return QPAT_OK;
 }
 
@@ -1028,8 +1333,8 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
 
 namespace {
 
-// Optional CUDA-event timing of the fine-level smoothing launches (the
-// multigrid cycle's dominant kernel); the events of one cycle are read after
+// Optional CUDA-event timing of the fine level's smoothing products (degree 1:
+// its residual kernel; higher degrees: the smoothing steps); the events of one cycle are read after
 // the next stream synchronisation of the CG loop.
 struct FineTimer {
     bool on = false;
@@ -1075,17 +1380,15 @@ struct VCycle {
     const AmgHierDev& H;
     const AmgValues& V;
     AmgVecs& W;
-    const OpState& st;
     int deg;
     double ratio;
     cudaStream_t s;
     FineTimer* timer = nullptr;
-    bool pre_done = false;  // the fine level's first smoothing step was taken by the CG update
 
     static constexpr bool F64 = std::is_same<T, double>::value;
     const T* av(int l, int v) const {
         if constexpr (F64)
-            return l == 0 ? st.v64[v] : V.A[size_t(l)][size_t(v)];
+            return V.A[size_t(l)][size_t(v)];
         else
             return V.A32[size_t(l)][size_t(v)];
     }
@@ -1124,27 +1427,6 @@ struct VCycle {
             k_cheb<T, R, NV, false, 1><<<blocks_of(A.n), 256, 0, s>>>(A, a0, a1, di, hi, ratio, k, x_in, x_out, d, b);
     }
 
-    // the fine level's first smoothing step on b (before the first iteration)
-    void first_fine(const T* b) {
-        if (H.lv.size() < 2) return;
-        const LevelDev& d = H.lv[0];
-        note_launch(1);
-        k_cheb<T, R, NV, true, 1><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, av(0, 0), av(0, 1), dinv(0), V.hi, ratio, 0,
-                                                                  nullptr, static_cast<T*>(W.xa[0]),
-                                                                  static_cast<T*>(W.d[0]), b);
-    }
-
-    PreStep<T, NV> pre_step(float* b32) const {
-        PreStep<T, NV> p;
-        p.dinv = dinv(0);
-        p.hi = V.hi;
-        p.ratio = ratio;
-        p.x = static_cast<T*>(W.xa[0]);
-        p.d = deg > 1 ? static_cast<T*>(W.d[0]) : nullptr;
-        p.b32 = b32;
-        return p;
-    }
-
     const T* run(int l, const T* b) {
         const LevelDev& d = H.lv[size_t(l)];
         const int L = int(H.lv.size());
@@ -1158,11 +1440,9 @@ struct VCycle {
         }
         const double* hi = V.hi + 2 * l;
         const T *a0 = av(l, 0), *a1 = av(l, 1);
-        if (!(l == 0 && pre_done)) {
-            note_launch(1);
-            k_cheb<T, R, NV, true, 1><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, a0, a1, dinv(l), hi, ratio, 0, nullptr,
-                                                                      x, dd, b);
-        }
+        note_launch(1);
+        k_cheb<T, R, NV, true, 1><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, a0, a1, dinv(l), hi, ratio, 0, nullptr, x, dd,
+                                                                  b);
         for (int k = 1; k < deg; ++k) {
             if (l == 0 && timer) timer->before();
             cheb(d.A, a0, a1, dinv(l), hi, k, x, y, dd, b);
@@ -1185,16 +1465,109 @@ struct VCycle {
     }
 };
 
+// The degree-1 cycle (see k_level): per level the residual, its restriction
+// and, on the way back, prolongation with the post-smoothing step; the fine
+// level's last kernel (k_top) belongs to the CG.
+template <typename T, int R, int NV>
+struct FastCycle {
+    const AmgHierDev& H;
+    const AmgValues& V;
+    AmgVecs& W;
+    cudaStream_t s;
+    FineTimer* timer = nullptr;
+
+    static constexpr bool F64 = std::is_same<T, double>::value;
+    static constexpr int LPR = R / kLaneRhs<T, R>, GX = 32 / LPR, GM = GX < 8 ? GX : 8;
+    const T* val(const std::vector<std::array<double*, 2>>& a, const std::vector<std::array<float*, 2>>& b, int l,
+                 int v) const {
+        if constexpr (F64) return a[size_t(l)][size_t(v)];
+        else return b[size_t(l)][size_t(v)];
+    }
+    const T* wd(int l) const {
+        if constexpr (F64) return V.wd[size_t(l)];
+        else return V.wd32[size_t(l)];
+    }
+    SellDev p2(int l) const {
+        const LevelDev& d = H.lv[size_t(l)];
+        SellDev p;
+        p.n = d.A.n;
+        p.ptr = d.ap_ptr;
+        p.col = d.ap_col;
+        p.entries = d.ap_nnz;
+        p.maxlen = d.ap_maxlen;
+        p.rowmajor = 1;
+        return p;
+    }
+    // Groups that share a row's entries.  FP64 issue is the scarce resource
+    // (16 cycles of an SM for each warp instruction, idle lanes included), so
+    // rows are shared by several groups only as far as the GPU would not be
+    // filled otherwise, or two where rows of one lane lie row by row in memory
+    // (coalescing); FP32 shares row-major rows by up to 8.  Long rows of the
+    // smallest levels get a block each.
+    template <int MODE>
+    void launch(const SellDev& A, const T* v0, const T* v1, const T* x, const T* w, const T* b, const T* res, T* y) {
+        note_launch(1);
+        const double avg = double(A.entries) / double(std::max<int64_t>(1, A.n));
+        const int64_t fill = 152 * 1024, threads = A.n * LPR;
+        auto go = [&](auto gw, auto wpr) {
+            using Map = RowMap<T, R, decltype(gw)::value, decltype(wpr)::value>;
+            k_level<T, R, NV, MODE, decltype(gw)::value, decltype(wpr)::value>
+                <<<blocks_of(A.n, Map::RPB), 256, 0, s>>>(A, v0, v1, x, w, b, res, y);
+        };
+        using std::integral_constant;
+        constexpr int GS = F64 ? (LPR == 1 ? 2 : 1) : GM;
+        if (A.n <= 1024 && avg >= 8 * GX)
+            go(integral_constant<int, GX>(), integral_constant<int, 8>());
+        else if (threads * GM < fill && avg >= 2 * GX)
+            go(integral_constant<int, GX>(), integral_constant<int, 1>());
+        else if (threads * GS < fill)
+            go(integral_constant<int, GM>(), integral_constant<int, 1>());
+        else if (A.rowmajor)
+            go(integral_constant<int, GS>(), integral_constant<int, 1>());
+        else
+            go(integral_constant<int, 1>(), integral_constant<int, 1>());
+    }
+
+    // leaves the fine level's residual in W.r[0] and the coarse correction in the returned vector
+    const T* run(const T* b0) {
+        const int L = int(H.lv.size());
+        for (int l = 0; l + 1 < L; ++l) {
+            const LevelDev& d = H.lv[size_t(l)];
+            const T* b = l == 0 ? b0 : static_cast<const T*>(W.b[size_t(l)]);
+            T* res = static_cast<T*>(W.r[size_t(l)]);
+            if (l == 0 && timer) timer->before();
+            launch<0>(d.A, val(V.S, V.S32, l, 0), val(V.S, V.S32, l, 1), b, nullptr, b, nullptr, res);
+            if (l == 0 && timer) timer->after();
+            launch<1>(d.R, val(V.R, V.R32, l, 0), val(V.R, V.R32, l, 1), res, nullptr, nullptr, nullptr,
+                      static_cast<T*>(W.b[size_t(l + 1)]));
+        }
+        const T* inv;
+        if constexpr (F64) inv = V.inv;
+        else inv = V.inv32;
+        const int nc = int(H.lv.back().A.n);
+        T* x = static_cast<T*>(W.xa[size_t(L - 1)]);
+        note_launch(1);
+        k_dense_apply<T, R, NV><<<blocks_of(nc * R, 128), 128, 0, s>>>(nc, inv, static_cast<const T*>(W.b[size_t(L - 1)]), x);
+        for (int l = L - 2; l >= 1; --l) {
+            T* y = static_cast<T*>(W.xa[size_t(l)]);
+            launch<2>(p2(l), val(V.P2, V.P232, l, 0), val(V.P2, V.P232, l, 1), x, wd(l), static_cast<const T*>(W.b[size_t(l)]),
+                      static_cast<const T*>(W.r[size_t(l)]), y);
+            x = y;
+        }
+        return x;
+    }
+};
+
 // Conjugate gradients on the fine operator with one V-cycle per iteration
 // as the preconditioner; X0 (or 0) to start, each right-hand side stops at
 // |r| <= rtol |b| (the recursive residual, as the persistent PCG does).
 // After the start, every iteration is
 //   z = B r, beta = r.z / (r.z)_old, p = z + beta p, q = A p,
 //   alpha = r.z / p.q, x += alpha p, r -= alpha q, check,
-// launched from the host one kernel at a time when the fine-level smoothing
-// is being timed, and otherwise replayed from a captured graph whose
-// "while" node runs on the device until the check ends it (no host round
-// trip per iteration).  Both forms launch the same kernels on the same data.
+// launched from the host one kernel at a time when the fine level is being
+// timed, and otherwise replayed from a captured graph whose "while" node runs
+// on the device until the check ends it (no host round trip per iteration).
+// Both forms launch the same kernels on the same data.
 template <int R, int NV>
 struct CgSolve {
     qpat_mesh_s* M;
@@ -1210,60 +1583,57 @@ struct CgSolve {
     int64_t n = 0;
     int G = 0;
 
-    // kernels of one iteration: per level above the coarsest 2 deg + 3
-    // (smoothing, residual, restriction, prolongation), 1 on the coarsest,
-    // 2 casts for the FP32 cycle, 7 of the CG itself
-    // (the fine level's first smoothing step, and for the FP32 cycle the cast
-    // of r, are taken by the CG update)
-    int body_kernels() const {
-        const int deg = std::max(1, so.mg_degree);
-        const int L = int(H.lv.size());
-        return (L - 1) * (2 * deg + 3) - (L > 1 ? 1 : 0) + 1 + (f32 ? 1 : 0) + 7;
+    bool fast() const { return so.mg_degree <= 1 && H.lv.size() > 1; }
+
+    // z = B r and beta on stream t; returns the kernels launched beyond those that the cycles count themselves
+    template <typename T>
+    void precondition(cudaStream_t t) {
+        constexpr bool F32 = std::is_same<T, float>::value;
+        const T* b;
+        if constexpr (F32) b = static_cast<const T*>(W.b[0]);
+        else b = C.r;
+        note_launch(1);
+        if (fast()) {
+            FastCycle<T, R, NV> c{H, V, W, t, timer};
+            const T* e = c.run(b);
+            k_top<T, R, NV, 1><<<full_grid(k_top<T, R, NV, 1>, G), 256, 0, t>>>(c.p2(0), c.val(V.P2, V.P232, 0, 0), c.val(V.P2, V.P232, 0, 1), e, c.wd(0), b,
+                                                  static_cast<const T*>(W.r[0]), C.r, C.q, C.z, C.part, C.count, C.rz,
+                                                  C.alpha, C.beta, C.ctl);
+            return;
+        }
+        VCycle<T, R, NV> c{H, V, W, std::max(1, so.mg_degree), so.mg_ratio, t, timer};
+        const T* x = c.run(0, b);
+        const double* z;
+        if constexpr (F32) {
+            note_launch(1);
+            k_f2d_vec<<<G, 256, 0, t>>>(n * R, x, C.z);
+            z = C.z;
+        } else {
+            z = x;
+        }
+        k_cg_dots<R, F32><<<full_grid(k_cg_dots<R, F32>, G), 256, 0, t>>>(n, C.r, z, C.q, C.part, C.count, C.rz, C.alpha, C.beta, C.ctl);
+        zp = z;
     }
+    const double* zp = nullptr;  // z where it is not C.z
 
     // one iteration on stream t; use_graph: the check sets the loop condition
     void body(cudaStream_t t, cudaGraphConditionalHandle cond, int use_graph) {
-        const int deg = std::max(1, so.mg_degree);
-        const LevelDev& d0 = H.lv[0];
-        const double* z;
-        const bool multi = H.lv.size() > 1;
-        if (!f32) {
-            VCycle<double, R, NV> c{H, V, W, st, deg, so.mg_ratio, t, timer, multi};
-            z = c.run(0, C.r);
-        } else {
-            VCycle<float, R, NV> c{H, V, W, st, deg, so.mg_ratio, t, timer, multi};
-            const float* x0 = c.run(0, static_cast<float*>(W.b[0]));
-            note_launch(1);
-            k_f2d_vec<<<G, 256, 0, t>>>(n * R, x0, C.z);
-            z = C.z;
-        }
-        note_launch(7);
-        if (f32) {
-            k_cg_dots<R, true><<<G, 256, 0, t>>>(n, C.r, z, C.zo, C.part);
-            k_cg_beta<R, true><<<1, 32 * R, 0, t>>>(C.part, G, C.rz, C.beta, C.ctl);
-            k_cg_dir<R, true><<<G, 256, 0, t>>>(n, C.beta, z, C.p, C.zo);
-        } else {
-            k_cg_dots<R, false><<<G, 256, 0, t>>>(n, C.r, z, nullptr, C.part);
-            k_cg_beta<R, false><<<1, 32 * R, 0, t>>>(C.part, G, C.rz, C.beta, C.ctl);
-            k_cg_dir<R, false><<<G, 256, 0, t>>>(n, C.beta, z, C.p, nullptr);
-        }
-        k_cg_apply<R, NV><<<G, 256, 0, t>>>(d0.A, st.v64[0], st.v64[1], C.p, C.q, C.part);
-        k_cg_alpha<R><<<1, 32 * R, 0, t>>>(C.part, G, C.rz, C.alpha, C.ctl);
-        if (!f32) {
-            VCycle<double, R, NV> c{H, V, W, st, deg, so.mg_ratio, t, timer};
-            k_cg_update<R, NV, double><<<G, 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, C.part, c.pre_step(nullptr));
-        } else {
-            VCycle<float, R, NV> c{H, V, W, st, deg, so.mg_ratio, t, timer};
-            float* b0 = static_cast<float*>(W.b[0]);
-            k_cg_update<R, NV, float><<<G, 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, C.part, c.pre_step(b0));
-        }
-        k_cg_check<R><<<1, 32 * R, 0, t>>>(C.part, G, C.bb, C.rtol2, C.rr, C.ctl, cond, use_graph);
+        zp = C.z;
+        if (f32) precondition<float>(t);
+        else precondition<double>(t);
+        note_launch(3);
+        k_cg_dir<R><<<full_grid(k_cg_dir<R>, G), 256, 0, t>>>(n, C.beta, zp, C.p);
+        // K's rows hold 15 entries, M_delta's 7: one group per row, the lanes of its right-hand sides side by side
+        k_cg_apply<R, NV, 1><<<full_grid(k_cg_apply<R, NV, 1>, G), 256, 0, t>>>(NV == 1 ? H.K : H.lv[0].A, st.v64[0], st.v64[1], C.p, C.q, C.part, C.count,
+                                               C.rz, C.alpha, C.ctl);
+        k_cg_update<R><<<full_grid(k_cg_update<R>, G), 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, f32 ? static_cast<float*>(W.b[0]) : nullptr,
+                                         C.part, C.count, C.bb, C.rtol2, C.rr, C.ctl, cond, use_graph);
     }
 
     int run(AmgState& A, const std::string& key, const double* B, double* X, const double* X0, int* iters) {
-        const LevelDev& d0 = H.lv[0];
-        n = d0.A.n;
-        G = int(std::min<int64_t>(blocks_of(n), kRedMaxGrid));
+        const SellDev& A0 = NV == 1 ? H.K : H.lv[0].A;
+        n = A0.n;
+        G = int(std::min<int64_t>(blocks_of(n * R, 512), kRedMaxGrid));
         int* hc = reinterpret_cast<int*>(M->host_scratch + 240);
         cudaError_t e = cudaSuccess;
         auto read_ctl = [&]() -> cudaError_t {
@@ -1280,24 +1650,16 @@ struct CgSolve {
             return cuda_fail(e, "multigrid start");
         note_launch(2);
         if (X0)
-            k_cg_init_x0<R, NV><<<G, 256, 0, s>>>(d0.A, st.v64[0], st.v64[1], B, X0, C.x, C.r, C.part);
+            k_cg_init_x0<R, NV><<<G, 256, 0, s>>>(A0, st.v64[0], st.v64[1], B, X0, C.x, C.r, C.part);
         else
             k_cg_init<R><<<G, 256, 0, s>>>(n, B, C.x, C.r, C.part);
         k_cg_start<R><<<1, 32 * R, 0, s>>>(C.part, G, C.bb, C.ctl);
         if ((e = read_ctl()) != cudaSuccess) return cuda_fail(e, "multigrid cg");
         if (hc[0] != QPAT_OK) return fail(hc[0], "multigrid cg: right-hand side not finite");
         if (hc[1] > 0) {
-            // the first cycle's first fine smoothing step (later ones come with the CG update)
-            const int deg = std::max(1, so.mg_degree);
-            if (!f32) {
-                VCycle<double, R, NV> c{H, V, W, st, deg, so.mg_ratio, s, timer};
-                c.first_fine(C.r);
-            } else {
-                VCycle<float, R, NV> c{H, V, W, st, deg, so.mg_ratio, s, timer};
-                float* b0 = static_cast<float*>(W.b[0]);
+            if (f32) {
                 note_launch(1);
-                k_d2f_vec<<<G, 256, 0, s>>>(n * R, C.r, b0);
-                c.first_fine(b0);
+                k_d2f_vec<<<G, 256, 0, s>>>(n * R, C.r, static_cast<float*>(W.b[0]));
             }
             if (!timer->on) {
                 AmgGraph& g = A.graphs[key];
@@ -1345,8 +1707,9 @@ struct CgSolve {
         if ((e = cudaStreamBeginCaptureToGraph(A.capture, bodyg, nullptr, nullptr, 0,
                                                cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
             return cuda_fail(e, "multigrid capture");
+        const int64_t before = thread_launches();
         body(A.capture, cond, 1);
-        g.body_kernels = body_kernels();
+        g.body_kernels = int(thread_launches() - before);
         cudaGraph_t out = nullptr;
         const cudaError_t e1 = cudaGetLastError();
         e = cudaStreamEndCapture(A.capture, &out);
@@ -1386,20 +1749,21 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         return fail(QPAT_EINVAL, "multigrid: mg_degree must lie in [1, 8] and mg_ratio exceed 1");
     if (!M->amg) M->amg = new AmgState();
     AmgState& A = *M->amg;
-    const int pat = st.kind == OP_PRIOR ? 1 : 0;
-    AmgHierDev& H = A.hier[pat];
+    AmgHierDev& H = A.hier;
     if (!H.tried) {
-        const int rc = build_hier(M, pat, H);
+        const int rc = build_hier(M, H);
         if (rc != QPAT_OK) return rc;
     } else if (!H.error.empty()) {
         return fail(QPAT_EINVAL, H.error);
     }
     const bool f32 = so.multigrid == 2 && st.kind == OP_K;
     AmgValues& V = A.vals[st.v64[0]];
-    int rc = numeric(M, H, st, V, f32, s);
+    const bool fast = so.mg_degree <= 1 && H.lv.size() > 1;
+    H.used[st.kind == OP_PRIOR] = true;
+    int rc = numeric(M, H, st, V, fast, so.mg_ratio, f32, s);
     if (rc != QPAT_OK) return rc;
     cudaError_t e = cudaSuccess;
-    AmgVecs& W = A.vecs[{pat * 64 + R, f32 ? 1 : 0}];
+    AmgVecs& W = A.vecs[{R, f32 ? 1 : 0}];
     if (W.xa.empty()) {
         const size_t esz = f32 ? sizeof(float) : sizeof(double);
         for (const LevelDev& d : H.lv) {
@@ -1420,10 +1784,12 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         C.p = dalloc<double>(C.allocs, nR, e);
         C.q = dalloc<double>(C.allocs, nR, e);
         C.z = dalloc<double>(C.allocs, nR, e);
-        C.zo = dalloc<double>(C.allocs, nR, e);
         C.part = dalloc<double>(C.allocs, size_t(kRedMaxGrid) * 32, e);
         double* sc = dalloc<double>(C.allocs, 5 * 16 + 1, e);
         C.ctl = dalloc<int>(C.allocs, kCtlActive + 16, e);
+        C.count = dalloc<unsigned>(C.allocs, 1, e);
+        if (e == cudaSuccess) e = cudaMemsetAsync(C.count, 0, sizeof(unsigned), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(C.q, 0, sizeof(double) * nR, s);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
         C.bb = sc;
         C.rz = sc + 16;
@@ -1434,7 +1800,7 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
     }
     // the captured iteration depends on these buffers and settings only
     char key[256];
-    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%d/%.17g/%p/%p/%p", pat, R, st.nv, int(f32), so.mg_degree, so.mg_ratio,
+    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%.17g/%p/%p/%p", R, st.nv, int(f32), so.mg_degree, so.mg_ratio,
                   static_cast<const void*>(&V), static_cast<const void*>(st.v64[0]),
                   static_cast<const void*>(st.v64[1]));
     FineTimer timer;
@@ -1467,7 +1833,8 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
 
 int amg_levels(qpat_mesh_s* M, int prior, int64_t* rows, int max_levels) {
     if (!M->amg) return 0;
-    const AmgHierDev& H = M->amg->hier[prior ? 1 : 0];
+    const AmgHierDev& H = M->amg->hier;
+    if (!H.used[prior ? 1 : 0]) return 0;
     const int L = int(H.lv.size());
     for (int l = 0; l < std::min(L, max_levels); ++l) rows[l] = H.lv[size_t(l)].A.n;
     return L;
@@ -1476,8 +1843,7 @@ int amg_levels(qpat_mesh_s* M, int prior, int64_t* rows, int max_levels) {
 void amg_release(qpat_mesh_s* M) {
     if (!M->amg) return;
     AmgState& A = *M->amg;
-    for (auto& H : A.hier)
-        for (void* p : H.allocs) cudaFree(p);
+    for (void* p : A.hier.allocs) cudaFree(p);
     for (auto& kv : A.vals)
         for (void* p : kv.second.allocs) cudaFree(p);
     for (auto& kv : A.vecs)

@@ -3,9 +3,11 @@
 // selected by qpat_params.multigrid.
 //
 // The method is the textbook smoothed aggregation of Vanek, Mandel and
-// Brezina (Computing 56, 1996): aggregates of the matrix graph, a piecewise-
-// constant tentative prolongator smoothed by one damped Jacobi step,
-// P = (I - omega D^-1 A) P_tent with omega = 4 / (3 rho(D^-1 A)), Galerkin
+// Brezina (Computing 56, 1996): aggregates of the matrix graph (here of 8
+// nodes, by three rounds of pairwise matching), a piecewise-constant tentative prolongator smoothed by one damped Jacobi step,
+// a damped Jacobi step along the couplings between graph neighbours, weighted
+// so that the constants are kept (which keeps the coarse rows at ~30 to 70
+// entries), Galerkin
 // coarse operators A_c = P^T A P, Chebyshev smoothing in D^-1 A on each level
 // and an exact solve on the coarsest level; applied as one symmetric V-cycle
 // per CG iteration.
@@ -57,6 +59,8 @@ struct SellPattern {
 // applied by 8 lanes per row.
 constexpr int kAmgRowMajorLen = 24;
 
+constexpr uint16_t kAmgDropped = 0xffff;
+
 // Host plan of one level: the level's operator pattern and, except on the
 // coarsest level, the transfer to the next one.
 struct AmgLevelPlan {
@@ -65,7 +69,8 @@ struct AmgLevelPlan {
     int64_t nc = 0;                // rows of the next level (0 on the coarsest)
     std::vector<int32_t> agg;      // aggregate of each row
     SellPattern P;                 // prolongator pattern (n rows, next-level columns)
-    std::vector<uint16_t> a2p;      // per A entry (SELL position): slot in its row of P holding agg(col)
+    std::vector<uint16_t> a2p;      // per A entry (position): slot in its row of P holding agg(col); kAmgDropped if
+                                    // the entry is not in the graph (P then has it on the diagonal)
     std::vector<uint16_t> pself;    // per row: slot of agg(row) in its row of P
     // A P (n rows, next-level columns; CSR, columns sorted): the product's
     // pattern and, per row i, for every A entry k < len(i) and every P entry
@@ -90,25 +95,42 @@ struct AmgPlan {
     std::string error;                 // non-empty: no hierarchy (the caller keeps its other preconditioner)
 };
 
+// Damping of the step that smooths the prolongator (2/3 times a margin; 0.6 gave the fewest iterations on M_delta).
+constexpr double kAmgOmega = 0.6;
 // Largest coarsest level solved exactly (dense inverse in one CTA).
 constexpr int kAmgCoarsest = 128;
 // Most levels of a hierarchy.
 constexpr int kAmgMaxLevels = 12;
 
+// A graph with edge weights and the order in which matching visits its nodes.
+struct AmgGraphPlan {
+    std::vector<int64_t> ptr;
+    std::vector<int32_t> col;
+    std::vector<int32_t> w;      // number of fine edges behind the edge
+    std::vector<int32_t> order;
+};
+
 // Builds the plan from the fine pattern in SELL form with global column ids
 // (entries of a row in any order, the diagonal present, the pattern
 // symmetric).  The fine level's A keeps the given positions, so the assembled
 // values of the mesh's pattern serve as level 0 unchanged.
-AmgPlan amg_build_plan(const SellPattern& fine);
+// graph: the graph whose aggregates the hierarchy uses (the fine pattern's).
+AmgPlan amg_build_plan(const SellPattern& fine, AmgGraphPlan graph);
 
 // Checks every invariant the device kernels rely on (diagonal slots,
 // non-empty aggregates, P, a2p, pself, the A P and Galerkin slots, R = P^T,
 // symmetric coarse patterns, the coarsest size); "" if all hold.
 std::string amg_check_plan(const AmgPlan& plan);
 
-// The fine pattern of a prepared host mesh (K: prior = 0; the prior's
-// stiffness-only pattern: prior = 1) with global column ids.
+// The fine pattern of a prepared host mesh with global column ids, for K and
+// for M_delta alike: the prior's stiffness-only pattern.  K is taken into it by
+// adding the couplings outside it (mass terms without stiffness, on Kuhn
+// meshes 8 of a row's 14) to the diagonal: half the products of a cycle, and a
+// matrix that is spectrally equivalent to K (a lumped against a consistent
+// mass: within [1/5, 1] of it, and within a percent where diffusion rules).
 struct HostMesh;
-SellPattern amg_fine_pattern(const HostMesh& h, int prior);
+SellPattern amg_fine_pattern(const HostMesh& h);
+// Its graph, visited along the coordinates (the aggregates then follow a structured grid).
+AmgGraphPlan amg_fine_graph(const HostMesh& h, const SellPattern& fine);
 
 }  // namespace qpat

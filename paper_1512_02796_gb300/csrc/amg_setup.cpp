@@ -18,10 +18,13 @@ int host_threads() {
     return int(std::max(1u, std::min(h, 16u)));
 }
 
+// Threads for n rows (coarse levels have few, long rows).
+int threads_for(int64_t n) { return n < 256 ? 1 : host_threads(); }
+
 // fn(t, begin, end) over nt contiguous ranges of [0, n).
 template <typename F>
 void parallel_ranges(int64_t n, int nt, const F& fn) {
-    if (nt <= 1 || n < 8192) {
+    if (nt <= 1) {
         fn(0, int64_t(0), n);
         return;
     }
@@ -59,7 +62,7 @@ struct Marker {
 // gather(i, marker) adds.
 template <typename G>
 Csr build_rows(int64_t n, int64_t ncols, const G& gather) {
-    const int nt = n < 8192 ? 1 : host_threads();
+    const int nt = threads_for(n);
     std::vector<std::vector<int32_t>> cols(static_cast<size_t>(nt));
     std::vector<std::vector<int64_t>> lens(static_cast<size_t>(nt));
     parallel_ranges(n, nt, [&](int t, int64_t b, int64_t e) {
@@ -145,58 +148,126 @@ bool sell_from_csr(const Csr& c, SellPattern& s, std::string& err) {
     return true;
 }
 
-// Aggregates of the graph of A (Vanek, Mandel, Brezina 1996, without a
-// strength threshold: the pattern alone decides).  1: every node whose
-// neighbours are all free forms an aggregate with them; 2: a free node joins
-// the aggregate of step 1 it has most neighbours in (ties: the lower id);
-// 3: what is left forms aggregates with its free neighbours.
-std::vector<int32_t> aggregate(const SellPattern& A, int64_t& nagg) {
-    const int64_t n = A.n;
-    std::vector<int32_t> agg(size_t(n), -1);
-    int32_t na = 0;
-    for (int64_t i = 0; i < n; ++i) {
-        if (agg[size_t(i)] >= 0) continue;
-        bool free_ = true;
-        for (int k = 0; k < A.len[size_t(i)] && free_; ++k) {
-            const int32_t j = A.col[size_t(A.pos(i, k))];
-            if (j != i && agg[size_t(j)] >= 0) free_ = false;
+// One round of pairwise matching on a weighted graph (w: number of fine edges
+// between two nodes): nodes in the given order take the free neighbour they
+// share most edges with (ties: first in the order); a node without a free
+// neighbour joins the pair it shares most edges with.
+std::vector<int32_t> match(const AmgGraphPlan& G, int64_t& npairs) {
+    const int64_t n = int64_t(G.order.size());
+    std::vector<int32_t> rank(static_cast<size_t>(n)), to(size_t(n), -1);
+    for (int64_t q = 0; q < n; ++q) rank[size_t(G.order[size_t(q)])] = int32_t(q);
+    auto best = [&](int32_t i, bool taken) {
+        int32_t j = -1;
+        int64_t at = 0;
+        for (int64_t k = G.ptr[size_t(i)]; k < G.ptr[size_t(i + 1)]; ++k) {
+            const int32_t c = G.col[size_t(k)];
+            if ((to[size_t(c)] >= 0) != taken) continue;
+            if (j < 0 || G.w[size_t(k)] > G.w[size_t(at)] ||
+                (G.w[size_t(k)] == G.w[size_t(at)] && rank[size_t(c)] < rank[size_t(j)])) {
+                j = c;
+                at = k;
+            }
         }
-        if (!free_) continue;
-        agg[size_t(i)] = na;
-        for (int k = 0; k < A.len[size_t(i)]; ++k) agg[size_t(A.col[size_t(A.pos(i, k))])] = na;
-        ++na;
-    }
-    const std::vector<int32_t> agg1 = agg;
-    std::vector<std::pair<int32_t, int>> cnt;
-    for (int64_t i = 0; i < n; ++i) {
-        if (agg1[size_t(i)] >= 0) continue;
-        cnt.clear();
-        for (int k = 0; k < A.len[size_t(i)]; ++k) {
-            const int32_t j = A.col[size_t(A.pos(i, k))];
-            const int32_t a = j == i ? -1 : agg1[size_t(j)];
-            if (a < 0) continue;
-            auto it = std::find_if(cnt.begin(), cnt.end(), [a](const std::pair<int32_t, int>& p) { return p.first == a; });
-            if (it == cnt.end())
-                cnt.push_back({a, 1});
-            else
-                ++it->second;
+        return j;
+    };
+    int32_t np = 0;
+    std::vector<int32_t> alone;
+    for (int32_t i : G.order) {
+        if (to[size_t(i)] >= 0) continue;
+        const int32_t j = best(i, false);
+        if (j < 0) {
+            alone.push_back(i);
+            continue;
         }
-        if (cnt.empty()) continue;
-        std::pair<int32_t, int> best = cnt[0];
-        for (const auto& p : cnt)
-            if (p.second > best.second || (p.second == best.second && p.first < best.first)) best = p;
-        agg[size_t(i)] = best.first;
+        to[size_t(i)] = to[size_t(j)] = np++;
     }
-    for (int64_t i = 0; i < n; ++i) {
-        if (agg[size_t(i)] >= 0) continue;
-        agg[size_t(i)] = na;
-        for (int k = 0; k < A.len[size_t(i)]; ++k) {
-            const int32_t j = A.col[size_t(A.pos(i, k))];
-            if (agg[size_t(j)] < 0) agg[size_t(j)] = na;
+    std::vector<int32_t> joins(alone.size());
+    for (size_t q = 0; q < alone.size(); ++q) {
+        const int32_t j = best(alone[q], true);
+        joins[q] = j < 0 ? -1 : to[size_t(j)];
+    }
+    for (size_t q = 0; q < alone.size(); ++q) to[size_t(alone[q])] = joins[q] >= 0 ? joins[q] : np++;
+    npairs = np;
+    return to;
+}
+
+// The graph of the sets `to`: edge counts between different sets, rows sorted; sets keep their numbers as order.
+AmgGraphPlan merge(const AmgGraphPlan& G, const std::vector<int32_t>& to, int64_t nc) {
+    const int64_t n = int64_t(to.size());
+    std::vector<int64_t> mptr(size_t(nc + 1), 0);
+    std::vector<int32_t> members(static_cast<size_t>(n));
+    for (int32_t t : to) ++mptr[size_t(t + 1)];
+    for (int64_t I = 0; I < nc; ++I) mptr[size_t(I + 1)] += mptr[size_t(I)];
+    {
+        std::vector<int64_t> at(mptr.begin(), mptr.end() - 1);
+        for (int64_t i = 0; i < n; ++i) members[size_t(at[size_t(to[size_t(i)])]++)] = int32_t(i);
+    }
+    auto gather = [&](int64_t I, Marker& mk) {
+        for (int64_t q = mptr[size_t(I)]; q < mptr[size_t(I + 1)]; ++q) {
+            const int32_t i = members[size_t(q)];
+            for (int64_t k = G.ptr[size_t(i)]; k < G.ptr[size_t(i + 1)]; ++k) {
+                const int32_t J = to[size_t(G.col[size_t(k)])];
+                if (J != I) mk.add(J, I);
+            }
         }
-        ++na;
+    };
+    const Csr c = build_rows(nc, nc, gather);
+    AmgGraphPlan out;
+    out.w.assign(c.col.size(), 0);
+    parallel_ranges(nc, threads_for(nc), [&](int, int64_t b, int64_t e) {
+        for (int64_t I = b; I < e; ++I)
+            for (int64_t q = mptr[size_t(I)]; q < mptr[size_t(I + 1)]; ++q) {
+                const int32_t i = members[size_t(q)];
+                for (int64_t k = G.ptr[size_t(i)]; k < G.ptr[size_t(i + 1)]; ++k) {
+                    const int32_t J = to[size_t(G.col[size_t(k)])];
+                    if (J != I)
+                        out.w[size_t(c.ptr[size_t(I)] + slot_of(c.col.data(), c.ptr[size_t(I)], c.ptr[size_t(I + 1)], J))] +=
+                            G.w[size_t(k)];
+                }
+            }
+    });
+    out.ptr = c.ptr;
+    out.col = c.col;
+    out.order.resize(size_t(nc));
+    for (int64_t I = 0; I < nc; ++I) out.order[size_t(I)] = int32_t(I);
+    return out;
+}
+
+// Aggregates of 8: three rounds of pairwise matching, heaviest neighbours
+// first and in the order of the grid the nodes come from, which on a
+// structured grid gives its 2 x 2 x 2 blocks.  The graph becomes the next
+// level's.  Aggregates are numbered by their first node.
+std::vector<int32_t> aggregate(AmgGraphPlan& G, int64_t& nagg) {
+    const int64_t n = int64_t(G.order.size());
+    std::vector<int32_t> agg(static_cast<size_t>(n));
+    for (int64_t i = 0; i < n; ++i) agg[size_t(i)] = int32_t(i);
+    int64_t nc = n;
+    for (int round = 0; round < 3; ++round) {
+        const std::vector<int32_t> to = match(G, nc);
+        G = merge(G, to, nc);
+        for (int32_t& a : agg) a = to[size_t(a)];
     }
-    nagg = na;
+    std::vector<int32_t> name(size_t(nc), -1);
+    int32_t next = 0;
+    for (int32_t& a : agg) {
+        if (name[size_t(a)] < 0) name[size_t(a)] = next++;
+        a = name[size_t(a)];
+    }
+    // the graph in the new numbers, visited in the old order
+    AmgGraphPlan H;
+    H.order = name;
+    H.ptr.assign(size_t(nc + 1), 0);
+    H.col.resize(G.col.size());
+    H.w.resize(G.w.size());
+    for (int64_t I = 0; I < nc; ++I) H.ptr[size_t(name[size_t(I)] + 1)] = G.ptr[size_t(I + 1)] - G.ptr[size_t(I)];
+    for (int64_t I = 0; I < nc; ++I) H.ptr[size_t(I + 1)] += H.ptr[size_t(I)];
+    for (int64_t I = 0; I < nc; ++I)
+        for (int64_t k = G.ptr[size_t(I)], o = H.ptr[size_t(name[size_t(I)])]; k < G.ptr[size_t(I + 1)]; ++k, ++o) {
+            H.col[size_t(o)] = name[size_t(G.col[size_t(k)])];
+            H.w[size_t(o)] = G.w[size_t(k)];
+        }
+    G = std::move(H);
+    nagg = nc;
     return agg;
 }
 
@@ -218,30 +289,36 @@ bool set_diag(AmgLevelPlan& L) {
 
 // The transfer from level L to the next one; `coarse` receives the next
 // level's pattern (rows sorted).
-bool build_transfer(AmgLevelPlan& L, Csr& coarse, std::string& err) {
+bool build_transfer(AmgLevelPlan& L, AmgGraphPlan& graph, Csr& coarse, std::string& err) {
     const SellPattern& A = L.A;
     const int64_t n = A.n;
-    const int nt = n < 8192 ? 1 : host_threads();
+    const int nt = threads_for(n);
     int64_t nc = 0;
-    L.agg = aggregate(A, nc);
+    const AmgGraphPlan fine = graph;
+    L.agg = aggregate(graph, nc);
     L.nc = nc;
     if (nc <= 0 || nc >= n) {
         err = "multigrid: aggregation made no progress";
         return false;
     }
-    // P = (I - omega D^-1 A) P_tent: row i holds the aggregates of i's row of A
+    // P: row i holds the aggregates of i and of its graph neighbours
     const Csr Pc = build_rows(n, nc, [&](int64_t i, Marker& mk) {
-        for (int k = 0; k < A.len[size_t(i)]; ++k) mk.add(L.agg[size_t(A.col[size_t(A.pos(i, k))])], i);
+        mk.add(L.agg[size_t(i)], i);
+        for (int64_t k = fine.ptr[size_t(i)]; k < fine.ptr[size_t(i + 1)]; ++k) mk.add(L.agg[size_t(fine.col[size_t(k)])], i);
     });
     if (!sell_from_csr(Pc, L.P, err)) return false;
-    L.a2p.assign(size_t(A.entries()), 0);
+    L.a2p.assign(size_t(A.entries()), kAmgDropped);
     L.pself.assign(size_t(n), 0);
     parallel_ranges(n, nt, [&](int, int64_t b, int64_t e) {
+        std::vector<int64_t> kept(size_t(n), -1);
         for (int64_t i = b; i < e; ++i) {
             const int64_t pb = Pc.ptr[size_t(i)], pe = Pc.ptr[size_t(i + 1)];
+            kept[size_t(i)] = i;
+            for (int64_t k = fine.ptr[size_t(i)]; k < fine.ptr[size_t(i + 1)]; ++k) kept[size_t(fine.col[size_t(k)])] = i;
             for (int k = 0; k < A.len[size_t(i)]; ++k) {
                 const int64_t at = A.pos(i, k);
-                L.a2p[size_t(at)] = uint16_t(slot_of(Pc.col.data(), pb, pe, L.agg[size_t(A.col[size_t(at)])]));
+                const int32_t j = A.col[size_t(at)];
+                if (kept[size_t(j)] == i) L.a2p[size_t(at)] = uint16_t(slot_of(Pc.col.data(), pb, pe, L.agg[size_t(j)]));
             }
             L.pself[size_t(i)] = uint16_t(slot_of(Pc.col.data(), pb, pe, L.agg[size_t(i)]));
         }
@@ -266,13 +343,15 @@ bool build_transfer(AmgLevelPlan& L, Csr& coarse, std::string& err) {
     }
     L.ap_slot.assign(size_t(L.ap_sptr[size_t(n)]), 0);
     parallel_ranges(n, nt, [&](int, int64_t b, int64_t e) {
+        std::vector<uint16_t> where(static_cast<size_t>(nc));
         for (int64_t i = b; i < e; ++i) {
+            for (int64_t q = APc.ptr[size_t(i)]; q < APc.ptr[size_t(i + 1)]; ++q)
+                where[size_t(APc.col[size_t(q)])] = uint16_t(q - APc.ptr[size_t(i)]);
             int64_t o = L.ap_sptr[size_t(i)];
             for (int k = 0; k < A.len[size_t(i)]; ++k) {
                 const int32_t j = A.col[size_t(A.pos(i, k))];
                 for (int64_t q = Pc.ptr[size_t(j)]; q < Pc.ptr[size_t(j + 1)]; ++q)
-                    L.ap_slot[size_t(o++)] = uint16_t(
-                        slot_of(APc.col.data(), APc.ptr[size_t(i)], APc.ptr[size_t(i + 1)], Pc.col[size_t(q)]));
+                    L.ap_slot[size_t(o++)] = where[size_t(Pc.col[size_t(q)])];
             }
         }
     });
@@ -311,14 +390,16 @@ bool build_transfer(AmgLevelPlan& L, Csr& coarse, std::string& err) {
         L.g_ptr[size_t(I + 1)] = L.g_ptr[size_t(I)] + s;
     }
     L.g_slot.assign(size_t(L.g_ptr[size_t(nc)]), 0);
-    parallel_ranges(nc, nc < 8192 ? 1 : nt, [&](int, int64_t b, int64_t e) {
+    parallel_ranges(nc, threads_for(nc), [&](int, int64_t b, int64_t e) {
+        std::vector<uint16_t> where(static_cast<size_t>(nc));
         for (int64_t I = b; I < e; ++I) {
+            for (int64_t q = coarse.ptr[size_t(I)]; q < coarse.ptr[size_t(I + 1)]; ++q)
+                where[size_t(coarse.col[size_t(q)])] = uint16_t(q - coarse.ptr[size_t(I)]);
             int64_t o = L.g_ptr[size_t(I)];
             for (int64_t q = Rc.ptr[size_t(I)]; q < Rc.ptr[size_t(I + 1)]; ++q) {
                 const int32_t i = Rc.col[size_t(q)];
                 for (int64_t a = APc.ptr[size_t(i)]; a < APc.ptr[size_t(i + 1)]; ++a)
-                    L.g_slot[size_t(o++)] = uint16_t(slot_of(coarse.col.data(), coarse.ptr[size_t(I)],
-                                                             coarse.ptr[size_t(I + 1)], APc.col[size_t(a)]));
+                    L.g_slot[size_t(o++)] = where[size_t(APc.col[size_t(a)])];
             }
         }
     });
@@ -329,7 +410,7 @@ bool build_transfer(AmgLevelPlan& L, Csr& coarse, std::string& err) {
 
 }  // namespace
 
-AmgPlan amg_build_plan(const SellPattern& fine) {
+AmgPlan amg_build_plan(const SellPattern& fine, AmgGraphPlan graph) {
     AmgPlan plan;
     plan.levels.reserve(kAmgMaxLevels);
     plan.levels.emplace_back();
@@ -344,7 +425,7 @@ AmgPlan amg_build_plan(const SellPattern& fine) {
             return plan;
         }
         Csr coarse;
-        if (!build_transfer(plan.levels.back(), coarse, plan.error)) return plan;
+        if (!build_transfer(plan.levels.back(), graph, coarse, plan.error)) return plan;
         plan.levels.emplace_back();
         if (!sell_from_csr(coarse, plan.levels.back().A, plan.error)) return plan;
         if (!set_diag(plan.levels.back())) {
@@ -359,33 +440,59 @@ AmgPlan amg_build_plan(const SellPattern& fine) {
 
 namespace qpat {
 
-SellPattern amg_fine_pattern(const HostMesh& h, int prior) {
-    const auto& ptr = prior ? h.psell_ptr : h.sell_ptr;
-    const auto& col = prior ? h.psell_col : h.sell_col;
-    const auto& len = prior ? h.psell_len : h.sell_len;
+SellPattern amg_fine_pattern(const HostMesh& h) {
     SellPattern f;
     f.n = h.N;
-    f.nslices = int64_t(ptr.size()) - 1;
-    f.ptr = ptr;
-    f.col.assign(size_t(32 * ptr.back()), 0);
-    f.len.assign(len.begin(), len.end());
+    f.nslices = int64_t(h.psell_ptr.size()) - 1;
+    f.ptr = h.psell_ptr;
+    f.col.assign(size_t(32 * h.psell_ptr.back()), 0);
+    f.len.assign(h.psell_len.begin(), h.psell_len.end());
     f.maxlen = 0;
     for (int64_t s = 0; s < f.nslices; ++s) {
-        const int64_t w = ptr[size_t(s + 1)] - ptr[size_t(s)];
+        const int64_t w = f.ptr[size_t(s + 1)] - f.ptr[size_t(s)];
         f.maxlen = std::max(f.maxlen, int(w));
-        const int p = h.patch_of_slice[size_t(s)];
-        const int nb = h.node_ptr[size_t(p)];
+        const int nb = h.node_ptr[size_t(h.patch_of_slice[size_t(s)])];
         for (int lane = 0; lane < 32; ++lane) {
             const int64_t g = 32 * s + lane;
             for (int64_t k = 0; k < w; ++k) {
-                const int64_t at = (ptr[size_t(s)] + k) * 32 + lane;
-                f.col[size_t(at)] = g < h.N ? h.nodes[size_t(nb + col[size_t(at)])] : 0;
+                const int64_t at = (f.ptr[size_t(s)] + k) * 32 + lane;
+                f.col[size_t(at)] = g < h.N ? h.nodes[size_t(nb + h.psell_col[size_t(at)])] : 0;
             }
         }
     }
     return f;
 }
 
+AmgGraphPlan amg_fine_graph(const HostMesh& h, const SellPattern& fine) {
+    AmgGraphPlan G;
+    const int64_t n = fine.n;
+    G.ptr.assign(size_t(n + 1), 0);
+    for (int64_t i = 0; i < n; ++i) G.ptr[size_t(i + 1)] = G.ptr[size_t(i)] + fine.len[size_t(i)] - 1;  // without the diagonal
+    G.col.reserve(size_t(G.ptr[size_t(n)]));
+    for (int64_t i = 0; i < n; ++i)
+        for (int k = 0; k < fine.len[size_t(i)]; ++k) {
+            const int32_t j = fine.col[size_t(fine.pos(i, k))];
+            if (j != i) G.col.push_back(j);
+        }
+    G.w.assign(G.col.size(), 1);
+    // by z, then y, then x, on the lattice of the Morton order (which absorbs the rounding of grid coordinates)
+    double lo[3] = {h.xyz[0], h.xyz[1], h.xyz[2]};
+    for (int64_t i = 0; i < n; ++i)
+        for (int c = 0; c < 3; ++c) lo[c] = std::min(lo[c], h.xyz[size_t(3 * i + c)]);
+    std::vector<std::pair<uint64_t, int32_t>> key(static_cast<size_t>(n));
+    for (int64_t i = 0; i < n; ++i) {
+        uint64_t code = 0;
+        for (int c = 2; c >= 0; --c) {
+            const double t = (h.xyz[size_t(3 * i + c)] - lo[c]) / std::max(h.extent, 1e-300);
+            code = code << 21 | uint64_t(std::min(std::max(t, 0.0), 1.0) * double((1u << 21) - 1) + 0.5);
+        }
+        key[size_t(i)] = {code, int32_t(i)};
+    }
+    std::sort(key.begin(), key.end());
+    G.order.resize(size_t(n));
+    for (int64_t q = 0; q < n; ++q) G.order[size_t(q)] = key[size_t(q)].second;
+    return G;
+}
 
 std::string amg_check_plan(const AmgPlan& plan) {
     if (!plan.error.empty()) return plan.error;
@@ -420,6 +527,7 @@ std::string amg_check_plan(const AmgPlan& plan) {
             for (int k = 0; k < A.len[size_t(i)]; ++k) {
                 const int64_t e = A.pos(i, k);
                 const int s = L.a2p[size_t(e)];
+                if (s == kAmgDropped && A.col[size_t(e)] != i) continue;
                 if (s >= LP || L.P.col[size_t(L.P.pos(i, s))] != L.agg[size_t(A.col[size_t(e)])]) return at + "a2p";
             }
         }

@@ -194,19 +194,31 @@ __global__ void __launch_bounds__(kT) k_tet_prior(ElemDev el, const double* __re
     double s[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) s[c] = el.s[6 * t + c];
-    const double f = -1.0 / (30.0 * el.vm[t]);
-    double w[2];
+    // |grad u|^2 = e / vm with e = -sum_ab s_ab (u_a - u_b)^2 / 30
+    const double vm = el.vm[t];
+    double e[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         const double* u = r == 0 ? u1 : u2;
         const double x[4] = {u[v.x], u[v.y], u[v.z], u[v.w]};
-        double g2 = 0.0;
+        double a = 0.0;
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             const double d = x[edge_a(c)] - x[edge_b(c)];
-            g2 = fma(s[c] * d, d, g2);
+            a = fma(s[c] * d, d, a);
         }
-        w[r] = 4.0 * (r == 0 ? 1.0 : scale1) * prior_weight<double>(kind, fmax(f * g2, 0.0), inv_T2, q);
+        e[r] = fmax(a * (-1.0 / 30.0), 0.0);
+    }
+    double w[2];
+    if (kind == 0) {
+        // 1 / (1 + |grad u|^2 / T^2) = vm / (vm + e / T^2) of both blocks by one division
+        const double a = fma(e[0], inv_T2, vm), b = fma(e[1], inv_T2, vm);
+        const double f = 4.0 * vm / (a * b);
+        w[0] = f * b;
+        w[1] = scale1 * (f * a);
+    } else {
+        w[0] = 4.0 * prior_weight<double>(kind, e[0] / vm, inv_T2, q);
+        w[1] = 4.0 * scale1 * prior_weight<double>(kind, e[1] / vm, inv_T2, q);
     }
     tq[t] = make_double2(w[0], w[1]);
 }

@@ -15,6 +15,7 @@ namespace qpat {
 // Counts kernel launches of this library (one per launch statement; a
 // replayed CUDA graph counts its kernel nodes); read by qpat_launch_count.
 void note_launch(int n = 1);
+int64_t thread_launches();  // of the calling thread
 
 // Lets kernel `func` launch with `smem` bytes of dynamic shared memory.  The
 // attribute this sets is one value per kernel for the whole process, so it is
