@@ -74,7 +74,9 @@ typedef struct {
     int fp32_operator;     /* FP32 inner operator of precision 1: 0 = matrix-free
                               element recomputation, 1 = assembled FP32 values */
     int pcg_variant;       /* PCG on assembled operators: 0 = library choice
-                              (currently 1, the fastest measured), 1 = two grid
+                              (the fastest measured: variant 1, or the multigrid
+                              CG below where that is faster; see multigrid),
+                              1 = two grid
                               reductions per iteration (textbook order),
                               2 = one grid reduction per iteration
                               (Chronopoulos-Gear recurrences; the same iterates
@@ -129,7 +131,12 @@ typedef struct {
                               paper, which prescribes no linear solver; every choice
                               reaches the same pcg_rtol):
                               0 = the persistent PCG above (poly_degree,
-                              prior_poly_degree);
+                              prior_poly_degree), or, where nothing above picks
+                              a solver (pcg_variant 0, polynomial degrees,
+                              mixed_restart and barrier_spin_limit at their
+                              defaults), whichever of it and 1 (precision 1:
+                              K solves as 2) was measured faster at the size;
+                              pcg_variant = 1 always runs the persistent PCG;
                               1 = conjugate gradients with one V-cycle of
                               smoothed-aggregation algebraic multigrid per
                               iteration (Vanek, Mandel, Brezina 1996: aggregates
@@ -137,7 +144,7 @@ typedef struct {
                               by one damped Jacobi step that keeps the constants,
                               Galerkin coarse operators P^T A P, Chebyshev
                               smoothing in D^-1 A, an exact dense solve on the
-                              coarsest level of <= 128 rows; the cycle of K works
+                              coarsest level of <= 64 rows; the cycle of K works
                               on K with its couplings outside the stiffness
                               pattern lumped on the diagonal), all in FP64; the K
                               solves then run FP64 iterates whatever `precision`
@@ -220,7 +227,7 @@ int qpat_mesh_host_info(const double* xyz, int64_t N, const int32_t* tets, int64
  * aggregates, the level patterns and the index plans of the device set-up
  * and verifies every invariant the device relies on (P rows, R = P^T, the
  * slots of A P and P^T A P, symmetric coarse patterns, a coarsest level of
- * at most 128 rows).  Writes the rows of each level (finest first, up to
+ * at most 64 rows).  Writes the rows of each level (finest first, up to
  * max_levels) and returns the level count, or QPAT_EINVAL with a message. */
 int qpat_multigrid_host_info(const double* xyz, int64_t N, const int32_t* tets, int64_t E,
                              int patch_nodes, int prior, int64_t* rows, int max_levels);

@@ -249,6 +249,28 @@ static int pcg_status(int st, const char* what) {
     return fail(st, std::string(what) + ": PCG failed");
 }
 
+// The library's choice for solves that ask for neither solver (multigrid = 0,
+// pcg_variant = 0, the default polynomial degree, no barrier limit, no
+// restarts): multigrid-preconditioned CG where it is the faster one, with the
+// cycle in FP32 for the K solves of precision 1 (which may iterate in FP32).
+// Measured on GB300, whole calls, persistent against multigrid:
+//   M_delta: 2.4 / 1.5 ms (11^3), 5.1 / 1.9 (24^3), 27 / 6.5 (64^3), cylinders 8.3 / 4.5 (21 x 21 x 27), 41 / 17 (49 x 49 x 61);
+//   K, FP64 on grids (the stiffness pattern well below K's): R = 8 1.6 / 1.2 ms (11^3), R = 4 1.5 / 1.5 (16^3),
+//   2.7 / 1.8 (24^3), R = 1 1.9 / 1.8 (32^3), 3.8 / 2.4 (48^3), R = 8 40 / 9.2 (64^3);
+//   on cylinders, whose cycle keeps K's whole pattern: R = 4 3.8 / 3.7 (21 x 21 x 27), 9.7 / 8.3 (33 x 33 x 41),
+//   R = 1 5.1 / 6.2, R = 8 15 / 10 (33 x 33 x 41);
+//   K, precision 1 against the FP32 cycle: 1.7 / 1.1 ms (11^3, R = 1), 14 / 6.3 (64^3, R = 8).
+// Below 512 nodes the hierarchy has no second level worth its set-up.
+static bool prefers_multigrid(const qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R) {
+    const int deg = st.kind == OP_PRIOR ? so.poly_prior : so.poly_k;
+    if (so.multigrid || so.pcg_variant != 0 || so.mixed_restart || so.spin_limit > 0 || deg != kDefaultPolyDegree) return false;
+    const int64_t N = M->h.N;
+    if (st.kind == OP_PRIOR || so.precision == 1) return N >= 512;
+    const bool lean = 3 * M->dp.sell_entries < 2 * M->d.sell_entries;
+    if (R == 1) return N >= (lean ? 48000 : 150000);
+    return N * R >= (lean ? 12000 : 64000);
+}
+
 // Solves A X = B for R right-hand sides (library order, N x R node-major,
 // FP64 in and out).  precision 0: FP64 PCG to rtol.  precision 1: X = 0,
 // then sweeps of  r = B - A X (FP64 element apply), d = A32^-1 (r / |r|)
@@ -263,6 +285,12 @@ int solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so_in, int R, cons
     if (st.kind == OP_PRIOR) so.precision = 0;
     // multigrid-preconditioned CG (FP64 iterates whatever the precision mode)
     if (so.multigrid) return amg_solve(M, st, so, R, B, X, s, X0);
+    if (prefers_multigrid(M, st, so_in, R)) {
+        SolveOpts mg = so;
+        mg.multigrid = st.kind == OP_K && so_in.precision == 1 ? 2 : 1;
+        if (amg_solve(M, st, mg, R, B, X, s, X0) == QPAT_OK) return QPAT_OK;
+        // no hierarchy for this mesh, coefficients beyond the FP32 cycle, a breakdown: the persistent solver decides
+    }
     // the prior's assembled blocks live in the stiffness-only pattern
     const MeshDev& md = st.kind == OP_PRIOR ? M->dp : M->d;
     const int64_t N = M->h.N;
@@ -596,8 +624,8 @@ void qpat_default_params(qpat_params* p) {
     p->patch_nodes = 0;
     p->prior = 0;
     p->prior_q = 1.0;
-    p->poly_degree = 2;        // fastest measured on a 64^3 cube (GB300)
-    p->prior_poly_degree = 2;
+    p->poly_degree = kDefaultPolyDegree;  // fastest measured on a 64^3 cube (GB300)
+    p->prior_poly_degree = kDefaultPolyDegree;
     p->lsqr_reorth = 1;        // exact-arithmetic LSQR iterates (see qpat.h)
     p->multigrid = 0;
     p->mg_degree = 1;          // fewer FP64 fine-level products per cycle; fastest measured at 64^3 and 128^3

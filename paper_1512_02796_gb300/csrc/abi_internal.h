@@ -50,6 +50,8 @@ struct OpState {
     uint64_t stamp = 0;             // new for every preparation (keys values derived from the operator)
 };
 
+constexpr int kDefaultPolyDegree = 2;  // poly_degree and prior_poly_degree
+
 struct SolveOpts {
     int precision = 0;        // 0 FP64 PCG, 1 FP32 PCG + FP64 refinement
     double rtol = 1e-13;

@@ -286,38 +286,74 @@ __global__ void k_galerkin(SellDev R, SellDev C, const int64_t* r_src, const int
     for (int k = lane; k < LC; k += 32) out[spos(C, I, k)] = acc[k];
 }
 
-// In-place Gauss-Jordan inversion of the (symmetric positive definite)
-// coarsest operator, one CTA per value set, without pivoting: the pivots of
-// an SPD matrix are its positive Schur complements.
+// Gauss-Jordan inversion of the (symmetric positive definite) coarsest
+// operator, one CTA per value set, without pivoting: the pivots of an SPD
+// matrix are its positive Schur complements.  The matrix stays in registers
+// (thread (w, lane) holds rows w + 32 u, columns lane + 32 v); a step passes
+// its pivot row and column through shared memory, double-buffered, with one
+// barrier.  n^3 multiply-adds on one SM's FP64 pipe bound it (64 rows: ~70 us).
+constexpr int kInvTiles = kAmgCoarsest / 32;
 template <int NV>
-__global__ void k_dense_inv(SellDev A, const double* v0, const double* v1, double* inv) {
-    extern __shared__ double a[];
-    const int n = int(A.n);
-    const int v = blockIdx.x;
-    const double* val = v == 0 ? v0 : v1;
-    double* fcol = a + n * n;
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) a[t] = 0.0;
+__global__ void __launch_bounds__(1024) k_dense_inv(SellDev A, const double* v0, const double* v1, double* inv) {
+    extern __shared__ double dense[];
+    __shared__ double row[2][kAmgCoarsest], col[2][kAmgCoarsest], piv[2];
+    const int n = int(A.n), w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double* val = blockIdx.x == 0 ? v0 : v1;
+    for (int t = threadIdx.x; t < n * n; t += blockDim.x) dense[t] = 0.0;
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x)
         for (int k = 0; k < A.len[i]; ++k) {
             const int64_t at = spos(A, i, k);
-            a[i * n + A.col[at]] += val[at];
+            dense[i * n + A.col[at]] += val[at];
         }
     __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        const double rp = 1.0 / a[k * n + k];
-        __syncthreads();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) a[k * n + j] = j == k ? rp : a[k * n + j] * rp;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) fcol[i] = a[i * n + k];
-        __syncthreads();
-        for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-            const int i = t / n, j = t % n;
-            if (i == k) continue;
-            a[t] = j == k ? -fcol[i] * a[k * n + k] : a[t] - fcol[i] * a[k * n + j];
+    double a[kInvTiles][kInvTiles];
+#pragma unroll
+    for (int u = 0; u < kInvTiles; ++u)
+#pragma unroll
+        for (int v = 0; v < kInvTiles; ++v) {
+            const int i = w + 32 * u, j = lane + 32 * v;
+            a[u][v] = i < n && j < n ? dense[i * n + j] : 0.0;
         }
+    auto publish = [&](int k) {
+        const int b = k & 1;
+#pragma unroll
+        for (int u = 0; u < kInvTiles; ++u)
+#pragma unroll
+            for (int v = 0; v < kInvTiles; ++v) {
+                const int i = w + 32 * u, j = lane + 32 * v;
+                if (i == k) row[b][j] = a[u][v];
+                if (j == k) col[b][i] = a[u][v];
+                if (i == k && j == k) piv[b] = 1.0 / a[u][v];
+            }
+    };
+    publish(0);
+    for (int k = 0; k < n; ++k) {
         __syncthreads();
+        const int b = k & 1;
+        const double rp = piv[b];
+        double r[kInvTiles];
+#pragma unroll
+        for (int v = 0; v < kInvTiles; ++v) r[v] = row[b][lane + 32 * v] * rp;
+#pragma unroll
+        for (int u = 0; u < kInvTiles; ++u) {
+            const int i = w + 32 * u;
+            const double c = col[b][i];
+#pragma unroll
+            for (int v = 0; v < kInvTiles; ++v) {
+                const int j = lane + 32 * v;
+                a[u][v] = i == k ? (j == k ? rp : r[v]) : j == k ? -c * rp : fma(-c, r[v], a[u][v]);
+            }
+        }
+        if (k + 1 < n) publish(k + 1);
     }
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) inv[int64_t(v) * n * n + t] = a[t];
+#pragma unroll
+    for (int u = 0; u < kInvTiles; ++u)
+#pragma unroll
+        for (int v = 0; v < kInvTiles; ++v) {
+            const int i = w + 32 * u, j = lane + 32 * v;
+            if (i < n && j < n) inv[int64_t(blockIdx.x) * n * n + i * n + j] = a[u][v];
+        }
 }
 
 __global__ void k_d2f(int64_t n, const double* in, float* out) {
@@ -1188,11 +1224,11 @@ cudaError_t numeric_levels(const qpat_mesh_s* M, const AmgHierDev& H, const OpSt
     }
     const LevelDev& c = H.lv[size_t(L - 1)];
     const int n = int(c.A.n);
-    const size_t smem = size_t(n) * size_t(n + 1) * sizeof(double);
+    const size_t smem = size_t(n) * size_t(n) * sizeof(double);
     if ((e = allow_smem(reinterpret_cast<const void*>(&k_dense_inv<NV>), smem)) != cudaSuccess) return e;
     const double *a0 = V.A[size_t(L - 1)][0], *a1 = V.A[size_t(L - 1)][1];
     note_launch(1);
-    k_dense_inv<NV><<<NV, 256, smem, s>>>(c.A, a0, a1, V.inv);
+    k_dense_inv<NV><<<NV, 1024, smem, s>>>(c.A, a0, a1, V.inv);
     return cudaGetLastError();
 }
 

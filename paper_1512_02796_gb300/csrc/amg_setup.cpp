@@ -421,7 +421,7 @@ AmgPlan amg_build_plan(const SellPattern& fine, AmgGraphPlan graph) {
     }
     while (plan.levels.back().A.n > kAmgCoarsest) {
         if (int(plan.levels.size()) >= kAmgMaxLevels) {
-            plan.error = "multigrid: no coarsest level of at most 128 rows within 12 levels";
+            plan.error = "multigrid: no coarsest level of at most 64 rows within 12 levels";
             return plan;
         }
         Csr coarse;
