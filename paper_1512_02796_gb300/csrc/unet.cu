@@ -10,6 +10,7 @@
 // 8): log(mu / 0.01), log(kappa / 0.33) and the load vector of the
 // illumination (2 integral Phi lambda_i, Appendix) divided by h^2; target:
 // the fluence phi of that illumination.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <random>
@@ -28,8 +29,7 @@ struct Conv {
     int cin = 0, cout = 0, lvl = 0, relu = 1;
     float *w32 = nullptr, *b32 = nullptr;      // masters
     bf16 *w = nullptr, *wt = nullptr;           // bf16 copy and its flipped transpose
-    float *gw = nullptr, *gb = nullptr;         // gradient of the last sample
-    float *aw = nullptr, *ab = nullptr;         // accumulated gradient
+    float *aw = nullptr, *ab = nullptr;         // gradient summed over the samples
     float *mw = nullptr, *vw = nullptr, *mb = nullptr, *vb = nullptr;
     int64_t nw() const { return int64_t(27) * cin * cout; }
 };
@@ -58,7 +58,7 @@ __global__ void k_take_channel0(int64_t nvox, const float* y32, float* y, float 
         y[v] = log_floor > 0.f ? expf(y32[v * 16]) : y32[v * 16];
 }
 
-// mean-squared error of channel 0 and its gradient (bf16, 16 channels); in
+// mean-squared error of the predictions y32 and its gradient (bf16, channel 0 of 16); in
 // log mode against log(max(t, log_floor))
 __global__ void k_mse(int64_t nvox, const float* y32, const float* t, float scale, bf16* dy, float* loss,
                       float log_floor) {
@@ -66,10 +66,12 @@ __global__ void k_mse(int64_t nvox, const float* y32, const float* t, float scal
     float s = 0.f;
     for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < nvox; v += int64_t(gridDim.x) * blockDim.x) {
         const float tv = log_floor > 0.f ? logf(fmaxf(t[v], log_floor)) : t[v];
-        const float d = y32[v * 16] - tv;
+        const float d = y32[v] - tv;
         s += d * d;
-        dy[v * 16] = __float2bfloat16(2.f * d * scale);
-        for (int c = 1; c < 16; ++c) dy[v * 16 + c] = __float2bfloat16(0.f);
+        const __nv_bfloat162 g = __halves2bfloat162(__float2bfloat16(2.f * d * scale), __float2bfloat16(0.f));
+        uint4* o = reinterpret_cast<uint4*>(dy + v * 16);
+        o[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&g), 0u, 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
     red[threadIdx.x] = s;
     __syncthreads();
@@ -78,11 +80,6 @@ __global__ void k_mse(int64_t nvox, const float* y32, const float* t, float scal
         __syncthreads();
     }
     if (threadIdx.x == 0) atomicAdd(loss, red[0] * scale);
-}
-
-__global__ void k_axpy32(int64_t n, float a, const float* x, float* y, int overwrite) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        y[i] = overwrite ? a * x[i] : y[i] + a * x[i];
 }
 
 __global__ void k_f32_to_f64(int64_t n, const float* in, double* out) {
@@ -101,14 +98,22 @@ struct qpat_unet_s {
     std::vector<Conv> conv;
     std::vector<void*> allocs;
     int lv[4] = {0, 0, 0, 0};  // grid side per level
-    // activations (bf16 channels-last) and their gradients
-    bf16 *xin, *a0, *s0, *p0, *a1, *s1, *p1, *a2, *s2, *p2, *a3, *bt, *cat2, *a4, *d2, *cat1, *a5, *d1, *cat0, *a6,
-        *d0, *yb;
+    // activations (bf16 channels-last) of up to cap samples, one behind the
+    // other, and (train_cap samples) the concatenations and gradients that
+    // training needs; see reserve
+    int cap = 0, train_cap = 0;
+    std::vector<void*> acts, train_acts;
+    bf16 *xin, *a0, *s0, *p0, *a1, *s1, *p1, *a2, *s2, *p2, *a3, *bt, *a4, *d2, *a5, *d1, *a6, *d0;
+    bf16 *cat2, *cat1, *cat0;
     bf16 *g_y, *g_d0, *g_a6, *g_cat0, *g_d1, *g_s0, *g_a5, *g_cat1, *g_d2, *g_s1, *g_a4, *g_cat2, *g_bt, *g_s2, *g_a3,
         *g_p2, *g_a2, *g_p1, *g_a1, *g_p0, *g_a0;
-    float* y32 = nullptr;
+    float* y = nullptr;        // predictions of a training batch
+    float* partial = nullptr;  // wgrad scratch
     float log_floor = 0.f;  // > 0: the network learns log(max(phi, log_floor)) (qpat_unet_set_log_output)
-    float* partial = nullptr;
+    // mma.sync engine only: concatenation, bf16 and fp32 output of one sample
+    bf16 *mcat = nullptr, *mout = nullptr;
+    float* mout32 = nullptr;
+    float* grad = nullptr;     // every aw and ab in the order of the parameters
     float* loss = nullptr;
     float* hloss = nullptr;
 };
@@ -116,13 +121,20 @@ struct qpat_unet_s {
 namespace {
 
 template <typename T>
-int ualloc(qpat_unet_s* U, T** p, size_t count) {
+int alloc_in(std::vector<void*>& list, T** p, size_t count) {
     void* v = nullptr;
-    cudaError_t e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(T));
+    const cudaError_t e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(T));
     if (e != cudaSuccess) return cuda_fail(e, "qpat_unet: cudaMalloc");
-    U->allocs.push_back(v);
+    list.push_back(v);
     *p = static_cast<T*>(v);
-    e = cudaMemset(v, 0, std::max<size_t>(count, 1) * sizeof(T));
+    return QPAT_OK;
+}
+
+template <typename T>
+int ualloc(qpat_unet_s* U, T** p, size_t count) {
+    const int rc = alloc_in(U->allocs, p, count);
+    if (rc != QPAT_OK) return rc;
+    const cudaError_t e = cudaMemset(*p, 0, std::max<size_t>(count, 1) * sizeof(T));
     return e == cudaSuccess ? QPAT_OK : cuda_fail(e, "qpat_unet: memset");
 }
 
@@ -132,83 +144,177 @@ int ualloc(qpat_unet_s* U, T** p, size_t count) {
         if (e_ != cudaSuccess) return cuda_fail(e_, #x); \
     } while (0)
 
-int conv_fwd(const Conv& c, const bf16* in, bf16* out, float* out32, int n, cudaStream_t s) {
-    UCK(unet::conv3d_fwd(in, c.cin, c.w, c.b32, c.cout, c.relu, out, out32, n, s));
+// Samples that go through the network at once: all of a call's, as far as
+// their activations take at most kActBytes (at least one sample; the layers of
+// a coarse level of one sample fill a few SMs only).
+constexpr size_t kActBytes = size_t(8) << 30;
+constexpr int kMaxSamples = 64;
+
+// Room for min(B, what kActBytes holds) samples, also for training; kept for
+// later calls, grown (after the stream has finished with it) on demand.
+int reserve(qpat_unet_s* U, int B, bool train, cudaStream_t s) {
+    const int64_t v0 = int64_t(U->n) * U->n * U->n, v1 = v0 / 8, v2 = v1 / 8, v3 = v2 / 8;
+    const size_t fwd = 2 * size_t(v0 * 80 + v1 * 176 + v2 * 352 + v3 * 320);
+    const size_t bwd = 2 * size_t(v0 * 176 + v1 * 352 + v2 * 704 + v3 * 320) + 4 * size_t(v0);
+    auto fit = [&](size_t bytes) { return int(std::max<size_t>(1, std::min<size_t>(size_t(std::min(B, kMaxSamples)), kActBytes / bytes))); };
+    auto release = [&](std::vector<void*>& list, int& cap) {
+        for (void* p : list) cudaFree(p);
+        list.clear();
+        cap = 0;
+    };
+    int want = fit(train ? fwd + bwd : fwd), rc = QPAT_OK;
+    if (want > U->cap) {
+        UCK(cudaStreamSynchronize(s));
+        for (;; want = 1) {  // not enough memory for several: one
+            release(U->acts, U->cap);
+            rc = QPAT_OK;
+            auto A = [&](bf16** p, int64_t nv, int ch) { if (!rc) rc = alloc_in(U->acts, p, size_t(nv) * ch * want); };
+            A(&U->xin, v0, 16); A(&U->a0, v0, 16); A(&U->s0, v0, 16); A(&U->p0, v1, 16); A(&U->a1, v1, 32);
+            A(&U->s1, v1, 32); A(&U->p1, v2, 32); A(&U->a2, v2, 64); A(&U->s2, v2, 64); A(&U->p2, v3, 64);
+            A(&U->a3, v3, 128); A(&U->bt, v3, 128); A(&U->a4, v2, 64); A(&U->d2, v2, 64); A(&U->a5, v1, 32);
+            A(&U->d1, v1, 32); A(&U->a6, v0, 16); A(&U->d0, v0, 16);
+            if (!rc || want == 1) break;
+        }
+        if (rc) {
+            release(U->acts, U->cap);
+            return rc;
+        }
+        U->cap = want;
+    }
+    if (train && std::min(want, U->cap) > U->train_cap) {
+        UCK(cudaStreamSynchronize(s));
+        for (want = std::min(want, U->cap);; want = 1) {
+            release(U->train_acts, U->train_cap);
+            rc = QPAT_OK;
+            auto A = [&](bf16** p, int64_t nv, int ch) { if (!rc) rc = alloc_in(U->train_acts, p, size_t(nv) * ch * want); };
+            A(&U->cat2, v2, 192); A(&U->cat1, v1, 96); A(&U->cat0, v0, 48);
+            A(&U->g_y, v0, 16); A(&U->g_d0, v0, 16); A(&U->g_a6, v0, 16); A(&U->g_cat0, v0, 48); A(&U->g_d1, v1, 32);
+            A(&U->g_s0, v0, 16); A(&U->g_a5, v1, 32); A(&U->g_cat1, v1, 96); A(&U->g_d2, v2, 64); A(&U->g_s1, v1, 32);
+            A(&U->g_a4, v2, 64); A(&U->g_cat2, v2, 192); A(&U->g_bt, v3, 128); A(&U->g_s2, v2, 64); A(&U->g_a3, v3, 128);
+            A(&U->g_p2, v3, 64); A(&U->g_a2, v2, 64); A(&U->g_p1, v2, 32); A(&U->g_a1, v1, 32); A(&U->g_p0, v1, 16);
+            A(&U->g_a0, v0, 16);
+            if (!rc) rc = alloc_in(U->train_acts, &U->y, size_t(v0) * want);
+            size_t scratch = 0;
+            for (int b = 1; b <= want; ++b)  // the chunking of a smaller batch may need more
+                for (const Conv& c : U->conv) scratch = std::max(scratch, unet::wgrad_scratch(U->lv[c.lvl], c.cin, c.cout, b));
+            if (!rc) rc = alloc_in(U->train_acts, &U->partial, scratch);
+            if (!rc || want == 1) break;
+        }
+        if (rc) {
+            release(U->train_acts, U->train_cap);
+            return rc;
+        }
+        U->train_cap = want;
+    }
     return QPAT_OK;
+}
+
+// One convolution of B samples.  On the tcgen05 engine one launch, which reads
+// a concatenation from its two parts; the mma.sync engine goes sample by
+// sample through materialised tensors.
+int conv_fwd(qpat_unet_s* U, const Conv& c, const bf16* w, int Cout, const float* bias, int relu,
+             const unet::ConvInput& in, const unet::ConvOutput& out, int n, int B, cudaStream_t s) {
+    const int Cin = in.Clo + in.Cskip;
+    if (unet::conv_engine() == 0 && unet::conv3d_fwd_tc_supported(Cin, Cout)) {
+        UCK(unet::conv3d_fwd_tc(in, w, bias, Cout, relu, out, n, B, s));
+        return QPAT_OK;
+    }
+    const int64_t v0 = int64_t(U->n) * U->n * U->n, nv = int64_t(n) * n * n;
+    int rc = QPAT_OK;
+    if (!U->mcat && (rc = ualloc(U, &U->mcat, size_t(v0) * 48))) return rc;
+    if (!U->mout && (rc = ualloc(U, &U->mout, size_t(v0) * 16))) return rc;
+    if (!U->mout32 && (rc = ualloc(U, &U->mout32, size_t(v0) * 16))) return rc;
+    for (int b = 0; b < B; ++b) {
+        const bf16* x = in.skip + b * nv * in.Cskip;
+        if (in.lo) {
+            UCK(unet::upcat(in.lo + b * (nv / 8) * in.Clo, in.Clo, x, in.Cskip, n, 1, U->mcat, s));
+            x = U->mcat;
+        }
+        UCK(unet::conv3d_fwd(x, Cin, w, bias, Cout, relu, out.bf ? out.bf + b * nv * Cout : U->mout,
+                             out.first ? U->mout32 : out.f32, n, s));
+        if (out.first) {
+            qpat::note_launch(1);
+            k_take_channel0<<<g1(nv), 256, 0, s>>>(nv, U->mout32, out.first + b * nv, out.first_exp ? 1.f : 0.f);
+        }
+    }
+    (void)c;
+    return QPAT_OK;
+}
+
+int conv_fwd(qpat_unet_s* U, const Conv& c, const unet::ConvInput& in, bf16* out, int n, int B, cudaStream_t s) {
+    return conv_fwd(U, c, c.w, c.cout, c.b32, c.relu, in, unet::ConvOutput{out}, n, B, s);
 }
 
 // backward of one conv: gout (gradient of its output, masked here by the
-// ReLU through `out`) -> weight/bias gradient, and gin if not null
-int conv_bwd(qpat_unet_s* U, Conv& c, const bf16* in, const bf16* out, bf16* gout, bf16* gin, int n,
+// ReLU through `out`) -> weight/bias gradient (added to what is there when
+// add is set), and gin if not null
+int conv_bwd(qpat_unet_s* U, Conv& c, const bf16* in, const bf16* out, bf16* gout, bf16* gin, int n, int B, int add,
              cudaStream_t s) {
-    const int64_t nv = int64_t(n) * n * n;
+    const int64_t nv = int64_t(n) * n * n * B;
     if (c.relu) UCK(unet::relu_mask(gout, out, nv * c.cout, s));
-    UCK(unet::conv3d_wgrad(in, c.cin, gout, c.cout, c.gw, c.gb, U->partial, n, s));
-    if (gin) UCK(unet::conv3d_fwd(gout, c.cout, c.wt, nullptr, c.cin, 0, gin, nullptr, n, s));
+    UCK(unet::conv3d_wgrad(in, c.cin, gout, c.cout, c.aw, c.ab, U->partial, n, B, add, s));
+    if (gin) return conv_fwd(U, c, c.wt, c.cin, nullptr, 0, unet::ConvInput{gout, c.cout}, unet::ConvOutput{gin}, n, B, s);
     return QPAT_OK;
 }
 
-int unet_forward(qpat_unet_s* U, cudaStream_t s) {
+// The network on B samples in xin; y (B n^3 floats) receives channel 0 of the
+// last layer (y_exp: its exponential).  train: the concatenations are also
+// written out for the backward pass.
+int unet_forward(qpat_unet_s* U, int B, bool train, float* y, int y_exp, cudaStream_t s) {
     auto& C = U->conv;
+    using In = unet::ConvInput;
     const int n0 = U->lv[0], n1 = U->lv[1], n2 = U->lv[2], n3 = U->lv[3];
     int rc;
-    if ((rc = conv_fwd(C[0], U->xin, U->a0, nullptr, n0, s)) || (rc = conv_fwd(C[1], U->a0, U->s0, nullptr, n0, s)))
+    if ((rc = conv_fwd(U, C[0], In{U->xin, 16}, U->a0, n0, B, s)) || (rc = conv_fwd(U, C[1], In{U->a0, 16}, U->s0, n0, B, s)))
         return rc;
-    UCK(unet::avgpool(U->s0, 16, n0, U->p0, s));
-    if ((rc = conv_fwd(C[2], U->p0, U->a1, nullptr, n1, s)) || (rc = conv_fwd(C[3], U->a1, U->s1, nullptr, n1, s)))
+    UCK(unet::avgpool(U->s0, 16, n0, B, U->p0, s));
+    if ((rc = conv_fwd(U, C[2], In{U->p0, 16}, U->a1, n1, B, s)) || (rc = conv_fwd(U, C[3], In{U->a1, 32}, U->s1, n1, B, s)))
         return rc;
-    UCK(unet::avgpool(U->s1, 32, n1, U->p1, s));
-    if ((rc = conv_fwd(C[4], U->p1, U->a2, nullptr, n2, s)) || (rc = conv_fwd(C[5], U->a2, U->s2, nullptr, n2, s)))
+    UCK(unet::avgpool(U->s1, 32, n1, B, U->p1, s));
+    if ((rc = conv_fwd(U, C[4], In{U->p1, 32}, U->a2, n2, B, s)) || (rc = conv_fwd(U, C[5], In{U->a2, 64}, U->s2, n2, B, s)))
         return rc;
-    UCK(unet::avgpool(U->s2, 64, n2, U->p2, s));
-    if ((rc = conv_fwd(C[6], U->p2, U->a3, nullptr, n3, s)) || (rc = conv_fwd(C[7], U->a3, U->bt, nullptr, n3, s)))
+    UCK(unet::avgpool(U->s2, 64, n2, B, U->p2, s));
+    if ((rc = conv_fwd(U, C[6], In{U->p2, 64}, U->a3, n3, B, s)) || (rc = conv_fwd(U, C[7], In{U->a3, 128}, U->bt, n3, B, s)))
         return rc;
-    UCK(unet::upcat(U->bt, 128, U->s2, 64, n2, U->cat2, s));
-    if ((rc = conv_fwd(C[8], U->cat2, U->a4, nullptr, n2, s)) || (rc = conv_fwd(C[9], U->a4, U->d2, nullptr, n2, s)))
-        return rc;
-    UCK(unet::upcat(U->d2, 64, U->s1, 32, n1, U->cat1, s));
-    if ((rc = conv_fwd(C[10], U->cat1, U->a5, nullptr, n1, s)) ||
-        (rc = conv_fwd(C[11], U->a5, U->d1, nullptr, n1, s)))
-        return rc;
-    UCK(unet::upcat(U->d1, 32, U->s0, 16, n0, U->cat0, s));
-    if ((rc = conv_fwd(C[12], U->cat0, U->a6, nullptr, n0, s)) ||
-        (rc = conv_fwd(C[13], U->a6, U->d0, nullptr, n0, s)) || (rc = conv_fwd(C[14], U->d0, U->yb, U->y32, n0, s)))
-        return rc;
-    return QPAT_OK;
+    auto cat = [&](const bf16* lo, int clo, const bf16* skip, int cs, int n, bf16* to, In& in) -> cudaError_t {
+        in = train ? In{to, clo + cs} : In{skip, cs, lo, clo};
+        return train ? unet::upcat(lo, clo, skip, cs, n, B, to, s) : cudaSuccess;
+    };
+    In in{};
+    UCK(cat(U->bt, 128, U->s2, 64, n2, U->cat2, in));
+    if ((rc = conv_fwd(U, C[8], in, U->a4, n2, B, s)) || (rc = conv_fwd(U, C[9], In{U->a4, 64}, U->d2, n2, B, s))) return rc;
+    UCK(cat(U->d2, 64, U->s1, 32, n1, U->cat1, in));
+    if ((rc = conv_fwd(U, C[10], in, U->a5, n1, B, s)) || (rc = conv_fwd(U, C[11], In{U->a5, 32}, U->d1, n1, B, s))) return rc;
+    UCK(cat(U->d1, 32, U->s0, 16, n0, U->cat0, in));
+    if ((rc = conv_fwd(U, C[12], in, U->a6, n0, B, s)) || (rc = conv_fwd(U, C[13], In{U->a6, 16}, U->d0, n0, B, s))) return rc;
+    unet::ConvOutput out;
+    out.first = y;
+    out.first_exp = y_exp;
+    return conv_fwd(U, C[14], C[14].w, 16, C[14].b32, 0, In{U->d0, 16}, out, n0, B, s);
 }
 
-int unet_backward(qpat_unet_s* U, cudaStream_t s) {
+int unet_backward(qpat_unet_s* U, int B, int add, cudaStream_t s) {
     auto& C = U->conv;
     const int n0 = U->lv[0], n1 = U->lv[1], n2 = U->lv[2], n3 = U->lv[3];
     int rc;
-    if ((rc = conv_bwd(U, C[14], U->d0, U->yb, U->g_y, U->g_d0, n0, s)) ||
-        (rc = conv_bwd(U, C[13], U->a6, U->d0, U->g_d0, U->g_a6, n0, s)) ||
-        (rc = conv_bwd(U, C[12], U->cat0, U->a6, U->g_a6, U->g_cat0, n0, s)))
+    auto bwd = [&](int i, const bf16* in, const bf16* out, bf16* gout, bf16* gin, int n) {
+        return rc = conv_bwd(U, C[size_t(i)], in, out, gout, gin, n, B, add, s);
+    };
+    if (bwd(14, U->d0, nullptr, U->g_y, U->g_d0, n0) || bwd(13, U->a6, U->d0, U->g_d0, U->g_a6, n0) ||
+        bwd(12, U->cat0, U->a6, U->g_a6, U->g_cat0, n0))
         return rc;
-    UCK(unet::upcat_bwd(U->g_cat0, 32, 16, n0, U->g_d1, U->g_s0, 0, s));
-    if ((rc = conv_bwd(U, C[11], U->a5, U->d1, U->g_d1, U->g_a5, n1, s)) ||
-        (rc = conv_bwd(U, C[10], U->cat1, U->a5, U->g_a5, U->g_cat1, n1, s)))
-        return rc;
-    UCK(unet::upcat_bwd(U->g_cat1, 64, 32, n1, U->g_d2, U->g_s1, 0, s));
-    if ((rc = conv_bwd(U, C[9], U->a4, U->d2, U->g_d2, U->g_a4, n2, s)) ||
-        (rc = conv_bwd(U, C[8], U->cat2, U->a4, U->g_a4, U->g_cat2, n2, s)))
-        return rc;
-    UCK(unet::upcat_bwd(U->g_cat2, 128, 64, n2, U->g_bt, U->g_s2, 0, s));
-    if ((rc = conv_bwd(U, C[7], U->a3, U->bt, U->g_bt, U->g_a3, n3, s)) ||
-        (rc = conv_bwd(U, C[6], U->p2, U->a3, U->g_a3, U->g_p2, n3, s)))
-        return rc;
-    UCK(unet::avgpool_bwd(U->g_p2, 64, n2, U->g_s2, 1, s));
-    if ((rc = conv_bwd(U, C[5], U->a2, U->s2, U->g_s2, U->g_a2, n2, s)) ||
-        (rc = conv_bwd(U, C[4], U->p1, U->a2, U->g_a2, U->g_p1, n2, s)))
-        return rc;
-    UCK(unet::avgpool_bwd(U->g_p1, 32, n1, U->g_s1, 1, s));
-    if ((rc = conv_bwd(U, C[3], U->a1, U->s1, U->g_s1, U->g_a1, n1, s)) ||
-        (rc = conv_bwd(U, C[2], U->p0, U->a1, U->g_a1, U->g_p0, n1, s)))
-        return rc;
-    UCK(unet::avgpool_bwd(U->g_p0, 16, n0, U->g_s0, 1, s));
-    if ((rc = conv_bwd(U, C[1], U->a0, U->s0, U->g_s0, U->g_a0, n0, s)) ||
-        (rc = conv_bwd(U, C[0], U->xin, U->a0, U->g_a0, nullptr, n0, s)))
-        return rc;
+    UCK(unet::upcat_bwd(U->g_cat0, 32, 16, n0, B, U->g_d1, U->g_s0, 0, s));
+    if (bwd(11, U->a5, U->d1, U->g_d1, U->g_a5, n1) || bwd(10, U->cat1, U->a5, U->g_a5, U->g_cat1, n1)) return rc;
+    UCK(unet::upcat_bwd(U->g_cat1, 64, 32, n1, B, U->g_d2, U->g_s1, 0, s));
+    if (bwd(9, U->a4, U->d2, U->g_d2, U->g_a4, n2) || bwd(8, U->cat2, U->a4, U->g_a4, U->g_cat2, n2)) return rc;
+    UCK(unet::upcat_bwd(U->g_cat2, 128, 64, n2, B, U->g_bt, U->g_s2, 0, s));
+    if (bwd(7, U->a3, U->bt, U->g_bt, U->g_a3, n3) || bwd(6, U->p2, U->a3, U->g_a3, U->g_p2, n3)) return rc;
+    UCK(unet::avgpool_bwd(U->g_p2, 64, n2, B, U->g_s2, 1, s));
+    if (bwd(5, U->a2, U->s2, U->g_s2, U->g_a2, n2) || bwd(4, U->p1, U->a2, U->g_a2, U->g_p1, n2)) return rc;
+    UCK(unet::avgpool_bwd(U->g_p1, 32, n1, B, U->g_s1, 1, s));
+    if (bwd(3, U->a1, U->s1, U->g_s1, U->g_a1, n1) || bwd(2, U->p0, U->a1, U->g_a1, U->g_p0, n1)) return rc;
+    UCK(unet::avgpool_bwd(U->g_p0, 16, n0, B, U->g_s0, 1, s));
+    if (bwd(1, U->a0, U->s0, U->g_s0, U->g_a0, n0) || bwd(0, U->xin, U->a0, U->g_a0, nullptr, n0)) return rc;
     return QPAT_OK;
 }
 
@@ -239,7 +345,6 @@ int qpat_unet_create(int n, uint64_t seed, qpat_unet_t* out) {
                              {96, 32, 1, 1},  {32, 32, 1, 1},  {48, 16, 0, 1},  {16, 16, 0, 1},  {16, 16, 0, 0}};
     std::mt19937_64 rng(seed);
     int rc = QPAT_OK;
-    const int64_t v0 = int64_t(n) * n * n, v1 = v0 / 8, v2 = v1 / 8, v3 = v2 / 8;
     for (int i = 0; i < 15 && rc == QPAT_OK; ++i) {
         Conv c;
         c.cin = spec[i][0];
@@ -248,9 +353,7 @@ int qpat_unet_create(int n, uint64_t seed, qpat_unet_t* out) {
         c.relu = spec[i][3];
         const int64_t nw = c.nw();
         if ((rc = ualloc(U, &c.w32, nw)) || (rc = ualloc(U, &c.b32, c.cout)) || (rc = ualloc(U, &c.w, nw)) ||
-            (rc = ualloc(U, &c.wt, nw)) || (rc = ualloc(U, &c.gw, nw)) || (rc = ualloc(U, &c.gb, c.cout)) ||
-            (rc = ualloc(U, &c.aw, nw)) || (rc = ualloc(U, &c.ab, c.cout)) || (rc = ualloc(U, &c.mw, nw)) ||
-            (rc = ualloc(U, &c.vw, nw)) || (rc = ualloc(U, &c.mb, c.cout)) || (rc = ualloc(U, &c.vb, c.cout)))
+            (rc = ualloc(U, &c.wt, nw)) || (rc = ualloc(U, &c.mw, nw)) || (rc = ualloc(U, &c.vw, nw)) || (rc = ualloc(U, &c.mb, c.cout)) || (rc = ualloc(U, &c.vb, c.cout)))
             break;
         // He-normal initialisation over the real fan-in (the first conv sees 3 channels)
         const int fan = 27 * (i == 0 ? 3 : c.cin);
@@ -264,19 +367,18 @@ int qpat_unet_create(int n, uint64_t seed, qpat_unet_t* out) {
             rc = cuda_fail(cudaGetLastError(), "qpat_unet_create: upload");
         U->conv.push_back(c);
     }
-    auto A = [&](bf16** p, int64_t nv, int ch) { return rc ? rc : (rc = ualloc(U, p, size_t(nv) * ch)); };
-    A(&U->xin, v0, 16); A(&U->a0, v0, 16); A(&U->s0, v0, 16); A(&U->p0, v1, 16); A(&U->a1, v1, 32);
-    A(&U->s1, v1, 32); A(&U->p1, v2, 32); A(&U->a2, v2, 64); A(&U->s2, v2, 64); A(&U->p2, v3, 64);
-    A(&U->a3, v3, 128); A(&U->bt, v3, 128); A(&U->cat2, v2, 192); A(&U->a4, v2, 64); A(&U->d2, v2, 64);
-    A(&U->cat1, v1, 96); A(&U->a5, v1, 32); A(&U->d1, v1, 32); A(&U->cat0, v0, 48); A(&U->a6, v0, 16);
-    A(&U->d0, v0, 16); A(&U->yb, v0, 16);
-    A(&U->g_y, v0, 16); A(&U->g_d0, v0, 16); A(&U->g_a6, v0, 16); A(&U->g_cat0, v0, 48); A(&U->g_d1, v1, 32);
-    A(&U->g_s0, v0, 16); A(&U->g_a5, v1, 32); A(&U->g_cat1, v1, 96); A(&U->g_d2, v2, 64); A(&U->g_s1, v1, 32);
-    A(&U->g_a4, v2, 64); A(&U->g_cat2, v2, 192); A(&U->g_bt, v3, 128); A(&U->g_s2, v2, 64); A(&U->g_a3, v3, 128);
-    A(&U->g_p2, v3, 64); A(&U->g_a2, v2, 64); A(&U->g_p1, v2, 32); A(&U->g_a1, v1, 32); A(&U->g_p0, v1, 16);
-    A(&U->g_a0, v0, 16);
-    if (!rc) rc = ualloc(U, &U->y32, size_t(v0) * 16);
-    if (!rc) rc = ualloc(U, &U->partial, size_t(unet::wgrad_chunks(n)) * 27 * 192 * 128);
+    size_t total = 0;
+    for (const Conv& c : U->conv) total += size_t(c.nw()) + c.cout;
+    if (!rc) rc = ualloc(U, &U->grad, total);
+    if (!rc) {
+        float* g = U->grad;
+        for (Conv& c : U->conv) {
+            c.aw = g;
+            c.ab = g + c.nw();
+            g = c.ab + c.cout;
+        }
+        rc = reserve(U, 1, false, nullptr);
+    }
     if (!rc) rc = ualloc(U, &U->loss, 1);
     if (!rc && cudaMallocHost(&U->hloss, sizeof(float)) != cudaSuccess) rc = fail(QPAT_ECUDA, "qpat_unet: pinned");
     if (!rc) rc = refresh_bf16(U, nullptr);
@@ -293,7 +395,8 @@ void qpat_unet_free(qpat_unet_t U) {
     if (!U) return;
     DeviceGuard dg(U->device);
     cudaDeviceSynchronize();
-    for (void* p : U->allocs) cudaFree(p);
+    for (auto* list : {&U->allocs, &U->acts, &U->train_acts})
+        for (void* p : *list) cudaFree(p);
     if (U->hloss) cudaFreeHost(U->hloss);
     delete U;
 }
@@ -337,13 +440,13 @@ int qpat_unet_predict_dev(qpat_unet_t U, const float* x, int B, float* y, void* 
     DeviceGuard dg(U->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t nv = int64_t(U->n) * U->n * U->n;
-    for (int b = 0; b < B; ++b) {
+    int rc = reserve(U, B, false, s);
+    if (rc) return rc;
+    for (int b = 0; b < B; b += U->cap) {
+        const int nb = std::min(U->cap, B - b);
         qpat::note_launch(1);
-        k_pack_input<<<g1(nv * 16), 256, 0, s>>>(nv, x + b * nv * 3, U->xin);
-        int rc = unet_forward(U, s);
-        if (rc) return rc;
-        qpat::note_launch(1);
-        k_take_channel0<<<g1(nv), 256, 0, s>>>(nv, U->y32, y + b * nv, U->log_floor);
+        k_pack_input<<<g1(nv * nb * 16), 256, 0, s>>>(nv * nb, x + b * nv * 3, U->xin);
+        if ((rc = unet_forward(U, nb, false, y + b * nv, U->log_floor > 0.f, s))) return rc;
     }
     UCK(cudaGetLastError());
     return QPAT_OK;
@@ -354,21 +457,18 @@ int qpat_unet_predict_dev(qpat_unet_t U, const float* x, int B, float* y, void* 
 // aw, ab (summed over the samples).
 static int unet_loss_grad(qpat_unet_s* U, const float* x, const float* t, int B, cudaStream_t s) {
     const int64_t nv = int64_t(U->n) * U->n * U->n;
+    int rc = reserve(U, B, true, s);
+    if (rc) return rc;
     UCK(cudaMemsetAsync(U->loss, 0, sizeof(float), s));
-    for (int b = 0; b < B; ++b) {
+    const int cap = std::min(U->cap, U->train_cap);
+    for (int b = 0; b < B; b += cap) {
+        const int nb = std::min(cap, B - b);
         qpat::note_launch(1);
-        k_pack_input<<<g1(nv * 16), 256, 0, s>>>(nv, x + b * nv * 3, U->xin);
-        int rc = unet_forward(U, s);
-        if (rc) return rc;
+        k_pack_input<<<g1(nv * nb * 16), 256, 0, s>>>(nv * nb, x + b * nv * 3, U->xin);
+        if ((rc = unet_forward(U, nb, true, U->y, 0, s))) return rc;
         qpat::note_launch(1);
-        k_mse<<<g1(nv), 256, 0, s>>>(nv, U->y32, t + b * nv, 1.f / float(nv * B), U->g_y, U->loss, U->log_floor);
-        if ((rc = unet_backward(U, s))) return rc;
-        for (auto& c : U->conv) {
-            qpat::note_launch(1);
-            k_axpy32<<<g1(c.nw()), 256, 0, s>>>(c.nw(), 1.f, c.gw, c.aw, b == 0);
-            qpat::note_launch(1);
-            k_axpy32<<<1, 256, 0, s>>>(c.cout, 1.f, c.gb, c.ab, b == 0);
-        }
+        k_mse<<<g1(nv * nb), 256, 0, s>>>(nv * nb, U->y, t + b * nv, 1.f / float(nv * B), U->g_y, U->loss, U->log_floor);
+        if ((rc = unet_backward(U, nb, b > 0, s))) return rc;
     }
     UCK(cudaGetLastError());
     return QPAT_OK;
@@ -381,13 +481,7 @@ int qpat_unet_grad_dev(qpat_unet_t U, const float* x, const float* t, int B, flo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int rc = unet_loss_grad(U, x, t, B, s);
     if (rc) return rc;
-    size_t o = 0;
-    for (auto& c : U->conv) {
-        UCK(cudaMemcpyAsync(grad + o, c.aw, sizeof(float) * c.nw(), cudaMemcpyDeviceToHost, s));
-        o += c.nw();
-        UCK(cudaMemcpyAsync(grad + o, c.ab, sizeof(float) * c.cout, cudaMemcpyDeviceToHost, s));
-        o += c.cout;
-    }
+    UCK(cudaMemcpyAsync(grad, U->grad, sizeof(float) * size_t(qpat_unet_num_params(U)), cudaMemcpyDeviceToHost, s));
     UCK(cudaMemcpyAsync(U->hloss, U->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
     UCK(cudaStreamSynchronize(s));
     if (loss) *loss = *U->hloss;
@@ -466,7 +560,7 @@ int qpat_conv3d_bf16_dev(const void* in, int Cin, const void* w, const float* bi
 int qpat_conv3d_bf16_wgrad_dev(const void* in, int Cin, const void* dy, int Cout, int n, float* dw, float* db,
                                float* partial, void* stream) {
     if (!in || !dy || !dw || !partial) return fail(QPAT_EINVAL, "qpat_conv3d_bf16_wgrad_dev: NULL argument");
-    UCK(unet::conv3d_wgrad(static_cast<const bf16*>(in), Cin, static_cast<const bf16*>(dy), Cout, dw, db, partial, n,
+    UCK(unet::conv3d_wgrad(static_cast<const bf16*>(in), Cin, static_cast<const bf16*>(dy), Cout, dw, db, partial, n, 1, 0,
                            static_cast<cudaStream_t>(stream)));
     return QPAT_OK;
 }
@@ -480,7 +574,7 @@ int qpat_conv3d_set_engine(int engine) {
 int qpat_conv3d_tc_timeouts(void) { return unet::tc_timeouts(); }
 
 int64_t qpat_conv3d_bf16_wgrad_scratch(int n, int Cin, int Cout) {
-    return int64_t(unet::wgrad_chunks(n)) * 27 * Cin * Cout;
+    return int64_t(unet::wgrad_scratch(n, Cin, Cout, 1));
 }
 
 }  // extern "C"

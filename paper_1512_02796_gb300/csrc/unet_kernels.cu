@@ -119,49 +119,99 @@ cudaError_t conv_fwd_t(const bf16* in, int Cin, const bf16* w, const float* bias
     return cudaGetLastError();
 }
 
-// partial[chunk][tap][co][ci] = sum_{v in chunk} dy[v][co] * in[nbr(v, tap)][ci]
-constexpr int kWgradVox = 8192;  // voxels per chunk
+// Weight gradient: partial[chunk][tap][co][ci] = sum_{v in chunk} dy[v][co] in[nbr(v, tap)][ci]
+// and, from the centre tap's CTAs, bias[chunk][co] = sum dy[v][co].  A CTA
+// takes a chunk of voxels, a tap and 16 output channels; 64 voxels at a time
+// are copied to shared memory (16-byte cp.async, zeros outside the grid, the
+// next 64 under the current ones' MMAs), and each warp multiplies 16 of them:
+// both operands lie voxel by voxel, so their fragments come by transposed
+// ldmatrix.  Chunks are sized so that the CTAs fill the GPU (a grid of 4^3
+// voxels as well as one of 128^3); their sums are added in order by
+// k_sum_chunks.  Bound: shared-memory and L2 reads of `in`, once per tap.
+constexpr int kWgThreads = 128, kWgStep = 64;
+constexpr int kWgradVoxMin = 256, kWgradVoxMax = 8192;
+
+int64_t wgrad_chunk_voxels(int64_t voxels, int Cout) {
+    int64_t c = kWgradVoxMax;
+    while (c > kWgradVoxMin && (voxels + c - 1) / c * 27 * (Cout / 16) < 1024) c /= 2;
+    return c;
+}
+
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const bf16* p) {
+    const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+}
+
+__device__ __forceinline__ void copy16(bf16* dst, const bf16* src, bool ok) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
 
 template <int NCI>
-__global__ void __launch_bounds__(128) k_conv_wgrad(const bf16* __restrict__ in, int Cin,
-                                                    const bf16* __restrict__ dy, int Cout,
-                                                    float* __restrict__ partial, int n) {
-    __shared__ float red[16][NCI * 8 + 1];
-    const int nvox = n * n * n;
+__global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dy,
+                                                           int Cout, float* __restrict__ partial,
+                                                           float* __restrict__ bias, int n, int64_t voxels,
+                                                           int64_t chunk_voxels) {
+    constexpr int Cin = 8 * NCI, LI = Cin + 8, LD = 16 + 8;  // padded rows: fragment rows fall into different banks
+    extern __shared__ __align__(16) unsigned char wg_smem[];
+    bf16* sIn = reinterpret_cast<bf16*>(wg_smem);         // 2 x kWgStep x LI
+    bf16* sDy = sIn + 2 * kWgStep * LI;                   // 2 x kWgStep x LD
+    __shared__ float red[16][Cin + 1];
     const int chunk = blockIdx.x, tap = blockIdx.y, co0 = blockIdx.z * 16;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int vbeg = chunk * kWgradVox, vend = min(nvox, vbeg + kWgradVox);
+    const int64_t vbeg = chunk * chunk_voxels, vend = min(voxels, vbeg + chunk_voxels);
+    const int64_t shift = (int64_t(tap / 9 - 1) * n + (tap / 3 % 3 - 1)) * n + (tap % 3 - 1);
+    auto load = [&](int64_t v0, int st) {
+        for (int i = threadIdx.x; i < kWgStep * NCI; i += kWgThreads) {
+            const int64_t v = v0 + i / NCI;
+            bool ok = v < vend;
+            if (ok) {
+                const int x = int(v % n), y = int(v / n % n), z = int(v / (int64_t(n) * n) % n);
+                ok = nbr(z, y, x, tap, n) >= 0;
+            }
+            copy16(sIn + (st * kWgStep + i / NCI) * LI + i % NCI * 8, ok ? in + (v + shift) * Cin + i % NCI * 8 : in, ok);
+        }
+        for (int i = threadIdx.x; i < kWgStep * 2; i += kWgThreads) {
+            const int64_t v = v0 + i / 2;
+            const bool ok = v < vend;
+            copy16(sDy + (st * kWgStep + i / 2) * LD + i % 2 * 8, ok ? dy + v * Cout + co0 + i % 2 * 8 : dy, ok);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     float acc[NCI][4];
 #pragma unroll
     for (int i = 0; i < NCI; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-    for (int vb = vbeg + warp * 16; vb < vend; vb += 64) {
-        // A (16 c_out x 16 voxels): A[co][v] = dy[v][co]
-        const int va = vb + 2 * t, vc = vb + 2 * t + 8;
+    float db = 0.f;
+    load(vbeg, 0);
+    int st = 0;
+    for (int64_t v0 = vbeg; v0 < vend; v0 += kWgStep, st ^= 1) {
+        load(v0 + kWgStep, st ^ 1);  // past the end: zeros
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        const bf16* d = sDy + (st * kWgStep + warp * 16) * LD;
+        const bf16* x = sIn + (st * kWgStep + warp * 16) * LI;
+        // the four 8 x 8 blocks of a 16 (voxels) x 16 (channels) tile, transposed: lane l addresses row l % 8 of block l / 8
+        const int vr = lane & 7, hi8 = (lane >> 3) & 1, hi16 = lane >> 4;
         uint32_t a[4];
-        a[0] = pack2(dy[size_t(va) * Cout + co0 + g], dy[size_t(va + 1) * Cout + co0 + g]);
-        a[1] = pack2(dy[size_t(va) * Cout + co0 + g + 8], dy[size_t(va + 1) * Cout + co0 + g + 8]);
-        a[2] = pack2(dy[size_t(vc) * Cout + co0 + g], dy[size_t(vc + 1) * Cout + co0 + g]);
-        a[3] = pack2(dy[size_t(vc) * Cout + co0 + g + 8], dy[size_t(vc + 1) * Cout + co0 + g + 8]);
-        // B (16 voxels x 8 c_in): B[v][ci] = in[nbr(v, tap)][ci]
-        int nb[4];
-        const int vv[4] = {va, va + 1, vc, vc + 1};
+        ldsm4t(a, d + (vr + 8 * hi16) * LD + 8 * hi8);  // A[co][v]: blocks (co 0-7, v 0-7), (co 8-15, v 0-7), (.., v 8-15)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int v = vv[k];
-            nb[k] = nbr(v / (n * n), (v / n) % n, v % n, tap, n);
+        for (int c = 0; c < NCI; c += 2) {
+            uint32_t b[4];
+            ldsm4t(b, x + (vr + 8 * hi8) * LI + 8 * (c + hi16));  // B[v][ci]: (v 0-7, v 8-15) of ci block c, then of c + 1
+            const uint32_t b0[2] = {b[0], b[1]}, b1[2] = {b[2], b[3]};
+            mma_bf16(acc[c], a, b0);
+            mma_bf16(acc[c + 1], a, b1);
         }
-        const bf16 zero = __float2bfloat16(0.f);
-#pragma unroll
-        for (int nc = 0; nc < NCI; ++nc) {
-            const int ci = nc * 8 + g;
-            const bf16 e0 = nb[0] >= 0 ? in[size_t(nb[0]) * Cin + ci] : zero;
-            const bf16 e1 = nb[1] >= 0 ? in[size_t(nb[1]) * Cin + ci] : zero;
-            const bf16 e2 = nb[2] >= 0 ? in[size_t(nb[2]) * Cin + ci] : zero;
-            const bf16 e3 = nb[3] >= 0 ? in[size_t(nb[3]) * Cin + ci] : zero;
-            const uint32_t b[2] = {pack2(e0, e1), pack2(e2, e3)};
-            mma_bf16(acc[nc], a, b);
+        if (tap == 13) {
+            const int co = threadIdx.x & 15, part = threadIdx.x >> 4;
+            for (int v = part; v < kWgStep; v += kWgThreads / 16) db += __bfloat162float(sDy[(st * kWgStep + v) * LD + co]);
         }
+        __syncthreads();
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     // reduce the 4 warps in turn: C fragment rows co (g, g+8), columns ci (2t, 2t+1)
     for (int w = 0; w < 4; ++w) {
         if (warp == w) {
@@ -180,38 +230,43 @@ __global__ void __launch_bounds__(128) k_conv_wgrad(const bf16* __restrict__ in,
         const int r = i / Cin, c = i % Cin;
         partial[((size_t(chunk) * 27 + tap) * Cout + co0 + r) * Cin + c] = red[r][c];
     }
-}
-
-__global__ void k_sum_chunks(const float* partial, int chunks, int64_t count, float* out) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x) {
-        float s = 0.f;
-        for (int c = 0; c < chunks; ++c) s += partial[size_t(c) * count + i];
-        out[i] = s;
-    }
-}
-
-// db[co] = sum_v dy[v][co]
-__global__ void k_bias_grad(const bf16* dy, int Cout, int nvox, float* db) {
-    __shared__ float red[256];
-    const int co = blockIdx.x;
-    float s = 0.f;
-    for (int v = threadIdx.x; v < nvox; v += blockDim.x) s += __bfloat162float(dy[size_t(v) * Cout + co]);
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    if (tap == 13) {
         __syncthreads();
+        float* part = &red[0][0];  // 16 x (Cin + 1) floats, 128 of them used
+        part[threadIdx.x] = db;
+        __syncthreads();
+        if (threadIdx.x < 16) {
+            float s = 0.f;
+            for (int k = 0; k < kWgThreads / 16; ++k) s += part[16 * k + threadIdx.x];
+            bias[size_t(chunk) * Cout + co0 + threadIdx.x] = s;
+        }
     }
-    if (threadIdx.x == 0) db[co] = red[0];
+}
+
+// dw (27 Cout Cin) and db (Cout): sums over the chunks in order, added to what is there when add is set
+__global__ void k_sum_chunks(const float* __restrict__ partial, const float* __restrict__ bias, int chunks, int64_t count,
+                             int Cout, int add, float* __restrict__ dw, float* __restrict__ db) {
+    const int64_t total = count + (db ? Cout : 0);
+    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
+        const bool w = i < count;
+        const float* src = w ? partial + i : bias + (i - count);
+        const int64_t stride = w ? count : Cout;
+        float* to = w ? dw + i : db + (i - count);
+        float s = 0.f;
+        for (int c = 0; c < chunks; ++c) s += src[c * stride];
+        *to = add ? *to + s : s;
+    }
 }
 
 template <int NCI>
-cudaError_t wgrad_t(const bf16* in, int Cin, const bf16* dy, int Cout, float* partial, int n, cudaStream_t s) {
-    const int nvox = n * n * n;
-    const int chunks = (nvox + kWgradVox - 1) / kWgradVox;
-    dim3 grid(chunks, 27, Cout / 16);
+cudaError_t wgrad_t(const bf16* in, const bf16* dy, int Cout, float* partial, float* bias, int n, int64_t voxels,
+                    int64_t chunk, cudaStream_t s) {
+    const size_t smem = sizeof(bf16) * 2 * kWgStep * size_t(8 * NCI + 8 + 16 + 8);
+    const cudaError_t e = qpat::allow_smem((const void*)k_conv_wgrad<NCI>, smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid(unsigned((voxels + chunk - 1) / chunk), 27, unsigned(Cout / 16));
     qpat::note_launch(1);
-    k_conv_wgrad<NCI><<<grid, 128, 0, s>>>(in, Cin, dy, Cout, partial, n);
+    k_conv_wgrad<NCI><<<grid, kWgThreads, smem, s>>>(in, dy, Cout, partial, bias, n, voxels, chunk);
     return cudaGetLastError();
 }
 
@@ -231,9 +286,11 @@ __global__ void k_relu_mask(bf16* dy, const bf16* y, int64_t count) {
         if (!(__bfloat162float(y[i]) > 0.f)) dy[i] = __float2bfloat16(0.f);
 }
 
-__global__ void k_avgpool(const bf16* in, int C, int n, bf16* out) {
+// The pooling and concatenation kernels take B samples as one grid of B n planes: n is even, so no pair of planes
+// straddles two samples.
+__global__ void k_avgpool(const bf16* in, int C, int n, int B, bf16* out) {
     const int m = n / 2;
-    const int64_t total = int64_t(m) * m * m * C;
+    const int64_t total = int64_t(m) * m * m * C * B;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
         const int c = int(i % C);
         const int64_t v = i / C;
@@ -247,9 +304,9 @@ __global__ void k_avgpool(const bf16* in, int C, int n, bf16* out) {
     }
 }
 
-__global__ void k_avgpool_bwd(const bf16* dout, int C, int n, bf16* din, int accumulate) {
+__global__ void k_avgpool_bwd(const bf16* dout, int C, int n, int B, bf16* din, int accumulate) {
     const int m = n / 2;
-    const int64_t total = int64_t(n) * n * n * C;
+    const int64_t total = int64_t(n) * n * n * C * B;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
         const int c = int(i % C);
         const int64_t v = i / C;
@@ -260,9 +317,9 @@ __global__ void k_avgpool_bwd(const bf16* dout, int C, int n, bf16* din, int acc
     }
 }
 
-__global__ void k_upcat(const bf16* lo, int Clo, const bf16* skip, int Cs, int n, bf16* cat) {
+__global__ void k_upcat(const bf16* lo, int Clo, const bf16* skip, int Cs, int n, int B, bf16* cat) {
     const int m = n / 2, C = Clo + Cs;
-    const int64_t total = int64_t(n) * n * n * C;
+    const int64_t total = int64_t(n) * n * n * C * B;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
         const int c = int(i % C);
         const int64_t v = i / C;
@@ -275,9 +332,9 @@ __global__ void k_upcat(const bf16* lo, int Clo, const bf16* skip, int Cs, int n
     }
 }
 
-__global__ void k_upcat_bwd_lo(const bf16* dcat, int Clo, int Cs, int n, bf16* dlo) {
+__global__ void k_upcat_bwd_lo(const bf16* dcat, int Clo, int Cs, int n, int B, bf16* dlo) {
     const int m = n / 2, C = Clo + Cs;
-    const int64_t total = int64_t(m) * m * m * Clo;
+    const int64_t total = int64_t(m) * m * m * Clo * B;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
         const int c = int(i % Clo);
         const int64_t v = i / Clo;
@@ -291,9 +348,9 @@ __global__ void k_upcat_bwd_lo(const bf16* dcat, int Clo, int Cs, int n, bf16* d
     }
 }
 
-__global__ void k_upcat_bwd_skip(const bf16* dcat, int Clo, int Cs, int n, bf16* dskip, int accumulate) {
+__global__ void k_upcat_bwd_skip(const bf16* dcat, int Clo, int Cs, int n, int B, bf16* dskip, int accumulate) {
     const int C = Clo + Cs;
-    const int64_t total = int64_t(n) * n * n * Cs;
+    const int64_t total = int64_t(n) * n * n * Cs * B;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
         const int c = int(i % Cs);
         const int64_t v = i / Cs;
@@ -341,7 +398,7 @@ cudaError_t conv3d_fwd(const bf16* in, int Cin, const bf16* w, const float* bias
                        float* out32, int n, cudaStream_t s) {
     if (Cin % 16 || Cout % 8 || n % 2) return cudaErrorInvalidValue;
     if (g_conv_engine == 0 && conv3d_fwd_tc_supported(Cin, Cout))
-        return conv3d_fwd_tc(in, Cin, w, bias, Cout, relu, out, out32, n, s);
+        return conv3d_fwd_tc(ConvInput{in, Cin}, w, bias, Cout, relu, ConvOutput{out, out32}, n, 1, s);
     switch (Cout / 8) {
         case 1: return conv_fwd_t<1>(in, Cin, w, bias, Cout, relu, out, out32, n, s);
         case 2: return conv_fwd_t<2>(in, Cin, w, bias, Cout, relu, out, out32, n, s);
@@ -355,30 +412,32 @@ cudaError_t conv3d_fwd(const bf16* in, int Cin, const bf16* w, const float* bias
     }
 }
 
-int wgrad_chunks(int n) { return (n * n * n + kWgradVox - 1) / kWgradVox; }
+size_t wgrad_scratch(int n, int Cin, int Cout, int B) {
+    const int64_t voxels = int64_t(n) * n * n * B, chunk = wgrad_chunk_voxels(voxels, Cout);
+    return size_t((voxels + chunk - 1) / chunk) * (size_t(27) * Cin * Cout + size_t(Cout));
+}
 
 cudaError_t conv3d_wgrad(const bf16* in, int Cin, const bf16* dy, int Cout, float* dw, float* db, float* partial,
-                         int n, cudaStream_t s) {
+                         int n, int B, int add, cudaStream_t s) {
     if (Cin % 8 || Cout % 16 || (n * n * n) % 16) return cudaErrorInvalidValue;
+    const int64_t voxels = int64_t(n) * n * n * B, chunk = wgrad_chunk_voxels(voxels, Cout);
+    const int chunks = int((voxels + chunk - 1) / chunk);
+    const int64_t count = int64_t(27) * Cout * Cin;
+    float* bias = partial + chunks * count;
     cudaError_t e = cudaErrorInvalidValue;
     switch (Cin / 8) {
-        case 2: e = wgrad_t<2>(in, Cin, dy, Cout, partial, n, s); break;
-        case 4: e = wgrad_t<4>(in, Cin, dy, Cout, partial, n, s); break;
-        case 6: e = wgrad_t<6>(in, Cin, dy, Cout, partial, n, s); break;
-        case 8: e = wgrad_t<8>(in, Cin, dy, Cout, partial, n, s); break;
-        case 12: e = wgrad_t<12>(in, Cin, dy, Cout, partial, n, s); break;
-        case 16: e = wgrad_t<16>(in, Cin, dy, Cout, partial, n, s); break;
-        case 24: e = wgrad_t<24>(in, Cin, dy, Cout, partial, n, s); break;
+        case 2: e = wgrad_t<2>(in, dy, Cout, partial, bias, n, voxels, chunk, s); break;
+        case 4: e = wgrad_t<4>(in, dy, Cout, partial, bias, n, voxels, chunk, s); break;
+        case 6: e = wgrad_t<6>(in, dy, Cout, partial, bias, n, voxels, chunk, s); break;
+        case 8: e = wgrad_t<8>(in, dy, Cout, partial, bias, n, voxels, chunk, s); break;
+        case 12: e = wgrad_t<12>(in, dy, Cout, partial, bias, n, voxels, chunk, s); break;
+        case 16: e = wgrad_t<16>(in, dy, Cout, partial, bias, n, voxels, chunk, s); break;
+        case 24: e = wgrad_t<24>(in, dy, Cout, partial, bias, n, voxels, chunk, s); break;
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    const int64_t count = int64_t(27) * Cout * Cin;
     qpat::note_launch(1);
-    k_sum_chunks<<<grid1d(count), 256, 0, s>>>(partial, wgrad_chunks(n), count, dw);
-    if (db) {
-        qpat::note_launch(1);
-        k_bias_grad<<<Cout, 256, 0, s>>>(dy, Cout, n * n * n, db);
-    }
+    k_sum_chunks<<<grid1d(count + Cout), 256, 0, s>>>(partial, bias, chunks, count, Cout, add, dw, db);
     return cudaGetLastError();
 }
 
@@ -394,30 +453,30 @@ cudaError_t relu_mask(bf16* dy, const bf16* y, int64_t count, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t avgpool(const bf16* in, int C, int n, bf16* out, cudaStream_t s) {
+cudaError_t avgpool(const bf16* in, int C, int n, int B, bf16* out, cudaStream_t s) {
     qpat::note_launch(1);
-    k_avgpool<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * C), 256, 0, s>>>(in, C, n, out);
+    k_avgpool<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * C * B), 256, 0, s>>>(in, C, n, B, out);
     return cudaGetLastError();
 }
 
-cudaError_t avgpool_bwd(const bf16* dout, int C, int n, bf16* din, int accumulate, cudaStream_t s) {
+cudaError_t avgpool_bwd(const bf16* dout, int C, int n, int B, bf16* din, int accumulate, cudaStream_t s) {
     qpat::note_launch(1);
-    k_avgpool_bwd<<<grid1d(int64_t(n) * n * n * C), 256, 0, s>>>(dout, C, n, din, accumulate);
+    k_avgpool_bwd<<<grid1d(int64_t(n) * n * n * C * B), 256, 0, s>>>(dout, C, n, B, din, accumulate);
     return cudaGetLastError();
 }
 
-cudaError_t upcat(const bf16* lo, int Clo, const bf16* skip, int Cs, int n, bf16* cat, cudaStream_t s) {
+cudaError_t upcat(const bf16* lo, int Clo, const bf16* skip, int Cs, int n, int B, bf16* cat, cudaStream_t s) {
     qpat::note_launch(1);
-    k_upcat<<<grid1d(int64_t(n) * n * n * (Clo + Cs)), 256, 0, s>>>(lo, Clo, skip, Cs, n, cat);
+    k_upcat<<<grid1d(int64_t(n) * n * n * (Clo + Cs) * B), 256, 0, s>>>(lo, Clo, skip, Cs, n, B, cat);
     return cudaGetLastError();
 }
 
-cudaError_t upcat_bwd(const bf16* dcat, int Clo, int Cs, int n, bf16* dlo, bf16* dskip, int accumulate_skip,
+cudaError_t upcat_bwd(const bf16* dcat, int Clo, int Cs, int n, int B, bf16* dlo, bf16* dskip, int accumulate_skip,
                       cudaStream_t s) {
     qpat::note_launch(1);
-    k_upcat_bwd_lo<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * Clo), 256, 0, s>>>(dcat, Clo, Cs, n, dlo);
+    k_upcat_bwd_lo<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * Clo * B), 256, 0, s>>>(dcat, Clo, Cs, n, B, dlo);
     qpat::note_launch(1);
-    k_upcat_bwd_skip<<<grid1d(int64_t(n) * n * n * Cs), 256, 0, s>>>(dcat, Clo, Cs, n, dskip, accumulate_skip);
+    k_upcat_bwd_skip<<<grid1d(int64_t(n) * n * n * Cs * B), 256, 0, s>>>(dcat, Clo, Cs, n, B, dskip, accumulate_skip);
     return cudaGetLastError();
 }
 
