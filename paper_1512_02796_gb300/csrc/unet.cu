@@ -43,11 +43,13 @@ __global__ void k_features(int64_t nvox, const double* mu, const double* kappa, 
     }
 }
 
-// network input (channels-last, 16 channels, 3 used) from fp32 features
+// network input (channels-last, 16 channels, 3 used) from fp32 features, a voxel a thread
 __global__ void k_pack_input(int64_t nvox, const float* x, bf16* xin) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < nvox * 16; i += int64_t(gridDim.x) * blockDim.x) {
-        const int c = int(i % 16);
-        xin[i] = __float2bfloat16(c < 3 ? x[(i / 16) * 3 + c] : 0.f);
+    for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < nvox; v += int64_t(gridDim.x) * blockDim.x) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(x[3 * v], x[3 * v + 1]), b = __floats2bfloat162_rn(x[3 * v + 2], 0.f);
+        uint4* o = reinterpret_cast<uint4*>(xin + v * 16);
+        o[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b), 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -445,7 +447,7 @@ int qpat_unet_predict_dev(qpat_unet_t U, const float* x, int B, float* y, void* 
     for (int b = 0; b < B; b += U->cap) {
         const int nb = std::min(U->cap, B - b);
         qpat::note_launch(1);
-        k_pack_input<<<g1(nv * nb * 16), 256, 0, s>>>(nv * nb, x + b * nv * 3, U->xin);
+        k_pack_input<<<g1(nv * nb), 256, 0, s>>>(nv * nb, x + b * nv * 3, U->xin);
         if ((rc = unet_forward(U, nb, false, y + b * nv, U->log_floor > 0.f, s))) return rc;
     }
     UCK(cudaGetLastError());
@@ -464,7 +466,7 @@ static int unet_loss_grad(qpat_unet_s* U, const float* x, const float* t, int B,
     for (int b = 0; b < B; b += cap) {
         const int nb = std::min(cap, B - b);
         qpat::note_launch(1);
-        k_pack_input<<<g1(nv * nb * 16), 256, 0, s>>>(nv * nb, x + b * nv * 3, U->xin);
+        k_pack_input<<<g1(nv * nb), 256, 0, s>>>(nv * nb, x + b * nv * 3, U->xin);
         if ((rc = unet_forward(U, nb, true, U->y, 0, s))) return rc;
         qpat::note_launch(1);
         k_mse<<<g1(nv * nb), 256, 0, s>>>(nv * nb, U->y, t + b * nv, 1.f / float(nv * B), U->g_y, U->loss, U->log_floor);

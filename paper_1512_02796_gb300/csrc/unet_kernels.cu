@@ -150,10 +150,20 @@ __device__ __forceinline__ void copy16(bf16* dst, const bf16* src, bool ok) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
 
+// v / d for v < 2^31 by a multiplication (Granlund and Montgomery 1994)
+struct FastDiv {
+    uint32_t d, m, s;
+    explicit FastDiv(uint32_t div) : d(div), m(0), s(0) {
+        while ((uint64_t(1) << s) < d) ++s;
+        m = uint32_t(((uint64_t(1) << 32) * ((uint64_t(1) << s) - d)) / d + 1);
+    }
+    __device__ __forceinline__ uint32_t div(uint32_t v) const { return (__umulhi(m, v) + v) >> s; }
+};
+
 template <int NCI>
 __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dy,
                                                            int Cout, float* __restrict__ partial,
-                                                           float* __restrict__ bias, int n, int64_t voxels,
+                                                           float* __restrict__ bias, int n, FastDiv dn, int64_t voxels,
                                                            int64_t chunk_voxels) {
     constexpr int Cin = 8 * NCI, LI = Cin + 8, LD = 16 + 8;  // padded rows: fragment rows fall into different banks
     extern __shared__ __align__(16) unsigned char wg_smem[];
@@ -169,8 +179,10 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(const bf16* __restric
             const int64_t v = v0 + i / NCI;
             bool ok = v < vend;
             if (ok) {
-                const int x = int(v % n), y = int(v / n % n), z = int(v / (int64_t(n) * n) % n);
-                ok = nbr(z, y, x, tap, n) >= 0;
+                const uint32_t q = dn.div(uint32_t(v)), r = dn.div(q), w = dn.div(r);  // rows, planes, samples before v
+                const int x = int(uint32_t(v) - q * n) + tap % 3 - 1, y = int(q - r * n) + tap / 3 % 3 - 1,
+                          z = int(r - w * n) + tap / 9 - 1;
+                ok = x >= 0 && y >= 0 && z >= 0 && x < n && y < n && z < n;
             }
             copy16(sIn + (st * kWgStep + i / NCI) * LI + i % NCI * 8, ok ? in + (v + shift) * Cin + i % NCI * 8 : in, ok);
         }
@@ -266,7 +278,7 @@ cudaError_t wgrad_t(const bf16* in, const bf16* dy, int Cout, float* partial, fl
     if (e != cudaSuccess) return e;
     const dim3 grid(unsigned((voxels + chunk - 1) / chunk), 27, unsigned(Cout / 16));
     qpat::note_launch(1);
-    k_conv_wgrad<NCI><<<grid, kWgThreads, smem, s>>>(in, dy, Cout, partial, bias, n, voxels, chunk);
+    k_conv_wgrad<NCI><<<grid, kWgThreads, smem, s>>>(in, dy, Cout, partial, bias, n, FastDiv(uint32_t(n)), voxels, chunk);
     return cudaGetLastError();
 }
 
@@ -281,82 +293,125 @@ __global__ void k_flip(const bf16* w, int Cin, int Cout, bf16* wt) {
     }
 }
 
+// The element-wise kernels take 8 channels (16 bytes) a thread; every channel
+// count of the network is a multiple of 8.  Bound by HBM.
+struct Oct {
+    float f[8];
+};
+__device__ __forceinline__ Oct ld8(const bf16* p) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+    Oct o;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        o.f[2 * k] = __uint_as_float(w[k] << 16);
+        o.f[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+    }
+    return o;
+}
+__device__ __forceinline__ void st8(bf16* p, const Oct& o) {
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = pack2(__float2bfloat16(o.f[2 * k]), __float2bfloat16(o.f[2 * k + 1]));
+    *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+#define FOR_OCT(total) \
+    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < (total); i += int64_t(gridDim.x) * blockDim.x)
+
 __global__ void k_relu_mask(bf16* dy, const bf16* y, int64_t count) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x)
-        if (!(__bfloat162float(y[i]) > 0.f)) dy[i] = __float2bfloat16(0.f);
+    FOR_OCT(count / 8) {
+        const uint4 u = __ldg(reinterpret_cast<const uint4*>(y) + i);
+        uint4 d = reinterpret_cast<uint4*>(dy)[i];
+        auto keep = [](uint32_t v, uint32_t g) {  // halves of g whose v is above 0
+            return (__uint_as_float(v << 16) > 0.f ? g & 0xffffu : 0u) |
+                   (__uint_as_float(v & 0xffff0000u) > 0.f ? g & 0xffff0000u : 0u);
+        };
+        d = make_uint4(keep(u.x, d.x), keep(u.y, d.y), keep(u.z, d.z), keep(u.w, d.w));
+        reinterpret_cast<uint4*>(dy)[i] = d;
+    }
 }
 
 // The pooling and concatenation kernels take B samples as one grid of B n planes: n is even, so no pair of planes
 // straddles two samples.
 __global__ void k_avgpool(const bf16* in, int C, int n, int B, bf16* out) {
-    const int m = n / 2;
-    const int64_t total = int64_t(m) * m * m * C * B;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
-        const int c = int(i % C);
-        const int64_t v = i / C;
-        const int x = int(v % m), y = int((v / m) % m), z = int(v / (int64_t(m) * m));
-        float s = 0.f;
+    const int m = n / 2, c8 = C / 8;
+    FOR_OCT(int64_t(m) * m * m * c8 * B) {
+        const int c = int(i % c8) * 8;
+        const int64_t v = i / c8;
+        const int x = int(v % m), y = int(v / m % m);
+        const int64_t z = v / (int64_t(m) * m);
+        Oct s{};
         for (int d = 0; d < 8; ++d) {
-            const int zz = 2 * z + (d >> 2), yy = 2 * y + ((d >> 1) & 1), xx = 2 * x + (d & 1);
-            s += __bfloat162float(in[((size_t(zz) * n + yy) * n + xx) * C + c]);
+            const Oct q = ld8(in + (((2 * z + (d >> 2)) * n + 2 * y + ((d >> 1) & 1)) * n + 2 * x + (d & 1)) * C + c);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s.f[k] += q.f[k];
         }
-        out[i] = __float2bfloat16(0.125f * s);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s.f[k] *= 0.125f;
+        st8(out + v * C + c, s);
     }
 }
 
 __global__ void k_avgpool_bwd(const bf16* dout, int C, int n, int B, bf16* din, int accumulate) {
-    const int m = n / 2;
-    const int64_t total = int64_t(n) * n * n * C * B;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
-        const int c = int(i % C);
-        const int64_t v = i / C;
-        const int x = int(v % n), y = int((v / n) % n), z = int(v / (int64_t(n) * n));
-        float g = 0.125f * __bfloat162float(dout[((size_t(z / 2) * m + y / 2) * m + x / 2) * C + c]);
-        if (accumulate) g += __bfloat162float(din[i]);
-        din[i] = __float2bfloat16(g);
+    const int m = n / 2, c8 = C / 8;
+    FOR_OCT(int64_t(n) * n * n * c8 * B) {
+        const int c = int(i % c8) * 8;
+        const int64_t v = i / c8;
+        const int x = int(v % n), y = int(v / n % n);
+        const int64_t z = v / (int64_t(n) * n);
+        Oct g = ld8(dout + (((z / 2) * m + y / 2) * m + x / 2) * C + c);
+        Oct old{};
+        if (accumulate) old = ld8(din + v * C + c);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) g.f[k] = accumulate ? 0.125f * g.f[k] + old.f[k] : 0.125f * g.f[k];
+        st8(din + v * C + c, g);
     }
 }
 
 __global__ void k_upcat(const bf16* lo, int Clo, const bf16* skip, int Cs, int n, int B, bf16* cat) {
-    const int m = n / 2, C = Clo + Cs;
-    const int64_t total = int64_t(n) * n * n * C * B;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
-        const int c = int(i % C);
-        const int64_t v = i / C;
+    const int m = n / 2, C = Clo + Cs, c8 = C / 8;
+    FOR_OCT(int64_t(n) * n * n * c8 * B) {
+        const int c = int(i % c8) * 8;
+        const int64_t v = i / c8;
+        const bf16* src = skip + v * Cs + (c - Clo);
         if (c < Clo) {
-            const int x = int(v % n), y = int((v / n) % n), z = int(v / (int64_t(n) * n));
-            cat[i] = lo[((size_t(z / 2) * m + y / 2) * m + x / 2) * Clo + c];
-        } else {
-            cat[i] = skip[v * Cs + (c - Clo)];
+            const int x = int(v % n), y = int(v / n % n);
+            const int64_t z = v / (int64_t(n) * n);
+            src = lo + (((z / 2) * m + y / 2) * m + x / 2) * Clo + c;
         }
+        reinterpret_cast<uint4*>(cat)[i] = __ldg(reinterpret_cast<const uint4*>(src));
     }
 }
 
 __global__ void k_upcat_bwd_lo(const bf16* dcat, int Clo, int Cs, int n, int B, bf16* dlo) {
-    const int m = n / 2, C = Clo + Cs;
-    const int64_t total = int64_t(m) * m * m * Clo * B;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
-        const int c = int(i % Clo);
-        const int64_t v = i / Clo;
-        const int x = int(v % m), y = int((v / m) % m), z = int(v / (int64_t(m) * m));
-        float s = 0.f;
+    const int m = n / 2, C = Clo + Cs, c8 = Clo / 8;
+    FOR_OCT(int64_t(m) * m * m * c8 * B) {
+        const int c = int(i % c8) * 8;
+        const int64_t v = i / c8;
+        const int x = int(v % m), y = int(v / m % m);
+        const int64_t z = v / (int64_t(m) * m);
+        Oct s{};
         for (int d = 0; d < 8; ++d) {
-            const int zz = 2 * z + (d >> 2), yy = 2 * y + ((d >> 1) & 1), xx = 2 * x + (d & 1);
-            s += __bfloat162float(dcat[((size_t(zz) * n + yy) * n + xx) * C + c]);
+            const Oct q = ld8(dcat + (((2 * z + (d >> 2)) * n + 2 * y + ((d >> 1) & 1)) * n + 2 * x + (d & 1)) * C + c);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s.f[k] += q.f[k];
         }
-        dlo[i] = __float2bfloat16(s);
+        st8(dlo + v * Clo + c, s);
     }
 }
 
 __global__ void k_upcat_bwd_skip(const bf16* dcat, int Clo, int Cs, int n, int B, bf16* dskip, int accumulate) {
-    const int C = Clo + Cs;
-    const int64_t total = int64_t(n) * n * n * Cs * B;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total; i += int64_t(gridDim.x) * blockDim.x) {
-        const int c = int(i % Cs);
-        const int64_t v = i / Cs;
-        float g = __bfloat162float(dcat[v * C + Clo + c]);
-        if (accumulate) g += __bfloat162float(dskip[i]);
-        dskip[i] = __float2bfloat16(g);
+    const int C = Clo + Cs, c8 = Cs / 8;
+    FOR_OCT(int64_t(n) * n * n * c8 * B) {
+        const int c = int(i % c8) * 8;
+        const int64_t v = i / c8;
+        Oct g = ld8(dcat + v * C + Clo + c);
+        if (accumulate) {
+            const Oct old = ld8(dskip + v * Cs + c);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) g.f[k] += old.f[k];
+        }
+        st8(dskip + v * Cs + c, g);
     }
 }
 
@@ -420,6 +475,7 @@ size_t wgrad_scratch(int n, int Cin, int Cout, int B) {
 cudaError_t conv3d_wgrad(const bf16* in, int Cin, const bf16* dy, int Cout, float* dw, float* db, float* partial,
                          int n, int B, int add, cudaStream_t s) {
     if (Cin % 8 || Cout % 16 || (n * n * n) % 16) return cudaErrorInvalidValue;
+    if (int64_t(n) * n * n * B >= int64_t(1) << 31) return cudaErrorInvalidValue;  // 32-bit voxel numbers
     const int64_t voxels = int64_t(n) * n * n * B, chunk = wgrad_chunk_voxels(voxels, Cout);
     const int chunks = int((voxels + chunk - 1) / chunk);
     const int64_t count = int64_t(27) * Cout * Cin;
@@ -449,34 +505,34 @@ cudaError_t flip_weights(const bf16* w, int Cin, int Cout, bf16* w_t, cudaStream
 
 cudaError_t relu_mask(bf16* dy, const bf16* y, int64_t count, cudaStream_t s) {
     qpat::note_launch(1);
-    k_relu_mask<<<grid1d(count), 256, 0, s>>>(dy, y, count);
+    k_relu_mask<<<grid1d(count / 8), 256, 0, s>>>(dy, y, count);
     return cudaGetLastError();
 }
 
 cudaError_t avgpool(const bf16* in, int C, int n, int B, bf16* out, cudaStream_t s) {
     qpat::note_launch(1);
-    k_avgpool<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * C * B), 256, 0, s>>>(in, C, n, B, out);
+    k_avgpool<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * C / 8 * B), 256, 0, s>>>(in, C, n, B, out);
     return cudaGetLastError();
 }
 
 cudaError_t avgpool_bwd(const bf16* dout, int C, int n, int B, bf16* din, int accumulate, cudaStream_t s) {
     qpat::note_launch(1);
-    k_avgpool_bwd<<<grid1d(int64_t(n) * n * n * C * B), 256, 0, s>>>(dout, C, n, B, din, accumulate);
+    k_avgpool_bwd<<<grid1d(int64_t(n) * n * n * C / 8 * B), 256, 0, s>>>(dout, C, n, B, din, accumulate);
     return cudaGetLastError();
 }
 
 cudaError_t upcat(const bf16* lo, int Clo, const bf16* skip, int Cs, int n, int B, bf16* cat, cudaStream_t s) {
     qpat::note_launch(1);
-    k_upcat<<<grid1d(int64_t(n) * n * n * (Clo + Cs) * B), 256, 0, s>>>(lo, Clo, skip, Cs, n, B, cat);
+    k_upcat<<<grid1d(int64_t(n) * n * n * (Clo + Cs) / 8 * B), 256, 0, s>>>(lo, Clo, skip, Cs, n, B, cat);
     return cudaGetLastError();
 }
 
 cudaError_t upcat_bwd(const bf16* dcat, int Clo, int Cs, int n, int B, bf16* dlo, bf16* dskip, int accumulate_skip,
                       cudaStream_t s) {
     qpat::note_launch(1);
-    k_upcat_bwd_lo<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * Clo * B), 256, 0, s>>>(dcat, Clo, Cs, n, B, dlo);
+    k_upcat_bwd_lo<<<grid1d(int64_t(n / 2) * (n / 2) * (n / 2) * Clo / 8 * B), 256, 0, s>>>(dcat, Clo, Cs, n, B, dlo);
     qpat::note_launch(1);
-    k_upcat_bwd_skip<<<grid1d(int64_t(n) * n * n * Cs * B), 256, 0, s>>>(dcat, Clo, Cs, n, B, dskip, accumulate_skip);
+    k_upcat_bwd_skip<<<grid1d(int64_t(n) * n * n * Cs / 8 * B), 256, 0, s>>>(dcat, Clo, Cs, n, B, dskip, accumulate_skip);
     return cudaGetLastError();
 }
 

@@ -13,9 +13,9 @@
 // fall on the padding are computed and dropped.  Weights ([Cout][Cin] per tap,
 // the same layout) stay in shared memory when all 27 taps take at most
 // kResident bytes, else they are streamed through a ring of taps.  One thread
-// issues the MMAs (M = 128, N = Cout, K = 16), taps in order and channels in
-// order within a tap, for each 128-row tile of the box into its own columns
-// of tensor memory; the halo arrives in three groups of planes, and the taps
+// of a warp issues the MMAs (M = 128, N = Cout, K = 16) of the warp's 128-row
+// tiles, taps in order and channels in order within a tap, into the tile's
+// own columns of tensor memory; the halo arrives in three groups of planes, and the taps
 // of a plane start when it has arrived.  Each warp then reads its quarter of
 // the lanes with tcgen05.ld, adds the bias, applies ReLU and stores.
 // The input may be the concatenation of an upsampled coarser grid and a skip
@@ -147,8 +147,9 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 3; ++i)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_addr(&mbar[i])) : "memory");
+        for (int i = 0; i < 3; ++i)  // one arrival per issuing warp
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_addr(&mbar[i])), "r"(min(g.tiles, kTcThreads / 32))
+                         : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
 
@@ -206,21 +207,30 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
     const uint32_t tmem = tmem_base_s;
     const uint32_t idesc = instr_desc(kTcRows, a.Cout);
 
-    // MMAs of one tap for every tile (one thread)
+    // MMAs of one tap.  Issuing one takes a thread far longer than the tensor core takes to run it at N = 16 when the
+    // descriptors are built anew (150 cycles against 32), so the tiles go round the warps (a tile's MMAs stay with one
+    // thread and in order) and a descriptor is its predecessor plus a constant in the address field.
+    const int issuers = min(g.tiles, kTcThreads / 32);
+    const bool issuer = lane == 0 && warp < issuers;
+    const uint64_t descA = smem_desc(uA, uint32_t(g.lbo), 128u), descB = smem_desc(uW, uint32_t(g.wlbo), 128u);
+    const uint32_t stepA = uint32_t(2 * g.lbo) >> 4, stepB = uint32_t(2 * g.wlbo) >> 4;
     auto issue = [&](int tap, int stage) {
-        const int off = (tap / 9 * g.RY + tap / 3 % 3) * g.P + tap % 3;
-        for (int t = 0; t < g.tiles; ++t) {
-            const uint32_t a0 = uA + uint32_t((off + t * kTcRows) * 16), b0 = uW + uint32_t(stage * g.wtap);
+        const uint64_t da0 = descA + uint32_t((tap / 9 * g.RY + tap / 3 % 3) * g.P + tap % 3);
+        const uint64_t db0 = descB + (uint32_t(stage * g.wtap) >> 4);
+        for (int t = warp; t < g.tiles; t += issuers) {
+            uint64_t da = da0 + uint32_t(t * kTcRows), db = db0;
+            const uint32_t d = tmem + uint32_t(t * a.Cout);
+            uint32_t acc = tap > 0 ? 1u : 0u;
             for (int k = 0; k < Cin / 16; ++k) {
-                const uint64_t da = smem_desc(a0 + uint32_t(2 * k * g.lbo), uint32_t(g.lbo), 128u);
-                const uint64_t db = smem_desc(b0 + uint32_t(2 * k * g.wlbo), uint32_t(g.wlbo), 128u);
-                const uint32_t acc = (tap > 0 || k > 0) ? 1u : 0u;
                 asm volatile(
                     "{\n\t.reg .pred p;\n\t"
                     "setp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem + uint32_t(t * a.Cout)),
+                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
                     "l"(da), "l"(db), "r"(idesc), "r"(acc)
                     : "memory");
+                da += stepA;
+                db += stepB;
+                acc = 1u;
             }
         }
     };
@@ -243,7 +253,7 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
             else if (dz == 1) cp_wait<1>();
             else cp_wait<0>();
             publish();
-            if (threadIdx.x == 0) {
+            if (issuer) {
                 for (int t = 0; t < 9; ++t) issue(9 * dz + t, 9 * dz + t);
                 if (dz == 2) commit(0);
             }
@@ -256,7 +266,7 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
         for (; tap < 27; ++tap) {
             cp_wait<1>();
             if (!publish()) break;
-            if (threadIdx.x == 0) {
+            if (issuer) {
                 issue(tap, tap % S);
                 commit(tap % S);
             }
