@@ -12,19 +12,20 @@
 // any 128 consecutive voxels of the box form the rows of one MMA; rows that
 // fall on the padding are computed and dropped.  Weights ([Cout][Cin] per tap,
 // the same layout) stay in shared memory when all 27 taps take at most
-// kResident bytes, else they are streamed through a ring of taps.  One thread
-// of a warp issues the MMAs (M = 128, N = Cout, K = 16) of the warp's 128-row
+// kResident bytes, else they are streamed through a ring of taps.  A warp's
+// elected lane issues the MMAs (M = 128, N = Cout, K = 16) of the warp's 128-row
 // tiles, taps in order and channels in order within a tap, into the tile's
-// own columns of tensor memory; the halo arrives in three groups of planes, and the taps
-// of a plane start when it has arrived.  Each warp then reads its quarter of
-// the lanes with tcgen05.ld, adds the bias, applies ReLU and stores.
+// own columns of tensor memory.  Each warp then reads its quarter of the lanes
+// with tcgen05.ld, adds the bias, applies ReLU and stores.
 // The input may be the concatenation of an upsampled coarser grid and a skip
 // tensor, read directly from both.
 //
 // Bound: an MMA with few output channels reads its 4 KB of A at 128 bytes a
 // cycle (32 cycles) whatever N is, so a layer takes at least
-// 27 Cin / 16 x 32 cycles per 128 voxels; the form before this one copied
-// 27 x 128 rows per tile and waited for each copy.
+// 27 Cin / 16 x 32 cycles per 128 voxels: 49 us for 16 -> 16 channels at 128^3.
+// Measured there, one sample: MMAs alone 75 us over the empty kernel's 26, copies
+// alone 62, stores 23, together 137 (one box per CTA and no overlap: 192);
+// 48 -> 16: 374 (651); 64^3, 32 -> 32: 48 (97); 64^3, 96 -> 32, streamed: 212 (341).
 //
 // Tensor memory is allocated by warp 0 and freed on every exit path.  A wait
 // that gives up writes NaN into the tiles (the caller's parity checks see it)
@@ -105,12 +106,13 @@ __device__ __forceinline__ void cp_wait() {
 struct TcBox {
     int n, Tx, Ty, Tz;
     int P, RY;          // padded row (Tx + 2), padded rows per plane (Ty + 2)
-    int tiles;          // 128-row tiles per CTA
+    int tiles;          // 128-row tiles per box
     int lbo;            // bytes between 8-channel chunks of the halo
     int wlbo, wtap;     // bytes between chunks of a tap's weights, bytes of a tap
     int stages;         // 27: weights resident; else the ring's taps
     int ncols;          // tensor-memory columns
-    int nx, ny;         // boxes along x and y
+    int nx, ny, nz;     // boxes along x, y, z
+    int boxes;          // of all samples
 };
 
 struct TcArgs {
@@ -127,169 +129,72 @@ struct TcArgs {
     int first_exp;      //   its exponential
 };
 
-__global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
-    extern __shared__ __align__(128) unsigned char tc_smem[];
-    __shared__ uint64_t mbar[3];
-    __shared__ uint32_t tmem_base_s;
+struct Corner {
+    int x, y, z, sample;
+};
+__device__ __forceinline__ Corner corner_of(const TcBox& g, int box) {
+    Corner c;
+    c.x = box % g.nx * g.Tx;
+    box /= g.nx;
+    c.y = box % g.ny * g.Ty;
+    box /= g.ny;
+    c.z = box % g.nz * g.Tz;
+    c.sample = box / g.nz;
+    return c;
+}
+
+// One tensor's rows of the halo, kt 16-byte chunks a voxel, to shared address dst.  A row of voxels lies in one piece in memory, so a lane's address
+// advances by 32 chunks; up = 1: the row of the grid of half the side, every
+// voxel twice.
+__device__ __forceinline__ void load_rows(const TcBox& g, const Corner& c, const bf16* t, int kt, int up, uint32_t dst) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = g.n, m = n >> up;
+    const int dx = 32 / kt, dk = 32 % kt, x0 = lane / kt, q0 = lane % kt;
+    const int xa = c.x == 0 ? 1 : 0, xb = min(g.P, n - c.x + 1);  // padded columns inside the grid
+    const bf16* base = t + int64_t(c.sample) * m * m * m * kt * 8;
+    for (int row = warp; row < (g.Tz + 2) * g.RY; row += kTcThreads / 32) {
+        const int z = c.z + row / g.RY - 1, y = c.y + row % g.RY - 1;
+        const bool in = z >= 0 && z < n && y >= 0 && y < n;
+        const bf16* src = base + (in ? (int64_t(z >> up) * m + (y >> up)) * m * kt * 8 : 0);
+        const uint32_t to = dst + uint32_t(row * g.P * 16);
+        for (int x = x0, q = q0; x < g.P;) {
+            const bool ok = in && x >= xa && x < xb;
+            cp16(to + uint32_t(q * g.lbo + x * 16), src + (ok ? (((c.x + x - 1) >> up) * kt + q) * 8 : 0), ok);
+            x += dx;
+            q += dk;
+            if (q >= kt) {
+                q -= kt;
+                ++x;
+            }
+        }
+    }
+}
+
+// The halo of box c to shared address dst.
+__device__ __forceinline__ void load_halo(const TcArgs& a, const Corner& c, uint32_t dst) {
+    if (a.Clo) load_rows(a.g, c, a.lo, a.Clo / 8, 1, dst);
+    load_rows(a.g, c, a.skip, a.Cskip / 8, 0, dst + uint32_t(a.Clo / 8 * a.g.lbo));
+}
+
+// Weights of taps [t0, t0 + taps) to shared address dst.
+__device__ __forceinline__ void load_weights(const TcArgs& a, int t0, int taps, uint32_t dst) {
+    const int kc = (a.Clo + a.Cskip) / 8, per = a.Cout * kc;
+    const bf16* src = a.w + size_t(t0) * per * 8;
+    for (int i = threadIdx.x; i < taps * per; i += kTcThreads) {
+        const int tap = i / per, j = i - tap * per, row = j / kc;
+        cp16(dst + uint32_t(tap * a.g.wtap + (j - row * kc) * a.g.wlbo + row * 16), src + size_t(i) * 8, true);
+    }
+}
+
+// The results of box c from tensor memory: warps w and w + 4 own lanes 32 (w % 4) .. + 31 and take the tiles in turn.
+__device__ __forceinline__ void store_box(const TcArgs& a, const Corner& c, uint32_t tmem, bool ok) {
     const TcBox& g = a.g;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n = g.n, Cin = a.Clo + a.Cskip, kc = Cin / 8, lc = a.Clo / 8;
-    const int x0 = int(blockIdx.x % g.nx) * g.Tx, y0 = int(blockIdx.x / g.nx) * g.Ty, z0 = int(blockIdx.y) * g.Tz;
-    const int64_t nvox = int64_t(n) * n * n, sample = blockIdx.z;
-    unsigned char* sA = tc_smem;
-    unsigned char* sW = sA + size_t(kc) * g.lbo;
-    const uint32_t uA = s_addr(sA), uW = s_addr(sW);
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_addr(&tmem_base_s)),
-                     "r"(g.ncols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 3; ++i)  // one arrival per issuing warp
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_addr(&mbar[i])), "r"(min(g.tiles, kTcThreads / 32))
-                         : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-
-    // halo planes [p0, p1) of the box: a warp per padded row, 16 bytes per lane
-    auto load_planes = [&](int p0, int p1) {
-        const bf16* skip = a.skip + sample * nvox * a.Cskip;
-        const bf16* lo = a.lo ? a.lo + sample * (nvox >> 3) * a.Clo : nullptr;
-        const int m = n >> 1, dx = 32 / kc, dc = 32 % kc;
-        for (int row = p0 * g.RY + warp; row < p1 * g.RY; row += kTcThreads / 32) {
-            const int z = z0 + row / g.RY - 1, y = y0 + row % g.RY - 1;
-            const bool in = z >= 0 && z < n && y >= 0 && y < n;
-            int x = lane / kc, c = lane % kc;
-            for (; x < g.P; ) {
-                const int xx = x0 + x - 1;
-                const bool ok = in && xx >= 0 && xx < n;
-                const void* src = a.skip;
-                if (ok)
-                    src = c < lc ? static_cast<const void*>(lo + ((int64_t(z >> 1) * m + (y >> 1)) * m + (xx >> 1)) * a.Clo + c * 8)
-                                 : static_cast<const void*>(skip + ((int64_t(z) * n + y) * n + xx) * a.Cskip + (c - lc) * 8);
-                cp16(uA + uint32_t(c * g.lbo + (row * g.P + x) * 16), src, ok);
-                x += dx;
-                c += dc;
-                if (c >= kc) {
-                    c -= kc;
-                    ++x;
-                }
-            }
-        }
-    };
-    auto load_weights = [&](int tap, int stage) {
-        const bf16* src = a.w + size_t(tap) * a.Cout * Cin;
-        const uint32_t dst = uW + uint32_t(stage * g.wtap);
-        for (int i = threadIdx.x; i < a.Cout * kc; i += kTcThreads)
-            cp16(dst + uint32_t((i % kc) * g.wlbo + (i / kc) * 16), src + size_t(i) * 8, true);
-    };
-    const bool resident = g.stages == 27;
-    load_planes(0, g.Tz);
-    if (resident) {
-        for (int t = 0; t < 27; ++t) load_weights(t, t);
-        cp_commit();
-        load_planes(g.Tz, g.Tz + 1);
-        cp_commit();
-        load_planes(g.Tz + 1, g.Tz + 2);
-        cp_commit();
-    } else {
-        load_planes(g.Tz, g.Tz + 2);
-        load_weights(0, 0);
-        cp_commit();
-        load_weights(1, 1);
-        cp_commit();
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_base_s;
-    const uint32_t idesc = instr_desc(kTcRows, a.Cout);
-
-    // MMAs of one tap.  Issuing one takes a thread far longer than the tensor core takes to run it at N = 16 when the
-    // descriptors are built anew (150 cycles against 32), so the tiles go round the warps (a tile's MMAs stay with one
-    // thread and in order) and a descriptor is its predecessor plus a constant in the address field.
-    const int issuers = min(g.tiles, kTcThreads / 32);
-    const bool issuer = lane == 0 && warp < issuers;
-    const uint64_t descA = smem_desc(uA, uint32_t(g.lbo), 128u), descB = smem_desc(uW, uint32_t(g.wlbo), 128u);
-    const uint32_t stepA = uint32_t(2 * g.lbo) >> 4, stepB = uint32_t(2 * g.wlbo) >> 4;
-    auto issue = [&](int tap, int stage) {
-        const uint64_t da0 = descA + uint32_t((tap / 9 * g.RY + tap / 3 % 3) * g.P + tap % 3);
-        const uint64_t db0 = descB + (uint32_t(stage * g.wtap) >> 4);
-        for (int t = warp; t < g.tiles; t += issuers) {
-            uint64_t da = da0 + uint32_t(t * kTcRows), db = db0;
-            const uint32_t d = tmem + uint32_t(t * a.Cout);
-            uint32_t acc = tap > 0 ? 1u : 0u;
-            for (int k = 0; k < Cin / 16; ++k) {
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\t"
-                    "setp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-                    "l"(da), "l"(db), "r"(idesc), "r"(acc)
-                    : "memory");
-                da += stepA;
-                db += stepB;
-                acc = 1u;
-            }
-        }
-    };
-    auto commit = [&](int i) {
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_addr(&mbar[i]))
-                     : "memory");
-    };
-    // this thread's copies have arrived -> visible to the tensor core (async proxy) for everybody; false (in every
-    // thread) once a wait of some thread has given up
-    bool mine = true;
-    auto publish = [&]() -> bool {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        const bool all = __syncthreads_and(mine);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        return all;
-    };
-    if (resident) {
-        for (int dz = 0; dz < 3; ++dz) {
-            if (dz == 0) cp_wait<2>();
-            else if (dz == 1) cp_wait<1>();
-            else cp_wait<0>();
-            publish();
-            if (issuer) {
-                for (int t = 0; t < 9; ++t) issue(9 * dz + t, 9 * dz + t);
-                if (dz == 2) commit(0);
-            }
-        }
-        mine = mbar_wait_parity(&mbar[0], 0u);
-    } else {
-        // ring of 2 or 3 taps; completion of tap t is phase t / stages of mbar[t % stages]
-        const int S = g.stages;
-        int tap = 0;
-        for (; tap < 27; ++tap) {
-            cp_wait<1>();
-            if (!publish()) break;
-            if (issuer) {
-                issue(tap, tap % S);
-                commit(tap % S);
-            }
-            const int next = tap + 2;  // goes to the stage of tap next - S, whose MMAs must have read it
-            if (next >= S && next < 27 && !mbar_wait_parity(&mbar[(next - S) % S], uint32_t(((next - S) / S) & 1))) mine = false;
-            if (next < 27) load_weights(next, next % S);
-            cp_commit();
-        }
-        cp_wait<0>();
-        // the last taps' MMAs (or, after a give-up, those in flight) finish before TMEM is read and freed
-        for (int t = max(0, tap - S); t < tap; ++t)
-            if (!mbar_wait_parity(&mbar[t % S], uint32_t((t / S) & 1))) mine = false;
-    }
-    const bool ok = __syncthreads_and(mine);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-
-    // ---- epilogue: warps w and w + 4 own TMEM lanes 32 (w % 4) .. + 31 and take the tiles in turn
-    if (!ok && threadIdx.x == 0) atomicAdd(&g_tc_timeouts, 1);
-    for (int t = warp >> 2; t < g.tiles; t += 2) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = g.n;
+    const int64_t nvox = int64_t(n) * n * n;
+    for (int t = warp >> 2; t < g.tiles; t += kTcThreads / 128) {
         const int p = t * kTcRows + (warp & 3) * 32 + lane;
         const int x = p % g.P, y = p / g.P % g.RY, z = p / (g.P * g.RY);
-        const bool valid = x < g.Tx && y < g.Ty && z < g.Tz && x0 + x < n && y0 + y < n && z0 + z < n;
-        const int64_t v = sample * nvox + (int64_t(z0 + z) * n + (y0 + y)) * n + x0 + x;
+        const bool valid = x < g.Tx && y < g.Ty && z < g.Tz && c.x + x < n && c.y + y < n && c.z + z < n;
+        const int64_t v = c.sample * nvox + (int64_t(c.z + z) * n + (c.y + y)) * n + c.x + x;
         for (int c0 = 0; c0 < a.Cout; c0 += 16) {
             uint32_t r[16];
             const uint32_t taddr = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(t * a.Cout + c0);
@@ -330,26 +235,232 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
             }
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.ncols) : "memory");
 }
 
-// The box of a launch with the least estimated time per SM: whole waves of
-// CTAs, each its halo's bytes at ~48 a cycle, its MMAs at 32 cycles (more
-// above 128 output channels) and its stores; two CTAs share an SM where their
-// shared memory (<= half) lets one's loads run under the other's MMAs.
-// false: no box fits.
+__device__ __forceinline__ void tmem_alloc(uint32_t* base, int ncols) {  // one warp
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_addr(base)), "r"(ncols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(uint32_t base, int ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void mbar_init(uint64_t* bar, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(bar)) : "memory");
+}
+// Executed by a whole warp, issued by its elected lane: bar completes a phase when that lane's MMAs so far are done.
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(s_addr(bar))
+        : "memory");
+}
+__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void to_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// The MMAs of one tap for tiles first, first + step, ... of a box, by one warp:
+// every lane walks the loop with warp-uniform values and the elected one
+// issues, so that the descriptors stay in uniform registers (a single lane
+// that builds them takes 100 to 200 cycles an MMA, several times what the
+// tensor core takes at N = 16); each descriptor is its predecessor plus a
+// constant in the address field.
+struct TapIssue {
+    uint64_t descA, descB;
+    uint32_t stepA, stepB, idesc;
+    __device__ TapIssue(const TcArgs& a, uint32_t uA, uint32_t uW)
+        : descA(smem_desc(uA, uint32_t(a.g.lbo), 128u)), descB(smem_desc(uW, uint32_t(a.g.wlbo), 128u)),
+          stepA(uint32_t(2 * a.g.lbo) >> 4), stepB(uint32_t(2 * a.g.wlbo) >> 4), idesc(instr_desc(kTcRows, a.Cout)) {}
+    __device__ __forceinline__ void operator()(const TcArgs& a, int tap, uint32_t halo_off, uint32_t w_off, uint32_t acc_at,
+                                               int first, int step) const {
+        const TcBox& g = a.g;
+        const int ks = (a.Clo + a.Cskip) / 16;
+        const uint64_t da0 = descA + (halo_off >> 4) + uint32_t((tap / 9 * g.RY + tap / 3 % 3) * g.P + tap % 3);
+        const uint64_t db0 = descB + (w_off >> 4);
+        for (int t = first; t < g.tiles; t += step) {
+            uint64_t da = da0 + uint32_t(t * kTcRows), db = db0;
+            const uint32_t d = acc_at + uint32_t(t * a.Cout);
+            uint32_t acc = tap > 0 ? 1u : 0u;
+            for (int k = 0; k < ks; ++k) {
+                asm volatile(
+                    "{\n\t.reg .pred p, q;\n\t"
+                    "elect.sync _|q, 0xffffffff;\n\t"
+                    "setp.ne.b32 p, %4, 0;\n\t"
+                    "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+                    "l"(da), "l"(db), "r"(idesc), "r"(acc)
+                    : "memory");
+                da += stepA;
+                db += stepB;
+                acc = 1u;
+            }
+        }
+    }
+};
+
+// Resident weights: a CTA goes through its boxes with two halos and two sets of
+// accumulators.  Eight warps copy halos and store results; four more only issue
+// MMAs (a thread that issues waits while the tensor core's queue is full, so it
+// cannot be one that copies).  Box `it` uses halo, accumulators and barriers
+// it % 2: full (its halo is there), done (its MMAs are over), stored (its
+// accumulators have been read).  Every wait is bounded; once one gives up, no
+// thread waits again and what is stored is NaN.
+constexpr int kIssueWarps = 4;
+constexpr int kStayThreads = kTcThreads + 32 * kIssueWarps;
+
+__global__ void __launch_bounds__(kStayThreads) k_conv_fwd_tc_stay(const TcArgs a) {
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    __shared__ uint64_t full[2], done[2], stored[2];
+    __shared__ uint32_t tmem_base_s;
+    __shared__ volatile int gave_up;
+    const TcBox& g = a.g;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);  // warp-uniform for the compiler
+    const int halo = (a.Clo + a.Cskip) / 8 * g.lbo, set = g.tiles * a.Cout;
+    const uint32_t uA = s_addr(tc_smem), uW = uA + uint32_t(halo * 2);
+    if (warp == 0) tmem_alloc(&tmem_base_s, g.ncols);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&full[i], kTcThreads);
+            mbar_init(&done[i], kIssueWarps);
+            mbar_init(&stored[i], kTcThreads);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        gave_up = 0;
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base_s, 0);
+    auto wait = [&](uint64_t* bar, int phase) {
+        if (!gave_up && !mbar_wait_parity(bar, uint32_t(phase & 1))) {
+            gave_up = 1;
+            atomicAdd(&g_tc_timeouts, 1);
+        }
+    };
+    const int boxes = g.boxes, stride = int(gridDim.x), mine = int(blockIdx.x);
+    const int count = mine < boxes ? (boxes - 1 - mine) / stride + 1 : 0;
+    if (warp >= kTcThreads / 32) {
+        const TapIssue issue(a, uA, uW);
+        for (int it = 0; it < count; ++it) {
+            const int buf = it & 1;
+            wait(&full[buf], it >> 1);
+            if (it >= 2) wait(&stored[buf], (it >> 1) - 1);
+            __syncwarp();
+            tc_after();
+            for (int t = 0; t < 27; ++t)
+                issue(a, t, uint32_t(buf * halo), uint32_t(t * g.wtap), tmem + uint32_t(buf * set), warp - kTcThreads / 32,
+                      kIssueWarps);
+            mma_commit(&done[buf]);
+        }
+    } else {
+        load_halo(a, corner_of(g, mine), uA);
+        load_weights(a, 0, 27, uW);
+        cp_commit();
+        for (int it = 0; it <= count; ++it) {
+            const int buf = it & 1;
+            if (it < count) {
+                cp_wait<0>();
+                to_async_proxy();
+                mbar_arrive(&full[buf]);
+            }
+            if (it > 0) {
+                wait(&done[buf ^ 1], (it - 1) >> 1);
+                tc_after();
+            }
+            if (it + 1 < count) {
+                load_halo(a, corner_of(g, mine + (it + 1) * stride), uA + uint32_t((buf ^ 1) * halo));
+                cp_commit();
+            }
+            if (it > 0) {
+                store_box(a, corner_of(g, mine + (it - 1) * stride), tmem + uint32_t((buf ^ 1) * set), !gave_up);
+                tc_before();
+                mbar_arrive(&stored[buf ^ 1]);
+            }
+        }
+    }
+    tc_before();
+    __syncthreads();
+    if (warp == 0) tmem_free(tmem, g.ncols);
+}
+
+// Streamed weights: one box per CTA, a ring of 2 or 3 taps; the tiles go round
+// the warps (a tile's MMAs stay with one lane, in order).
+__global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    __shared__ uint64_t mbar[3];
+    __shared__ uint32_t tmem_base_s;
+    const TcBox& g = a.g;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);
+    const int halo = (a.Clo + a.Cskip) / 8 * g.lbo;
+    const uint32_t uA = s_addr(tc_smem), uW = uA + uint32_t(halo);
+    const int issuers = min(g.tiles, kTcThreads / 32);
+    const bool issuer = warp < issuers;
+    if (warp == 0) tmem_alloc(&tmem_base_s, g.ncols);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 3; ++i) mbar_init(&mbar[i], issuers);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const Corner at = corner_of(g, blockIdx.x);
+    load_halo(a, at, uA);
+    load_weights(a, 0, 1, uW);
+    cp_commit();
+    load_weights(a, 1, 1, uW + uint32_t(g.wtap));
+    cp_commit();
+    tc_before();
+    __syncthreads();
+    tc_after();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base_s, 0);
+    const TapIssue issue(a, uA, uW);
+    // completion of tap t is phase t / S of mbar[t % S]; a thread whose wait gives up says so at the next barrier,
+    // where all leave together
+    const int S = g.stages;
+    bool mine = true;
+    int tap = 0;
+    for (; tap < 27; ++tap) {
+        cp_wait<1>();
+        to_async_proxy();
+        if (!__syncthreads_and(mine)) break;
+        if (issuer) {
+            tc_after();
+            issue(a, tap, 0u, uint32_t(tap % S * g.wtap), tmem, warp, issuers);
+            mma_commit(&mbar[tap % S]);
+        }
+        const int next = tap + 2;  // goes to the stage of tap next - S, whose MMAs must have read it
+        if (next >= S && next < 27 && !mbar_wait_parity(&mbar[(next - S) % S], uint32_t(((next - S) / S) & 1))) mine = false;
+        if (next < 27) load_weights(a, next, 1, uW + uint32_t(next % S * g.wtap));
+        cp_commit();
+    }
+    cp_wait<0>();
+    // the last taps' MMAs (or, after a give-up, those in flight) finish before TMEM is read and freed
+    for (int t = max(0, tap - S); t < tap; ++t)
+        if (!mbar_wait_parity(&mbar[t % S], uint32_t((t / S) & 1))) mine = false;
+    const bool good = __syncthreads_and(mine);
+    tc_after();
+    if (!good && threadIdx.x == 0) atomicAdd(&g_tc_timeouts, 1);
+    store_box(a, at, tmem, good);
+    tc_before();
+    __syncthreads();
+    if (warp == 0) tmem_free(tmem, g.ncols);
+}
+
+// The box of a launch with the least estimated time.  An MMA takes 32 cycles
+// (more above 128 output channels), a halo about its bytes / 24 to issue and
+// bring in, the results their bytes / 16.  Resident weights: per box the
+// larger of the MMAs and the copies; streamed: the sum, and ~8,000 cycles for
+// a CTA's start and its first tap (measured at 128^3, 16 -> 16 channels), two
+// CTAs sharing an SM where their shared memory allows.  false: no box fits.
 bool search_box(int n, int Cin, int Cout, int B, TcBox& best, size_t& best_smem) {
     const int kc = Cin / 8;
     const int wlbo = Cout * 16 + 16, wtap = kc * wlbo;
+    const bool stay = 27 * wtap <= kResident;
     double best_t = 0.0;
     bool found = false;
     for (int sx = 0; sx < 10; ++sx) {
         const int Tx = (n + (1 << sx) - 1) >> sx;
         if (sx > 0 && Tx < 8) break;
-        for (int Tz : {1, 2, 4, 8})
+        for (int Tz : {1, 2, 3, 4, 6, 8})
             for (int Ty = 1; Ty <= std::min(n, 64); ++Ty) {
                 if (Tz > n && Tz > 1) continue;
                 TcBox g{};
@@ -361,30 +472,35 @@ bool search_box(int n, int Cin, int Cout, int B, TcBox& best, size_t& best_smem)
                 g.RY = Ty + 2;
                 const int span = ((Tz - 1) * g.RY + Ty - 1) * g.P + Tx;
                 g.tiles = (span + kTcRows - 1) / kTcRows;
-                if (g.tiles * Cout > 512) break;
+                const int cols = g.tiles * Cout * (stay ? 2 : 1);
+                if (cols > 512) break;
                 // every row that an MMA reads (the last tap shifts the last tile by this much) lies in the buffer
                 const int rows = std::max((Tz + 2) * g.RY * g.P, g.tiles * kTcRows + (2 * g.RY + 2) * g.P + 2);
                 g.lbo = (rows * 16 + 127) / 128 * 128 + 64;
                 g.wlbo = wlbo;
                 g.wtap = wtap;
-                g.stages = 27 * wtap <= kResident ? 27 : 3;
-                size_t smem = size_t(kc) * g.lbo + size_t(g.stages) * wtap;
-                if (smem > size_t(kTcSmem) && g.stages == 3) {
+                g.stages = stay ? 27 : 3;
+                size_t smem = size_t(kc) * g.lbo * (stay ? 2 : 1) + size_t(g.stages) * wtap;
+                if (smem > size_t(kTcSmem) && !stay) {
                     g.stages = 2;
                     smem -= wtap;
                 }
                 if (smem > size_t(kTcSmem)) break;
                 g.ncols = 32;
-                while (g.ncols < g.tiles * Cout) g.ncols *= 2;
+                while (g.ncols < cols) g.ncols *= 2;
                 g.nx = (n + Tx - 1) / Tx;
                 g.ny = (n + Ty - 1) / Ty;
-                const double ctas = double(g.nx) * g.ny * ((n + Tz - 1) / Tz) * B;
-                const int share = smem <= size_t(kTcSmem) / 2 && g.ncols <= 256 ? 2 : 1;
+                g.nz = (n + Tz - 1) / Tz;
+                const double boxes = double(g.nx) * g.ny * g.nz * B;
+                if (boxes >= 2147483648.0) continue;
+                g.boxes = int(boxes);
                 const double mma = g.tiles * 27.0 * (Cin / 16) * std::max(32.0, Cout / 4.0);
-                const double load = ((Tz + 2.0) * g.RY * g.P * Cin * 2 + 27.0 * wtap) / 48.0 + 1500.0;
-                const double store = g.tiles * 128.0 * Cout * 2 / 32.0 + 500.0;
-                const double waves = std::max(1.0, double(int64_t((ctas + 152 * share - 1) / (152 * share))));
-                const double t = waves * (share == 2 ? std::max(2 * mma, mma + load + store) : mma + load + store);
+                const double load = (Tz + 2.0) * g.RY * g.P * Cin * 2 / 24.0 + 800.0;
+                const double store = g.tiles * 128.0 * Cout * 2 / 16.0 + 300.0;
+                const int share = !stay && smem <= size_t(kTcSmem) / 2 && g.ncols <= 256 ? 2 : 1;
+                const double waves = std::max(1.0, double(int64_t((boxes + 152 * share - 1) / (152 * share))));
+                const double t = stay ? waves * std::max(mma + 600.0, load + store) + load + store
+                                      : waves * (share * std::max(mma, 27.0 * wtap / 24.0) + load + store + 8000.0);
                 if (!found || t < best_t) {
                     found = true;
                     best_t = t;
@@ -434,10 +550,11 @@ cudaError_t conv3d_fwd_tc(const ConvInput& in, const bf16* w, const float* bias,
     const int Cin = in.Clo + in.Cskip;
     TcArgs a{};
     size_t smem = 0;
-    if (!conv3d_fwd_tc_supported(Cin, Cout) || in.Clo % 8 || in.Cskip % 8 || B < 1 || B > 65535 || n > 65535 ||
+    if (!conv3d_fwd_tc_supported(Cin, Cout) || in.Clo % 8 || in.Cskip % 8 || B < 1 || n < 1 ||
         !choose_box(n, Cin, Cout, B, a.g, smem))
         return cudaErrorInvalidValue;
-    cudaError_t e = qpat::allow_smem((const void*)k_conv_fwd_tc, smem);
+    const bool stay = a.g.stages == 27;
+    cudaError_t e = qpat::allow_smem(stay ? (const void*)k_conv_fwd_tc_stay : (const void*)k_conv_fwd_tc, smem);
     if (e != cudaSuccess) return e;
     a.skip = in.skip;
     a.lo = in.lo;
@@ -452,7 +569,17 @@ cudaError_t conv3d_fwd_tc(const ConvInput& in, const bf16* w, const float* bias,
     a.first = out.first;
     a.first_exp = out.first_exp;
     qpat::note_launch(1);
-    k_conv_fwd_tc<<<dim3(unsigned(a.g.nx * a.g.ny), unsigned((n + a.g.Tz - 1) / a.g.Tz), unsigned(B)), kTcThreads, smem, s>>>(a);
+    if (stay) {
+        int dev = 0, nsm = 0, per = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_conv_fwd_tc_stay, kStayThreads, smem)) != cudaSuccess)
+            return e;
+        per = std::max(1, std::min(per, 512 / a.g.ncols));  // resident CTAs share the 512 columns of tensor memory
+        k_conv_fwd_tc_stay<<<std::min(a.g.boxes, nsm * per), kStayThreads, smem, s>>>(a);
+    } else {
+        k_conv_fwd_tc<<<a.g.boxes, kTcThreads, smem, s>>>(a);
+    }
     return cudaGetLastError();
 }
 
