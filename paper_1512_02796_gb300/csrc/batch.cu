@@ -6,7 +6,7 @@
 // records the whole sequence -- per problem the layout change, the assembly
 // of K, the load vector; then the single batched PCG launch; then the output
 // layout change -- into a CUDA graph on the caller's stream; every later call
-// replays that graph.  Illuminations per problem are padded to a common R.
+// replays that graph.  Each problem's illuminations are padded to 1, 2, 4 or 8.
 #include <algorithm>
 #include <cstring>
 #include <string>
@@ -17,16 +17,16 @@
 struct qpat_batch_s {
     struct Prob {
         qpat_mesh_s* mesh = nullptr;
-        int K = 0;
+        int K = 0, R = 0;
         double *kappa = nullptr, *mu = nullptr, *flux = nullptr, *phi = nullptr;   // caller layout
         double *kl = nullptr, *ml = nullptr, *vals = nullptr, *inv = nullptr;     // library layout
         double *f = nullptr, *x = nullptr, *r = nullptr, *p0 = nullptr, *p1 = nullptr, *q = nullptr;
         double *partials = nullptr, *ctl = nullptr;
         qpat::ElemScratch scratch;                 // of this problem's assembly
-        double *z = nullptr, *gb = nullptr;  // patch-local Chebyshev preconditioner
+        double *z = nullptr;   // preconditioned residual
+        double *gb = nullptr;  // patch-local Chebyshev preconditioner
     };
     int device = 0;
-    int R = 0;
     double rtol = 1e-13;
     int maxit = 20000;
     int poly_deg = 0;
@@ -72,16 +72,16 @@ int batch_sequence(qpat_batch_s* B, cudaStream_t s) {
         if ((e = launch_assemble_K(m, P.mesh->el, P.scratch, P.kl, P.ml, P.vals, nullptr, P.inv, nullptr, s,
                                    B->poly_deg > 0 ? P.gb : nullptr)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: assemble");
-        if ((e = cudaMemsetAsync(P.f, 0, sizeof(double) * N * B->R, s)) != cudaSuccess)
+        if ((e = cudaMemsetAsync(P.f, 0, sizeof(double) * N * P.R, s)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: memset");
-        if ((e = launch_load(m, P.K, B->R, P.flux, P.f, s)) != cudaSuccess)
+        if ((e = launch_load(m, P.K, P.R, P.flux, P.f, s)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: load");
         if ((e = cudaMemsetAsync(P.ctl, 0, sizeof(double) * 8, s)) != cudaSuccess)  // barrier, status, iterations
             return cuda_fail(e, "qpat_batch_forward: memset");
     }
     if ((e = pcg_batch_launch(B->plan, s)) != cudaSuccess) return cuda_fail(e, "qpat_batch_forward: batched pcg");
     for (auto& P : B->probs)
-        if ((e = launch_from_lib<double, double>(P.mesh->d, P.K, B->R, P.x, P.phi, s)) != cudaSuccess)
+        if ((e = launch_from_lib<double, double>(P.mesh->d, P.K, P.R, P.x, P.phi, s)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: from_lib");
     return QPAT_OK;
 }
@@ -103,7 +103,6 @@ int qpat_batch_create(int nprob, const qpat_mesh_t* meshes, const int* K, const 
     }
     auto* B = new qpat_batch_s();
     B->device = meshes[0]->device;
-    B->R = round_rhs(Kmax);
     const SolveOpts so = solve_opts(prm);
     B->rtol = so.rtol;
     B->maxit = so.maxit;
@@ -115,7 +114,8 @@ int qpat_batch_create(int nprob, const qpat_mesh_t* meshes, const int* K, const 
         qpat_batch_s::Prob P;
         P.mesh = meshes[j];
         P.K = K[j];
-        const size_t N = P.mesh->h.N, F = P.mesh->h.F, R = B->R;
+        P.R = round_rhs(P.K);
+        const size_t N = P.mesh->h.N, F = P.mesh->h.F, R = P.R;
         if ((rc = batch_alloc(B, &P.kappa, N)) || (rc = batch_alloc(B, &P.mu, N)) ||
             (rc = batch_alloc(B, &P.flux, size_t(P.K) * F)) || (rc = batch_alloc(B, &P.phi, size_t(P.K) * N)) ||
             (rc = batch_alloc(B, &P.kl, N)) || (rc = batch_alloc(B, &P.ml, N)) ||
@@ -129,9 +129,10 @@ int qpat_batch_create(int nprob, const qpat_mesh_t* meshes, const int* K, const 
         if ((rc = batch_alloc(B, &tq, 2 * size_t(P.mesh->el.E))) || (rc = batch_alloc(B, &ev, 2 * size_t(P.mesh->el.NE))))
             break;
         P.scratch = {reinterpret_cast<double2*>(tq), reinterpret_cast<double2*>(ev)};
-        if (B->poly_deg > 0 && ((rc = batch_alloc(B, &P.z, N * R)) || (rc = batch_alloc(B, &P.gb, 1)))) break;
+        if ((rc = batch_alloc(B, &P.z, N * R)) || (B->poly_deg > 0 && (rc = batch_alloc(B, &P.gb, 1)))) break;
         PcgBatchProblem q;
         q.m = P.mesh->d;
+        q.R = P.R;
         q.vals = P.vals;
         q.invdiag = P.inv;
         q.w.b = P.f;
@@ -154,7 +155,7 @@ int qpat_batch_create(int nprob, const qpat_mesh_t* meshes, const int* K, const 
         B->probs.push_back(P);
     }
     if (rc == QPAT_OK) {
-        cudaError_t e = pcg_batch_prepare(B->R, pp, B->plan);
+        cudaError_t e = pcg_batch_prepare(round_rhs(Kmax), pp, B->plan);
         if (e != cudaSuccess) rc = cuda_fail(e, "qpat_batch_create: too many problems or patches too large");
     }
     if (rc != QPAT_OK) {

@@ -144,7 +144,8 @@ struct PcgBatchProblem {
     MeshDev m;
     const double* vals;     // assembled K values
     const double* invdiag;  // N
-    PcgWork w;              // b, x, r, p0, p1, q, partials, bar, status, iters, stats
+    PcgWork w;              // b, x, r, p0, p1, q, z (optional), partials, bar, status, iters, stats
+    int R;                  // right-hand sides: 1, 2, 4 or 8
     double rtol;
     int maxit;
 };

@@ -22,6 +22,7 @@
 // wherever R allows.  Scalars are accumulated in FP64 for either T.
 #include <cuda/atomic>
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 #include <vector>
@@ -68,6 +69,7 @@ struct PcgArgs {
     // an upper bound of the spectrum of D^-1 A
     int poly_deg = 0;
     const double* poly_hi = nullptr;
+    int R = 0;  // right-hand sides of this problem (k_pcg_batch)
 };
 
 // kMaxGrid, kMaxNS and kDefaultSpinLimit: launch.h
@@ -208,13 +210,17 @@ __device__ __forceinline__ void sell_row(const MeshDev& m, const OpParams<T>& op
 // (across warps, then across CTAs in a fixed order) run in FP64.  GB300
 // issues FP64 at 1/64 of the FP32 rate, so per-element FP64 terms, FP32->FP64
 // conversions and FP64 warp shuffles would dominate an FP32 iteration.
+__device__ __forceinline__ int* reduce_flags() {
+    __shared__ int f[2];
+    return f;
+}
 template <int NQ, int VW, int NP, typename T>
 __device__ __forceinline__ bool grid_reduce(T (&acc)[NQ][VW], double* scratch, double* partials, int& red_id,
                                             unsigned* bar, int* status, long long limit, double* out, int cta,
                                             int ncta) {
     constexpr int R = VW * NP, NS = NQ * R;
-    __shared__ int s_last;
-    __shared__ int s_ok;
+    int* flags = reduce_flags();
+    int &s_last = flags[0], &s_ok = flags[1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     // Warp sums by reduce-scatter: the NQ x VW values of a thread are padded
     // to P2 (a power of two); at each shuffle level the lanes whose level bit
@@ -399,7 +405,23 @@ __device__ __forceinline__ T* cheb_patch(const PcgArgs<T>& a, int ob, int nown, 
 }
 
 // ---------------------------------------------------------------- the solver
-template <typename T, int R, int OP, bool kPoly = false, int NT = kThreads>
+// The solver's static shared memory, for at most RM right-hand sides: one
+// block for all instantiations of pcg_body in a kernel.
+template <int RM, int NT, bool kPoly>
+struct PcgShared {
+    double scratch[(NT / 32) * kMaxNS];
+    double red[kMaxNS];
+    double bb[RM], rz[RM], rz_old[RM], rr[RM], alpha[RM], beta[RM], zcoef[RM];
+    int flag;
+    double pco[kPoly ? kMaxPolyDegree + 1 : 1];
+};
+template <int RM, int NT, bool kPoly>
+__device__ __forceinline__ PcgShared<RM, NT, kPoly>& pcg_shared() {
+    __shared__ PcgShared<RM, NT, kPoly> s;
+    return s;
+}
+
+template <typename T, int R, int OP, bool kPoly = false, int NT = kThreads, int RM = R>
 __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, const int ncta) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr bool kCsr = (OP == OP_CSR1 || OP == OP_CSR2);
@@ -411,10 +433,10 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
     } else {
         s.carve(reinterpret_cast<T*>(smem_raw), a.m.max_touched, a.m.max_own);
     }
-    __shared__ double scratch[(NT / 32) * kMaxNS];
-    __shared__ double red[kMaxNS];
-    __shared__ double bb[R], rz[R], rz_old[R], rr[R], alpha[R], beta[R], zcoef[R];
-    __shared__ int s_flag;
+    PcgShared<RM, NT, kPoly>& sh = pcg_shared<RM, NT, kPoly>();
+    double *scratch = sh.scratch, *red = sh.red, *bb = sh.bb, *rz = sh.rz, *rz_old = sh.rz_old, *rr = sh.rr;
+    double *alpha = sh.alpha, *beta = sh.beta, *zcoef = sh.zcoef, *pco = sh.pco;
+    int& s_flag = sh.flag;
 
     const MeshDev& m = a.m;
     const int P = m.P;
@@ -430,7 +452,6 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
     // overlay the staged p (phase A is over whenever they are in use)
     const int deg = (kPoly && kCsr && zs) ? a.poly_deg : 0;  // kPoly: a separate instantiation keeps
                                                               // the Jacobi kernel's registers unchanged
-    __shared__ double pco[kMaxPolyDegree + 1];
     T *cV = nullptr, *cW0 = nullptr, *cW1 = nullptr;
     bool top_neg = false;  // a_deg = -1: the Horner start is -v
     if (deg > 0) {
@@ -1411,11 +1432,15 @@ __global__ void __launch_bounds__(kThreads, 4) k_pcg_ring(PcgArgs<T> a, RingLayo
     pcg_ring_body<T, R, OP>(a, L, blockIdx.x, gridDim.x);
 }
 
-// Independent problems (meshes of different sizes) in one cooperative
-// launch: CTAs [cta_begin[j], cta_begin[j+1]) solve problem j, and each
-// problem's barriers and reductions involve only its own CTAs.
-template <typename T, int R, int OP, bool kPoly = false>
-__global__ void __launch_bounds__(kThreads) k_pcg_batch(const PcgArgs<T>* __restrict__ probs,
+// Independent problems (meshes of different sizes, each with its own number
+// of right-hand sides, at most RM) in one cooperative launch: CTAs
+// [cta_begin[j], cta_begin[j+1]) solve problem j, and each problem's barriers
+// and reductions involve only its own CTAs.  FP64 multiply-adds bound a
+// problem with several patches per CTA, so padding its right-hand sides to
+// the batch's largest number would cost in proportion.  Three CTAs per SM (70
+// registers for Jacobi, no spills) instead of the two that 102 registers allow.
+template <typename T, int RM, int OP, bool kPoly = false>
+__global__ void __launch_bounds__(kThreads, 3) k_pcg_batch(const PcgArgs<T>* __restrict__ probs,
                                                         const int* __restrict__ cta_begin, int nprob) {
     int lo = 0, hi = nprob - 1;
     while (lo < hi) {
@@ -1427,7 +1452,14 @@ __global__ void __launch_bounds__(kThreads) k_pcg_batch(const PcgArgs<T>* __rest
     }
     const int b0 = cta_begin[lo];
     const PcgArgs<T> a = probs[lo];
-    pcg_body<T, R, OP, kPoly>(a, int(blockIdx.x) - b0, cta_begin[lo + 1] - b0);
+    const int cta = int(blockIdx.x) - b0, ncta = cta_begin[lo + 1] - b0;
+    if (RM == 1 || a.R == 1) pcg_body<T, 1, OP, kPoly, kThreads, RM>(a, cta, ncta);
+    if constexpr (RM >= 2)
+        if (a.R == 2) pcg_body<T, 2, OP, kPoly, kThreads, RM>(a, cta, ncta);
+    if constexpr (RM >= 4)
+        if (a.R == 4) pcg_body<T, 4, OP, kPoly, kThreads, RM>(a, cta, ncta);
+    if constexpr (RM >= 8)
+        if (a.R == 8) pcg_body<T, 8, OP, kPoly, kThreads, RM>(a, cta, ncta);
 }
 
 template <int R>
@@ -1438,8 +1470,9 @@ cudaError_t batch_prepare_t(const std::vector<PcgBatchProblem>& probs, PcgBatchP
     size_t smem = 0;
     for (const auto& p : probs) {
         if (p.w.poly_deg < 0 || p.w.poly_deg > kMaxPolyDegree) return cudaErrorInvalidValue;
-        smem = std::max(smem, sizeof(double) * size_t(p.m.max_touched) * R);
-        if (poly) smem = std::max(smem, 3 * sizeof(double) * size_t(p.m.max_own) * R);
+        if (p.R < 1 || p.R > R) return cudaErrorInvalidValue;
+        smem = std::max(smem, sizeof(double) * size_t(p.m.max_touched) * p.R);
+        if (poly) smem = std::max(smem, 3 * sizeof(double) * size_t(p.m.max_own) * p.R);
     }
     auto kern = poly ? k_pcg_batch<double, R, OP_CSR1, true> : k_pcg_batch<double, R, OP_CSR1>;
     cudaError_t err = qpat::allow_smem((const void*)kern, size_t(smem));
@@ -1453,30 +1486,33 @@ cudaError_t batch_prepare_t(const std::vector<PcgBatchProblem>& probs, PcgBatchP
     const int nprob = int(probs.size());
     int resident = std::min(per_sm * nsm, kMaxGrid);
     if (resident < nprob) return cudaErrorInvalidConfiguration;
-    // CTAs proportional to the work (nodes), at least one per problem and at
-    // most one per patch
-    double total = 0;
-    for (const auto& p : probs) total += double(p.m.N);
-    std::vector<int> cnt(nprob);
-    int used = 0;
-    for (int j = 0; j < nprob; ++j) {
-        int c = int(double(resident - nprob) * double(probs[j].m.N) / total) + 1;
-        c = std::min(c, probs[j].m.P);
-        cnt[j] = c;
-        used += c;
-    }
-    // hand the remaining CTAs to the problems with the most nodes per CTA
-    for (int guard = 0; used < resident && guard < resident; ++guard) {
-        int best = -1;
+    // The launch lasts as long as its slowest problem: the next CTAs go to
+    // the problem with the largest estimated time, as many as take one patch
+    // off its fullest CTA.  A problem's iterations grow with its mesh side
+    // (N^(1/3)); an iteration costs each CTA its patches in turn, dearer with
+    // more right-hand sides, and two barriers (about two patches' time).
+    // 12 meshes of 16 to 48 nodes a side, 1 to 4 illuminations: 33 ms split by
+    // nodes alone with every problem at 4 right-hand sides and two CTAs per SM,
+    // 19.8 ms now.
+    std::vector<int> cnt(nprob, 1);
+    int used = nprob;
+    for (;;) {
+        int worst = -1;
         double load = 0;
-        for (int j = 0; j < nprob; ++j)
-            if (cnt[j] < probs[j].m.P && double(probs[j].m.N) / cnt[j] > load) {
-                load = double(probs[j].m.N) / cnt[j];
-                best = j;
+        for (int j = 0; j < nprob; ++j) {
+            const int most = (probs[j].m.P + cnt[j] - 1) / cnt[j];
+            const double t = std::cbrt(double(probs[j].m.N)) * (most * (1.0 + probs[j].R) + 4.0);
+            if (t > load) {
+                load = t;
+                worst = most > 1 ? j : -1;
             }
-        if (best < 0) break;
-        ++cnt[best];
-        ++used;
+        }
+        if (worst < 0) break;
+        const int Pw = probs[worst].m.P, most = (Pw + cnt[worst] - 1) / cnt[worst];
+        const int want = (Pw + most - 2) / (most - 1);
+        if (used + want - cnt[worst] > resident) break;
+        used += want - cnt[worst];
+        cnt[worst] = want;
     }
     std::vector<int> begin(nprob + 1, 0);
     for (int j = 0; j < nprob; ++j) begin[j + 1] = begin[j] + cnt[j];
@@ -1501,8 +1537,9 @@ cudaError_t batch_prepare_t(const std::vector<PcgBatchProblem>& probs, PcgBatchP
         a.rtol2 = p.rtol * p.rtol;
         a.maxit = p.maxit;
         a.spin_limit = p.w.spin_limit > 0 ? p.w.spin_limit : kDefaultSpinLimit;
+        a.R = p.R;
+        a.z = static_cast<double*>(p.w.z);
         if (poly) {
-            a.z = static_cast<double*>(p.w.z);
             a.poly_deg = p.w.poly_deg;
             a.poly_hi = p.w.poly_hi;
         }
