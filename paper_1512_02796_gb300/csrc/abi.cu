@@ -341,7 +341,6 @@ int solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so_in, int R, cons
     w.p1 = M->ws.get_bytes(nm("p1"), n * esz, s, &e);
     w.q = M->ws.get_bytes(nm("q"), n * esz, s, &e);
     w.partials = M->ws.get<double>("pcg.partials", pcg_partials_doubles(), s, &e);
-    w.bar = M->ws.get<unsigned>("pcg.bar", 2, s, &e);
     w.status = M->ws.get<int>("pcg.status", 1, s, &e);
     w.iters = M->ws.get<int>("pcg.iters", 1, s, &e);
     w.stats = M->ws.get<double>("pcg.stats", 32, s, &e);

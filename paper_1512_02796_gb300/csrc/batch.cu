@@ -21,7 +21,7 @@ struct qpat_batch_s {
         double *kappa = nullptr, *mu = nullptr, *flux = nullptr, *phi = nullptr;   // caller layout
         double *kl = nullptr, *ml = nullptr, *vals = nullptr, *inv = nullptr;     // library layout
         double *f = nullptr, *x = nullptr, *r = nullptr, *p0 = nullptr, *p1 = nullptr, *q = nullptr;
-        double *partials = nullptr, *ctl = nullptr;
+        double* ctl = nullptr;  // status, iterations, statistics; from kCtlDoubles on the reductions' slots
         qpat::ElemScratch scratch;                 // of this problem's assembly
         double *z = nullptr;   // preconditioned residual
         double *gb = nullptr;  // patch-local Chebyshev preconditioner
@@ -40,6 +40,8 @@ struct qpat_batch_s {
 using namespace qpat;
 
 namespace {
+
+constexpr size_t kCtlDoubles = 64;
 
 int batch_alloc(qpat_batch_s* B, double** p, size_t n) {
     void* v = nullptr;
@@ -63,7 +65,8 @@ void batch_release(qpat_batch_s* B) {
 // the recorded sequence (also valid eagerly)
 int batch_sequence(qpat_batch_s* B, cudaStream_t s) {
     cudaError_t e;
-    for (auto& P : B->probs) {
+    for (size_t j = 0; j < B->probs.size(); ++j) {
+        auto& P = B->probs[j];
         const MeshDev& m = P.mesh->d;
         const int64_t N = m.N;
         if ((e = launch_to_lib<double, double>(m, 1, 1, P.kappa, P.kl, s)) != cudaSuccess ||
@@ -76,7 +79,9 @@ int batch_sequence(qpat_batch_s* B, cudaStream_t s) {
             return cuda_fail(e, "qpat_batch_forward: memset");
         if ((e = launch_load(m, P.K, P.R, P.flux, P.f, s)) != cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: load");
-        if ((e = cudaMemsetAsync(P.ctl, 0, sizeof(double) * 8, s)) != cudaSuccess)  // barrier, status, iterations
+        // status, iterations and, behind them, the reductions' slots
+        if ((e = cudaMemsetAsync(P.ctl, 0, kCtlDoubles * sizeof(double) + pcg_slots_bytes(B->plan.cta_count[j], P.R), s)) !=
+            cudaSuccess)
             return cuda_fail(e, "qpat_batch_forward: memset");
     }
     if ((e = pcg_batch_launch(B->plan, s)) != cudaSuccess) return cuda_fail(e, "qpat_batch_forward: batched pcg");
@@ -123,7 +128,7 @@ int qpat_batch_create(int nprob, const qpat_mesh_t* meshes, const int* K, const 
             (rc = batch_alloc(B, &P.f, N * R)) || (rc = batch_alloc(B, &P.x, N * R)) ||
             (rc = batch_alloc(B, &P.r, N * R)) || (rc = batch_alloc(B, &P.p0, N * R)) ||
             (rc = batch_alloc(B, &P.p1, N * R)) || (rc = batch_alloc(B, &P.q, N * R)) ||
-            (rc = batch_alloc(B, &P.partials, pcg_partials_doubles())) || (rc = batch_alloc(B, &P.ctl, 64)))
+            (rc = batch_alloc(B, &P.ctl, kCtlDoubles + pcg_partials_doubles(std::min(P.mesh->d.P, pcg_max_grid()), P.R))))
             break;
         double *tq = nullptr, *ev = nullptr;
         if ((rc = batch_alloc(B, &tq, 2 * size_t(P.mesh->el.E))) || (rc = batch_alloc(B, &ev, 2 * size_t(P.mesh->el.NE))))
@@ -141,8 +146,7 @@ int qpat_batch_create(int nprob, const qpat_mesh_t* meshes, const int* K, const 
         q.w.p0 = P.p0;
         q.w.p1 = P.p1;
         q.w.q = P.q;
-        q.w.partials = P.partials;
-        q.w.bar = reinterpret_cast<unsigned*>(P.ctl);
+        q.w.partials = P.ctl + kCtlDoubles;
         q.w.status = reinterpret_cast<int*>(P.ctl + 1);
         q.w.iters = reinterpret_cast<int*>(P.ctl + 2);
         q.w.stats = P.ctl + 8;

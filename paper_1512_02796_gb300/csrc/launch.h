@@ -79,11 +79,22 @@ cudaError_t launch_cast_d2f(int64_t n, const double* in, float* out, cudaStream_
 constexpr int kMaxPolyDegree = 8;
 
 // Bounds of the persistent PCG kernels' grid reductions: at most kMaxGrid
-// CTAs, each contributing kMaxNS doubles (3 quantities x 16 RHS).  The
-// partials buffer holds 2 x kMaxGrid x kMaxNS + 2 x kMaxNS doubles
-// (pcg_partials_doubles).
+// CTAs, each contributing kMaxNS doubles (3 quantities x 16 RHS).
 constexpr int kMaxGrid = 152 * 8;
 constexpr int kMaxNS = 48;
+// CTAs of a group whose partial sums its first member adds up (1: no groups),
+// the slots of one reduction, and the bytes that a launch of ncta CTAs with R
+// right-hand sides uses (and zeroes) of PcgWork::partials.
+__host__ __device__ constexpr int reduce_group(int ncta) { return ncta <= 64 ? 1 : ncta <= 512 ? 16 : 64; }
+__host__ __device__ constexpr int reduce_slots(int ncta) {
+    const int g = reduce_group(ncta);
+    return g == 1 ? ncta : ncta + (ncta + g - 1) / g;
+}
+constexpr size_t pcg_slots_bytes(int ncta, int R) { return size_t(2) * reduce_slots(ncta) * (3 * R) * 16; }
+// Size of PcgWork::partials for launches of up to ncta CTAs and R right-hand sides.
+constexpr size_t pcg_partials_doubles(int ncta = kMaxGrid, int R = 16) {
+    return size_t(2) * (ncta + 64) * (3 * R) * 2;
+}
 // Default bound of a grid-barrier wait: polls of ~32 ns sleep (about 2 s).
 constexpr long long kDefaultSpinLimit = 40000000LL;
 
@@ -110,8 +121,7 @@ struct PcgWork {
     // upper bound of the spectrum of D^-1 A
     int poly_deg = 0;
     const double* poly_hi = nullptr;
-    double* partials;   // 2 x max_grid x 3R
-    unsigned* bar;      // 2
+    double* partials;   // pcg_partials_doubles(); 16-byte aligned
     int* status;        // 1
     int* iters;         // 1
     double* stats;      // 2R: final r.r, b.b
@@ -144,7 +154,7 @@ struct PcgBatchProblem {
     MeshDev m;
     const double* vals;     // assembled K values
     const double* invdiag;  // N
-    PcgWork w;              // b, x, r, p0, p1, q, z (optional), partials, bar, status, iters, stats
+    PcgWork w;              // b, x, r, p0, p1, q, z (optional), partials (for P CTAs and R), status, iters, stats
     int R;                  // right-hand sides: 1, 2, 4 or 8
     double rtol;
     int maxit;
@@ -168,6 +178,5 @@ bool pcg_fits(const MeshDev& m, int OP, int R, int deg);
 template <typename T>
 bool apply_csr_fits(const MeshDev& m, int R);
 int pcg_max_grid();            // upper bound of the cooperative grid
-size_t pcg_partials_doubles();  // size of PcgWork::partials (per-CTA partials + totals)
 
 }  // namespace qpat

@@ -21,11 +21,11 @@ namespace {
 // Node count times padded right-hand sides that the scratch can hold.
 constexpr int64_t kNoallocMaxNR = int64_t(1) << 19;
 // Scratch layout in doubles: kappa, mu, inverse diagonal (N each, N <= max),
-// then six N x R vectors (f, x, r, p0, p1, q), two reduction buffers and a
-// small control block (barrier, status, iteration count, statistics).
-constexpr int64_t kPartials = int64_t(2) * kMaxGrid * kMaxNS + 2 * kMaxNS;  // = pcg_partials_doubles()
+// then six N x R vectors (f, x, r, p0, p1, q), the reductions' slots and a
+// small control block (status, iteration count, statistics).
+constexpr int64_t kPartials = int64_t(pcg_partials_doubles());
 constexpr int64_t kCtl = 64;
-// control block: barrier and status words in ctl[0..2], then 2 x 16 doubles
+// control block: status and iteration words in ctl[1..2], then 2 x 16 doubles
 // of solver statistics from ctl[8]
 static_assert(8 + 2 * 16 <= kCtl, "control block too small for the solver statistics");
 constexpr int64_t kNoallocDoubles = 3 * kNoallocMaxNR + 6 * kNoallocMaxNR + kPartials + kCtl;
@@ -93,7 +93,6 @@ extern "C" int qpat_forward_noalloc_dev(qpat_mesh_t M, const double* kappa, cons
     w.p1 = p1;
     w.q = q;
     w.partials = partials;
-    w.bar = reinterpret_cast<unsigned*>(ctl);        // 2 x unsigned in ctl[0]
     w.status = reinterpret_cast<int*>(ctl + 1);
     w.iters = reinterpret_cast<int*>(ctl + 2);
     w.stats = ctl + 8;                               // 32 doubles

@@ -12,15 +12,14 @@
 //   phase B: x += alpha p, r -= alpha q on its owned nodes, z = M^-1 r
 //            (Jacobi D^-1, or the patch-local Chebyshev polynomial below),
 //            accumulating r.z and r.r.
-// Each phase ends with a grid-wide reduction behind a bounded grid barrier:
-// every CTA writes its partial sums, the last CTA to arrive adds all of them
-// in a fixed order, publishes the totals and releases the others, so every
-// CTA takes the same decisions from bit-identical scalars.  R right-hand
+// Each phase ends with a grid-wide reduction with bounded waits: every CTA
+// publishes its partial sums, waits for those of all the others and adds them
+// in a fixed order, so every CTA takes the same decisions from bit-identical
+// scalars.  R right-hand
 // sides share one launch with their own alpha and beta (block form of the
 // stacked illuminations of Sec. 4); node vectors are N x R node-major and
 // are moved as 16-byte vectors (4 floats or 2 doubles of consecutive RHS)
 // wherever R allows.  Scalars are accumulated in FP64 for either T.
-#include <cuda/atomic>
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -45,7 +44,6 @@ struct PcgArgs {
     T* p1;
     T* q;
     double* partials;
-    unsigned* bar;
     int* status;
     int* iters;
     double* stats;
@@ -203,6 +201,90 @@ __device__ __forceinline__ void sell_row(const MeshDev& m, const OpParams<T>& op
 }
 
 // ---------------------------------------------------------------- grid reduction
+// Slots of the grid reductions: a partial sum travels as two 64-bit words,
+// each half of the double beside the reduction's number, so that a reader
+// that sees the number in both words has the value: no counter, no flag and no
+// second read.  The slots are zeroed before a launch (numbers start at 1) and
+// used alternately by even and odd reductions; a CTA writes reduction k + 2
+// only after it has the totals of k + 1, which every CTA entered after it had
+// read those of k.
+__device__ __forceinline__ void slot_store(ulonglong2* p, double v, unsigned tag) {
+    const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
+    const unsigned long long lo = (b << 32) | tag, hi = (b & 0xffffffff00000000ull) | tag;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(__cvta_generic_to_global(p)), "l"(lo), "l"(hi)
+                 : "memory");
+}
+__device__ __forceinline__ ulonglong2 slot_load(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
+                 : "=l"(v.x), "=l"(v.y)
+                 : "l"(__cvta_generic_to_global(p))
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ double slot_value(const ulonglong2& v) {
+    return __longlong_as_double((long long)((v.y & 0xffffffff00000000ull) | (v.x >> 32)));
+}
+__device__ __forceinline__ int* reduce_flags() {
+    __shared__ int f[1];
+    return f;
+}
+
+// Publishes the CTA's sums (scratch, one row of NS a warp) and forms the totals
+// of all CTAs in out; set: the half of the slots that this reduction uses.
+// kOrder: what any CTA wrote before is visible to all after.
+template <int NS, int R, bool kOrder>
+__device__ __forceinline__ bool share_sums(double* scratch, double* partials, int set, unsigned tag, int* status,
+                                           long long limit, double* out, int cta, int ncta) {
+    constexpr int C = NS * 8 <= kThreads ? 8 : kThreads / NS;  // chains of additions per quantity
+    const int t = threadIdx.x, group = reduce_group(ncta), ng = (ncta + group - 1) / group;
+    // the groups' slots, then (where there are groups) one per CTA
+    ulonglong2* tops = reinterpret_cast<ulonglong2*>(partials) + set * reduce_slots(ncta) * (3 * R);
+    double a = 0.0;
+    if (t < NS)
+        for (int w = 0; w < int(blockDim.x >> 5); ++w) a += scratch[w * NS + t];
+    bool up = group > 1;  // first to the group's first member, which goes round twice
+    for (;;) {
+        if (t < NS) {
+            if (kOrder) __threadfence();
+            slot_store(tops + ((up ? ng + cta : cta / group) * NS + t), a, tag);
+        }
+        if (up && cta % group != 0) up = false;
+        __syncthreads();
+        const int n = up ? min(group, ncta - cta) : ng;
+        const ulonglong2* from = tops + (up ? (ng + cta) * NS : 0);
+        if (t < NS * C) {
+            double sum = 0.0;
+            for (int j = t / NS; j < n; j += C) {
+                ulonglong2 v = slot_load(from + j * NS + t % NS);
+                for (long long spins = 0; unsigned(v.x) != tag || unsigned(v.y) != tag; v = slot_load(from + j * NS + t % NS)) {
+                    if (++spins > limit) {
+                        atomicExch(status, QPAT_ETIMEOUT);
+                        reduce_flags()[0] = 0;
+                        break;
+                    }
+                    if (spins > 16) __nanosleep(32);
+                }
+                sum += slot_value(v);
+            }
+            if (kOrder) __threadfence();
+            scratch[t] = sum;
+        }
+        __syncthreads();
+        if (!reduce_flags()[0]) return false;
+        if (t < NS) {
+            a = 0.0;
+#pragma unroll
+            for (int c = 0; c < C; ++c) a += scratch[c * NS + t];
+        }
+        if (!up) break;
+        up = false;
+    }
+    if (t < NS) out[t] = a;
+    __syncthreads();
+    return true;
+}
+
 // Sum over the grid of NQ x R values; thread t holds acc[q][c] for RHS
 // (t % NP) * VW + c.  Totals land in out[q * R + r] (shared) in every CTA.
 // Each thread's partial sums (a few terms) and the sums across a warp are
@@ -210,17 +292,22 @@ __device__ __forceinline__ void sell_row(const MeshDev& m, const OpParams<T>& op
 // (across warps, then across CTAs in a fixed order) run in FP64.  GB300
 // issues FP64 at 1/64 of the FP32 rate, so per-element FP64 terms, FP32->FP64
 // conversions and FP64 warp shuffles would dominate an FP32 iteration.
-__device__ __forceinline__ int* reduce_flags() {
-    __shared__ int f[2];
-    return f;
-}
-template <int NQ, int VW, int NP, typename T>
+//
+// Bound by round trips to L2.  Every CTA reads the partial sums of all CTAs
+// (at most 64) or of all groups of CTAs, whose first members have read their
+// group's: one or two trips after the last CTA's store.  The form before (an
+// arrival counter, the last CTA adding and publishing the totals, a generation
+// word to poll) took about six.  A PCG iteration (two reductions, three
+// operator sweeps) on 1331 nodes, 42 CTAs: 17.4 -> 15.1 us; on 11,907 nodes
+// x 4 RHS, 304 CTAs: 23.5 -> 19.8 us.  Above 64 CTAs the additions of all
+// partial sums in every CTA (two a clock and SM in FP64) would cost more than
+// the trip that the groups add.
+//
+// kOrder: what any CTA wrote before the reduction is visible to all after it.
+template <int NQ, int VW, int NP, bool kOrder = true, typename T>
 __device__ __forceinline__ bool grid_reduce(T (&acc)[NQ][VW], double* scratch, double* partials, int& red_id,
-                                            unsigned* bar, int* status, long long limit, double* out, int cta,
-                                            int ncta) {
+                                            int* status, long long limit, double* out, int cta, int ncta) {
     constexpr int R = VW * NP, NS = NQ * R;
-    int* flags = reduce_flags();
-    int &s_last = flags[0], &s_ok = flags[1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     // Warp sums by reduce-scatter: the NQ x VW values of a thread are padded
     // to P2 (a power of two); at each shuffle level the lanes whose level bit
@@ -261,69 +348,10 @@ __device__ __forceinline__ bool grid_reduce(T (&acc)[NQ][VW], double* scratch, d
             if (f < V) scratch[warp * NS + (f / VW) * R + part * VW + (f % VW)] = double(v[i]);
         }
     }
+    if (threadIdx.x == 0) reduce_flags()[0] = 1;
     __syncthreads();
-    double* part = partials + size_t(red_id & 1) * kMaxGrid * kMaxNS;
-    double* res = partials + size_t(2) * kMaxGrid * kMaxNS + (red_id & 1) * kMaxNS;
     ++red_id;
-    if (threadIdx.x < NS) {
-        double a = 0.0;
-        for (int w = 0; w < nw; ++w) a += scratch[w * NS + threadIdx.x];
-        part[size_t(cta) * NS + threadIdx.x] = a;
-    }
-    __syncthreads();
-    cuda::atomic_ref<unsigned, cuda::thread_scope_device> cnt(bar[0]);
-    cuda::atomic_ref<unsigned, cuda::thread_scope_device> gen(bar[1]);
-    unsigned g = 0;
-    if (threadIdx.x == 0) {
-        g = gen.load(cuda::memory_order_acquire);
-        __threadfence();
-        const unsigned old = cnt.fetch_add(1u, cuda::memory_order_acq_rel);
-        s_last = old == unsigned(ncta) - 1;
-        s_ok = 1;
-    }
-    __syncthreads();
-    if (s_last) {
-        // the last CTA adds the partials of every CTA in a fixed order
-        __threadfence();
-        for (int s = warp; s < NS; s += nw) {
-            // four independent chains keep four loads per lane in flight
-            double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-            int j = lane;
-            for (; j + 96 < ncta; j += 128) {
-                a0 += __ldcg(part + size_t(j) * NS + s);
-                a1 += __ldcg(part + size_t(j + 32) * NS + s);
-                a2 += __ldcg(part + size_t(j + 64) * NS + s);
-                a3 += __ldcg(part + size_t(j + 96) * NS + s);
-            }
-            for (; j < ncta; j += 32) a0 += __ldcg(part + size_t(j) * NS + s);
-            double a = (a0 + a1) + (a2 + a3);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (lane == 0) res[s] = a;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            cnt.store(0u, cuda::memory_order_relaxed);
-            gen.fetch_add(1u, cuda::memory_order_release);
-        }
-    } else if (threadIdx.x == 0) {
-        long long spins = 0;
-        while (gen.load(cuda::memory_order_acquire) == g) {
-            if (++spins > limit) {
-                atomicExch(status, QPAT_ETIMEOUT);
-                s_ok = 0;
-                break;
-            }
-            __nanosleep(32);
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    if (!s_ok) return false;
-    if (threadIdx.x < NS) out[threadIdx.x] = __ldcg(res + threadIdx.x);
-    __syncthreads();
-    return true;
+    return share_sums<NS, R, kOrder>(scratch, partials, red_id & 1, unsigned(red_id), status, limit, out, cta, ncta);
 }
 
 // ---------------------------------------------------------------- preconditioner
@@ -511,7 +539,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
         }
 #pragma unroll
         for (int c = 0; c < VW; ++c) acc[2][c] = acc[0][c];
-        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta,
+        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta,
                                     ncta))
             return;
         if (threadIdx.x < R) {
@@ -634,7 +662,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
                 __syncthreads();
             }
         }
-        if (!grid_reduce<1, VW, NP>(accA, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta,
+        if (!grid_reduce<1, VW, NP, false>(accA, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta,
                                     ncta))
             return;
         if (threadIdx.x == 0) {
@@ -713,7 +741,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
                 }
             }
         }
-        if (!grid_reduce<2, VW, NP>(accB, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta,
+        if (!grid_reduce<2, VW, NP>(accB, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta,
                                     ncta))
             return;
         if (threadIdx.x < R) {
@@ -746,8 +774,13 @@ constexpr int min_ctas() {
     return (OP == OP_CSR1 || OP == OP_CSR2) ? 4 : 1;
 }
 
+// FP64 on the assembled operators: three resident CTAs per SM (80 registers).
+template <typename T, int OP, bool kPoly>
+constexpr int pcg_ctas() {
+    return sizeof(T) == 8 && (OP == OP_CSR1 || (OP == OP_CSR2 && !kPoly)) ? 3 : 1;
+}
 template <typename T, int R, int OP, bool kPoly = false>
-__global__ void __launch_bounds__(kThreads) k_pcg(PcgArgs<T> a) {
+__global__ void __launch_bounds__(kThreads, pcg_ctas<T, OP, kPoly>()) k_pcg(PcgArgs<T> a) {
     pcg_body<T, R, OP, kPoly>(a, blockIdx.x, gridDim.x);
 }
 
@@ -841,7 +874,7 @@ __device__ __forceinline__ void pcg1_body(const PcgArgs<T>& a, const int cta, co
             __syncthreads();
         }
         // r = b, so |r|^2 = |b|^2
-        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta, ncta))
+        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta, ncta))
             return;
         if (threadIdx.x == 0) {
             int bad = 0;
@@ -963,7 +996,7 @@ __device__ __forceinline__ void pcg1_body(const PcgArgs<T>& a, const int cta, co
             }
             __syncthreads();
         }
-        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta, ncta))
+        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta, ncta))
             return;
         if (threadIdx.x == 0) {
             int bad = 0;
@@ -1188,7 +1221,7 @@ __device__ __forceinline__ void pcg_ring_body(const PcgArgs<T>& a, const RingLay
         }
 #pragma unroll
         for (int c = 0; c < VW; ++c) acc[2][c] = acc[0][c];
-        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta,
+        if (!grid_reduce<3, VW, NP>(acc, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta,
                                     ncta)) {
             drain();
             return;
@@ -1341,7 +1374,7 @@ __device__ __forceinline__ void pcg_ring_body(const PcgArgs<T>& a, const RingLay
         double accA[1][VW];
 #pragma unroll
         for (int c = 0; c < VW; ++c) accA[0][c] = threadIdx.x < NP ? dot_s[threadIdx.x][c] : 0.0;
-        if (!grid_reduce<1, VW, NP>(accA, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta,
+        if (!grid_reduce<1, VW, NP, false>(accA, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta,
                                     ncta)) {
             drain();
             return;
@@ -1402,7 +1435,7 @@ __device__ __forceinline__ void pcg_ring_body(const PcgArgs<T>& a, const RingLay
                 }
             }
         }
-        if (!grid_reduce<2, VW, NP>(accB, scratch, a.partials, red_id, a.bar, a.status, a.spin_limit, red, cta,
+        if (!grid_reduce<2, VW, NP>(accB, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta,
                                     ncta)) {
             drain();
             return;
@@ -1530,7 +1563,6 @@ cudaError_t batch_prepare_t(const std::vector<PcgBatchProblem>& probs, PcgBatchP
         a.p1 = static_cast<double*>(p.w.p1);
         a.q = static_cast<double*>(p.w.q);
         a.partials = p.w.partials;
-        a.bar = p.w.bar;
         a.status = p.w.status;
         a.iters = p.w.iters;
         a.stats = p.w.stats;
@@ -1632,7 +1664,6 @@ cudaError_t launch_pcg_t(const MeshDev& m, const OpParams<T>& op, const T* invdi
     a.p1 = static_cast<T*>(w.p1);
     a.q = static_cast<T*>(w.q);
     a.partials = w.partials;
-    a.bar = w.bar;
     a.status = w.status;
     a.iters = w.iters;
     a.stats = w.stats;
@@ -1650,7 +1681,7 @@ cudaError_t launch_pcg_t(const MeshDev& m, const OpParams<T>& op, const T* invdi
     a.poly_deg = deg;
     a.poly_hi = w.poly_hi;
     if (kSingle && !(a.r1 && a.s0 && a.s1 && a.w1)) return cudaErrorInvalidValue;
-    err = cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), s);
+    err = cudaMemsetAsync(w.partials, 0, pcg_slots_bytes(grid, R), s);
     if (err != cudaSuccess) return err;
     err = cudaMemsetAsync(w.status, 0, sizeof(int), s);
     if (err != cudaSuccess) return err;
@@ -1702,14 +1733,13 @@ cudaError_t launch_pcg_ring_t(const MeshDev& m, const OpParams<T>& op, const T* 
     a.p1 = static_cast<T*>(w.p1);
     a.q = static_cast<T*>(w.q);
     a.partials = w.partials;
-    a.bar = w.bar;
     a.status = w.status;
     a.iters = w.iters;
     a.stats = w.stats;
     a.rtol2 = rtol * rtol;
     a.maxit = maxit;
     a.spin_limit = w.spin_limit > 0 ? w.spin_limit : kDefaultSpinLimit;
-    err = cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), s);
+    err = cudaMemsetAsync(w.partials, 0, pcg_slots_bytes(grid, R), s);
     if (err != cudaSuccess) return err;
     err = cudaMemsetAsync(w.status, 0, sizeof(int), s);
     if (err != cudaSuccess) return err;
@@ -1770,8 +1800,6 @@ void pcg_batch_release(PcgBatchPlan& plan) {
     plan.dev_args = nullptr;
     plan.dev_cta_begin = nullptr;
 }
-
-size_t pcg_partials_doubles() { return size_t(2) * kMaxGrid * kMaxNS + 2 * kMaxNS; }
 
 template <typename T>
 cudaError_t launch_pcg(const MeshDev& m, int OP, int R, const OpParams<T>& op, const T* invdiag,

@@ -51,7 +51,6 @@ int time_candidate(qpat_mesh_s* M, const double* kap_h, const double* mu_h, int 
     w.p1 = p1;
     w.q = q;
     w.partials = part;
-    w.bar = reinterpret_cast<unsigned*>(ctl);
     w.status = reinterpret_cast<int*>(ctl + 1);
     w.iters = reinterpret_cast<int*>(ctl + 2);
     w.stats = ctl + 8;
