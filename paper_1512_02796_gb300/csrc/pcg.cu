@@ -230,19 +230,28 @@ __device__ __forceinline__ int* reduce_flags() {
     return f;
 }
 
+// Sum of buf[c * stride], c < 8, as a tree (a chain of eight dependent FP64 additions takes three times as long).
+__device__ __forceinline__ double sum8(const double* buf, int stride) {
+    return ((buf[0] + buf[stride]) + (buf[2 * stride] + buf[3 * stride])) +
+           ((buf[4 * stride] + buf[5 * stride]) + (buf[6 * stride] + buf[7 * stride]));
+}
+
 // Publishes the CTA's sums (scratch, one row of NS a warp) and forms the totals
 // of all CTAs in out; set: the half of the slots that this reduction uses.
+// Up to 64 threads wait for the slots of each quantity, so that all slots of a
+// small launch are in flight at once (six one after the other: 3 us).
 // kOrder: what any CTA wrote before is visible to all after.
 template <int NS, int R, bool kOrder>
 __device__ __forceinline__ bool share_sums(double* scratch, double* partials, int set, unsigned tag, int* status,
                                            long long limit, double* out, int cta, int ncta) {
-    constexpr int C = NS * 8 <= kThreads ? 8 : kThreads / NS;  // chains of additions per quantity
+    constexpr int C = NS <= 4 ? 64 : NS <= 16 ? kThreads / (8 * NS) * 8 : NS <= 32 ? 8 : 4;  // slots at a time
+    static_assert(C * NS <= (kThreads / 32) * kMaxNS, "scratch too small");
     const int t = threadIdx.x, group = reduce_group(ncta), ng = (ncta + group - 1) / group;
     // the groups' slots, then (where there are groups) one per CTA
     ulonglong2* tops = reinterpret_cast<ulonglong2*>(partials) + set * reduce_slots(ncta) * (3 * R);
     double a = 0.0;
     if (t < NS)
-        for (int w = 0; w < int(blockDim.x >> 5); ++w) a += scratch[w * NS + t];
+        for (int w = 0; w < int(blockDim.x >> 5); w += 8) a += sum8(scratch + w * NS + t, NS);
     bool up = group > 1;  // first to the group's first member, which goes round twice
     for (;;) {
         if (t < NS) {
@@ -272,10 +281,22 @@ __device__ __forceinline__ bool share_sums(double* scratch, double* partials, in
         }
         __syncthreads();
         if (!reduce_flags()[0]) return false;
-        if (t < NS) {
-            a = 0.0;
+        if constexpr (C > 8) {
+            constexpr int S = C / 8;  // groups of eight
+            if (t < NS * S) a = sum8(scratch + t, NS * S);
+            __syncthreads();
+            if (t < NS * S) scratch[t] = a;
+            __syncthreads();
+            if (t < NS) {
+                if constexpr (S == 8) {
+                    a = sum8(scratch + t, NS);
+                } else {
 #pragma unroll
-            for (int c = 0; c < C; ++c) a += scratch[c * NS + t];
+                    for (int c = 1; c < S; ++c) a += scratch[c * NS + t];
+                }
+            }
+        } else if (t < NS) {
+            a = C == 8 ? sum8(scratch + t, NS) : (scratch[t] + scratch[NS + t]) + (scratch[2 * NS + t] + scratch[3 * NS + t]);
         }
         if (!up) break;
         up = false;
@@ -298,8 +319,8 @@ __device__ __forceinline__ bool share_sums(double* scratch, double* partials, in
 // group's: one or two trips after the last CTA's store.  The form before (an
 // arrival counter, the last CTA adding and publishing the totals, a generation
 // word to poll) took about six.  A PCG iteration (two reductions, three
-// operator sweeps) on 1331 nodes, 42 CTAs: 17.4 -> 15.1 us; on 11,907 nodes
-// x 4 RHS, 304 CTAs: 23.5 -> 19.8 us.  Above 64 CTAs the additions of all
+// operator sweeps) on 1331 nodes, 42 CTAs: 17.4 -> 11.8 us; on 11,907 nodes
+// x 4 RHS, 304 CTAs: 23.5 -> 17.0 us.  Above 64 CTAs the additions of all
 // partial sums in every CTA (two a clock and SM in FP64) would cost more than
 // the trip that the groups add.
 //
@@ -308,7 +329,7 @@ template <int NQ, int VW, int NP, bool kOrder = true, typename T>
 __device__ __forceinline__ bool grid_reduce(T (&acc)[NQ][VW], double* scratch, double* partials, int& red_id,
                                             int* status, long long limit, double* out, int cta, int ncta) {
     constexpr int R = VW * NP, NS = NQ * R;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // Warp sums by reduce-scatter: the NQ x VW values of a thread are padded
     // to P2 (a power of two); at each shuffle level the lanes whose level bit
     // is clear keep the lower half of their set and the others the upper
@@ -440,7 +461,6 @@ struct PcgShared {
     double scratch[(NT / 32) * kMaxNS];
     double red[kMaxNS];
     double bb[RM], rz[RM], rz_old[RM], rr[RM], alpha[RM], beta[RM], zcoef[RM];
-    int flag;
     double pco[kPoly ? kMaxPolyDegree + 1 : 1];
 };
 template <int RM, int NT, bool kPoly>
@@ -464,7 +484,6 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
     PcgShared<RM, NT, kPoly>& sh = pcg_shared<RM, NT, kPoly>();
     double *scratch = sh.scratch, *red = sh.red, *bb = sh.bb, *rz = sh.rz, *rz_old = sh.rz_old, *rr = sh.rr;
     double *alpha = sh.alpha, *beta = sh.beta, *zcoef = sh.zcoef, *pco = sh.pco;
-    int& s_flag = sh.flag;
 
     const MeshDev& m = a.m;
     const int P = m.P;
@@ -557,13 +576,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
     int it = 0;
     for (;;) {
         // ---- convergence / cap (uniform over CTAs)
-        if (threadIdx.x == 0) {
-            int any = 0;
-            for (int r = 0; r < R; ++r) any |= (rr[r] > a.rtol2 * bb[r]) ? 1 : 0;
-            s_flag = any;
-        }
-        __syncthreads();
-        if (!s_flag) break;
+        if (!__syncthreads_or(threadIdx.x < R && rr[threadIdx.x] > a.rtol2 * bb[threadIdx.x])) break;
         if (it >= a.maxit) {
             if (cta == 0 && threadIdx.x == 0) atomicCAS(a.status, 0, QPAT_ENOCONV);
             break;
@@ -665,18 +678,15 @@ __device__ __forceinline__ void pcg_body(const PcgArgs<T>& a, const int cta, con
         if (!grid_reduce<1, VW, NP, false>(accA, scratch, a.partials, red_id, a.status, a.spin_limit, red, cta,
                                     ncta))
             return;
-        if (threadIdx.x == 0) {
-            int bad = 0;
-            for (int r = 0; r < R; ++r) {
-                const bool act = rr[r] > a.rtol2 * bb[r];
-                const double pq = red[r];
-                if (act && !(pq > 0.0 && isfinite(pq))) bad = 1;
-                alpha[r] = act && pq > 0.0 ? rz[r] / pq : 0.0;
-            }
-            s_flag = bad;
+        int bad = 0;
+        if (threadIdx.x < R) {
+            const int r = threadIdx.x;
+            const bool act = rr[r] > a.rtol2 * bb[r];
+            const double pq = red[r];
+            bad = act && !(pq > 0.0 && isfinite(pq));
+            alpha[r] = act && pq > 0.0 ? rz[r] / pq : 0.0;
         }
-        __syncthreads();
-        if (s_flag) {
+        if (__syncthreads_or(bad)) {
             if (cta == 0 && threadIdx.x == 0) atomicCAS(a.status, 0, QPAT_EBREAKDOWN);
             break;
         }
