@@ -254,21 +254,23 @@ static int pcg_status(int st, const char* what) {
 // restarts): multigrid-preconditioned CG where it is the faster one, with the
 // cycle in FP32 for the K solves of precision 1 (which may iterate in FP32).
 // Measured on GB300, whole calls, persistent against multigrid:
-//   M_delta: 2.4 / 1.5 ms (11^3), 5.1 / 1.9 (24^3), 27 / 6.5 (64^3), cylinders 8.3 / 4.5 (21 x 21 x 27), 41 / 17 (49 x 49 x 61);
-//   K, FP64 on grids (the stiffness pattern well below K's): R = 8 1.6 / 1.2 ms (11^3), R = 4 1.5 / 1.5 (16^3),
-//   2.7 / 1.8 (24^3), R = 1 1.9 / 1.8 (32^3), 3.8 / 2.4 (48^3), R = 8 40 / 9.2 (64^3);
-//   on cylinders, whose cycle keeps K's whole pattern: R = 4 3.8 / 3.7 (21 x 21 x 27), 9.7 / 8.3 (33 x 33 x 41),
-//   R = 1 5.1 / 6.2, R = 8 15 / 10 (33 x 33 x 41);
-//   K, precision 1 against the FP32 cycle: 1.7 / 1.1 ms (11^3, R = 1), 14 / 6.3 (64^3, R = 8).
-// Below 512 nodes the hierarchy has no second level worth its set-up.
+//   M_delta: 1.5 / 1.5 ms (11^3), 2.1 / 1.6 (13^3), 4.0 / 1.9 (24^3), 27 / 6.5 (64^3), cylinders 3.3 / 2.7 (11 x 11 x 14),
+//   6.5 / 4.5 (21 x 21 x 27), 41 / 17 (49 x 49 x 61);
+//   K, FP64 on grids (the stiffness pattern well below K's): R = 1 1.6 / 1.7 ms (32^3), 2.4 / 2.1 (40^3),
+//   R = 2 1.1 / 1.4 (16^3), 1.9 / 1.7 (24^3), R = 4 1.1 / 1.5 (16^3), 1.7 / 1.6 (20^3), 2.1 / 1.8 (24^3),
+//   R = 8 0.9 / 1.2 (11^3), 1.1 / 1.5 (16^3), 1.8 / 1.75 (20^3), 7.3 / 3.9 (40^3);
+//   on cylinders, whose cycle keeps K's whole pattern: R = 1 4.4 / 5.9 (33 x 33 x 41), 10.7 / 11.5 (49 x 49 x 61),
+//   R = 2 5.3 / 6.9 (33 x 33 x 41), R = 4 8.1 / 8.2, R = 8 12.2 / 10.3, 3.6 / 4.4 (21 x 21 x 27);
+//   K, precision 1 against the FP32 cycle: 1.4 / 1.1 ms (9^3, R = 1), 24 / 3.3 (40^3, R = 8).
 static bool prefers_multigrid(const qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R) {
     const int deg = st.kind == OP_PRIOR ? so.poly_prior : so.poly_k;
     if (so.multigrid || so.pcg_variant != 0 || so.mixed_restart || so.spin_limit > 0 || deg != kDefaultPolyDegree) return false;
     const int64_t N = M->h.N;
-    if (st.kind == OP_PRIOR || so.precision == 1) return N >= 512;
+    if (st.kind == OP_PRIOR) return N >= 1500;
+    if (so.precision == 1) return N >= 512;
     const bool lean = 3 * M->dp.sell_entries < 2 * M->d.sell_entries;
     if (R == 1) return N >= (lean ? 48000 : 150000);
-    return N * R >= (lean ? 12000 : 64000);
+    return lean ? N >= 8000 : N * R >= 180000;
 }
 
 // Solves A X = B for R right-hand sides (library order, N x R node-major,

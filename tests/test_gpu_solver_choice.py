@@ -17,8 +17,8 @@ Q = pytest.importorskip("paper_1512_02796_gb300")
 
 pytestmark = pytest.mark.gpu
 
-# nodes below, around and above the lines of the choice (512 nodes; 12,000 and 64,000 nodes x right-hand sides)
-MESHES = {"cube7": (7, None), "cube9": (9, None), "cube17": (17, None), "cube25": (25, None), "cyl9x7": (9, 7),
+# nodes below, around and above the lines of the choice (512, 1,500 and 8,000 nodes; 180,000 nodes x right-hand sides)
+MESHES = {"cube7": (7, None), "cube9": (9, None), "cube17": (17, None), "cube13": (13, None), "cube21": (21, None), "cube25": (25, None), "cyl9x7": (9, 7),
           "cyl25x27": (25, 27)}
 
 
