@@ -184,8 +184,8 @@ cudaError_t apply_csr_t(const MeshDev& m, const T* v0, const T* v1, const T* x, 
 // f_i += 2/3 sum over the boundary faces F of node i of Phi_F |F|, gathered per
 // (node, illumination) over the node's faces in a fixed order.  Bound by the
 // latency of a face's two loads behind its index and of FP64: three faces in
-// flight and one division a node (one face at a time, a division each: 49 us on
-// 91,125 nodes x 4).
+// flight and one division a node (91,125 nodes x 4: 16 us; one face at a time
+// with a division each: 49).
 __global__ void k_load(MeshDev m, int K, int R, const double* __restrict__ flux, double* f) {
     constexpr int U = 3;
     const int64_t total = int64_t(m.N) * K;
