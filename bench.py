@@ -850,7 +850,7 @@ def run_ours(args):
 
     # ---- the same step with the persistent Jacobi / patch-local PCG (FP64)
     if args.pcg_steps > 0 and prm.multigrid:
-        pp = Q.qpat_default_params(precision=0, poly_degree=0)
+        pp = Q.qpat_default_params(precision=0, poly_degree=0, pcg_variant=1)
         rp = time_steps(Q, torch, d, pp, args.pcg_steps, 3)
         kp, _ = kernel_table(d, pp, 0, rp["kernels"], sm_mhz, nsm, hbm_peak, sum(rp["step_ms"]))
         dp = max(kp, key=lambda k: kp[k]["ms"])
@@ -871,7 +871,7 @@ def run_ours(args):
                         "roofline": mg_roofline(km, "pair", f64_peak, hbm_peak, hbm_kind, sm_mhz, nsm, args.workload),
                         "kernels": km}
         # and FP32 PCG inside FP64 refinement (persistent kernels)
-        pr = Q.qpat_default_params(precision=1, fp32_operator=1)
+        pr = Q.qpat_default_params(precision=1, fp32_operator=1, pcg_variant=1)
         rr = time_steps(Q, torch, d, pr, args.mixed_steps, 3)
         kr, _ = kernel_table(d, pr, 1, rr["kernels"], sm_mhz, nsm, hbm_peak, sum(rr["step_ms"]))
         out["mixed_pcg"] = {"value": args.mixed_steps / (sum(rr["step_ms"]) / 1e3), "unit": UNIT,
@@ -909,7 +909,7 @@ def c2_leg(Q, torch, nsm, hbm_peak, hbm_kind, sm_mhz, steps: int = 5):
         pg = Q.qpat_default_params(precision=0, multigrid=1)
         rg = time_steps(Q, torch, d, pg, steps, 3)
         kg, f64_peak = mg_kernel_table(d, pg, rg["kernels"], sm_mhz, nsm, hbm_peak, sum(rg["step_ms"]))
-        pm = Q.qpat_default_params(precision=1, fp32_operator=1)
+        pm = Q.qpat_default_params(precision=1, fp32_operator=1, pcg_variant=1)
         r = time_steps(Q, torch, d, pm, steps, 3)
         km, f64_peak = kernel_table(d, pm, 1, r["kernels"], sm_mhz, nsm, hbm_peak, sum(r["step_ms"]))
         return {"value": steps / (sum(rg["step_ms"]) / 1e3), "unit": UNIT, "steps": steps,
@@ -1059,7 +1059,7 @@ def concurrent_recon_leg(Q, torch, count: int = 32, threads: int = 16, patch_nod
                 sig = 0.01 * np.abs(h) + 1e-3 * np.abs(h).max()
                 chi = h + sig * S.noise_draws(cfg.seed + 7, h.shape)
             sets[key].append((m, flux, chi, sig, (float(np.median(kap)), float(np.median(mu)))))
-    prm = Q.qpat_default_params(precision=0, T=2e-2, max_lin=3, max_lsqr=10, fixed_counts=1)
+    prm = Q.qpat_default_params(precision=0, T=2e-2, max_lin=3, max_lsqr=10, fixed_counts=1, pcg_variant=1)
     run = lambda p: Q.qpat_reconstruct(p[0], p[1], p[2], p[3], prm, p[4])
     rel = lambda a, b: float(np.linalg.norm(a - b) / np.linalg.norm(b))
     try:
@@ -1162,13 +1162,13 @@ def recon_leg(Q, torch, n: int = 64, seed: int = 7, T: float = 2e-2, cap: int = 
     # K solves with Jacobi instead of the degree-2 patch polynomial, both to
     # the same 1e-13 residual): how far two FP64 runs lie apart measures the
     # method's own sensitivity to solve-level rounding at this size
-    for name, prm in (("fp64", Q.qpat_default_params(precision=0, T=T, max_lsqr=cap)),
-                      ("fp64_alt", Q.qpat_default_params(precision=0, T=T, max_lsqr=cap, poly_degree=0)),
-                      ("mixed", Q.qpat_default_params(precision=1, fp32_operator=1, T=T, max_lsqr=cap)),
+    for name, prm in (("fp64", Q.qpat_default_params(precision=0, T=T, max_lsqr=cap, pcg_variant=1)),
+                      ("fp64_alt", Q.qpat_default_params(precision=0, T=T, max_lsqr=cap, poly_degree=0, pcg_variant=1)),
+                      ("mixed", Q.qpat_default_params(precision=1, fp32_operator=1, T=T, max_lsqr=cap, pcg_variant=1)),
                       ("fp64_mg", Q.qpat_default_params(precision=0, T=T, max_lsqr=cap, multigrid=1)),
                       ("mixed_mg", Q.qpat_default_params(precision=0, T=T, max_lsqr=cap, multigrid=2))):
         warm = Q.qpat_default_params(precision=prm.precision, fp32_operator=1, max_lin=1, max_lsqr=2, fixed_counts=1,
-                                     multigrid=prm.multigrid)
+                                     multigrid=prm.multigrid, pcg_variant=prm.pcg_variant)
         Q.qpat_reconstruct(mesh, flux, chi, sig, warm)         # warm-up (workspace, kernels)
         t0 = time.perf_counter()
         try:
@@ -1500,9 +1500,9 @@ def run_profile_case(args):
     for name, prm in (("pair_mg64", Q.qpat_default_params(precision=0, multigrid=1)),
                       ("prior_mg64", Q.qpat_default_params(precision=0, multigrid=1)),
                       ("pair_mg32", Q.qpat_default_params(precision=0, multigrid=2)),
-                      ("pair_fp64", Q.qpat_default_params(precision=0, poly_degree=0)),
-                      ("prior_fp64", Q.qpat_default_params(precision=0)),
-                      ("pair_fp32", Q.qpat_default_params(precision=1, fp32_operator=1))):
+                      ("pair_fp64", Q.qpat_default_params(precision=0, poly_degree=0, pcg_variant=1)),
+                      ("prior_fp64", Q.qpat_default_params(precision=0, pcg_variant=1)),
+                      ("pair_fp32", Q.qpat_default_params(precision=1, fp32_operator=1, pcg_variant=1))):
         mesh.reset_stats()
         n0 = Q.qpat_launch_count()
         if name.startswith("prior"):
