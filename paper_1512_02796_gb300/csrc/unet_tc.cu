@@ -385,11 +385,12 @@ __global__ void __launch_bounds__(kStayThreads) k_conv_fwd_tc_stay(const TcArgs 
     if (warp == 0) tmem_free(tmem, g.ncols);
 }
 
-// Streamed weights: one box per CTA, a ring of 2 or 3 taps; the tiles go round
+// Streamed weights: one box per CTA, a ring of 2 to 4 taps (with 4, the stage that a copy goes to was read by the
+// MMAs of two taps ago, so that nothing waits for the tap just issued); the tiles go round
 // the warps (a tile's MMAs stay with one lane, in order).
 __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    __shared__ uint64_t mbar[3];
+    __shared__ uint64_t mbar[4];
     __shared__ uint32_t tmem_base_s;
     const TcBox& g = a.g;
     const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
     const bool issuer = warp < issuers;
     if (warp == 0) tmem_alloc(&tmem_base_s, g.ncols);
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 3; ++i) mbar_init(&mbar[i], issuers);
+        for (int i = 0; i < 4; ++i) mbar_init(&mbar[i], issuers);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const Corner at = corner_of(g, blockIdx.x);
@@ -445,12 +446,14 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const TcArgs a) {
     if (warp == 0) tmem_free(tmem, g.ncols);
 }
 
-// The box of a launch with the least estimated time.  An MMA takes 32 cycles
-// (more above 128 output channels), a halo about its bytes / 24 to issue and
-// bring in, the results their bytes / 16.  Resident weights: per box the
-// larger of the MMAs and the copies; streamed: the sum, and ~8,000 cycles for
-// a CTA's start and its first tap (measured at 128^3, 16 -> 16 channels), two
-// CTAs sharing an SM where their shared memory allows.  false: no box fits.
+// The box of a launch with the least estimated time, in cycles as measured at
+// 128^3 (16 -> 16 and 48 -> 16 channels, one part at a time): an MMA 40 (more
+// above 160 output channels), but a warp issues one every 118, halos come in at
+// 13 bytes a cycle, results leave at 16.  Resident weights: per box the larger
+// of the MMAs and the copies with their waits; streamed: the sum, ~8,000 for a
+// CTA's start and its first tap and, where the ring has fewer than 4 taps,
+// ~1,000 a tap for the MMAs that a copy waits for; two CTAs share an SM where
+// their shared memory allows.  false: no box fits.
 bool search_box(int n, int Cin, int Cout, int B, TcBox& best, size_t& best_smem) {
     const int kc = Cin / 8;
     const int wlbo = Cout * 16 + 16, wtap = kc * wlbo;
@@ -479,10 +482,10 @@ bool search_box(int n, int Cin, int Cout, int B, TcBox& best, size_t& best_smem)
                 g.lbo = (rows * 16 + 127) / 128 * 128 + 64;
                 g.wlbo = wlbo;
                 g.wtap = wtap;
-                g.stages = stay ? 27 : 3;
+                g.stages = stay ? 27 : 4;
                 size_t smem = size_t(kc) * g.lbo * (stay ? 2 : 1) + size_t(g.stages) * wtap;
-                if (smem > size_t(kTcSmem) && !stay) {
-                    g.stages = 2;
+                while (smem > size_t(kTcSmem) && !stay && g.stages > 2) {
+                    --g.stages;
                     smem -= wtap;
                 }
                 if (smem > size_t(kTcSmem)) break;
@@ -494,13 +497,16 @@ bool search_box(int n, int Cin, int Cout, int B, TcBox& best, size_t& best_smem)
                 const double boxes = double(g.nx) * g.ny * g.nz * B;
                 if (boxes >= 2147483648.0) continue;
                 g.boxes = int(boxes);
-                const double mma = g.tiles * 27.0 * (Cin / 16) * std::max(32.0, Cout / 4.0);
-                const double load = (Tz + 2.0) * g.RY * g.P * Cin * 2 / 24.0 + 800.0;
+                const int issuers = stay ? kIssueWarps : kTcThreads / 32;
+                const double mma = 27.0 * (Cin / 16) * std::max(g.tiles * std::max(40.0, Cout / 4.0),
+                                                                118.0 * ((g.tiles + issuers - 1) / issuers));
+                const double load = (Tz + 2.0) * g.RY * g.P * Cin * 2 / 13.0 + 800.0;
                 const double store = g.tiles * 128.0 * Cout * 2 / 16.0 + 300.0;
                 const int share = !stay && smem <= size_t(kTcSmem) / 2 && g.ncols <= 256 ? 2 : 1;
                 const double waves = std::max(1.0, double(int64_t((boxes + 152 * share - 1) / (152 * share))));
-                const double t = stay ? waves * std::max(mma + 600.0, load + store) + load + store
-                                      : waves * (share * std::max(mma, 27.0 * wtap / 24.0) + load + store + 8000.0);
+                const double tap = g.stages < 4 ? 1000.0 : 0.0;
+                const double t = stay ? waves * std::max(mma + 600.0, load + store + 2500.0) + load + store
+                                      : waves * (share * std::max(mma, 27.0 * wtap / 24.0) + 27.0 * tap + load + store + 8000.0);
                 if (!found || t < best_t) {
                     found = true;
                     best_t = t;
