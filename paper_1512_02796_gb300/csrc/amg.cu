@@ -743,13 +743,13 @@ __global__ void __launch_bounds__(256) k_cg_init(int64_t n, const double* b, dou
     block_partials<R>(acc, part);
 }
 
-// x = x0, r = b - A x0, partials of b.b (the stopping target stays rtol |b|)
+// x = x0, r = b - A x0, partials of b.b and of r.r (the stopping target stays rtol |b|)
 template <int R, int NV>
 __global__ void __launch_bounds__(256) k_cg_init_x0(SellDev A, const double* v0, const double* v1, const double* b,
                                                     const double* x0, double* x, double* r, double* part) {
-    double acc[R];
+    double acc[2 * R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) acc[q] = 0.0;
+    for (int q = 0; q < 2 * R; ++q) acc[q] = 0.0;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < A.n; i += int64_t(gridDim.x) * blockDim.x) {
         double bv[R], av[R], xv[R];
         row_apply<double, R, NV, 1>(A, v0, v1, x0, i, 0, true, av);
@@ -759,36 +759,58 @@ __global__ void __launch_bounds__(256) k_cg_init_x0(SellDev A, const double* v0,
         for (int q = 0; q < R; ++q) {
             acc[q] = fma(bv[q], bv[q], acc[q]);
             av[q] = bv[q] - av[q];
+            acc[R + q] = fma(av[q], av[q], acc[R + q]);
         }
         stR<double, R>(r + i * R, av);
         stR<double, R>(x + i * R, xv);
     }
-    block_partials<R>(acc, part);
+    block_partials<2 * R>(acc, part);
+}
+
+// x = r = 0 on the right-hand sides with b = 0, whatever the guess was
+template <int R>
+__global__ void __launch_bounds__(256) k_cg_clear(int64_t n, const double* bb, double* x, double* r) {
+    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n * R; i += int64_t(gridDim.x) * blockDim.x)
+        if (bb[i % R] == 0.0) x[i] = r[i] = 0.0;
 }
 
 // Control words of a CG solve (int ctl[]): [0] status, [1] right-hand sides
 // still running, [2] iterations done, [3] 1 before the first direction,
-// [4] iteration cap; the per-RHS running flags follow at ctl + kCtlActive.
+// [4] iteration cap, [5] right-hand sides with b = 0 and a residual (from a
+// guess); the per-RHS running flags follow at ctl + kCtlActive.
 constexpr int kCtlActive = 8;
 
-// bb = totals; a right-hand side with b = 0 is solved by x = 0 and never runs
-template <int R>
-__global__ void k_cg_start(const double* part, int G, double* bb, int* ctl) {
+// bb = totals of b.b.  A right-hand side with b = 0 is solved by x = 0, and
+// one whose guess already meets the target by that guess: neither runs (a
+// residual of 0 would have no direction).  Q: quantities per right-hand side
+// in the partials (2: r.r behind b.b; 1: r = b).
+template <int R, int Q>
+__global__ void k_cg_start(const double* part, int G, const double* rtol2, double* bb, int* ctl) {
     int* active = ctl + kCtlActive;
+    __shared__ int clear[R];
     const int r = threadIdx.x >> 5;
-    const double t = total_of(part, G, R, r);
+    const double t = total_of(part, G, Q * R, r);
+    const double rr = Q == 1 ? t : total_of(part, G, Q * R, (Q - 1) * R + r);
     if ((threadIdx.x & 31) == 0) {
         bb[r] = t;
-        active[r] = t > 0.0 ? 1 : 0;
-        if (!isfinite(t)) atomicExch(ctl, int(QPAT_EINVAL));
+        active[r] = t > 0.0 && rr > *rtol2 * t ? 1 : 0;
+        clear[r] = t == 0.0 && rr > 0.0 ? 1 : 0;
+        if (!isfinite(t))
+            atomicExch(ctl, int(QPAT_EINVAL));
+        else if (!isfinite(rr))
+            atomicExch(ctl, int(QPAT_EBREAKDOWN));
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        int c = 0;
-        for (int q = 0; q < R; ++q) c += active[q];
+        int c = 0, z = 0;
+        for (int q = 0; q < R; ++q) {
+            c += active[q];
+            z += clear[q];
+        }
         ctl[1] = c;
         ctl[2] = 0;
         ctl[3] = 1;
+        ctl[5] = z;
     }
 }
 
@@ -1673,7 +1695,7 @@ struct CgSolve {
         int* hc = reinterpret_cast<int*>(M->host_scratch + 240);
         cudaError_t e = cudaSuccess;
         auto read_ctl = [&]() -> cudaError_t {
-            cudaError_t x = cudaMemcpyAsync(hc, C.ctl, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
+            cudaError_t x = cudaMemcpyAsync(hc, C.ctl, 6 * sizeof(int), cudaMemcpyDeviceToHost, s);
             if (x == cudaSuccess) x = cudaStreamSynchronize(s);
             return x;
         };
@@ -1685,13 +1707,21 @@ struct CgSolve {
             (e = cudaMemsetAsync(C.p, 0, sizeof(double) * n * R, s)) != cudaSuccess)
             return cuda_fail(e, "multigrid start");
         note_launch(2);
-        if (X0)
+        if (X0) {
             k_cg_init_x0<R, NV><<<G, 256, 0, s>>>(A0, st.v64[0], st.v64[1], B, X0, C.x, C.r, C.part);
-        else
+            k_cg_start<R, 2><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.ctl);
+        } else {
             k_cg_init<R><<<G, 256, 0, s>>>(n, B, C.x, C.r, C.part);
-        k_cg_start<R><<<1, 32 * R, 0, s>>>(C.part, G, C.bb, C.ctl);
+            k_cg_start<R, 1><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.ctl);
+        }
         if ((e = read_ctl()) != cudaSuccess) return cuda_fail(e, "multigrid cg");
-        if (hc[0] != QPAT_OK) return fail(hc[0], "multigrid cg: right-hand side not finite");
+        if (hc[0] != QPAT_OK)
+            return fail(hc[0], hc[0] == QPAT_EINVAL ? "multigrid cg: right-hand side not finite"
+                                                    : "multigrid cg: residual of the initial guess not finite");
+        if (hc[5] > 0) {
+            note_launch(1);
+            k_cg_clear<R><<<G, 256, 0, s>>>(n, C.bb, C.x, C.r);
+        }
         if (hc[1] > 0) {
             if (f32) {
                 note_launch(1);
