@@ -253,6 +253,16 @@ int64_t qpat_mesh_rhs_iterations(qpat_mesh_t mesh);
  * multigrid solve of that kind).  Not in the paper (diagnostics). */
 int qpat_mesh_multigrid_levels(qpat_mesh_t mesh, int prior, int64_t* rows, int max_levels);
 
+/* Device memory (bytes) that the multigrid solver of this mesh may hold; 0
+ * (the default): as much as the device gives.  A solve that names multigrid
+ * and would need more fails with QPAT_ECUDA, as one for which the device has
+ * no memory left; a solve that leaves the choice to the library then takes the
+ * persistent PCG.  qpat_mesh_multigrid_bytes: what it holds now (a solve that
+ * failed for want of memory holds nothing of its own); -1 for a NULL mesh.
+ * Not in the paper. */
+int qpat_mesh_set_multigrid_limit(qpat_mesh_t mesh, int64_t bytes);
+int64_t qpat_mesh_multigrid_bytes(qpat_mesh_t mesh);
+
 /* With timing on (qpat_mesh_set_timing): the summed device time (ms) and
  * the count of the fine level's smoothing products in the multigrid cycles
  * since the last reset (mg_degree 1: the residual after the pre-smoothing

@@ -906,6 +906,14 @@ int qpat_mesh_multigrid_levels(qpat_mesh_t M, int prior, int64_t* rows, int max_
     return qpat::amg_levels(M, prior, rows, max_levels);
 }
 
+int qpat_mesh_set_multigrid_limit(qpat_mesh_t M, int64_t bytes) {
+    if (!M || bytes < 0) return fail(QPAT_EINVAL, "qpat_mesh_set_multigrid_limit: NULL mesh or negative limit");
+    qpat::amg_set_limit(M, size_t(bytes));
+    return QPAT_OK;
+}
+
+int64_t qpat_mesh_multigrid_bytes(qpat_mesh_t M) { return M ? int64_t(qpat::amg_bytes(M)) : -1; }
+
 int qpat_mesh_reset_stats(qpat_mesh_t M) {
     if (!M) return fail(QPAT_EINVAL, "qpat_mesh_reset_stats: NULL mesh");
     M->stats = SolveStats();

@@ -135,6 +135,8 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
               cudaStream_t s, const double* X0 = nullptr);
 // rows of each level of the hierarchy of the K (prior = 0) or prior pattern; returns the level count
 int amg_levels(qpat_mesh_s* M, int prior, int64_t* rows, int max_levels);
+void amg_set_limit(qpat_mesh_s* M, size_t bytes);  // device memory the solver may hold (0: no limit)
+size_t amg_bytes(const qpat_mesh_s* M);            // device memory it holds
 void amg_release(qpat_mesh_s* M);
 SolveOpts solve_opts(const qpat_params* prm);
 

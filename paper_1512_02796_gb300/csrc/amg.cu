@@ -1048,16 +1048,92 @@ __global__ void k_f2d_vec(int64_t n, const float* in, double* out) {
 
 // ---------------------------------------------------------------- host side
 
+// Device memory that the multigrid solver of a mesh holds, and the most that
+// it may hold (0: no limit).
+struct MemLedger {
+    size_t used = 0, limit = 0;
+};
+
+// A set of device allocations that is released as a whole.  Every part of the
+// state below is allocated into a local one and put in its place only when all
+// of it is there, so that a failed allocation leaves nothing half-built.
+class DevMem {
+  public:
+    explicit DevMem(MemLedger* l) : ledger_(l) {}
+    DevMem(DevMem&& o) noexcept : ledger_(o.ledger_) { list_.swap(o.list_); }
+    DevMem& operator=(DevMem&& o) noexcept {
+        std::swap(ledger_, o.ledger_);
+        list_.swap(o.list_);
+        return *this;
+    }
+    ~DevMem() {
+        for (const auto& a : list_) {
+            cudaFree(a.first);
+            ledger_->used -= a.second;
+        }
+    }
+    // count values of T; nothing (and e unchanged) once e reports a failure
+    template <typename T>
+    T* get(size_t count, cudaError_t& e) {
+        if (e != cudaSuccess) return nullptr;
+        const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
+        if (ledger_->limit && ledger_->used + bytes > ledger_->limit) {
+            e = cudaErrorMemoryAllocation;
+            return nullptr;
+        }
+        list_.emplace_back(nullptr, 0);
+        void* p = nullptr;
+        if ((e = cudaMalloc(&p, bytes)) != cudaSuccess) {
+            list_.pop_back();
+            return nullptr;
+        }
+        list_.back() = {p, bytes};
+        ledger_->used += bytes;
+        return static_cast<T*>(p);
+    }
+    template <typename T>
+    const T* put(const std::vector<T>& h, cudaError_t& e) {
+        T* d = get<T>(h.size(), e);
+        if (e == cudaSuccess && !h.empty()) e = cudaMemcpy(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
+        return d;
+    }
+
+  private:
+    MemLedger* ledger_;
+    std::vector<std::pair<void*, size_t>> list_;
+};
+
 struct AmgHierDev {
-    bool tried = false;
+    explicit AmgHierDev(MemLedger* l) : mem(l) {}
+    bool ready = false;
     bool used[2] = {false, false};  // a K (M_delta) solve has run on it
-    std::string error;
+    std::string error;              // non-empty: this mesh has no hierarchy
     std::vector<LevelDev> lv;
     SellDev K;                      // the full pattern of K (the products of its CG)
-    std::vector<void*> allocs;
+    DevMem mem;
+};
+
+// One CG iteration captured once as the body of a graph "while" node, per
+// operator values, right-hand-side count and cycle settings; the check
+// kernel of the body sets the loop condition on the device.
+struct AmgGraph {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    int body_kernels = 0;
+    AmgGraph() = default;
+    AmgGraph(AmgGraph&& o) noexcept : graph(o.graph), exec(o.exec), body_kernels(o.body_kernels) {
+        o.graph = nullptr;
+        o.exec = nullptr;
+    }
+    AmgGraph& operator=(AmgGraph&&) = delete;
+    ~AmgGraph() {
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
+    }
 };
 
 struct AmgValues {
+    explicit AmgValues(MemLedger* l) : mem(l) {}
     uint64_t stamp = 0;
     bool valid = false;
     bool has32 = false;
@@ -1070,65 +1146,42 @@ struct AmgValues {
     std::vector<std::array<float*, 2>> A32, P32, R32, S32, P232;
     std::vector<float*> dinv32, wd32;
     float* inv32 = nullptr;
-    std::vector<void*> allocs;
+    std::map<std::string, AmgGraph> graphs;  // iterations captured on these values
+    DevMem mem;
 };
 
 struct AmgVecs {
+    explicit AmgVecs(MemLedger* l) : mem(l) {}
     std::vector<void*> b, xa, xb, d, r;
-    std::vector<void*> allocs;
+    DevMem mem;
 };
 
 struct AmgCg {
+    explicit AmgCg(MemLedger* l) : mem(l) {}
     double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *part = nullptr;
     double *bb = nullptr, *rz = nullptr, *alpha = nullptr, *beta = nullptr, *rr = nullptr, *rtol2 = nullptr;
     int* ctl = nullptr;  // control words (see k_cg_start)
     unsigned* count = nullptr;  // blocks that have finished (see last_block_totals)
-    std::vector<void*> allocs;
-};
-
-// One CG iteration captured once as the body of a graph "while" node, per
-// operator values, right-hand-side count and cycle settings; the check
-// kernel of the body sets the loop condition on the device.
-struct AmgGraph {
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    int body_kernels = 0;
+    DevMem mem;
 };
 
 struct AmgState {
-    AmgHierDev hier;     // on the prior's pattern, for K and M_delta
-    std::map<const void*, AmgValues> vals;
+    MemLedger ledger;
+    AmgHierDev hier{&ledger};     // on the prior's pattern, for K and M_delta
     std::map<std::pair<int, int>, AmgVecs> vecs;  // (R, FP32 V-cycle)
     std::map<int, AmgCg> cg;                       // R
-    std::map<std::string, AmgGraph> graphs;
+    std::map<const void*, AmgValues> vals;         // per operator; their graphs work on vecs and cg too
     cudaStream_t capture = nullptr;                // a non-default stream to capture on
 };
 
 namespace {
 
-template <typename T>
-T* dalloc(std::vector<void*>& list, size_t count, cudaError_t& e) {
-    if (e != cudaSuccess) return nullptr;
-    void* p = nullptr;
-    e = cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(T));
-    if (e != cudaSuccess) return nullptr;
-    list.push_back(p);
-    return static_cast<T*>(p);
-}
-
-template <typename T>
-const T* upload(std::vector<void*>& list, const std::vector<T>& h, cudaError_t& e) {
-    T* d = dalloc<T>(list, h.size(), e);
-    if (e == cudaSuccess && !h.empty()) e = cudaMemcpy(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
-    return d;
-}
-
-SellDev upload_sell(std::vector<void*>& list, const SellPattern& S, cudaError_t& e) {
+SellDev upload_sell(DevMem& mem, const SellPattern& S, cudaError_t& e) {
     SellDev d;
     d.n = S.n;
-    d.ptr = upload(list, S.ptr, e);
-    d.col = upload(list, S.col, e);
-    d.len = upload(list, S.len, e);
+    d.ptr = mem.put(S.ptr, e);
+    d.col = mem.put(S.col, e);
+    d.len = mem.put(S.len, e);
     d.entries = S.entries();
     d.maxlen = S.maxlen;
     d.rowmajor = S.rowmajor ? 1 : 0;
@@ -1150,7 +1203,6 @@ int full_grid(K kernel, int most) {
 inline int blocks_of(int64_t n, int per = 256) { return int(std::max<int64_t>(1, (n + per - 1) / per)); }
 
 int build_hier(qpat_mesh_s* M, AmgHierDev& H) {
-    H.tried = true;
     const SellPattern fine = amg_fine_pattern(M->h);
     const AmgPlan plan = amg_build_plan(fine, amg_fine_graph(M->h, fine));
     if (!plan.error.empty()) {
@@ -1160,24 +1212,24 @@ int build_hier(qpat_mesh_s* M, AmgHierDev& H) {
     cudaError_t e = cudaSuccess;
     for (const AmgLevelPlan& L : plan.levels) {
         LevelDev d;
-        d.A = upload_sell(H.allocs, L.A, e);
-        d.diag = upload(H.allocs, L.diag, e);
+        d.A = upload_sell(H.mem, L.A, e);
+        d.diag = H.mem.put(L.diag, e);
         d.nc = L.nc;
         if (L.nc > 0) {
-            d.P = upload_sell(H.allocs, L.P, e);
-            d.a2p = upload(H.allocs, L.a2p, e);
-            d.pself = upload(H.allocs, L.pself, e);
-            d.ap_ptr = upload(H.allocs, L.ap_ptr, e);
-            d.ap_col = upload(H.allocs, L.ap_col, e);
-            d.ap_sptr = upload(H.allocs, L.ap_sptr, e);
-            d.ap_slot = upload(H.allocs, L.ap_slot, e);
+            d.P = upload_sell(H.mem, L.P, e);
+            d.a2p = H.mem.put(L.a2p, e);
+            d.pself = H.mem.put(L.pself, e);
+            d.ap_ptr = H.mem.put(L.ap_ptr, e);
+            d.ap_col = H.mem.put(L.ap_col, e);
+            d.ap_sptr = H.mem.put(L.ap_sptr, e);
+            d.ap_slot = H.mem.put(L.ap_slot, e);
             d.ap_nnz = int64_t(L.ap_col.size());
             for (size_t i = 0; i + 1 < L.ap_ptr.size(); ++i)
                 d.ap_maxlen = std::max<int>(d.ap_maxlen, int(L.ap_ptr[i + 1] - L.ap_ptr[i]));
-            d.R = upload_sell(H.allocs, L.R, e);
-            d.r_src = upload(H.allocs, L.r_src, e);
-            d.g_ptr = upload(H.allocs, L.g_ptr, e);
-            d.g_slot = upload(H.allocs, L.g_slot, e);
+            d.R = upload_sell(H.mem, L.R, e);
+            d.r_src = H.mem.put(L.r_src, e);
+            d.g_ptr = H.mem.put(L.g_ptr, e);
+            d.g_slot = H.mem.put(L.g_slot, e);
         }
         H.lv.push_back(d);
     }
@@ -1185,13 +1237,11 @@ int build_hier(qpat_mesh_s* M, AmgHierDev& H) {
     H.K.n = M->h.N;
     H.K.ptr = M->d.sell_ptr;
     H.K.col = M->el.ent_col;
-    H.K.len = upload(H.allocs, len, e);
+    H.K.len = H.mem.put(len, e);
     H.K.entries = M->d.sell_entries;
     H.K.maxlen = M->d.sell_wmax;
-    if (e != cudaSuccess) {
-        H.error = std::string("multigrid upload: ") + cudaGetErrorString(e);
-        return cuda_fail(e, "multigrid upload");
-    }
+    if (e != cudaSuccess) return cuda_fail(e, "multigrid upload");
+    H.ready = true;
     return QPAT_OK;
 }
 
@@ -1262,7 +1312,8 @@ cudaError_t cast_to_f32(const double* in, float* out, int64_t n, cudaStream_t s)
 
 // Values of the hierarchy for the operator st (allocated once per operator
 // buffer, recomputed when st was prepared again or the cycle's form changed).
-// fast: the degree-1 cycle's S, wd and P2 too.
+// fast: the degree-1 cycle's S, wd and P2 too.  After a failure V is incomplete
+// and must be dropped.
 int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V, bool fast, double ratio, bool need32,
             cudaStream_t s) {
     const int L = int(H.lv.size());
@@ -1279,18 +1330,18 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
             const LevelDev& d = H.lv[size_t(l)];
             for (int v = 0; v < NV; ++v) {
                 V.A[size_t(l)][size_t(v)] =
-                    l == 0 && NV == 2 ? st.v64[v] : dalloc<double>(V.allocs, size_t(d.A.entries), e);
+                    l == 0 && NV == 2 ? st.v64[v] : V.mem.get<double>(size_t(d.A.entries), e);
                 if (l + 1 < L) {
-                    V.P[size_t(l)][size_t(v)] = dalloc<double>(V.allocs, size_t(d.P.entries), e);
-                    V.R[size_t(l)][size_t(v)] = dalloc<double>(V.allocs, size_t(d.R.entries), e);
+                    V.P[size_t(l)][size_t(v)] = V.mem.get<double>(size_t(d.P.entries), e);
+                    V.R[size_t(l)][size_t(v)] = V.mem.get<double>(size_t(d.R.entries), e);
                 }
             }
-            if (l + 1 < L) V.AP[size_t(l)] = dalloc<double>(V.allocs, size_t(d.ap_nnz) * NV, e);
-            V.dinv[size_t(l)] = dalloc<double>(V.allocs, size_t(d.A.n) * NV, e);
+            if (l + 1 < L) V.AP[size_t(l)] = V.mem.get<double>(size_t(d.ap_nnz) * NV, e);
+            V.dinv[size_t(l)] = V.mem.get<double>(size_t(d.A.n) * NV, e);
         }
-        V.hi = dalloc<double>(V.allocs, size_t(2 * L), e);
+        V.hi = V.mem.get<double>(size_t(2 * L), e);
         const int64_t nco = H.lv.back().A.n;
-        V.inv = dalloc<double>(V.allocs, size_t(NV * nco * nco), e);
+        V.inv = V.mem.get<double>(size_t(NV * nco * nco), e);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
         // padding entries are never written: keep them 0
         for (int l = 0; l < L && e == cudaSuccess; ++l)
@@ -1309,10 +1360,10 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         V.wd.assign(size_t(L), nullptr);
         for (int l = 0; l + 1 < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
-            for (int v = 0; v < NV; ++v) V.S[size_t(l)][size_t(v)] = dalloc<double>(V.allocs, size_t(d.A.entries), e);
-            double* p2 = dalloc<double>(V.allocs, size_t(d.ap_nnz) * NV, e);
+            for (int v = 0; v < NV; ++v) V.S[size_t(l)][size_t(v)] = V.mem.get<double>(size_t(d.A.entries), e);
+            double* p2 = V.mem.get<double>(size_t(d.ap_nnz) * NV, e);
             V.P2[size_t(l)] = {p2, NV == 2 ? p2 + d.ap_nnz : nullptr};
-            V.wd[size_t(l)] = dalloc<double>(V.allocs, size_t(d.A.n) * NV, e);
+            V.wd[size_t(l)] = V.mem.get<double>(size_t(d.A.n) * NV, e);
         }
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
         V.valid = false;
@@ -1325,16 +1376,16 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         for (int l = 0; l < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
             for (int v = 0; v < NV; ++v) {
-                V.A32[size_t(l)][size_t(v)] = dalloc<float>(V.allocs, size_t(d.A.entries), e);
+                V.A32[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.A.entries), e);
                 if (l + 1 < L) {
-                    V.P32[size_t(l)][size_t(v)] = dalloc<float>(V.allocs, size_t(d.P.entries), e);
-                    V.R32[size_t(l)][size_t(v)] = dalloc<float>(V.allocs, size_t(d.R.entries), e);
+                    V.P32[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.P.entries), e);
+                    V.R32[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.R.entries), e);
                 }
             }
-            V.dinv32[size_t(l)] = dalloc<float>(V.allocs, size_t(d.A.n) * NV, e);
+            V.dinv32[size_t(l)] = V.mem.get<float>(size_t(d.A.n) * NV, e);
         }
         const int64_t nco = H.lv.back().A.n;
-        V.inv32 = dalloc<float>(V.allocs, size_t(NV * nco * nco), e);
+        V.inv32 = V.mem.get<float>(size_t(NV * nco * nco), e);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
         V.has32 = true;
         V.valid = false;
@@ -1346,10 +1397,10 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         for (int l = 0; l + 1 < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
             for (int v = 0; v < NV; ++v) {
-                V.S32[size_t(l)][size_t(v)] = dalloc<float>(V.allocs, size_t(d.A.entries), e);
-                V.P232[size_t(l)][size_t(v)] = dalloc<float>(V.allocs, size_t(d.ap_nnz), e);
+                V.S32[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.A.entries), e);
+                V.P232[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.ap_nnz), e);
             }
-            V.wd32[size_t(l)] = dalloc<float>(V.allocs, size_t(d.A.n) * NV, e);
+            V.wd32[size_t(l)] = V.mem.get<float>(size_t(d.A.n) * NV, e);
         }
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
         V.valid = false;
@@ -1632,7 +1683,7 @@ struct CgSolve {
     const OpState& st;
     const SolveOpts& so;
     const AmgHierDev& H;
-    const AmgValues& V;
+    AmgValues& V;
     bool f32;
     AmgVecs& W;
     AmgCg& C;
@@ -1728,14 +1779,16 @@ struct CgSolve {
                 k_d2f_vec<<<G, 256, 0, s>>>(n * R, C.r, static_cast<float*>(W.b[0]));
             }
             if (!timer->on) {
-                AmgGraph& g = A.graphs[key];
-                if (!g.exec) {
-                    const int rc = capture(A, g);
+                auto g = V.graphs.find(key);
+                if (g == V.graphs.end()) {
+                    AmgGraph fresh;
+                    const int rc = capture(A, fresh);
                     if (rc != QPAT_OK) return rc;
+                    g = V.graphs.emplace(key, std::move(fresh)).first;
                 }
-                if ((e = cudaGraphLaunch(g.exec, s)) != cudaSuccess) return cuda_fail(e, "multigrid graph");
+                if ((e = cudaGraphLaunch(g->second.exec, s)) != cudaSuccess) return cuda_fail(e, "multigrid graph");
                 if ((e = read_ctl()) != cudaSuccess) return cuda_fail(e, "multigrid cg");
-                note_launch(hc[2] * g.body_kernels);
+                note_launch(hc[2] * g->second.body_kernels);
             } else {
                 while (true) {
                     body(s, 0, 0);
@@ -1790,7 +1843,7 @@ struct CgSolve {
 
 template <int NV>
 int dispatch(int R, AmgState& A, const std::string& key, qpat_mesh_s* M, const OpState& st, const SolveOpts& so,
-             const AmgHierDev& H, const AmgValues& V, bool f32, AmgVecs& W, AmgCg& C, const double* B, double* X,
+             const AmgHierDev& H, AmgValues& V, bool f32, AmgVecs& W, AmgCg& C, const double* B, double* X,
              const double* X0, cudaStream_t s, FineTimer* timer, int* iters) {
     if constexpr (NV == 2) {
         return CgSolve<2, 2>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, iters);
@@ -1816,44 +1869,56 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
     if (!M->amg) M->amg = new AmgState();
     AmgState& A = *M->amg;
     AmgHierDev& H = A.hier;
-    if (!H.tried) {
-        const int rc = build_hier(M, H);
-        if (rc != QPAT_OK) return rc;
-    } else if (!H.error.empty()) {
-        return fail(QPAT_EINVAL, H.error);
+    if (!H.ready) {
+        if (!H.error.empty()) return fail(QPAT_EINVAL, H.error);
+        AmgHierDev fresh(&A.ledger);
+        const int rc = build_hier(M, fresh);
+        if (rc != QPAT_OK) {
+            H.error = fresh.error;  // no hierarchy for this mesh; empty where only memory is short
+            return rc;
+        }
+        H = std::move(fresh);
     }
     const bool f32 = so.multigrid == 2 && st.kind == OP_K;
-    AmgValues& V = A.vals[st.v64[0]];
     const bool fast = so.mg_degree <= 1 && H.lv.size() > 1;
     H.used[st.kind == OP_PRIOR] = true;
+    const void* const op = st.v64[0];
+    AmgValues& V = A.vals.try_emplace(op, &A.ledger).first->second;
     int rc = numeric(M, H, st, V, fast, so.mg_ratio, f32, s);
-    if (rc != QPAT_OK) return rc;
+    if (rc != QPAT_OK) {
+        A.vals.erase(op);
+        return rc;
+    }
     cudaError_t e = cudaSuccess;
-    AmgVecs& W = A.vecs[{R, f32 ? 1 : 0}];
-    if (W.xa.empty()) {
+    auto vecs = A.vecs.find({R, f32 ? 1 : 0});
+    if (vecs == A.vecs.end()) {
+        AmgVecs fresh(&A.ledger);
         const size_t esz = f32 ? sizeof(float) : sizeof(double);
         for (const LevelDev& d : H.lv) {
             const size_t cnt = size_t(d.A.n) * R * esz;
-            W.b.push_back(dalloc<char>(W.allocs, cnt, e));
-            W.xa.push_back(dalloc<char>(W.allocs, cnt, e));
-            W.xb.push_back(dalloc<char>(W.allocs, cnt, e));
-            W.d.push_back(dalloc<char>(W.allocs, cnt, e));
-            W.r.push_back(dalloc<char>(W.allocs, cnt, e));
+            fresh.b.push_back(fresh.mem.get<char>(cnt, e));
+            fresh.xa.push_back(fresh.mem.get<char>(cnt, e));
+            fresh.xb.push_back(fresh.mem.get<char>(cnt, e));
+            fresh.d.push_back(fresh.mem.get<char>(cnt, e));
+            fresh.r.push_back(fresh.mem.get<char>(cnt, e));
         }
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
+        vecs = A.vecs.emplace(std::make_pair(R, f32 ? 1 : 0), std::move(fresh)).first;
     }
-    AmgCg& C = A.cg[R];
-    if (!C.r) {
+    AmgVecs& W = vecs->second;
+    auto cg = A.cg.find(R);
+    if (cg == A.cg.end()) {
+        AmgCg C(&A.ledger);
         const size_t nR = size_t(M->h.N) * R;
-        C.x = dalloc<double>(C.allocs, nR, e);
-        C.r = dalloc<double>(C.allocs, nR, e);
-        C.p = dalloc<double>(C.allocs, nR, e);
-        C.q = dalloc<double>(C.allocs, nR, e);
-        C.z = dalloc<double>(C.allocs, nR, e);
-        C.part = dalloc<double>(C.allocs, size_t(kRedMaxGrid) * 32, e);
-        double* sc = dalloc<double>(C.allocs, 5 * 16 + 1, e);
-        C.ctl = dalloc<int>(C.allocs, kCtlActive + 16, e);
-        C.count = dalloc<unsigned>(C.allocs, 1, e);
+        C.x = C.mem.get<double>(nR, e);
+        C.r = C.mem.get<double>(nR, e);
+        C.p = C.mem.get<double>(nR, e);
+        C.q = C.mem.get<double>(nR, e);
+        C.z = C.mem.get<double>(nR, e);
+        C.part = C.mem.get<double>(size_t(kRedMaxGrid) * 32, e);
+        double* sc = C.mem.get<double>(5 * 16 + 1, e);
+        C.ctl = C.mem.get<int>(kCtlActive + 16, e);
+        C.count = C.mem.get<unsigned>(1, e);
         if (e == cudaSuccess) e = cudaMemsetAsync(C.count, 0, sizeof(unsigned), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(C.q, 0, sizeof(double) * nR, s);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
@@ -1863,11 +1928,12 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         C.beta = sc + 48;
         C.rr = sc + 64;
         C.rtol2 = sc + 80;
+        cg = A.cg.emplace(R, std::move(C)).first;
     }
-    // the captured iteration depends on these buffers and settings only
+    AmgCg& C = cg->second;
+    // an iteration captured on V depends on these settings and buffers beside it
     char key[256];
-    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%.17g/%p/%p/%p", R, st.nv, int(f32), so.mg_degree, so.mg_ratio,
-                  static_cast<const void*>(&V), static_cast<const void*>(st.v64[0]),
+    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%.17g/%p", R, st.nv, int(f32), so.mg_degree, so.mg_ratio,
                   static_cast<const void*>(st.v64[1]));
     FineTimer timer;
     timer.on = M->timing != 0;
@@ -1906,21 +1972,16 @@ int amg_levels(qpat_mesh_s* M, int prior, int64_t* rows, int max_levels) {
     return L;
 }
 
+void amg_set_limit(qpat_mesh_s* M, size_t bytes) {
+    if (!M->amg) M->amg = new AmgState();
+    M->amg->ledger.limit = bytes;
+}
+
+size_t amg_bytes(const qpat_mesh_s* M) { return M->amg ? M->amg->ledger.used : 0; }
+
 void amg_release(qpat_mesh_s* M) {
     if (!M->amg) return;
-    AmgState& A = *M->amg;
-    for (void* p : A.hier.allocs) cudaFree(p);
-    for (auto& kv : A.vals)
-        for (void* p : kv.second.allocs) cudaFree(p);
-    for (auto& kv : A.vecs)
-        for (void* p : kv.second.allocs) cudaFree(p);
-    for (auto& kv : A.cg)
-        for (void* p : kv.second.allocs) cudaFree(p);
-    for (auto& kv : A.graphs) {
-        if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
-        if (kv.second.graph) cudaGraphDestroy(kv.second.graph);
-    }
-    if (A.capture) cudaStreamDestroy(A.capture);
+    if (M->amg->capture) cudaStreamDestroy(M->amg->capture);
     delete M->amg;
     M->amg = nullptr;
 }

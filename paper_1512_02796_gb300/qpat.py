@@ -97,6 +97,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
         "qpat_mesh_multigrid_fine_time": (ctypes.c_int, [vp, ctypes.POINTER(ctypes.c_double), _c_int64_p]),
         "qpat_multigrid_host_info": (ctypes.c_int, [_c_double_p, ctypes.c_int64, _c_int32_p, ctypes.c_int64, ctypes.c_int,
                                                     ctypes.c_int, _c_int64_p, ctypes.c_int]),
+        "qpat_mesh_set_multigrid_limit": (ctypes.c_int, [vp, ctypes.c_int64]),
+        "qpat_mesh_multigrid_bytes": (ctypes.c_int64, [vp]),
         "qpat_mesh_reset_stats": (ctypes.c_int, [vp]),
         "qpat_mesh_set_timing": (ctypes.c_int, [vp, ctypes.c_int]),
         "qpat_mesh_pcg_time": (ctypes.c_int, [vp, _c_double_p]),
@@ -179,6 +181,7 @@ def exported_names() -> Sequence[str]:
         "qpat_mesh_num_entries", "qpat_mesh_num_prior_entries", "qpat_mesh_num_local_entries",
         "qpat_mesh_faces", "qpat_mesh_permutation", "qpat_mesh_stats", "qpat_mesh_fp64_fallbacks",
         "qpat_mesh_rhs_iterations", "qpat_mesh_multigrid_levels", "qpat_mesh_multigrid_fine_time", "qpat_multigrid_host_info", "qpat_mesh_reset_stats",
+        "qpat_mesh_set_multigrid_limit", "qpat_mesh_multigrid_bytes",
         "qpat_mesh_set_timing", "qpat_mesh_pcg_time",
         "qpat_flux_patch", "qpat_flux_side", "qpat_apply_K_dev", "qpat_forward", "qpat_forward_dev", "qpat_forward_noalloc_dev",
         "qpat_forward_guess_dev",
@@ -418,6 +421,14 @@ class Mesh:
         if n < 0:
             _check(n)
         return [int(r) for r in rows[:min(n, 16)]]
+
+    def set_multigrid_limit(self, limit: int):
+        """Bounds the device memory of the multigrid solver (bytes, 0: no limit)."""
+        _check(load().qpat_mesh_set_multigrid_limit(self.handle, limit))
+
+    def multigrid_bytes(self) -> int:
+        """Device memory that the multigrid solver holds."""
+        return int(load().qpat_mesh_multigrid_bytes(self.handle))
 
     def set_timing(self, on: bool = True):
         _check(load().qpat_mesh_set_timing(self.handle, 1 if on else 0))
