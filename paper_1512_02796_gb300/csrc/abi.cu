@@ -263,6 +263,7 @@ static int pcg_status(int st, const char* what) {
 //   R = 2 5.3 / 6.9 (33 x 33 x 41), R = 4 8.1 / 8.2, R = 8 12.2 / 10.3, 3.6 / 4.4 (21 x 21 x 27);
 //   K, precision 1 against the FP32 cycle: 1.4 / 1.1 ms (9^3, R = 1), 24 / 3.3 (40^3, R = 8).
 static bool prefers_multigrid(const qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R) {
+    if (M->multigrid_refused) return false;
     const int deg = st.kind == OP_PRIOR ? so.poly_prior : so.poly_k;
     if (so.multigrid || so.pcg_variant != 0 || so.mixed_restart || so.spin_limit > 0 || deg != kDefaultPolyDegree) return false;
     const int64_t N = M->h.N;
@@ -271,6 +272,34 @@ static bool prefers_multigrid(const qpat_mesh_s* M, const OpState& st, const Sol
     const bool lean = 3 * M->dp.sell_entries < 2 * M->d.sell_entries;
     if (R == 1) return N >= (lean ? 48000 : 150000);
     return lean ? N >= 8000 : N * R >= 180000;
+}
+
+// Iterations that the library's own attempt at multigrid may take: the most
+// that any mesh above needed is 85, and a system that takes several times as
+// many is not one for which this choice is the faster.
+constexpr int kAttemptIterations = 400;
+
+// The multigrid CG where the library chose it: true if that settles the call
+// (*rc).  Where multigrid cannot solve the system (no hierarchy for this mesh,
+// no memory, coefficients beyond the FP32 cycle, a breakdown, more iterations
+// than above) the call goes on with the persistent solver as if it had not been
+// tried: no counts, no message.  A mesh without hierarchy or memory is not
+// tried again.
+static bool multigrid_settles(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, const double* B, double* X,
+                              cudaStream_t s, const double* X0, int* rc) {
+    SolveOpts mg = so;
+    mg.multigrid = st.kind == OP_K && so.precision == 1 ? 2 : 1;
+    mg.maxit = std::min(so.maxit, kAttemptIterations);
+    const SolveStats before = M->stats;
+    const std::string message = g_err;
+    *rc = amg_solve(M, st, mg, R, B, X, s, X0);
+    if (*rc == QPAT_OK) return true;
+    const AmgOutcome why = amg_outcome(M);
+    if (*rc == QPAT_ECUDA && why != AmgOutcome::no_memory) return true;
+    if (why != AmgOutcome::ran) M->multigrid_refused = true;
+    M->stats = before;
+    g_err = message;
+    return false;
 }
 
 // Solves A X = B for R right-hand sides (library order, N x R node-major,
@@ -287,11 +316,10 @@ int solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so_in, int R, cons
     if (st.kind == OP_PRIOR) so.precision = 0;
     // multigrid-preconditioned CG (FP64 iterates whatever the precision mode)
     if (so.multigrid) return amg_solve(M, st, so, R, B, X, s, X0);
-    if (prefers_multigrid(M, st, so_in, R)) {
-        SolveOpts mg = so;
-        mg.multigrid = st.kind == OP_K && so_in.precision == 1 ? 2 : 1;
-        if (amg_solve(M, st, mg, R, B, X, s, X0) == QPAT_OK) return QPAT_OK;
-        // no hierarchy for this mesh, coefficients beyond the FP32 cycle, a breakdown: the persistent solver decides
+    if (prefers_multigrid(M, st, so, R)) {
+        int rc = QPAT_OK;
+        if (multigrid_settles(M, st, so, R, B, X, s, X0, &rc)) return rc;
+        so.pcg_variant = 1;  // the persistent solver, also where it calls this function for parts of the system
     }
     // the prior's assembled blocks live in the stiffness-only pattern
     const MeshDev& md = st.kind == OP_PRIOR ? M->dp : M->d;
@@ -325,7 +353,7 @@ int solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so_in, int R, cons
                     k_take_rhs<<<grid_of(N * Rh), 256, 0, s>>>(N, R, half * Rh, Rh, X0, X0h);
                 }
                 if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "split");
-                const int rc = solve(M, st, so_in, Rh, Bh, Xh, s, X0h);
+                const int rc = solve(M, st, so, Rh, Bh, Xh, s, X0h);
                 if (rc != QPAT_OK) return rc;
                 qpat::note_launch(1);
                 k_put_rhs<<<grid_of(N * Rh), 256, 0, s>>>(N, R, half * Rh, Rh, Xh, X);
@@ -909,6 +937,7 @@ int qpat_mesh_multigrid_levels(qpat_mesh_t M, int prior, int64_t* rows, int max_
 int qpat_mesh_set_multigrid_limit(qpat_mesh_t M, int64_t bytes) {
     if (!M || bytes < 0) return fail(QPAT_EINVAL, "qpat_mesh_set_multigrid_limit: NULL mesh or negative limit");
     qpat::amg_set_limit(M, size_t(bytes));
+    M->multigrid_refused = false;
     return QPAT_OK;
 }
 

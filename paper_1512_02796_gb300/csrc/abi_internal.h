@@ -102,6 +102,7 @@ struct qpat_mesh_s {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     double pcg_ms = 0.0;
     qpat::AmgState* amg = nullptr;   // built on the first multigrid solve
+    bool multigrid_refused = false;  // no hierarchy or no memory for it: not the library's choice any more
     double mg_fine_ms = 0.0;         // with timing on: fine-level smoothing launches of the multigrid cycle
     int64_t mg_fine_launches = 0;
 };
@@ -133,6 +134,10 @@ uint64_t next_op_stamp();
 // prepared operator.
 int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, const double* B, double* X,
               cudaStream_t s, const double* X0 = nullptr);
+// Why the last amg_solve ended as it did: it ran (with whatever result), this
+// mesh has no hierarchy, or the device had no memory for it.
+enum class AmgOutcome { ran, no_hierarchy, no_memory };
+AmgOutcome amg_outcome(const qpat_mesh_s* M);
 // rows of each level of the hierarchy of the K (prior = 0) or prior pattern; returns the level count
 int amg_levels(qpat_mesh_s* M, int prior, int64_t* rows, int max_levels);
 void amg_set_limit(qpat_mesh_s* M, size_t bytes);  // device memory the solver may hold (0: no limit)

@@ -1052,6 +1052,7 @@ __global__ void k_f2d_vec(int64_t n, const float* in, double* out) {
 // it may hold (0: no limit).
 struct MemLedger {
     size_t used = 0, limit = 0;
+    bool refused = false;  // an allocation failed
 };
 
 // A set of device allocations that is released as a whole.  Every part of the
@@ -1079,12 +1080,14 @@ class DevMem {
         const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
         if (ledger_->limit && ledger_->used + bytes > ledger_->limit) {
             e = cudaErrorMemoryAllocation;
+            ledger_->refused = true;
             return nullptr;
         }
         list_.emplace_back(nullptr, 0);
         void* p = nullptr;
         if ((e = cudaMalloc(&p, bytes)) != cudaSuccess) {
             list_.pop_back();
+            ledger_->refused = e == cudaErrorMemoryAllocation;
             return nullptr;
         }
         list_.back() = {p, bytes};
@@ -1868,6 +1871,7 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         return fail(QPAT_EINVAL, "multigrid: mg_degree must lie in [1, 8] and mg_ratio exceed 1");
     if (!M->amg) M->amg = new AmgState();
     AmgState& A = *M->amg;
+    A.ledger.refused = false;
     AmgHierDev& H = A.hier;
     if (!H.ready) {
         if (!H.error.empty()) return fail(QPAT_EINVAL, H.error);
@@ -1975,6 +1979,11 @@ int amg_levels(qpat_mesh_s* M, int prior, int64_t* rows, int max_levels) {
 void amg_set_limit(qpat_mesh_s* M, size_t bytes) {
     if (!M->amg) M->amg = new AmgState();
     M->amg->ledger.limit = bytes;
+}
+
+AmgOutcome amg_outcome(const qpat_mesh_s* M) {
+    if (!M->amg || M->amg->ledger.refused) return AmgOutcome::no_memory;
+    return M->amg->hier.ready ? AmgOutcome::ran : AmgOutcome::no_hierarchy;
 }
 
 size_t amg_bytes(const qpat_mesh_s* M) { return M->amg ? M->amg->ledger.used : 0; }
