@@ -783,9 +783,12 @@ constexpr int kCtlActive = 8;
 // bb = totals of b.b.  A right-hand side with b = 0 is solved by x = 0, and
 // one whose guess already meets the target by that guess: neither runs (a
 // residual of 0 would have no direction).  Q: quantities per right-hand side
-// in the partials (2: r.r behind b.b; 1: r = b).
+// in the partials (2: r.r behind b.b; 1: r = b).  scale: the power of two that
+// brings |r| to [1, 2); the FP32 cycle works on scale r, so that neither small
+// nor large right-hand sides leave FP32's range.  z, p and q then carry it too,
+// alpha its inverse, and beta and the iterates are the same to the bit.
 template <int R, int Q>
-__global__ void k_cg_start(const double* part, int G, const double* rtol2, double* bb, int* ctl) {
+__global__ void k_cg_start(const double* part, int G, const double* rtol2, double* bb, double* scale, int* ctl) {
     int* active = ctl + kCtlActive;
     __shared__ int clear[R];
     const int r = threadIdx.x >> 5;
@@ -793,6 +796,7 @@ __global__ void k_cg_start(const double* part, int G, const double* rtol2, doubl
     const double rr = Q == 1 ? t : total_of(part, G, Q * R, (Q - 1) * R + r);
     if ((threadIdx.x & 31) == 0) {
         bb[r] = t;
+        scale[r] = rr > 0.0 && isfinite(rr) ? scalbn(1.0, -(ilogb(rr) >> 1)) : 1.0;
         active[r] = t > 0.0 && rr > *rtol2 * t ? 1 : 0;
         clear[r] = t == 0.0 && rr > 0.0 ? 1 : 0;
         if (!isfinite(t))
@@ -976,7 +980,7 @@ __global__ void __launch_bounds__(256) k_cg_dir(int64_t n, const double* beta, c
     }
 }
 
-// x += alpha p, r -= alpha q (b32: and the FP32 copy of r), r.r.  The last
+// x += alpha p, r -= alpha q (b32: and the FP32 copy of scale r), r.r.  The last
 // block checks: a right-hand side stops once |r| <= rtol |b|; one more
 // iteration is done.  Inside a graph (use_graph) it also sets the loop's
 // condition: go on while some right-hand side runs, the status is clean and
@@ -985,16 +989,17 @@ __global__ void __launch_bounds__(256) k_cg_dir(int64_t n, const double* beta, c
 template <int R>
 __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alpha, const double* __restrict__ p,
                                                    const double* __restrict__ q, double* __restrict__ x,
-                                                   double* __restrict__ r, float* __restrict__ b32, double* part,
-                                                   unsigned* count, const double* bb, const double* rtol2, double* rr,
+                                                   double* __restrict__ r, const double* scale,
+                                                   float* __restrict__ b32, double* part, unsigned* count, const double* bb, const double* rtol2, double* rr,
                                                    int* ctl, cudaGraphConditionalHandle cond, int use_graph) {
     constexpr int C = FlatMap<R>::C;
     const FlatMap<R> m;
     __shared__ double tot[R];
-    double al[C], dot[C];
+    double al[C], sc[C], dot[C];
 #pragma unroll
     for (int t = 0; t < C; ++t) {
         al[t] = alpha[m.c0 + t];
+        sc[t] = scale[m.c0 + t];
         dot[t] = 0.0;
     }
     FOR_FLAT(n, R) {
@@ -1013,7 +1018,7 @@ __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alph
         stR<double, C>(r + o, rv);
         if (b32)
 #pragma unroll
-            for (int t = 0; t < C; ++t) b32[o + t] = float(rv[t]);
+            for (int t = 0; t < C; ++t) b32[o + t] = float(sc[t] * rv[t]);
     }
     m.template block_totals<1>(dot, part);
     if (!last_block_totals<R>(part, count, tot)) return;
@@ -1035,9 +1040,11 @@ __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alph
     }
 }
 
-__global__ void k_d2f_vec(int64_t n, const double* in, float* out) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        out[i] = float(in[i]);
+// b32 = scale r in FP32, N x R
+template <int R>
+__global__ void __launch_bounds__(256) k_cg_cast(int64_t n, const double* scale, const double* r, float* b32) {
+    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n * R; i += int64_t(gridDim.x) * blockDim.x)
+        b32[i] = float(scale[i % R] * r[i]);
 }
 __global__ void k_f2d_vec(int64_t n, const float* in, double* out) {
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
@@ -1162,7 +1169,8 @@ struct AmgVecs {
 struct AmgCg {
     explicit AmgCg(MemLedger* l) : mem(l) {}
     double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *part = nullptr;
-    double *bb = nullptr, *rz = nullptr, *alpha = nullptr, *beta = nullptr, *rr = nullptr, *rtol2 = nullptr;
+    double *bb = nullptr, *rz = nullptr, *alpha = nullptr, *beta = nullptr, *rr = nullptr, *scale = nullptr;
+    double* rtol2 = nullptr;
     int* ctl = nullptr;  // control words (see k_cg_start)
     unsigned* count = nullptr;  // blocks that have finished (see last_block_totals)
     DevMem mem;
@@ -1738,8 +1746,8 @@ struct CgSolve {
         // K's rows hold 15 entries, M_delta's 7: one group per row, the lanes of its right-hand sides side by side
         k_cg_apply<R, NV, 1><<<full_grid(k_cg_apply<R, NV, 1>, G), 256, 0, t>>>(NV == 1 ? H.K : H.lv[0].A, st.v64[0], st.v64[1], C.p, C.q, C.part, C.count,
                                                C.rz, C.alpha, C.ctl);
-        k_cg_update<R><<<full_grid(k_cg_update<R>, G), 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, f32 ? static_cast<float*>(W.b[0]) : nullptr,
-                                         C.part, C.count, C.bb, C.rtol2, C.rr, C.ctl, cond, use_graph);
+        k_cg_update<R><<<full_grid(k_cg_update<R>, G), 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, C.scale,
+                                         f32 ? static_cast<float*>(W.b[0]) : nullptr, C.part, C.count, C.bb, C.rtol2, C.rr, C.ctl, cond, use_graph);
     }
 
     int run(AmgState& A, const std::string& key, const double* B, double* X, const double* X0, int* iters) {
@@ -1763,10 +1771,10 @@ struct CgSolve {
         note_launch(2);
         if (X0) {
             k_cg_init_x0<R, NV><<<G, 256, 0, s>>>(A0, st.v64[0], st.v64[1], B, X0, C.x, C.r, C.part);
-            k_cg_start<R, 2><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.ctl);
+            k_cg_start<R, 2><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.scale, C.ctl);
         } else {
             k_cg_init<R><<<G, 256, 0, s>>>(n, B, C.x, C.r, C.part);
-            k_cg_start<R, 1><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.ctl);
+            k_cg_start<R, 1><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.scale, C.ctl);
         }
         if ((e = read_ctl()) != cudaSuccess) return cuda_fail(e, "multigrid cg");
         if (hc[0] != QPAT_OK)
@@ -1779,7 +1787,7 @@ struct CgSolve {
         if (hc[1] > 0) {
             if (f32) {
                 note_launch(1);
-                k_d2f_vec<<<G, 256, 0, s>>>(n * R, C.r, static_cast<float*>(W.b[0]));
+                k_cg_cast<R><<<G, 256, 0, s>>>(n, C.scale, C.r, static_cast<float*>(W.b[0]));
             }
             if (!timer->on) {
                 auto g = V.graphs.find(key);
@@ -1920,7 +1928,7 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         C.q = C.mem.get<double>(nR, e);
         C.z = C.mem.get<double>(nR, e);
         C.part = C.mem.get<double>(size_t(kRedMaxGrid) * 32, e);
-        double* sc = C.mem.get<double>(5 * 16 + 1, e);
+        double* sc = C.mem.get<double>(6 * 16 + 1, e);
         C.ctl = C.mem.get<int>(kCtlActive + 16, e);
         C.count = C.mem.get<unsigned>(1, e);
         if (e == cudaSuccess) e = cudaMemsetAsync(C.count, 0, sizeof(unsigned), s);
@@ -1931,7 +1939,8 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         C.alpha = sc + 32;
         C.beta = sc + 48;
         C.rr = sc + 64;
-        C.rtol2 = sc + 80;
+        C.scale = sc + 80;
+        C.rtol2 = sc + 96;
         cg = A.cg.emplace(R, std::move(C)).first;
     }
     AmgCg& C = cg->second;
