@@ -64,8 +64,9 @@ typedef struct {
     int fixed_counts;      /* 1: run exactly max_lin x max_lsqr, no Eq. (22) stop
                               (the step-4 acceptance of Algorithm 1 stays active) */
     int precision;         /* 0: FP64 PCG; 1: FP32 PCG inside FP64 refinement for
-                              the K solves (M_delta solves always run in FP64:
-                              their conditioning, set by delta, is beyond FP32) */
+                              the K solves, until the FP64 residual b - A x meets
+                              pcg_rtol (M_delta solves always run in FP64: their
+                              conditioning, set by delta, is beyond FP32) */
     int max_pcg_iter;      /* cap per PCG run (inner run for precision 1) */
     double pcg_rtol;       /* |b - A x| / |b| target of every K and M_delta solve */
     int fit_grid;          /* (kappa_0, mu_0) search grid per axis (Algorithm 1) */
@@ -238,7 +239,8 @@ int qpat_multigrid_host_info(const double* xyz, int64_t N, const int32_t* tets, 
 int qpat_mesh_stats(qpat_mesh_t mesh, int64_t* out4);
 /* Precision-1 solves of K whose FP32 inner PCG broke down, or whose FP64
  * refinement stalled, and that were therefore solved again by the FP64 PCG
- * (since the last reset); -1 for a NULL mesh. */
+ * (or, by the multigrid CG, whose iterates are FP64, taken as they were) since
+ * the last reset; -1 for a NULL mesh. */
 int64_t qpat_mesh_fp64_fallbacks(qpat_mesh_t mesh);
 int qpat_mesh_reset_stats(qpat_mesh_t mesh);
 /* Sum over the PCG launches since the last reset of iterations times the

@@ -278,6 +278,11 @@ static bool prefers_multigrid(const qpat_mesh_s* M, const OpState& st, const Sol
 // that any mesh above needed is 85, and a system that takes several times as
 // many is not one for which this choice is the faster.
 constexpr int kAttemptIterations = 400;
+// Sweeps of its refinement: two reach the target in the recursive residual, a
+// third takes off the rounding of their iterates.  What the FP64 residual is
+// above the target then, the FP64 solver that precision 1 falls back to (which
+// knows the recursive residual only) would leave as well.
+constexpr int kAttemptSweeps = 3;
 
 // The multigrid CG where the library chose it: true if that settles the call
 // (*rc).  Where multigrid cannot solve the system (no hierarchy for this mesh,
@@ -290,6 +295,13 @@ static bool multigrid_settles(qpat_mesh_s* M, const OpState& st, const SolveOpts
     SolveOpts mg = so;
     mg.multigrid = st.kind == OP_K && so.precision == 1 ? 2 : 1;
     mg.maxit = std::min(so.maxit, kAttemptIterations);
+    if (mg.multigrid == 2) {
+        // precision 1: refinement, as with the FP32 solver, until the FP64 residual b - A x meets the target.  The
+        // iterates are FP64, so that two sweeps can go as far as that solver's k sweeps to inner_rtol.
+        const double k = std::max(1.0, std::ceil(std::log(so.rtol) / std::log(so.inner_rtol)));
+        mg.sweep_rtol = std::pow(so.inner_rtol, k / 2);
+        mg.max_sweeps = std::min(so.max_sweeps, kAttemptSweeps);
+    }
     const SolveStats before = M->stats;
     const std::string message = g_err;
     *rc = amg_solve(M, st, mg, R, B, X, s, X0);
@@ -304,8 +316,10 @@ static bool multigrid_settles(qpat_mesh_s* M, const OpState& st, const SolveOpts
 
 // Solves A X = B for R right-hand sides (library order, N x R node-major,
 // FP64 in and out).  precision 0: FP64 PCG to rtol.  precision 1: X = 0,
-// then sweeps of  r = B - A X (FP64 element apply), d = A32^-1 (r / |r|)
-// (FP32 PCG to a loose tolerance), X += |r| d,  until |r_j| <= rtol |B_j|.
+// then sweeps of  r = B - A X (FP64 assembled product), d = A32^-1 (r / |r|)
+// (FP32 PCG to a loose tolerance), X += |r| d,  until |r_j| <= rtol |B_j|;
+// where the library chose multigrid, the sweeps' solver is FP64 CG with the
+// cycle in FP32.
 int solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so_in, int R, const double* B, double* X,
           cudaStream_t s, const double* X0) {
     // M_delta is solved in FP64 whatever the precision mode: its smallest

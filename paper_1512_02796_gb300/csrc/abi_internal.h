@@ -66,6 +66,7 @@ struct SolveOpts {
     long long spin_limit = 0; // grid-barrier polls before a timeout (0 = default)
     int multigrid = 0;        // 1: CG with the smoothed-aggregation V-cycle (FP64); 2: its K cycle in FP32
     int mg_degree = 1;        // Chebyshev degree of each smoothing
+    double sweep_rtol = 0.0;  // multigrid > 0: refinement by sweeps to this (0: one run to rtol)
     double mg_ratio = 30.0;   // smoothing interval [hi / mg_ratio, hi] of D^-1 A
 };
 

@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(256) k_cg_init(int64_t n, const double* b, dou
     block_partials<R>(acc, part);
 }
 
-// x = x0, r = b - A x0, partials of b.b and of r.r (the stopping target stays rtol |b|)
+// x = x0, r = b - A x0, partials of b.b and of r.r (the stopping target stays rtol |b|); x0 may be x
 template <int R, int NV>
 __global__ void __launch_bounds__(256) k_cg_init_x0(SellDev A, const double* v0, const double* v1, const double* b,
                                                     const double* x0, double* x, double* r, double* part) {
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(256) k_cg_init_x0(SellDev A, const double* v0,
             acc[R + q] = fma(av[q], av[q], acc[R + q]);
         }
         stR<double, R>(r + i * R, av);
-        stR<double, R>(x + i * R, xv);
+        if (x != x0) stR<double, R>(x + i * R, xv);
     }
     block_partials<2 * R>(acc, part);
 }
@@ -787,8 +787,12 @@ constexpr int kCtlActive = 8;
 // brings |r| to [1, 2); the FP32 cycle works on scale r, so that neither small
 // nor large right-hand sides leave FP32's range.  z, p and q then carry it too,
 // alpha its inverse, and beta and the iterates are the same to the bit.
+// stop: the |r|^2 at which the iteration leaves a right-hand side: the target
+// tol[0] |b|^2, or, in sweeps (tol[1] > 0), tol[1] times |r|^2 at the sweep's
+// start, but no less than two such sweeps from |b|^2 would leave.
 template <int R, int Q>
-__global__ void k_cg_start(const double* part, int G, const double* rtol2, double* bb, double* scale, int* ctl) {
+__global__ void k_cg_start(const double* part, int G, const double* tol, double* bb, double* stop, double* scale,
+                           int* ctl) {
     int* active = ctl + kCtlActive;
     __shared__ int clear[R];
     const int r = threadIdx.x >> 5;
@@ -797,7 +801,8 @@ __global__ void k_cg_start(const double* part, int G, const double* rtol2, doubl
     if ((threadIdx.x & 31) == 0) {
         bb[r] = t;
         scale[r] = rr > 0.0 && isfinite(rr) ? scalbn(1.0, -(ilogb(rr) >> 1)) : 1.0;
-        active[r] = t > 0.0 && rr > *rtol2 * t ? 1 : 0;
+        stop[r] = tol[1] > 0.0 ? fmax(tol[1] * rr, tol[1] * tol[1] * t) : tol[0] * t;
+        active[r] = t > 0.0 && rr > tol[0] * t ? 1 : 0;
         clear[r] = t == 0.0 && rr > 0.0 ? 1 : 0;
         if (!isfinite(t))
             atomicExch(ctl, int(QPAT_EINVAL));
@@ -981,7 +986,7 @@ __global__ void __launch_bounds__(256) k_cg_dir(int64_t n, const double* beta, c
 }
 
 // x += alpha p, r -= alpha q (b32: and the FP32 copy of scale r), r.r.  The last
-// block checks: a right-hand side stops once |r| <= rtol |b|; one more
+// block checks: a right-hand side stops once |r|^2 <= stop; one more
 // iteration is done.  Inside a graph (use_graph) it also sets the loop's
 // condition: go on while some right-hand side runs, the status is clean and
 // the cap is not reached (reaching it with a running right-hand side is
@@ -990,8 +995,9 @@ template <int R>
 __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alpha, const double* __restrict__ p,
                                                    const double* __restrict__ q, double* __restrict__ x,
                                                    double* __restrict__ r, const double* scale,
-                                                   float* __restrict__ b32, double* part, unsigned* count, const double* bb, const double* rtol2, double* rr,
-                                                   int* ctl, cudaGraphConditionalHandle cond, int use_graph) {
+                                                   float* __restrict__ b32, double* part, unsigned* count,
+                                                   const double* stop, double* rr, int* ctl,
+                                                   cudaGraphConditionalHandle cond, int use_graph) {
     constexpr int C = FlatMap<R>::C;
     const FlatMap<R> m;
     __shared__ double tot[R];
@@ -1027,7 +1033,7 @@ __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alph
         const double t = tot[threadIdx.x];
         rr[threadIdx.x] = t;
         if (!isfinite(t)) atomicExch(ctl, int(QPAT_EBREAKDOWN));
-        if (active[threadIdx.x] && t <= *rtol2 * bb[threadIdx.x]) active[threadIdx.x] = 0;
+        if (active[threadIdx.x] && t <= stop[threadIdx.x]) active[threadIdx.x] = 0;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1170,7 +1176,7 @@ struct AmgCg {
     explicit AmgCg(MemLedger* l) : mem(l) {}
     double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *part = nullptr;
     double *bb = nullptr, *rz = nullptr, *alpha = nullptr, *beta = nullptr, *rr = nullptr, *scale = nullptr;
-    double* rtol2 = nullptr;
+    double *stop = nullptr, *tol = nullptr;
     int* ctl = nullptr;  // control words (see k_cg_start)
     unsigned* count = nullptr;  // blocks that have finished (see last_block_totals)
     DevMem mem;
@@ -1678,6 +1684,13 @@ struct FastCycle {
     }
 };
 
+// What a solve took: iterations, the sweeps they came in, and whether the
+// refinement ended above its target.
+struct CgCount {
+    int iters = 0, sweeps = 0;
+    bool stalled = false;
+};
+
 // Conjugate gradients on the fine operator with one V-cycle per iteration
 // as the preconditioner; X0 (or 0) to start, each right-hand side stops at
 // |r| <= rtol |b| (the recursive residual, as the persistent PCG does).
@@ -1747,10 +1760,14 @@ struct CgSolve {
         k_cg_apply<R, NV, 1><<<full_grid(k_cg_apply<R, NV, 1>, G), 256, 0, t>>>(NV == 1 ? H.K : H.lv[0].A, st.v64[0], st.v64[1], C.p, C.q, C.part, C.count,
                                                C.rz, C.alpha, C.ctl);
         k_cg_update<R><<<full_grid(k_cg_update<R>, G), 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, C.scale,
-                                         f32 ? static_cast<float*>(W.b[0]) : nullptr, C.part, C.count, C.bb, C.rtol2, C.rr, C.ctl, cond, use_graph);
+                                         f32 ? static_cast<float*>(W.b[0]) : nullptr, C.part, C.count, C.stop, C.rr, C.ctl, cond, use_graph);
     }
 
-    int run(AmgState& A, const std::string& key, const double* B, double* X, const double* X0, int* iters) {
+    // With so.sweep_rtol the solve is a refinement: sweeps of the iteration,
+    // each to sweep_rtol of the residual b - A x that is formed at its start,
+    // until that residual meets the target or max_sweeps are over.  The
+    // iterates are FP64, so that what is left then is their rounding.
+    int run(AmgState& A, const std::string& key, const double* B, double* X, const double* X0, CgCount* count) {
         const SellDev& A0 = NV == 1 ? H.K : H.lv[0].A;
         n = A0.n;
         G = int(std::min<int64_t>(blocks_of(n * R, 512), kRedMaxGrid));
@@ -1761,30 +1778,37 @@ struct CgSolve {
             if (x == cudaSuccess) x = cudaStreamSynchronize(s);
             return x;
         };
-        const double rtol2 = so.rtol * so.rtol;
+        const bool refine = so.sweep_rtol > 0.0;
+        const double tol[2] = {so.rtol * so.rtol, refine ? so.sweep_rtol * so.sweep_rtol : 0.0};
         const int cap[1] = {so.maxit};
         if ((e = cudaMemsetAsync(C.ctl, 0, 8 * sizeof(int), s)) != cudaSuccess ||
             (e = cudaMemcpyAsync(C.ctl + 4, cap, sizeof(int), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(C.rtol2, &rtol2, sizeof(double), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(C.tol, tol, sizeof(tol), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(C.p, 0, sizeof(double) * n * R, s)) != cudaSuccess)
             return cuda_fail(e, "multigrid start");
-        note_launch(2);
-        if (X0) {
-            k_cg_init_x0<R, NV><<<G, 256, 0, s>>>(A0, st.v64[0], st.v64[1], B, X0, C.x, C.r, C.part);
-            k_cg_start<R, 2><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.scale, C.ctl);
-        } else {
-            k_cg_init<R><<<G, 256, 0, s>>>(n, B, C.x, C.r, C.part);
-            k_cg_start<R, 1><<<1, 32 * R, 0, s>>>(C.part, G, C.rtol2, C.bb, C.scale, C.ctl);
-        }
-        if ((e = read_ctl()) != cudaSuccess) return cuda_fail(e, "multigrid cg");
-        if (hc[0] != QPAT_OK)
-            return fail(hc[0], hc[0] == QPAT_EINVAL ? "multigrid cg: right-hand side not finite"
-                                                    : "multigrid cg: residual of the initial guess not finite");
-        if (hc[5] > 0) {
-            note_launch(1);
-            k_cg_clear<R><<<G, 256, 0, s>>>(n, C.bb, C.x, C.r);
-        }
-        if (hc[1] > 0) {
+        for (const double* from = X0;; from = C.x) {
+            note_launch(2);
+            if (from) {
+                k_cg_init_x0<R, NV><<<G, 256, 0, s>>>(A0, st.v64[0], st.v64[1], B, from, C.x, C.r, C.part);
+                k_cg_start<R, 2><<<1, 32 * R, 0, s>>>(C.part, G, C.tol, C.bb, C.stop, C.scale, C.ctl);
+            } else {
+                k_cg_init<R><<<G, 256, 0, s>>>(n, B, C.x, C.r, C.part);
+                k_cg_start<R, 1><<<1, 32 * R, 0, s>>>(C.part, G, C.tol, C.bb, C.stop, C.scale, C.ctl);
+            }
+            if ((e = read_ctl()) != cudaSuccess) return cuda_fail(e, "multigrid cg");
+            if (hc[0] != QPAT_OK)
+                return fail(hc[0], hc[0] == QPAT_EINVAL ? "multigrid cg: right-hand side not finite"
+                                                        : "multigrid cg: residual at the start not finite");
+            if (hc[5] > 0) {
+                note_launch(1);
+                k_cg_clear<R><<<G, 256, 0, s>>>(n, C.bb, C.x, C.r);
+            }
+            if (hc[1] == 0) break;
+            if (refine && count->sweeps >= so.max_sweeps) {
+                count->stalled = true;
+                break;
+            }
+            ++count->sweeps;
             if (f32) {
                 note_launch(1);
                 k_cg_cast<R><<<G, 256, 0, s>>>(n, C.scale, C.r, static_cast<float*>(W.b[0]));
@@ -1808,10 +1832,11 @@ struct CgSolve {
                     if (hc[0] != QPAT_OK || hc[1] == 0) break;
                 }
             }
+            count->iters += hc[2];
+            if (hc[0] == QPAT_ENOCONV) return fail(QPAT_ENOCONV, "multigrid cg: iteration cap reached");
+            if (hc[0] != QPAT_OK) return fail(hc[0], "multigrid cg: breakdown (p.Ap <= 0 or not finite)");
+            if (!refine) break;
         }
-        *iters = hc[2];
-        if (hc[0] == QPAT_ENOCONV) return fail(QPAT_ENOCONV, "multigrid cg: iteration cap reached");
-        if (hc[0] != QPAT_OK) return fail(hc[0], "multigrid cg: breakdown (p.Ap <= 0 or not finite)");
         if ((e = cudaMemcpyAsync(X, C.x, sizeof(double) * n * R, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
             return cuda_fail(e, "copy");
         return QPAT_OK;
@@ -1855,16 +1880,16 @@ struct CgSolve {
 template <int NV>
 int dispatch(int R, AmgState& A, const std::string& key, qpat_mesh_s* M, const OpState& st, const SolveOpts& so,
              const AmgHierDev& H, AmgValues& V, bool f32, AmgVecs& W, AmgCg& C, const double* B, double* X,
-             const double* X0, cudaStream_t s, FineTimer* timer, int* iters) {
+             const double* X0, cudaStream_t s, FineTimer* timer, CgCount* count) {
     if constexpr (NV == 2) {
-        return CgSolve<2, 2>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, iters);
+        return CgSolve<2, 2>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, count);
     } else {
         switch (R) {
-            case 1: return CgSolve<1, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, iters);
-            case 2: return CgSolve<2, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, iters);
-            case 4: return CgSolve<4, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, iters);
-            case 8: return CgSolve<8, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, iters);
-            default: return CgSolve<16, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, iters);
+            case 1: return CgSolve<1, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, count);
+            case 2: return CgSolve<2, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, count);
+            case 4: return CgSolve<4, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, count);
+            case 8: return CgSolve<8, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, count);
+            default: return CgSolve<16, 1>{M, st, so, H, V, f32, W, C, s, timer}.run(A, key, B, X, X0, count);
         }
     }
 }
@@ -1928,7 +1953,7 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         C.q = C.mem.get<double>(nR, e);
         C.z = C.mem.get<double>(nR, e);
         C.part = C.mem.get<double>(size_t(kRedMaxGrid) * 32, e);
-        double* sc = C.mem.get<double>(6 * 16 + 1, e);
+        double* sc = C.mem.get<double>(7 * 16 + 2, e);
         C.ctl = C.mem.get<int>(kCtlActive + 16, e);
         C.count = C.mem.get<unsigned>(1, e);
         if (e == cudaSuccess) e = cudaMemsetAsync(C.count, 0, sizeof(unsigned), s);
@@ -1940,7 +1965,8 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         C.beta = sc + 48;
         C.rr = sc + 64;
         C.scale = sc + 80;
-        C.rtol2 = sc + 96;
+        C.stop = sc + 96;
+        C.tol = sc + 112;
         cg = A.cg.emplace(R, std::move(C)).first;
     }
     AmgCg& C = cg->second;
@@ -1952,9 +1978,9 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
     timer.on = M->timing != 0;
     timer.s = s;
     if (M->timing) cudaEventRecord(M->ev0, s);
-    int iters = 0;
-    rc = st.nv == 2 ? dispatch<2>(R, A, key, M, st, so, H, V, f32, W, C, B, X, X0, s, &timer, &iters)
-                    : dispatch<1>(R, A, key, M, st, so, H, V, f32, W, C, B, X, X0, s, &timer, &iters);
+    CgCount count;
+    rc = st.nv == 2 ? dispatch<2>(R, A, key, M, st, so, H, V, f32, W, C, B, X, X0, s, &timer, &count)
+                    : dispatch<1>(R, A, key, M, st, so, H, V, f32, W, C, B, X, X0, s, &timer, &count);
     if (timer.on) {
         cudaStreamSynchronize(s);
         timer.collect();
@@ -1969,10 +1995,12 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         cudaEventElapsedTime(&ms, M->ev0, M->ev1);
         M->pcg_ms += ms;
     }
-    M->stats.pcg_iters += iters;
-    M->stats.rhs_iters += int64_t(iters) * R;
+    M->stats.pcg_iters += count.iters;
+    M->stats.rhs_iters += int64_t(count.iters) * R;
     M->stats.solves += R;
-    M->stats.launches += 1;
+    M->stats.launches += std::max(1, count.sweeps);
+    if (so.sweep_rtol > 0.0) M->stats.refinements += count.sweeps;
+    if (count.stalled) M->stats.fp64_fallbacks += 1;
     return rc;
 }
 
