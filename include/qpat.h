@@ -72,8 +72,12 @@ typedef struct {
     int fit_grid;          /* (kappa_0, mu_0) search grid per axis (Algorithm 1) */
     int fit_gn_steps;      /* Gauss-Newton polish steps of that search */
     int patch_nodes;       /* owned nodes per CTA patch (0 = library choice) */
-    int fp32_operator;     /* FP32 inner operator of precision 1: 0 = matrix-free
-                              element recomputation, 1 = assembled FP32 values */
+    int fp32_operator;     /* operator of the FP32 PCG of precision 1: 0 = matrix-free
+                              element recomputation, 1 = assembled FP32 values.
+                              (Where the library takes the multigrid CG for such a
+                              solve, see multigrid, there is no FP32 PCG: its
+                              FP32 cycle works on assembled values.  pcg_variant = 1
+                              always runs the FP32 PCG with this operator.) */
     int pcg_variant;       /* PCG on assembled operators: 0 = library choice
                               (the fastest measured: variant 1, or the multigrid
                               CG below where that is faster; see multigrid),
@@ -136,7 +140,9 @@ typedef struct {
                               a solver (pcg_variant 0, polynomial degrees,
                               mixed_restart and barrier_spin_limit at their
                               defaults), whichever of it and 1 (precision 1:
-                              K solves as 2) was measured faster at the size;
+                              K solves as 2, in sweeps on the FP64 residual) was
+                              measured faster at the size, for the kind of mesh,
+                              the number of right-hand sides and fp32_operator;
                               pcg_variant = 1 always runs the persistent PCG;
                               1 = conjugate gradients with one V-cycle of
                               smoothed-aggregation algebraic multigrid per

@@ -252,26 +252,40 @@ static int pcg_status(int st, const char* what) {
 // The library's choice for solves that ask for neither solver (multigrid = 0,
 // pcg_variant = 0, the default polynomial degree, no barrier limit, no
 // restarts): multigrid-preconditioned CG where it is the faster one, with the
-// cycle in FP32 for the K solves of precision 1 (which may iterate in FP32).
-// Measured on GB300, whole calls, persistent against multigrid:
-//   M_delta: 1.5 / 1.5 ms (11^3), 2.1 / 1.6 (13^3), 4.0 / 1.9 (24^3), 27 / 6.5 (64^3), cylinders 3.3 / 2.7 (11 x 11 x 14),
-//   6.5 / 4.5 (21 x 21 x 27), 41 / 17 (49 x 49 x 61);
-//   K, FP64 on grids (the stiffness pattern well below K's): R = 1 1.6 / 1.7 ms (32^3), 2.4 / 2.1 (40^3),
-//   R = 2 1.1 / 1.4 (16^3), 1.9 / 1.7 (24^3), R = 4 1.1 / 1.5 (16^3), 1.7 / 1.6 (20^3), 2.1 / 1.8 (24^3),
-//   R = 8 0.9 / 1.2 (11^3), 1.1 / 1.5 (16^3), 1.8 / 1.75 (20^3), 7.3 / 3.9 (40^3);
-//   on cylinders, whose cycle keeps K's whole pattern: R = 1 4.4 / 5.9 (33 x 33 x 41), 10.7 / 11.5 (49 x 49 x 61),
-//   R = 2 5.3 / 6.9 (33 x 33 x 41), R = 4 8.1 / 8.2, R = 8 12.2 / 10.3, 3.6 / 4.4 (21 x 21 x 27);
-//   K, precision 1 against the FP32 cycle: 1.4 / 1.1 ms (9^3, R = 1), 24 / 3.3 (40^3, R = 8).
+// cycle in FP32 for the K solves of precision 1 (whose FP32 solver is another
+// one for each fp32_operator, so that the line is, too).  Lean: the stiffness
+// pattern, on which K's cycle works, is well below K's (grids of right-angled
+// tets); on other meshes the cycle costs twice as much and takes more iterations.
+// Measured on GB300, whole calls, persistent against multigrid, in ms; "jittered" are
+// grids with inner nodes displaced at random and renumbered, "Delaunay" those of random points:
+//   M_delta: 1.5 / 1.5 (11^3), 2.1 / 1.6 (13^3), 4.0 / 1.9 (24^3), 27 / 6.5 (64^3), cylinders 2.6 / 2.3 (11 x 11 x 14),
+//   6.8 / 4.4 (21 x 21 x 27), 39 / 18 (49 x 49 x 61), jittered 3.3 / 2.1 (13^3), 57 / 13 (64^3), Delaunay 8.5 / 5.7
+//   (2 k nodes), 41 / 38 (64 k), 150 / 92 (205 k);
+//   K, FP64, lean: R = 1 1.6 / 1.7 (32^3), 2.4 / 2.1 (40^3), R = 2 1.1 / 1.4 (16^3), 1.9 / 1.7 (24^3),
+//   R = 4 1.1 / 1.5 (16^3), 1.7 / 1.6 (20^3), 2.1 / 1.8 (24^3), R = 8 0.9 / 1.2 (11^3), 1.1 / 1.5 (16^3), 1.8 / 1.75 (20^3),
+//   7.3 / 3.9 (40^3);
+//   K, FP64, other meshes: R = 1 9.7 / 12.8 (49 x 49 x 61), 7.0 / 7.5 (jittered 64^3), 64 / 99 (Delaunay, 205 k);
+//   R = 2 14.4 / 15.3 (49 x 49 x 61); R = 4 4.4 / 5.5 (jittered 40^3), 24 / 21 (49 x 49 x 61), 38 / 42 (Delaunay, 64 k),
+//   193 / 137 (205 k); R = 8 11.2 / 10.7 (33 x 33 x 41), 7.1 / 6.8 (jittered 40^3), 66 / 56 (Delaunay, 64 k);
+//   R = 16 5.1 / 5.6 (21 x 21 x 27), 3.1 / 3.7 (jittered 24^3), 12.7 / 9.6 (jittered 40^3), 119 / 81 (Delaunay, 64 k);
+//   K, precision 1, matrix-free: R = 1 1.4 / 1.4 (11^3), 1.7 / 1.5 (13^3), R = 4 1.5 / 1.3 (9^3), 16 / 4.0 (48^3), cylinder
+//   11 x 11 x 14 R = 4 2.3 / 2.3, R = 8 3.4 / 2.4, jittered R = 1 1.5 / 1.8 (13^3), 2.8 / 2.6 (24^3), R = 4 1.9 / 1.9 (13^3);
+//   K, precision 1, assembled: R = 1 2.8 / 2.7 (48^3), 4.7 / 4.2 (64^3), R = 4 3.4 / 4.0 (48^3), 6.4 / 5.7 (64^3),
+//   R = 8 4.5 / 5.2 (48^3), 10.3 / 7.8 (64^3); jittered 64^3 R = 1 5.6 / 7.5, R = 8 12.0 / 12.5, R = 16 23.8 / 19.0;
+//   49 x 49 x 61 R = 1 8.2 / 11.7, R = 16 25.6 / 32.7; Delaunay, 64 k, R = 16 65 / 99.
 static bool prefers_multigrid(const qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R) {
     if (M->multigrid_refused) return false;
     const int deg = st.kind == OP_PRIOR ? so.poly_prior : so.poly_k;
     if (so.multigrid || so.pcg_variant != 0 || so.mixed_restart || so.spin_limit > 0 || deg != kDefaultPolyDegree) return false;
     const int64_t N = M->h.N;
     if (st.kind == OP_PRIOR) return N >= 1500;
-    if (so.precision == 1) return N >= 512;
     const bool lean = 3 * M->dp.sell_entries < 2 * M->d.sell_entries;
-    if (R == 1) return N >= (lean ? 48000 : 150000);
-    return lean ? N >= 8000 : N * R >= 180000;
+    if (so.precision == 1) {
+        if (so.fp32_assembled) return lean ? N >= 200000 : N * R >= 4000000;
+        return N * R >= (lean ? 2000 : 8000);
+    }
+    if (lean) return N >= (R == 1 ? 48000 : 8000);
+    return R > 1 && N * R >= 350000;
 }
 
 // Iterations that the library's own attempt at multigrid may take: the most

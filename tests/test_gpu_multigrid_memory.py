@@ -63,8 +63,7 @@ def test_every_allocation_can_fail(inputs, kind, named):
         mesh.close()
 
 
-@pytest.mark.parametrize("kind,prm,bits", [("K", {}, True), ("K", dict(precision=1), False),
-                                           ("K", dict(precision=1, fp32_operator=1), True), ("prior", {}, True)], ids=str)
+@pytest.mark.parametrize("kind,prm,bits", [("K", {}, True), ("K", dict(precision=1), False), ("prior", {}, True)], ids=str)
 def test_default_solves_go_on(inputs, kind, prm, bits):
     mesh = Q.qpat_mesh(*inputs[:2])
     chosen = solve(mesh, kind, inputs, **prm)
