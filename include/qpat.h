@@ -163,11 +163,12 @@ typedef struct {
                               The hierarchy's patterns are built on the host on the
                               first such solve of a mesh (seconds at 2 M nodes),
                               its values on the device once per prepared operator. */
-    int mg_degree;         /* Chebyshev degree of each multigrid smoothing, 1..8
-                              (default and 0: 1, i.e. one damped-Jacobi step
-                              before and after each coarse correction; on GB300
-                              every fine-level step is an FP64 sparse product,
-                              and degree 1 was the fastest measured) */
+    int mg_degree;         /* Chebyshev degree of the fine level's multigrid
+                              smoothing, 1..8 (default and 0: 1, i.e. one
+                              damped-Jacobi step before and after the coarse
+                              correction; on GB300 every fine-level step is an
+                              FP64 sparse product, and degree 1 was the fastest
+                              measured).  The coarser levels always take one step. */
     double mg_ratio;       /* the smoothing polynomial targets [hi / mg_ratio, hi] of
                               the spectrum of D^-1 A, hi its Gershgorin bound
                               times a margin of 1.13 (> 1; 0 = 30) */

@@ -411,22 +411,14 @@ __device__ __forceinline__ void stR(T* p, const T* v) {
     }
 }
 
-// acc = (A x)_i for the R columns of row i (NV = 2: column r uses value set
-// r).  G lanes share a row (G = 1: one thread per row; G = 8 for rows of a
-// few dozen entries and more): lane `sub` takes entries sub, sub + G, ...
-// and the group's sums are combined by a fixed xor tree, so every lane of
-// the group ends with the same, run-to-run identical, total.  Lanes past the
-// last row (valid = false) take part in the shuffles only.
-template <typename T, int R, int NV, int G>
-__device__ __forceinline__ void row_apply(const SellDev& A, const T* v0, const T* v1, const T* x, int64_t i, int sub,
-                                          bool valid, T* acc) {
+// acc = (A x)_i for the R columns of row i (NV = 2: column r uses value set r), by one thread.
+template <typename T, int R, int NV>
+__device__ __forceinline__ void row_apply(const SellDev& A, const T* v0, const T* v1, const T* x, int64_t i, T* acc) {
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = T(0);
-    const int L = valid ? row_len(A, i) : 0;
-    const int64_t base = !valid ? 0 : A.rowmajor ? A.ptr[i] : A.ptr[i >> 5] * 32 + (i & 31);
-    const int64_t stride = A.rowmajor ? 1 : 32;
-    for (int k = sub; k < L; k += G) {
-        const int64_t at = base + int64_t(k) * stride;
+    const int L = row_len(A, i);
+    for (int k = 0; k < L; ++k) {
+        const int64_t at = spos(A, i, k);
         const int64_t c = A.col[at];
         T xv[R];
         ldR<T, R>(x + c * R, xv);
@@ -439,90 +431,6 @@ __device__ __forceinline__ void row_apply(const SellDev& A, const T* v0, const T
             acc[1] = fma(v1[at], xv[1], acc[1]);
         }
     }
-    if constexpr (G > 1) {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
-    }
-}
-
-// MODE 0: y = A x;  1: y = b - A x;  2: y = b + A x (b may be y).
-template <typename T, int R, int NV, int MODE, int G>
-__global__ void __launch_bounds__(256) k_spmv(SellDev A, const T* v0, const T* v1, const T* x, const T* b, T* y) {
-    const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    const int64_t i = t / G;
-    const int sub = int(t % G);
-    const bool valid = i < A.n;
-    if (G == 1 && !valid) return;
-    T acc[R];
-    row_apply<T, R, NV, G>(A, v0, v1, x, i, sub, valid, acc);
-    if (!valid || sub != 0) return;
-    if constexpr (MODE != 0) {
-        T bv[R];
-        ldR<T, R>(b + i * R, bv);
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = MODE == 1 ? bv[r] - acc[r] : bv[r] + acc[r];
-    }
-    stR<T, R>(y + i * R, acc);
-}
-
-// Chebyshev smoothing step k (of a polynomial in D^-1 A on [hi / ratio, hi], hi with its margin):
-//   res = b - A x_in  (FIRST: x_in = 0, res = b),
-//   d = c_d d + c_r D^-1 res,  x_out = x_in + d,
-// with the coefficients of the three-term recurrence (Saad, Iterative
-// Methods for Sparse Linear Systems, Alg. 12.1): theta, delta the centre and
-// half-width of the interval, sigma = theta / delta, rho_0 = 1 / sigma,
-// rho_k = 1 / (2 sigma - rho_{k-1}); step 0: c_d = 0, c_r = 1 / theta;
-// step k: c_d = rho_k rho_{k-1}, c_r = 2 rho_k / delta.
-template <typename T, int R, int NV, bool FIRST, int G>
-__global__ void __launch_bounds__(256) k_cheb(SellDev A, const T* v0, const T* v1, const T* dinv, const double* hi,
-                                              double ratio, int k, const T* x_in, T* x_out, T* d, const T* b) {
-    const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    const int64_t i = t / G;
-    const int sub = int(t % G);
-    const bool valid = i < A.n;
-    if ((G == 1 || FIRST) && !valid) return;
-    T res[R];
-    if constexpr (!FIRST) row_apply<T, R, NV, G>(A, v0, v1, x_in, i, sub, valid, res);
-    if (!valid || sub != 0) return;
-    T cd[NV], cr[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const double h = kSmoothMargin * hi[v], lo = h / ratio;
-        const double theta = 0.5 * (h + lo), delta = 0.5 * (h - lo), sigma = theta / delta;
-        double rho_prev = 1.0 / sigma, rho = rho_prev;
-        for (int j = 1; j <= k; ++j) {
-            rho_prev = rho;
-            rho = 1.0 / (2.0 * sigma - rho_prev);
-        }
-        cd[v] = k == 0 ? T(0) : T(rho * rho_prev);
-        cr[v] = k == 0 ? T(1.0 / theta) : T(2.0 * rho / delta);
-    }
-    T bv[R], dv[R], xv[R];
-    ldR<T, R>(b + i * R, bv);
-    if constexpr (FIRST) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            res[r] = bv[r];
-            xv[r] = T(0);
-        }
-    } else {
-        ldR<T, R>(x_in + i * R, xv);
-#pragma unroll
-        for (int r = 0; r < R; ++r) res[r] = bv[r] - res[r];
-    }
-    if (k > 0) ldR<T, R>(d + i * R, dv);
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int v = NV == 2 ? r : 0;
-        const T di = dinv[i * NV + v];
-        const T upd = cr[v] * di * res[r];
-        dv[r] = k > 0 ? fma(cd[v], dv[r], upd) : upd;
-        xv[r] += dv[r];
-    }
-    stR<T, R>(d + i * R, dv);
-    stR<T, R>(x_out + i * R, xv);
 }
 
 // x = A^-1 b on the coarsest level (dense inverse, n <= kAmgCoarsest).
@@ -692,6 +600,7 @@ struct RowMap {
 //   MODE 1: y = R x                          (restriction)
 //   MODE 2: y = P2 e + wd (b + res)          (prolongation, correction and post-smoothing step: with x = wd b + P e,
 //                                             x + wd (b - A x) = wd (b + res) + (P - wd A P) e)
+//   MODE 3: y = b + A x
 // Three kernels a level; the smoothed iterate itself is never stored.  FP64: bound by FP64 issue (A, P and P2 rows
 // hold 7, 4 and 10 entries on a Kuhn mesh, 21 multiply-adds a node and right-hand side).
 template <typename T, int R, int NV, int MODE, int GW, int W>
@@ -711,6 +620,11 @@ __global__ void __launch_bounds__(256) k_level(SellDev A, const T* __restrict__ 
         ldR<T, C>(b + o, bv);
 #pragma unroll
         for (int r = 0; r < C; ++r) acc[r] = bv[r] - acc[r];
+    } else if constexpr (MODE == 3) {
+        T bv[C];
+        ldR<T, C>(b + o, bv);
+#pragma unroll
+        for (int r = 0; r < C; ++r) acc[r] = bv[r] + acc[r];
     } else if constexpr (MODE == 2) {
         T bv[C], rv[C];
         ldR<T, C>(b + o, bv);
@@ -719,6 +633,64 @@ __global__ void __launch_bounds__(256) k_level(SellDev A, const T* __restrict__ 
         for (int r = 0; r < C; ++r) acc[r] = fma(wd[i * NV + (NV == 2 ? m.c0 + r : 0)], bv[r] + rv[r], acc[r]);
     }
     stR<T, C>(y + o, acc);
+}
+
+// Chebyshev smoothing step k (of a polynomial in D^-1 A on [hi / ratio, hi], hi with its margin):
+//   res = b - A x_in  (FIRST: x_in = 0, res = b),
+//   d = c_d d + c_r D^-1 res,  x_out = x_in + d,
+// with the coefficients of the three-term recurrence (Saad, Iterative
+// Methods for Sparse Linear Systems, Alg. 12.1): theta, delta the centre and
+// half-width of the interval, sigma = theta / delta, rho_0 = 1 / sigma,
+// rho_k = 1 / (2 sigma - rho_{k-1}); step 0: c_d = 0, c_r = 1 / theta;
+// step k: c_d = rho_k rho_{k-1}, c_r = 2 rho_k / delta.
+template <typename T, int R, int NV, bool FIRST, int GW>
+__global__ void __launch_bounds__(256) k_cheb(SellDev A, const T* v0, const T* v1, const T* dinv, const double* hi,
+                                              double ratio, int k, const T* x_in, T* x_out, T* d, const T* b) {
+    const RowMap<T, R, GW, 1> m;
+    constexpr int C = RowMap<T, R, GW, 1>::C;
+    __shared__ T cd[NV], cr[NV];  // a block's threads share the divisions
+    if (threadIdx.x < NV) {
+        const double h = kSmoothMargin * hi[threadIdx.x], lo = h / ratio;
+        const double theta = 0.5 * (h + lo), delta = 0.5 * (h - lo), sigma = theta / delta;
+        double rho_prev = 1.0 / sigma, rho = rho_prev;
+        for (int j = 1; j <= k; ++j) {
+            rho_prev = rho;
+            rho = 1.0 / (2.0 * sigma - rho_prev);
+        }
+        cd[threadIdx.x] = k == 0 ? T(0) : T(rho * rho_prev);
+        cr[threadIdx.x] = k == 0 ? T(1.0 / theta) : T(2.0 * rho / delta);
+    }
+    __syncthreads();
+    const int64_t i = blockIdx.x * int64_t(m.RPB) + m.slot;
+    T res[C], bv[C], dv[C], xv[C];
+    if constexpr (!FIRST) {
+        row_part<T, R, NV>(A, v0, v1, x_in, i, m.c0, m.g, GW, i < A.n, res);
+        m.combine(res);
+    }
+    if (i >= A.n || m.g != 0) return;
+    const int64_t o = i * R + m.c0;
+    ldR<T, C>(b + o, bv);
+    if constexpr (FIRST) {
+#pragma unroll
+        for (int r = 0; r < C; ++r) {
+            res[r] = bv[r];
+            xv[r] = T(0);
+        }
+    } else {
+        ldR<T, C>(x_in + o, xv);
+#pragma unroll
+        for (int r = 0; r < C; ++r) res[r] = bv[r] - res[r];
+    }
+    if (k > 0) ldR<T, C>(d + o, dv);
+#pragma unroll
+    for (int r = 0; r < C; ++r) {
+        const int v = NV == 2 ? m.c0 + r : 0;
+        const T upd = cr[v] * dinv[i * NV + v] * res[r];
+        dv[r] = k > 0 ? fma(cd[v], dv[r], upd) : upd;
+        xv[r] += dv[r];
+    }
+    stR<T, C>(d + o, dv);
+    stR<T, C>(x_out + o, xv);
 }
 
 // ---- conjugate gradients (FP64), R right-hand sides; ctl[0] status, ctl[1] RHS still running
@@ -752,7 +724,7 @@ __global__ void __launch_bounds__(256) k_cg_init_x0(SellDev A, const double* v0,
     for (int q = 0; q < 2 * R; ++q) acc[q] = 0.0;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < A.n; i += int64_t(gridDim.x) * blockDim.x) {
         double bv[R], av[R], xv[R];
-        row_apply<double, R, NV, 1>(A, v0, v1, x0, i, 0, true, av);
+        row_apply<double, R, NV>(A, v0, v1, x0, i, av);
         ldR<double, R>(b + i * R, bv);
         ldR<double, R>(x0 + i * R, xv);
 #pragma unroll
@@ -1263,8 +1235,8 @@ int build_hier(qpat_mesh_s* M, AmgHierDev& H) {
 }
 
 template <int NV>
-cudaError_t numeric_levels(const qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V, bool fast,
-                           double ratio, cudaStream_t s) {
+cudaError_t numeric_levels(const qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V, double ratio,
+                           cudaStream_t s) {
     const int L = int(H.lv.size());
     cudaError_t e = cudaMemsetAsync(V.hi, 0, sizeof(double) * 2 * L, s);
     if (e != cudaSuccess) return e;
@@ -1275,14 +1247,14 @@ cudaError_t numeric_levels(const qpat_mesh_s* M, const AmgHierDev& H, const OpSt
     }
     for (int l = 0; l < L; ++l) {
         const LevelDev& d = H.lv[size_t(l)];
-                const double *a0 = V.A[size_t(l)][0], *a1 = V.A[size_t(l)][1];
+        const double *a0 = V.A[size_t(l)][0], *a1 = V.A[size_t(l)][1];
         double* hi = V.hi + 2 * l;
         note_launch(1);
         k_dinv_hi<NV><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, d.diag, a0, a1, V.dinv[size_t(l)], hi);
         if (l + 1 == L) break;
         const auto& Pv = V.P[size_t(l)];
         const auto& Rv = V.R[size_t(l)];
-        if (fast) {
+        if (V.wd[size_t(l)]) {
             note_launch(2);
             k_weights<NV><<<blocks_of(d.A.n * NV), 256, 0, s>>>(d.A.n, V.dinv[size_t(l)], hi, ratio, V.wd[size_t(l)]);
             k_scaled<NV><<<blocks_of(d.A.entries), 256, 0, s>>>(d.A.entries, d.A.col, V.wd[size_t(l)], a0, a1,
@@ -1299,7 +1271,7 @@ cudaError_t numeric_levels(const qpat_mesh_s* M, const AmgHierDev& H, const OpSt
             if ((e = allow_smem(reinterpret_cast<const void*>(&k_ap<NV>), smem)) != cudaSuccess) return e;
             k_ap<NV><<<blocks_of(d.A.n * NV, wpb * rpw), 32 * wpb, smem, s>>>(
                 d.A, d.P, d.diag, d.ap_ptr, d.ap_sptr, d.ap_slot, d.ap_nnz, d.ap_maxlen, a0, a1, Pv[0], Pv[1],
-                fast ? V.wd[size_t(l)] : nullptr, V.AP[size_t(l)], fast ? V.P2[size_t(l)][0] : nullptr);
+                V.wd[size_t(l)], V.AP[size_t(l)], V.P2[size_t(l)][0]);
         }
         const LevelDev& c = H.lv[size_t(l + 1)];
         int wpb = 8;
@@ -1329,18 +1301,39 @@ cudaError_t cast_to_f32(const double* in, float* out, int64_t n, cudaStream_t s)
 
 // Values of the hierarchy for the operator st (allocated once per operator
 // buffer, recomputed when st was prepared again or the cycle's form changed).
-// fast: the degree-1 cycle's S, wd and P2 too.  After a failure V is incomplete
-// and must be dropped.
+// fast: S, wd and P2 of the fine level too (degree 1; the coarser levels always
+// have theirs).  After a failure V is incomplete and must be dropped.
 int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V, bool fast, double ratio, bool need32,
             cudaStream_t s) {
     const int L = int(H.lv.size());
     const int NV = st.nv;
     cudaError_t e = cudaSuccess;
     auto set = [&](auto& list) { list.assign(size_t(L), {nullptr, nullptr}); };
+    // room for S, P2 and wd of a level with a transfer, and for their FP32 copies
+    auto smoothing = [&](int l) {
+        if (l + 1 == L) return;
+        const LevelDev& d = H.lv[size_t(l)];
+        for (int v = 0; v < NV; ++v) V.S[size_t(l)][size_t(v)] = V.mem.get<double>(size_t(d.A.entries), e);
+        double* p2 = V.mem.get<double>(size_t(d.ap_nnz) * NV, e);
+        V.P2[size_t(l)] = {p2, NV == 2 && p2 ? p2 + d.ap_nnz : nullptr};
+        V.wd[size_t(l)] = V.mem.get<double>(size_t(d.A.n) * NV, e);
+    };
+    auto smoothing32 = [&](int l) {
+        if (l + 1 == L) return;
+        const LevelDev& d = H.lv[size_t(l)];
+        for (int v = 0; v < NV; ++v) {
+            V.S32[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.A.entries), e);
+            V.P232[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.ap_nnz), e);
+        }
+        V.wd32[size_t(l)] = V.mem.get<float>(size_t(d.A.n) * NV, e);
+    };
     if (V.A.empty()) {
         set(V.A);
         set(V.P);
         set(V.R);
+        set(V.S);
+        set(V.P2);
+        V.wd.assign(size_t(L), nullptr);
         V.AP.assign(size_t(L), nullptr);
         V.dinv.assign(size_t(L), nullptr);
         for (int l = 0; l < L; ++l) {
@@ -1355,6 +1348,7 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
             }
             if (l + 1 < L) V.AP[size_t(l)] = V.mem.get<double>(size_t(d.ap_nnz) * NV, e);
             V.dinv[size_t(l)] = V.mem.get<double>(size_t(d.A.n) * NV, e);
+            if (l > 0) smoothing(l);
         }
         V.hi = V.mem.get<double>(size_t(2 * L), e);
         const int64_t nco = H.lv.back().A.n;
@@ -1371,17 +1365,8 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         if (e != cudaSuccess) return cuda_fail(e, "multigrid memset");
     }
     if (NV == 2) V.A[0] = {st.v64[0], st.v64[1]};
-    if (fast && V.S.empty()) {
-        set(V.S);
-        set(V.P2);
-        V.wd.assign(size_t(L), nullptr);
-        for (int l = 0; l + 1 < L; ++l) {
-            const LevelDev& d = H.lv[size_t(l)];
-            for (int v = 0; v < NV; ++v) V.S[size_t(l)][size_t(v)] = V.mem.get<double>(size_t(d.A.entries), e);
-            double* p2 = V.mem.get<double>(size_t(d.ap_nnz) * NV, e);
-            V.P2[size_t(l)] = {p2, NV == 2 ? p2 + d.ap_nnz : nullptr};
-            V.wd[size_t(l)] = V.mem.get<double>(size_t(d.A.n) * NV, e);
-        }
+    if (fast && L > 1 && !V.wd[0]) {
+        smoothing(0);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
         V.valid = false;
     }
@@ -1389,6 +1374,9 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         set(V.A32);
         set(V.P32);
         set(V.R32);
+        set(V.S32);
+        set(V.P232);
+        V.wd32.assign(size_t(L), nullptr);
         V.dinv32.assign(size_t(L), nullptr);
         for (int l = 0; l < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
@@ -1400,6 +1388,7 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
                 }
             }
             V.dinv32[size_t(l)] = V.mem.get<float>(size_t(d.A.n) * NV, e);
+            if (l > 0) smoothing32(l);
         }
         const int64_t nco = H.lv.back().A.n;
         V.inv32 = V.mem.get<float>(size_t(NV * nco * nco), e);
@@ -1407,25 +1396,14 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
         V.has32 = true;
         V.valid = false;
     }
-    if (fast && V.has32 && V.S32.empty()) {
-        set(V.S32);
-        set(V.P232);
-        V.wd32.assign(size_t(L), nullptr);
-        for (int l = 0; l + 1 < L; ++l) {
-            const LevelDev& d = H.lv[size_t(l)];
-            for (int v = 0; v < NV; ++v) {
-                V.S32[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.A.entries), e);
-                V.P232[size_t(l)][size_t(v)] = V.mem.get<float>(size_t(d.ap_nnz), e);
-            }
-            V.wd32[size_t(l)] = V.mem.get<float>(size_t(d.A.n) * NV, e);
-        }
+    if (fast && L > 1 && V.has32 && !V.wd32[0]) {
+        smoothing32(0);
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
         V.valid = false;
     }
-    if (V.valid && V.stamp == st.stamp && (!fast || V.ratio == ratio)) return QPAT_OK;
-    const bool scaled = !V.S.empty();  // once allocated kept up to date
-    if (fast || V.ratio == 0.0) V.ratio = ratio;
-    e = NV == 1 ? numeric_levels<1>(M, H, st, V, scaled, V.ratio, s) : numeric_levels<2>(M, H, st, V, scaled, V.ratio, s);
+    if (V.valid && V.stamp == st.stamp && V.ratio == ratio) return QPAT_OK;
+    V.ratio = ratio;
+    e = NV == 1 ? numeric_levels<1>(M, H, st, V, ratio, s) : numeric_levels<2>(M, H, st, V, ratio, s);
     if (e != cudaSuccess) return cuda_fail(e, "multigrid set-up");
     if (V.has32) {
         auto cast = [&](const double* in, float* out, int64_t n) {
@@ -1438,13 +1416,11 @@ int numeric(qpat_mesh_s* M, const AmgHierDev& H, const OpState& st, AmgValues& V
                 cast(V.A[i][j], V.A32[i][j], d.A.entries);
                 cast(V.P[i][j], V.P32[i][j], d.P.entries);
                 cast(V.R[i][j], V.R32[i][j], d.R.entries);
-                if (!V.S32.empty()) {
-                    cast(V.S[i][j], V.S32[i][j], d.A.entries);
-                    cast(V.P2[i][j], V.P232[i][j], d.ap_nnz);
-                }
+                cast(V.S[i][j], V.S32[i][j], d.A.entries);
+                cast(V.P2[i][j], V.P232[i][j], d.ap_nnz);
             }
             cast(V.dinv[size_t(l)], V.dinv32[size_t(l)], d.A.n * NV);
-            if (!V.wd32.empty()) cast(V.wd[size_t(l)], V.wd32[size_t(l)], d.A.n * NV);
+            cast(V.wd[size_t(l)], V.wd32[size_t(l)], d.A.n * NV);
         }
         const int64_t nco = H.lv.back().A.n;
         cast(V.inv, V.inv32, NV * nco * nco);
@@ -1495,99 +1471,6 @@ struct FineTimer {
     }
     ~FineTimer() {
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
-    }
-};
-
-// One V-cycle x = B b on level l and below (pre-smoothing from x = 0,
-// residual, restriction, the coarser cycle, prolongation, post-smoothing
-// with the same polynomial: B is symmetric).
-template <typename T, int R, int NV>
-struct VCycle {
-    const AmgHierDev& H;
-    const AmgValues& V;
-    AmgVecs& W;
-    int deg;
-    double ratio;
-    cudaStream_t s;
-    FineTimer* timer = nullptr;
-
-    static constexpr bool F64 = std::is_same<T, double>::value;
-    const T* av(int l, int v) const {
-        if constexpr (F64)
-            return V.A[size_t(l)][size_t(v)];
-        else
-            return V.A32[size_t(l)][size_t(v)];
-    }
-    const T* pv(int l, int v) const {
-        if constexpr (F64) return V.P[size_t(l)][size_t(v)];
-        else return V.P32[size_t(l)][size_t(v)];
-    }
-    const T* rv(int l, int v) const {
-        if constexpr (F64) return V.R[size_t(l)][size_t(v)];
-        else return V.R32[size_t(l)][size_t(v)];
-    }
-    const T* dinv(int l) const {
-        if constexpr (F64) return V.dinv[size_t(l)];
-        else return V.dinv32[size_t(l)];
-    }
-    const T* inv() const {
-        if constexpr (F64) return V.inv;
-        else return V.inv32;
-    }
-
-    template <int MODE>
-    void spmv(const SellDev& A, const T* a0, const T* a1, const T* x, const T* b, T* y) {
-        note_launch(1);
-        if (A.rowmajor)
-            k_spmv<T, R, NV, MODE, 8><<<blocks_of(A.n * 8), 256, 0, s>>>(A, a0, a1, x, b, y);
-        else
-            k_spmv<T, R, NV, MODE, 1><<<blocks_of(A.n), 256, 0, s>>>(A, a0, a1, x, b, y);
-    }
-    void cheb(const SellDev& A, const T* a0, const T* a1, const T* di, const double* hi, int k, const T* x_in,
-              T* x_out, T* d, const T* b) {
-        note_launch(1);
-        if (A.rowmajor)
-            k_cheb<T, R, NV, false, 8><<<blocks_of(A.n * 8), 256, 0, s>>>(A, a0, a1, di, hi, ratio, k, x_in, x_out, d,
-                                                                          b);
-        else
-            k_cheb<T, R, NV, false, 1><<<blocks_of(A.n), 256, 0, s>>>(A, a0, a1, di, hi, ratio, k, x_in, x_out, d, b);
-    }
-
-    const T* run(int l, const T* b) {
-        const LevelDev& d = H.lv[size_t(l)];
-        const int L = int(H.lv.size());
-        T* x = static_cast<T*>(W.xa[size_t(l)]);
-        T* y = static_cast<T*>(W.xb[size_t(l)]);
-        T* dd = static_cast<T*>(W.d[size_t(l)]);
-        if (l == L - 1) {
-            note_launch(1);
-            k_dense_apply<T, R, NV><<<1, 256, 0, s>>>(int(d.A.n), inv(), b, x);
-            return x;
-        }
-        const double* hi = V.hi + 2 * l;
-        const T *a0 = av(l, 0), *a1 = av(l, 1);
-        note_launch(1);
-        k_cheb<T, R, NV, true, 1><<<blocks_of(d.A.n), 256, 0, s>>>(d.A, a0, a1, dinv(l), hi, ratio, 0, nullptr, x, dd,
-                                                                  b);
-        for (int k = 1; k < deg; ++k) {
-            if (l == 0 && timer) timer->before();
-            cheb(d.A, a0, a1, dinv(l), hi, k, x, y, dd, b);
-            if (l == 0 && timer) timer->after();
-            std::swap(x, y);
-        }
-        T* res = static_cast<T*>(W.r[size_t(l)]);
-        T* bc = static_cast<T*>(W.b[size_t(l + 1)]);
-        spmv<1>(d.A, a0, a1, x, b, res);
-        spmv<0>(d.R, rv(l, 0), rv(l, 1), res, nullptr, bc);
-        const T* xc = run(l + 1, bc);
-        spmv<2>(d.P, pv(l, 0), pv(l, 1), xc, x, x);
-        for (int k = 0; k < deg; ++k) {
-            if (l == 0 && timer) timer->before();
-            cheb(d.A, a0, a1, dinv(l), hi, k, x, y, dd, b);
-            if (l == 0 && timer) timer->after();
-            std::swap(x, y);
-        }
-        return x;
     }
 };
 
@@ -1654,10 +1537,11 @@ struct FastCycle {
             go(integral_constant<int, 1>(), integral_constant<int, 1>());
     }
 
-    // leaves the fine level's residual in W.r[0] and the coarse correction in the returned vector
-    const T* run(const T* b0) {
+    // From the fine level (from = 0, right-hand side b0): leaves its residual in W.r[0] and returns the correction on
+    // level 1.  From level 1 (right-hand side in W.b[1]): returns the cycle's result there.
+    const T* run(const T* b0, int from) {
         const int L = int(H.lv.size());
-        for (int l = 0; l + 1 < L; ++l) {
+        for (int l = from; l + 1 < L; ++l) {
             const LevelDev& d = H.lv[size_t(l)];
             const T* b = l == 0 ? b0 : static_cast<const T*>(W.b[size_t(l)]);
             T* res = static_cast<T*>(W.r[size_t(l)]);
@@ -1680,6 +1564,92 @@ struct FastCycle {
                       static_cast<const T*>(W.r[size_t(l)]), y);
             x = y;
         }
+        return x;
+    }
+};
+
+// The cycle with a smoothing polynomial of higher degree on the fine level
+// (pre-smoothing from x = 0, residual, restriction, the degree-1 cycle of the
+// coarser levels, prolongation, post-smoothing with the same polynomial: B is
+// symmetric).  The coarser levels are bound by the number of their kernels: with
+// the polynomial there too (7 kernels a level at degree 2, 3 now), K with 4
+// right-hand sides on the 33 x 33 x 41 cylinder took 11.4 ms at degree 2, 7.0 now; at
+// degree 8 on 40^3 13.5 and 6.2; M_delta on 64^3 at degree 2 16.0 and 8.6.
+template <typename T, int R, int NV>
+struct PolyCycle {
+    const AmgHierDev& H;
+    const AmgValues& V;
+    AmgVecs& W;
+    int deg;
+    double ratio;
+    cudaStream_t s;
+    FineTimer* timer = nullptr;
+
+    static constexpr bool F64 = std::is_same<T, double>::value;
+    const T* av(int l, int v) const {
+        if constexpr (F64)
+            return V.A[size_t(l)][size_t(v)];
+        else
+            return V.A32[size_t(l)][size_t(v)];
+    }
+    const T* pv(int l, int v) const {
+        if constexpr (F64) return V.P[size_t(l)][size_t(v)];
+        else return V.P32[size_t(l)][size_t(v)];
+    }
+    const T* rv(int l, int v) const {
+        if constexpr (F64) return V.R[size_t(l)][size_t(v)];
+        else return V.R32[size_t(l)][size_t(v)];
+    }
+    const T* dinv(int l) const {
+        if constexpr (F64) return V.dinv[size_t(l)];
+        else return V.dinv32[size_t(l)];
+    }
+    const T* inv() const {
+        if constexpr (F64) return V.inv;
+        else return V.inv32;
+    }
+
+    const T* run(const T* b) {
+        const LevelDev& d = H.lv[0];
+        FastCycle<T, R, NV> coarse{H, V, W, s};
+        T* x = static_cast<T*>(W.xa[0]);
+        T* y = static_cast<T*>(W.xb[0]);
+        T* dd = static_cast<T*>(W.d[0]);
+        if (H.lv.size() == 1) {
+            note_launch(1);
+            k_dense_apply<T, R, NV><<<1, 256, 0, s>>>(int(d.A.n), inv(), b, x);
+            return x;
+        }
+        const T *a0 = av(0, 0), *a1 = av(0, 1);
+        note_launch(1);
+        k_cheb<T, R, NV, true, 1><<<blocks_of(d.A.n, RowMap<T, R, 1, 1>::RPB), 256, 0, s>>>(d.A, a0, a1, dinv(0), V.hi, ratio,
+                                                                                       0, nullptr, x, dd, b);
+        auto step = [&](int k) {
+            if (timer) timer->before();
+            note_launch(1);
+            auto go = [&](auto gw) {
+                constexpr int GW = decltype(gw)::value;
+                k_cheb<T, R, NV, false, GW><<<blocks_of(d.A.n, RowMap<T, R, GW, 1>::RPB), 256, 0, s>>>(
+                    d.A, a0, a1, dinv(0), V.hi, ratio, k, x, y, dd, b);
+            };
+            // a row's entries are shared by several groups only where the GPU would not be filled otherwise, in FP64 by two
+            // as soon as eight would fill it (see FastCycle::launch)
+            constexpr int GM = FastCycle<T, R, NV>::GM;
+            const int64_t fill = 152 * 1024, threads = d.A.n * coarse.LPR;
+            if (threads * (F64 ? GM : 1) < fill) go(std::integral_constant<int, GM>());
+            else if (threads < fill) go(std::integral_constant<int, 2>());
+            else go(std::integral_constant<int, 1>());
+            if (timer) timer->after();
+            std::swap(x, y);
+        };
+        for (int k = 1; k < deg; ++k) step(k);
+        T* res = static_cast<T*>(W.r[0]);
+        coarse.template launch<0>(d.A, a0, a1, x, nullptr, b, nullptr, res);
+        coarse.template launch<1>(d.R, rv(0, 0), rv(0, 1), res, nullptr, nullptr, nullptr, static_cast<T*>(W.b[1]));
+        const T* xc = coarse.run(nullptr, 1);
+        coarse.template launch<3>(d.P, pv(0, 0), pv(0, 1), xc, nullptr, x, nullptr, y);
+        std::swap(x, y);
+        for (int k = 0; k < deg; ++k) step(k);
         return x;
     }
 };
@@ -1728,14 +1698,14 @@ struct CgSolve {
         note_launch(1);
         if (fast()) {
             FastCycle<T, R, NV> c{H, V, W, t, timer};
-            const T* e = c.run(b);
+            const T* e = c.run(b, 0);
             k_top<T, R, NV, 1><<<full_grid(k_top<T, R, NV, 1>, G), 256, 0, t>>>(c.p2(0), c.val(V.P2, V.P232, 0, 0), c.val(V.P2, V.P232, 0, 1), e, c.wd(0), b,
                                                   static_cast<const T*>(W.r[0]), C.r, C.q, C.z, C.part, C.count, C.rz,
                                                   C.alpha, C.beta, C.ctl);
             return;
         }
-        VCycle<T, R, NV> c{H, V, W, std::max(1, so.mg_degree), so.mg_ratio, t, timer};
-        const T* x = c.run(0, b);
+        PolyCycle<T, R, NV> c{H, V, W, std::max(1, so.mg_degree), so.mg_ratio, t, timer};
+        const T* x = c.run(b);
         const double* z;
         if constexpr (F32) {
             note_launch(1);
