@@ -184,8 +184,24 @@ __global__ void __launch_bounds__(kT) k_rhs_jv(MeshDev m, ElemDev el, const doub
 
 // ---------------------------------------------------------------- prior
 
-// Per tet: 4 x the lagged weight of each block.
-__global__ void __launch_bounds__(kT) k_tet_prior(ElemDev el, const double* __restrict__ u1,
+// |grad u|^2 on a tet from coordinates: infinite only where it is beyond the range, never the difference of infinities.
+__device__ __noinline__ double tet_grad2(const double* xyz, const double* u, int4 v) {
+    const int id[4] = {v.x, v.y, v.z, v.w};
+    double p[4][3], c[4][3], x[4], g[3], ad;
+    for (int a = 0; a < 4; ++a) {
+        for (int k = 0; k < 3; ++k) p[a][k] = xyz[3 * int64_t(id[a]) + k];
+        x[a] = u[id[a]];
+    }
+    tet_cofactors(p, c, ad);
+    grad_vec(c, x, g);
+    return (g[0] * g[0] + g[1] * g[1] + g[2] * g[2]) / (ad * ad);
+}
+
+// Per tet: 4 x the lagged weight of each block.  Two weights by one division
+// where their products stay well inside the range; any other field, T or size
+// of tet (gradients of 1e70 and more against T) goes by the general formulas.
+__global__ void __launch_bounds__(kT) k_tet_prior(ElemDev el, const double* __restrict__ xyz,
+                                                  const double* __restrict__ u1,
                                                   const double* __restrict__ u2, double inv_T2, int kind, double q,
                                                   double scale1, double2* __restrict__ tq) {
     const int64_t t = thread_id();
@@ -207,13 +223,17 @@ __global__ void __launch_bounds__(kT) k_tet_prior(ElemDev el, const double* __re
             const double d = x[edge_a(c)] - x[edge_b(c)];
             a = fma(s[c] * d, d, a);
         }
-        e[r] = fmax(a * (-1.0 / 30.0), 0.0);
+        e[r] = a * (-1.0 / 30.0);
+        if (e[r] < 0.0) e[r] = 0.0;
     }
     double w[2];
-    if (kind == 0) {
-        // 1 / (1 + |grad u|^2 / T^2) = vm / (vm + e / T^2) of both blocks by one division
-        const double a = fma(e[0], inv_T2, vm), b = fma(e[1], inv_T2, vm);
-        const double f = 4.0 * vm / (a * b);
+    // 1 / (1 + |grad u|^2 / T^2) = vm / (vm + e / T^2)
+    const double a = fma(e[0], inv_T2, vm), b = fma(e[1], inv_T2, vm), ab = a * b;
+    if (!(ab > 1e-280 && ab < 1e280)) {  // NaN too
+        w[0] = 4.0 * prior_weight<double>(kind, tet_grad2(xyz, u1, v), inv_T2, q);
+        w[1] = 4.0 * scale1 * prior_weight<double>(kind, tet_grad2(xyz, u2, v), inv_T2, q);
+    } else if (kind == 0) {
+        const double f = 4.0 * vm / ab;
         w[0] = f * b;
         w[1] = scale1 * (f * a);
     } else {
@@ -399,7 +419,7 @@ cudaError_t launch_assemble_prior(const MeshDev& m, const ElemDev& el, const Ele
         if (e != cudaSuccess) return e;
     }
     note_launch(3);
-    k_tet_prior<<<blocks(el.E), kT, 0, s>>>(el, u1, u2, inv_T2, kind, q, scale1, w.tet);
+    k_tet_prior<<<blocks(el.E), kT, 0, s>>>(el, m.xyz64, u1, u2, inv_T2, kind, q, scale1, w.tet);
     k_edge_prior<<<blocks(el.NE), kT, 0, s>>>(el, w.tet, w.edge);
     k_row_prior<<<blocks(m.N), kT, 0, s>>>(m, el, w.edge, delta, val0, val1, inv64, inv32, gbound);
     return cudaGetLastError();
