@@ -446,7 +446,11 @@ int qpat_jvp_vjp_pair(qpat_mesh_t mesh, const qpat_params* prm,
  * train: one Adam step on the mean-squared error of B samples (targets t,
  * B x n^3 float, e.g. forward solutions); *loss (host, may be NULL) gets the
  * mean loss before the step.  Device pointers, asynchronous on stream except
- * when loss is requested.  Parameters: per convolution the fp32 weights
+ * when loss is requested; the first call with more samples than any before
+ * waits for the stream and allocates their activations (8 GB at most, and one
+ * sample's from qpat_unet_create on).  predict, and train without a loss, may be
+ * captured into a CUDA graph from the first call on (one sample at a time, or as
+ * many as an earlier call made room for).  Parameters: per convolution the fp32 weights
  * [27][c_out][c_in] then the bias [c_out]. */
 typedef struct qpat_unet_s* qpat_unet_t;
 int qpat_unet_create(int n, uint64_t seed, qpat_unet_t* out);

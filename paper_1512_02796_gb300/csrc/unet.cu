@@ -93,7 +93,19 @@ int g1(int64_t n) { return int(std::max<int64_t>(1, std::min<int64_t>((n + 255) 
 
 }  // namespace
 
-struct qpat_unet_s {
+// Activations of a batch of samples, and what training needs beside them.
+struct UnetActs {
+    bf16 *xin, *a0, *s0, *p0, *a1, *s1, *p1, *a2, *s2, *p2, *a3, *bt, *a4, *d2, *a5, *d1, *a6, *d0;
+};
+struct UnetTrainActs {
+    bf16 *cat2, *cat1, *cat0;
+    bf16 *g_y, *g_d0, *g_a6, *g_cat0, *g_d1, *g_s0, *g_a5, *g_cat1, *g_d2, *g_s1, *g_a4, *g_cat2, *g_bt, *g_s2, *g_a3,
+        *g_p2, *g_a2, *g_p1, *g_a1, *g_p0, *g_a0;
+    float* y;        // predictions of a training batch
+    float* partial;  // wgrad scratch
+};
+
+struct qpat_unet_s : UnetActs, UnetTrainActs {
     int n = 0;
     int device = 0;
     int step = 0;
@@ -104,17 +116,13 @@ struct qpat_unet_s {
     // other, and (train_cap samples) the concatenations and gradients that
     // training needs; see reserve
     int cap = 0, train_cap = 0;
+    int most = 0, train_most = 0;  // samples beyond which an allocation failed (0: none has)
     std::vector<void*> acts, train_acts;
-    bf16 *xin, *a0, *s0, *p0, *a1, *s1, *p1, *a2, *s2, *p2, *a3, *bt, *a4, *d2, *a5, *d1, *a6, *d0;
-    bf16 *cat2, *cat1, *cat0;
-    bf16 *g_y, *g_d0, *g_a6, *g_cat0, *g_d1, *g_s0, *g_a5, *g_cat1, *g_d2, *g_s1, *g_a4, *g_cat2, *g_bt, *g_s2, *g_a3,
-        *g_p2, *g_a2, *g_p1, *g_a1, *g_p0, *g_a0;
-    float* y = nullptr;        // predictions of a training batch
-    float* partial = nullptr;  // wgrad scratch
+    // Buffers that a captured call works on are kept for the graph's replays
+    // when later calls outgrow them.
+    bool acts_captured = false, train_captured = false;
+    std::vector<void*> kept;
     float log_floor = 0.f;  // > 0: the network learns log(max(phi, log_floor)) (qpat_unet_set_log_output)
-    // mma.sync engine only: concatenation, bf16 and fp32 output of one sample
-    bf16 *mcat = nullptr, *mout = nullptr;
-    float* mout32 = nullptr;
     float* grad = nullptr;     // every aw and ab in the order of the parameters
     float* loss = nullptr;
     float* hloss = nullptr;
@@ -152,99 +160,124 @@ int ualloc(qpat_unet_s* U, T** p, size_t count) {
 constexpr size_t kActBytes = size_t(8) << 30;
 constexpr int kMaxSamples = 64;
 
-// Room for min(B, what kActBytes holds) samples, also for training; kept for
-// later calls, grown (after the stream has finished with it) on demand.
-int reserve(qpat_unet_s* U, int B, bool train, cudaStream_t s) {
-    const int64_t v0 = int64_t(U->n) * U->n * U->n, v1 = v0 / 8, v2 = v1 / 8, v3 = v2 / 8;
-    const size_t fwd = 2 * size_t(v0 * 80 + v1 * 176 + v2 * 352 + v3 * 320);
-    const size_t bwd = 2 * size_t(v0 * 176 + v1 * 352 + v2 * 704 + v3 * 320) + 4 * size_t(v0);
-    auto fit = [&](size_t bytes) { return int(std::max<size_t>(1, std::min<size_t>(size_t(std::min(B, kMaxSamples)), kActBytes / bytes))); };
-    auto release = [&](std::vector<void*>& list, int& cap) {
-        for (void* p : list) cudaFree(p);
-        list.clear();
-        cap = 0;
-    };
-    int want = fit(train ? fwd + bwd : fwd), rc = QPAT_OK;
-    if (want > U->cap) {
-        UCK(cudaStreamSynchronize(s));
-        for (;; want = 1) {  // not enough memory for several: one
-            release(U->acts, U->cap);
-            rc = QPAT_OK;
-            auto A = [&](bf16** p, int64_t nv, int ch) { if (!rc) rc = alloc_in(U->acts, p, size_t(nv) * ch * want); };
-            A(&U->xin, v0, 16); A(&U->a0, v0, 16); A(&U->s0, v0, 16); A(&U->p0, v1, 16); A(&U->a1, v1, 32);
-            A(&U->s1, v1, 32); A(&U->p1, v2, 32); A(&U->a2, v2, 64); A(&U->s2, v2, 64); A(&U->p2, v3, 64);
-            A(&U->a3, v3, 128); A(&U->bt, v3, 128); A(&U->a4, v2, 64); A(&U->d2, v2, 64); A(&U->a5, v1, 32);
-            A(&U->d1, v1, 32); A(&U->a6, v0, 16); A(&U->d0, v0, 16);
-            if (!rc || want == 1) break;
+// Room for up to `want` samples in place of what `list` holds (the pointers in
+// P, which `each` allocates): halved where memory is short, and the room that
+// there was is given up only for more.
+template <typename P, typename F>
+int grow(qpat_unet_s* U, std::vector<void*>& list, int& cap, int& most, bool& captured, int want, const F& each) {
+    const P old = *U;
+    const std::string message = g_err;
+    for (; want > cap; want /= 2) {
+        std::vector<void*> fresh;
+        int rc = QPAT_OK;
+        each([&](auto** p, size_t count) {
+            if (!rc) rc = alloc_in(fresh, p, count * size_t(want));
+        }, want);
+        if (rc == QPAT_OK) {
+            if (captured)
+                U->kept.insert(U->kept.end(), list.begin(), list.end());
+            else
+                for (void* p : list) cudaFree(p);
+            list.swap(fresh);
+            captured = false;
+            cap = want;
+            break;
         }
-        if (rc) {
-            release(U->acts, U->cap);
-            return rc;
-        }
-        U->cap = want;
+        for (void* p : fresh) cudaFree(p);
+        static_cast<P&>(*U) = old;
+        most = std::max(cap, want / 2);
     }
-    if (train && std::min(want, U->cap) > U->train_cap) {
-        UCK(cudaStreamSynchronize(s));
-        for (want = std::min(want, U->cap);; want = 1) {
-            release(U->train_acts, U->train_cap);
-            rc = QPAT_OK;
-            auto A = [&](bf16** p, int64_t nv, int ch) { if (!rc) rc = alloc_in(U->train_acts, p, size_t(nv) * ch * want); };
-            A(&U->cat2, v2, 192); A(&U->cat1, v1, 96); A(&U->cat0, v0, 48);
-            A(&U->g_y, v0, 16); A(&U->g_d0, v0, 16); A(&U->g_a6, v0, 16); A(&U->g_cat0, v0, 48); A(&U->g_d1, v1, 32);
-            A(&U->g_s0, v0, 16); A(&U->g_a5, v1, 32); A(&U->g_cat1, v1, 96); A(&U->g_d2, v2, 64); A(&U->g_s1, v1, 32);
-            A(&U->g_a4, v2, 64); A(&U->g_cat2, v2, 192); A(&U->g_bt, v3, 128); A(&U->g_s2, v2, 64); A(&U->g_a3, v3, 128);
-            A(&U->g_p2, v3, 64); A(&U->g_a2, v2, 64); A(&U->g_p1, v2, 32); A(&U->g_a1, v1, 32); A(&U->g_p0, v1, 16);
-            A(&U->g_a0, v0, 16);
-            if (!rc) rc = alloc_in(U->train_acts, &U->y, size_t(v0) * want);
-            size_t scratch = 0;
-            for (int b = 1; b <= want; ++b)  // the chunking of a smaller batch may need more
-                for (const Conv& c : U->conv) scratch = std::max(scratch, unet::wgrad_scratch(U->lv[c.lvl], c.cin, c.cout, b));
-            if (!rc) rc = alloc_in(U->train_acts, &U->partial, scratch);
-            if (!rc || want == 1) break;
-        }
-        if (rc) {
-            release(U->train_acts, U->train_cap);
-            return rc;
-        }
-        U->train_cap = want;
-    }
+    if (cap < 1) return QPAT_ECUDA;  // not even one sample's: the allocation's message stands
+    g_err = message;
     return QPAT_OK;
+}
+
+// Room for min(B, what kActBytes holds) samples, also for training; kept for
+// later calls and grown on demand (the device finishes its work before memory
+// is released).  Where memory is short, for as many as it holds, and no more is
+// tried again.  A call that is being captured into a graph can neither allocate
+// nor wait: it takes the room that there is (one sample's from the start) in
+// groups.
+int reserve(qpat_unet_s* U, int B, bool train, cudaStream_t s) {
+    const size_t v0 = size_t(U->n) * U->n * U->n, v1 = v0 / 8, v2 = v1 / 8, v3 = v2 / 8;
+    const size_t fwd = 2 * (v0 * 80 + v1 * 176 + v2 * 352 + v3 * 320);
+    const size_t bwd = 2 * (v0 * 176 + v1 * 352 + v2 * 704 + v3 * 320) + 4 * v0;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t asked = cudaStreamIsCapturing(s, &capture);
+    if (asked != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        (void)cudaGetLastError();  // another stream's capture forbids the question on the default one
+        if (U->cap < 1 || U->train_cap < 1) return fail(QPAT_ECUDA, "qpat_unet: no activations, and none can be had in a capture");
+        U->acts_captured = U->train_captured = true;  // the mma.sync engine's scratch lies in the training buffers
+        return QPAT_OK;
+    }
+    auto fit = [&](size_t bytes, int most) {
+        const int want = int(std::max<size_t>(1, std::min<size_t>(size_t(std::min(B, kMaxSamples)), kActBytes / bytes)));
+        return most ? std::min(want, most) : want;
+    };
+    const int want = fit(train ? fwd + bwd : fwd, U->most);
+    const int want_train = std::min(fit(fwd + bwd, U->train_most), std::max(want, U->cap));
+    const bool more = want > U->cap, more_train = train && want_train > U->train_cap;
+    if (!more && !more_train) return QPAT_OK;
+    UCK(cudaStreamSynchronize(s));
+    int rc = QPAT_OK;
+    if (more)
+        rc = grow<UnetActs>(U, U->acts, U->cap, U->most, U->acts_captured, want, [&](auto A, int) {
+            A(&U->xin, v0 * 16); A(&U->a0, v0 * 16); A(&U->s0, v0 * 16); A(&U->p0, v1 * 16); A(&U->a1, v1 * 32);
+            A(&U->s1, v1 * 32); A(&U->p1, v2 * 32); A(&U->a2, v2 * 64); A(&U->s2, v2 * 64); A(&U->p2, v3 * 64);
+            A(&U->a3, v3 * 128); A(&U->bt, v3 * 128); A(&U->a4, v2 * 64); A(&U->d2, v2 * 64); A(&U->a5, v1 * 32);
+            A(&U->d1, v1 * 32); A(&U->a6, v0 * 16); A(&U->d0, v0 * 16);
+        });
+    if (!rc && more_train)
+        rc = grow<UnetTrainActs>(U, U->train_acts, U->train_cap, U->train_most, U->train_captured, want_train,
+                                 [&](auto A, int samples) {
+            A(&U->cat2, v2 * 192); A(&U->cat1, v1 * 96); A(&U->cat0, v0 * 48);
+            A(&U->g_y, v0 * 16); A(&U->g_d0, v0 * 16); A(&U->g_a6, v0 * 16); A(&U->g_cat0, v0 * 48); A(&U->g_d1, v1 * 32);
+            A(&U->g_s0, v0 * 16); A(&U->g_a5, v1 * 32); A(&U->g_cat1, v1 * 96); A(&U->g_d2, v2 * 64); A(&U->g_s1, v1 * 32);
+            A(&U->g_a4, v2 * 64); A(&U->g_cat2, v2 * 192); A(&U->g_bt, v3 * 128); A(&U->g_s2, v2 * 64); A(&U->g_a3, v3 * 128);
+            A(&U->g_p2, v3 * 64); A(&U->g_a2, v2 * 64); A(&U->g_p1, v2 * 32); A(&U->g_a1, v1 * 32); A(&U->g_p0, v1 * 16);
+            A(&U->g_a0, v0 * 16);
+            A(&U->y, v0);
+            size_t scratch = 0;
+            for (int b = 1; b <= samples; ++b)  // the chunking of a smaller batch may need more
+                for (const Conv& c : U->conv) scratch = std::max(scratch, unet::wgrad_scratch(U->lv[c.lvl], c.cin, c.cout, b));
+            A(&U->partial, (scratch + samples - 1) / samples);
+        });
+    return rc;
 }
 
 // One convolution of B samples.  On the tcgen05 engine one launch, which reads
 // a concatenation from its two parts; the mma.sync engine goes sample by
 // sample through materialised tensors.
-int conv_fwd(qpat_unet_s* U, const Conv& c, const bf16* w, int Cout, const float* bias, int relu,
+int conv_fwd(qpat_unet_s* U, const bf16* w, int Cout, const float* bias, int relu,
              const unet::ConvInput& in, const unet::ConvOutput& out, int n, int B, cudaStream_t s) {
     const int Cin = in.Clo + in.Cskip;
     if (unet::conv_engine() == 0 && unet::conv3d_fwd_tc_supported(Cin, Cout)) {
         UCK(unet::conv3d_fwd_tc(in, w, bias, Cout, relu, out, n, B, s));
         return QPAT_OK;
     }
-    const int64_t v0 = int64_t(U->n) * U->n * U->n, nv = int64_t(n) * n * n;
-    int rc = QPAT_OK;
-    if (!U->mcat && (rc = ualloc(U, &U->mcat, size_t(v0) * 48))) return rc;
-    if (!U->mout && (rc = ualloc(U, &U->mout, size_t(v0) * 16))) return rc;
-    if (!U->mout32 && (rc = ualloc(U, &U->mout32, size_t(v0) * 16))) return rc;
+    // one sample's concatenation and last layer, in training buffers that are free here: training writes its
+    // concatenations itself, and the gradients of the output and of cat0 after the forward pass
+    bf16 *const cat = U->cat0, *const last = U->g_y;
+    float* const last32 = reinterpret_cast<float*>(U->g_cat0);
+    const int64_t nv = int64_t(n) * n * n;
     for (int b = 0; b < B; ++b) {
         const bf16* x = in.skip + b * nv * in.Cskip;
         if (in.lo) {
-            UCK(unet::upcat(in.lo + b * (nv / 8) * in.Clo, in.Clo, x, in.Cskip, n, 1, U->mcat, s));
-            x = U->mcat;
+            UCK(unet::upcat(in.lo + b * (nv / 8) * in.Clo, in.Clo, x, in.Cskip, n, 1, cat, s));
+            x = cat;
         }
-        UCK(unet::conv3d_fwd(x, Cin, w, bias, Cout, relu, out.bf ? out.bf + b * nv * Cout : U->mout,
-                             out.first ? U->mout32 : out.f32, n, s));
+        UCK(unet::conv3d_fwd(x, Cin, w, bias, Cout, relu, out.bf ? out.bf + b * nv * Cout : last,
+                             out.first ? last32 : out.f32, n, s));
         if (out.first) {
             qpat::note_launch(1);
-            k_take_channel0<<<g1(nv), 256, 0, s>>>(nv, U->mout32, out.first + b * nv, out.first_exp ? 1.f : 0.f);
+            k_take_channel0<<<g1(nv), 256, 0, s>>>(nv, last32, out.first + b * nv, out.first_exp ? 1.f : 0.f);
         }
     }
-    (void)c;
     return QPAT_OK;
 }
 
 int conv_fwd(qpat_unet_s* U, const Conv& c, const unet::ConvInput& in, bf16* out, int n, int B, cudaStream_t s) {
-    return conv_fwd(U, c, c.w, c.cout, c.b32, c.relu, in, unet::ConvOutput{out}, n, B, s);
+    return conv_fwd(U, c.w, c.cout, c.b32, c.relu, in, unet::ConvOutput{out}, n, B, s);
 }
 
 // backward of one conv: gout (gradient of its output, masked here by the
@@ -255,7 +288,7 @@ int conv_bwd(qpat_unet_s* U, Conv& c, const bf16* in, const bf16* out, bf16* gou
     const int64_t nv = int64_t(n) * n * n * B;
     if (c.relu) UCK(unet::relu_mask(gout, out, nv * c.cout, s));
     UCK(unet::conv3d_wgrad(in, c.cin, gout, c.cout, c.aw, c.ab, U->partial, n, B, add, s));
-    if (gin) return conv_fwd(U, c, c.wt, c.cin, nullptr, 0, unet::ConvInput{gout, c.cout}, unet::ConvOutput{gin}, n, B, s);
+    if (gin) return conv_fwd(U, c.wt, c.cin, nullptr, 0, unet::ConvInput{gout, c.cout}, unet::ConvOutput{gin}, n, B, s);
     return QPAT_OK;
 }
 
@@ -292,7 +325,7 @@ int unet_forward(qpat_unet_s* U, int B, bool train, float* y, int y_exp, cudaStr
     unet::ConvOutput out;
     out.first = y;
     out.first_exp = y_exp;
-    return conv_fwd(U, C[14], C[14].w, 16, C[14].b32, 0, In{U->d0, 16}, out, n0, B, s);
+    return conv_fwd(U, C[14].w, 16, C[14].b32, 0, In{U->d0, 16}, out, n0, B, s);
 }
 
 int unet_backward(qpat_unet_s* U, int B, int add, cudaStream_t s) {
@@ -379,7 +412,7 @@ int qpat_unet_create(int n, uint64_t seed, qpat_unet_t* out) {
             c.ab = g + c.nw();
             g = c.ab + c.cout;
         }
-        rc = reserve(U, 1, false, nullptr);
+        rc = reserve(U, 1, true, nullptr);
     }
     if (!rc) rc = ualloc(U, &U->loss, 1);
     if (!rc && cudaMallocHost(&U->hloss, sizeof(float)) != cudaSuccess) rc = fail(QPAT_ECUDA, "qpat_unet: pinned");
@@ -397,7 +430,7 @@ void qpat_unet_free(qpat_unet_t U) {
     if (!U) return;
     DeviceGuard dg(U->device);
     cudaDeviceSynchronize();
-    for (auto* list : {&U->allocs, &U->acts, &U->train_acts})
+    for (auto* list : {&U->allocs, &U->acts, &U->train_acts, &U->kept})
         for (void* p : *list) cudaFree(p);
     if (U->hloss) cudaFreeHost(U->hloss);
     delete U;
