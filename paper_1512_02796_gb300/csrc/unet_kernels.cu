@@ -160,7 +160,13 @@ struct FastDiv {
     __device__ __forceinline__ uint32_t div(uint32_t v) const { return (__umulhi(m, v) + v) >> s; }
 };
 
-template <int NCI>
+// The same 16 bytes from an address that is a multiple of a bf16's size only.
+__device__ __forceinline__ void copy_bf16(bf16* dst, const bf16* src, bool ok) {
+    for (int e = 0; e < 8; ++e) dst[e] = ok ? src[e] : __float2bfloat16(0.f);
+}
+
+// kAligned: in and dy lie on 16-byte boundaries (a caller's tensors need not)
+template <int NCI, bool kAligned>
 __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dy,
                                                            int Cout, float* __restrict__ partial,
                                                            float* __restrict__ bias, int n, FastDiv dn, int64_t voxels,
@@ -174,6 +180,12 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(const bf16* __restric
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int64_t vbeg = chunk * chunk_voxels, vend = min(voxels, vbeg + chunk_voxels);
     const int64_t shift = (int64_t(tap / 9 - 1) * n + (tap / 3 % 3 - 1)) * n + (tap % 3 - 1);
+    auto copy = [](bf16* dst, const bf16* src, bool ok) {
+        if constexpr (kAligned)
+            copy16(dst, src, ok);
+        else
+            copy_bf16(dst, src, ok);
+    };
     auto load = [&](int64_t v0, int st) {
         for (int i = threadIdx.x; i < kWgStep * NCI; i += kWgThreads) {
             const int64_t v = v0 + i / NCI;
@@ -184,12 +196,12 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(const bf16* __restric
                           z = int(r - w * n) + tap / 9 - 1;
                 ok = x >= 0 && y >= 0 && z >= 0 && x < n && y < n && z < n;
             }
-            copy16(sIn + (st * kWgStep + i / NCI) * LI + i % NCI * 8, ok ? in + (v + shift) * Cin + i % NCI * 8 : in, ok);
+            copy(sIn + (st * kWgStep + i / NCI) * LI + i % NCI * 8, ok ? in + (v + shift) * Cin + i % NCI * 8 : in, ok);
         }
         for (int i = threadIdx.x; i < kWgStep * 2; i += kWgThreads) {
             const int64_t v = v0 + i / 2;
             const bool ok = v < vend;
-            copy16(sDy + (st * kWgStep + i / 2) * LD + i % 2 * 8, ok ? dy + v * Cout + co0 + i % 2 * 8 : dy, ok);
+            copy(sDy + (st * kWgStep + i / 2) * LD + i % 2 * 8, ok ? dy + v * Cout + co0 + i % 2 * 8 : dy, ok);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -274,11 +286,13 @@ template <int NCI>
 cudaError_t wgrad_t(const bf16* in, const bf16* dy, int Cout, float* partial, float* bias, int n, int64_t voxels,
                     int64_t chunk, cudaStream_t s) {
     const size_t smem = sizeof(bf16) * 2 * kWgStep * size_t(8 * NCI + 8 + 16 + 8);
-    const cudaError_t e = qpat::allow_smem((const void*)k_conv_wgrad<NCI>, smem);
+    const bool aligned = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(dy)) & 15) == 0;
+    const auto kernel = aligned ? k_conv_wgrad<NCI, true> : k_conv_wgrad<NCI, false>;
+    const cudaError_t e = qpat::allow_smem((const void*)kernel, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid(unsigned((voxels + chunk - 1) / chunk), 27, unsigned(Cout / 16));
     qpat::note_launch(1);
-    k_conv_wgrad<NCI><<<grid, kWgThreads, smem, s>>>(in, dy, Cout, partial, bias, n, FastDiv(uint32_t(n)), voxels, chunk);
+    kernel<<<grid, kWgThreads, smem, s>>>(in, dy, Cout, partial, bias, n, FastDiv(uint32_t(n)), voxels, chunk);
     return cudaGetLastError();
 }
 
