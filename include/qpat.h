@@ -496,7 +496,8 @@ int64_t qpat_conv3d_bf16_wgrad_scratch(int n, int Cin, int Cout);
  * 1 = mma.sync only.  QPAT_EINVAL for other values.  Not in the paper. */
 int qpat_conv3d_set_engine(int engine);
 /* Bounded waits of the tcgen05 convolution that gave up since the library
- * was loaded (their tiles are written as NaN); 0 in normal operation. */
+ * was loaded (their tiles are written as NaN, or 0 behind a ReLU); 0 in normal
+ * operation. */
 int qpat_conv3d_tc_timeouts(void);
 
 /* ---------------------------------------------------------- autotuner */

@@ -29,9 +29,10 @@
 // With boxes chosen by those rates and a ring of four taps, 8 samples through all
 // layers at 128^3 went from 11.2 to 8.9 ms; eight issuing warps instead of four: 9.0.
 //
-// Tensor memory is allocated by warp 0 and freed on every exit path.  A wait
-// that gives up writes NaN into the tiles (the caller's parity checks see it)
-// and counts the event in g_tc_timeouts.
+// Tensor memory is allocated by warp 0 and freed on every exit path, after the
+// MMAs in flight are done (or have been waited for as long as any wait lasts).
+// A wait that gives up counts the event in g_tc_timeouts and writes NaN into the
+// tiles (0 behind a ReLU, whose maximum with 0 drops it).
 #include <algorithm>
 #include <array>
 #include <cstdint>
@@ -314,7 +315,7 @@ constexpr int kStayThreads = kTcThreads + 32 * kIssueWarps;
 
 __global__ void __launch_bounds__(kStayThreads) k_conv_fwd_tc_stay(const TcArgs a) {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    __shared__ uint64_t full[2], done[2], stored[2];
+    __shared__ uint64_t full[2], done[2], stored[2], drained[kIssueWarps];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int gave_up;
     const TcBox& g = a.g;
@@ -328,6 +329,7 @@ __global__ void __launch_bounds__(kStayThreads) k_conv_fwd_tc_stay(const TcArgs 
             mbar_init(&done[i], kIssueWarps);
             mbar_init(&stored[i], kTcThreads);
         }
+        for (int i = 0; i < kIssueWarps; ++i) mbar_init(&drained[i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         gave_up = 0;
     }
@@ -384,6 +386,14 @@ __global__ void __launch_bounds__(kStayThreads) k_conv_fwd_tc_stay(const TcArgs 
     }
     tc_before();
     __syncthreads();
+    if (gave_up) {  // nobody has waited for the MMAs since: they end before tensor memory is freed
+        if (warp >= kTcThreads / 32) {
+            uint64_t* const end = &drained[warp - kTcThreads / 32];
+            mma_commit(end);
+            if (!mbar_wait_parity(end, 0u)) atomicAdd(&g_tc_timeouts, 1);
+        }
+        __syncthreads();
+    }
     if (warp == 0) tmem_free(tmem, g.ncols);
 }
 
