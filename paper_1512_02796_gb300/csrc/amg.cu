@@ -1140,7 +1140,7 @@ struct AmgValues {
 
 struct AmgVecs {
     explicit AmgVecs(MemLedger* l) : mem(l) {}
-    std::vector<void*> b, xa, xb, d, r;
+    std::vector<void*> b, xa, xb, d, r;  // nullptr where the form of the cycle has no use for one
     DevMem mem;
 };
 
@@ -1157,7 +1157,7 @@ struct AmgCg {
 struct AmgState {
     MemLedger ledger;
     AmgHierDev hier{&ledger};     // on the prior's pattern, for K and M_delta
-    std::map<std::pair<int, int>, AmgVecs> vecs;  // (R, FP32 V-cycle)
+    std::map<std::array<int, 3>, AmgVecs> vecs;   // (R, FP32 cycle, degree 1)
     std::map<int, AmgCg> cg;                       // R
     std::map<const void*, AmgValues> vals;         // per operator; their graphs work on vecs and cg too
     cudaStream_t capture = nullptr;                // a non-default stream to capture on
@@ -1897,20 +1897,25 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
         return rc;
     }
     cudaError_t e = cudaSuccess;
-    auto vecs = A.vecs.find({R, f32 ? 1 : 0});
+    const std::array<int, 3> form{R, f32 ? 1 : 0, fast ? 1 : 0};
+    auto vecs = A.vecs.find(form);
     if (vecs == A.vecs.end()) {
         AmgVecs fresh(&A.ledger);
-        const size_t esz = f32 ? sizeof(float) : sizeof(double);
-        for (const LevelDev& d : H.lv) {
-            const size_t cnt = size_t(d.A.n) * R * esz;
-            fresh.b.push_back(fresh.mem.get<char>(cnt, e));
-            fresh.xa.push_back(fresh.mem.get<char>(cnt, e));
-            fresh.xb.push_back(fresh.mem.get<char>(cnt, e));
-            fresh.d.push_back(fresh.mem.get<char>(cnt, e));
-            fresh.r.push_back(fresh.mem.get<char>(cnt, e));
+        const size_t esz = f32 ? sizeof(float) : sizeof(double), L = H.lv.size();
+        // the fine level's iterate and its partners belong to the polynomial (or, alone, to the dense solve), its
+        // right-hand side is CG's residual unless the cycle wants that in FP32
+        for (size_t l = 0; l < L; ++l) {
+            auto vec = [&](bool used) {
+                return used ? fresh.mem.get<char>(size_t(H.lv[l].A.n) * R * esz, e) : nullptr;
+            };
+            fresh.b.push_back(vec(l > 0 || f32));
+            fresh.xa.push_back(vec(l > 0 || !fast));
+            fresh.xb.push_back(vec(l == 0 && !fast));
+            fresh.d.push_back(vec(l == 0 && !fast));
+            fresh.r.push_back(vec(l + 1 < L));
         }
         if (e != cudaSuccess) return cuda_fail(e, "multigrid workspace");
-        vecs = A.vecs.emplace(std::make_pair(R, f32 ? 1 : 0), std::move(fresh)).first;
+        vecs = A.vecs.emplace(form, std::move(fresh)).first;
     }
     AmgVecs& W = vecs->second;
     auto cg = A.cg.find(R);

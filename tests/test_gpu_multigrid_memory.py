@@ -91,3 +91,17 @@ def test_failed_form_leaves_the_others(inputs):
         solve(mesh, "K", inputs, multigrid=2)
     np.testing.assert_array_equal(solve(mesh, "K", inputs, multigrid=1), a)
     mesh.close()
+
+
+@pytest.mark.parametrize("K", [8, 16])
+def test_vectors_of_the_default_cycle(inputs, K):
+    """Per unknown: CG's five vectors, the fine residual, and three vectors on levels that together have a sixth of the fine
+    level's rows."""
+    xyz, tets, kappa, mu, flux, _ = inputs
+    mesh = Q.qpat_mesh(xyz, tets)
+    p = Q.qpat_default_params(multigrid=1)
+    Q.qpat_forward(mesh, kappa, mu, flux[:1], p)
+    before = mesh.multigrid_bytes()
+    Q.qpat_forward(mesh, kappa, mu, np.tile(flux, (4, 1))[:K], p)
+    assert mesh.multigrid_bytes() - before < 8 * 6.6 * K * mesh.N + (1 << 20)
+    mesh.close()
