@@ -3,6 +3,8 @@
 // prior entry points.  Algorithm 1 lives in recon.cu.
 #include <algorithm>
 #include <atomic>
+#include <exception>
+#include <new>
 #include <set>
 #include <cmath>
 #include <cstring>
@@ -656,6 +658,18 @@ void note_launch(int n) {
 int64_t thread_launches() { return t_launches; }
 }  // namespace qpat
 
+// A call's host work: an exception (memory) becomes an error code, as none may leave a C entry point.
+template <typename F>
+static int guarded(const char* who, const F& fn) {
+    try {
+        return fn();
+    } catch (const std::bad_alloc&) {
+        return fail(QPAT_ENOMEM, std::string(who) + ": out of host memory");
+    } catch (const std::exception& ex) {
+        return fail(QPAT_ENOMEM, std::string(who) + ": " + ex.what());
+    }
+}
+
 extern "C" {
 
 const char* qpat_last_error(void) { return g_err.c_str(); }
@@ -693,28 +707,32 @@ static int mesh_create(const double* xyz, int64_t N, const int32_t* tets, int64_
                        int patch_multiple, qpat_mesh_t* out) {
     if (!out) return fail(QPAT_EINVAL, "qpat_mesh: out is NULL");
     *out = nullptr;
-    auto* M = new qpat_mesh_s();
-    std::string msg = build_host_mesh(xyz, N, tets, E, patch_nodes, patch_multiple, M->h);
-    if (!msg.empty()) {
-        delete M;
-        return fail(QPAT_EINVAL, msg);
-    }
-    int rc = upload_mesh(M);
+    qpat_mesh_t M = nullptr;
+    bool on_device = false;
+    const int rc = guarded("qpat_mesh", [&] {
+        M = new qpat_mesh_s();
+        const std::string msg = build_host_mesh(xyz, N, tets, E, patch_nodes, patch_multiple, M->h);
+        if (!msg.empty()) return fail(QPAT_EINVAL, msg);
+        on_device = true;
+        return upload_mesh(M);
+    });
     if (rc != QPAT_OK) {
-        qpat_mesh_free(M);
+        if (on_device)
+            qpat_mesh_free(M);
+        else
+            delete M;
         return rc;
     }
     *out = M;
     return QPAT_OK;
 }
 
-int qpat_multigrid_host_info(const double* xyz, int64_t N, const int32_t* tets, int64_t E, int patch_nodes,
-                             int prior, int64_t* rows, int max_levels) {
+static int multigrid_host_info(const double* xyz, int64_t N, const int32_t* tets, int64_t E, int patch_nodes, int64_t* rows,
+                               int max_levels) {
     if (max_levels < 0 || (max_levels > 0 && !rows)) return fail(QPAT_EINVAL, "qpat_multigrid_host_info: bad argument");
     HostMesh h;
     std::string msg = build_host_mesh(xyz, N, tets, E, patch_nodes, 0, h);
     if (!msg.empty()) return fail(QPAT_EINVAL, msg);
-    (void)prior;  // one hierarchy pattern serves K and M_delta
     const SellPattern fine = amg_fine_pattern(h);
     const AmgPlan plan = amg_build_plan(fine, amg_fine_graph(h, fine));
     msg = amg_check_plan(plan);
@@ -724,8 +742,14 @@ int qpat_multigrid_host_info(const double* xyz, int64_t N, const int32_t* tets, 
     return L;
 }
 
-int qpat_mesh_host_info(const double* xyz, int64_t N, const int32_t* tets, int64_t E, int patch_nodes,
-                        int64_t* info8, int32_t* faces, int32_t* perm) {  // info8: 11 entries
+int qpat_multigrid_host_info(const double* xyz, int64_t N, const int32_t* tets, int64_t E, int patch_nodes, int /*prior*/,
+                             int64_t* rows, int max_levels) {  // one hierarchy serves K and M_delta
+    return guarded("qpat_multigrid_host_info",
+                   [&] { return multigrid_host_info(xyz, N, tets, E, patch_nodes, rows, max_levels); });
+}
+
+static int mesh_host_info(const double* xyz, int64_t N, const int32_t* tets, int64_t E, int patch_nodes, int64_t* info8,
+                          int32_t* faces, int32_t* perm) {  // info8: 11 entries
     if (!info8) return fail(QPAT_EINVAL, "qpat_mesh_host_info: info is NULL");
     HostMesh h;
     std::string msg = build_host_mesh(xyz, N, tets, E, patch_nodes, 0, h);
@@ -850,6 +874,12 @@ int qpat_mesh_host_info(const double* xyz, int64_t N, const int32_t* tets, int64
         if (h.nodes[nb + h.sell_col[d]] != g) return fail(QPAT_EINVAL, "host check: diagonal slot");
     }
     return QPAT_OK;
+}
+
+int qpat_mesh_host_info(const double* xyz, int64_t N, const int32_t* tets, int64_t E, int patch_nodes,
+                        int64_t* info8, int32_t* faces, int32_t* perm) {
+    return guarded("qpat_mesh_host_info",
+                   [&] { return mesh_host_info(xyz, N, tets, E, patch_nodes, info8, faces, perm); });
 }
 
 static constexpr int kPatchesPerSm = 2;

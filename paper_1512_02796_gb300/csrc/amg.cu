@@ -12,6 +12,7 @@
 #include <array>
 #include <cmath>
 #include <cstdio>
+#include <exception>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -1191,9 +1192,15 @@ int full_grid(K kernel, int most) {
 
 inline int blocks_of(int64_t n, int per = 256) { return int(std::max<int64_t>(1, (n + per - 1) / per)); }
 
-int build_hier(qpat_mesh_s* M, AmgHierDev& H) {
-    const SellPattern fine = amg_fine_pattern(M->h);
-    const AmgPlan plan = amg_build_plan(fine, amg_fine_graph(M->h, fine));
+int build_hier(qpat_mesh_s* M, AmgHierDev& H, MemLedger& ledger) {
+    AmgPlan plan;
+    try {
+        const SellPattern fine = amg_fine_pattern(M->h);
+        plan = amg_build_plan(fine, amg_fine_graph(M->h, fine));
+    } catch (const std::exception& ex) {  // host memory
+        ledger.refused = true;
+        return fail(QPAT_ENOMEM, std::string("multigrid plan: ") + ex.what());
+    }
     if (!plan.error.empty()) {
         H.error = plan.error;
         return fail(QPAT_EINVAL, plan.error);
@@ -1879,7 +1886,7 @@ int amg_solve(qpat_mesh_s* M, const OpState& st, const SolveOpts& so, int R, con
     if (!H.ready) {
         if (!H.error.empty()) return fail(QPAT_EINVAL, H.error);
         AmgHierDev fresh(&A.ledger);
-        const int rc = build_hier(M, fresh);
+        const int rc = build_hier(M, fresh, A.ledger);
         if (rc != QPAT_OK) {
             H.error = fresh.error;  // no hierarchy for this mesh; empty where only memory is short
             return rc;

@@ -5,37 +5,16 @@
 // once per mesh and pattern, and is deterministic (row loops are split over
 // host threads in fixed contiguous ranges and concatenated in order).
 #include "amg.h"
+#include "host_threads.h"
 #include "qpat_internal.h"
 
 #include <algorithm>
-#include <thread>
 
 namespace qpat {
 namespace {
 
-int host_threads() {
-    const unsigned h = std::thread::hardware_concurrency();
-    return int(std::max(1u, std::min(h, 16u)));
-}
-
 // Threads for n rows (coarse levels have few, long rows).
 int threads_for(int64_t n) { return n < 256 ? 1 : host_threads(); }
-
-// fn(t, begin, end) over nt contiguous ranges of [0, n).
-template <typename F>
-void parallel_ranges(int64_t n, int nt, const F& fn) {
-    if (nt <= 1) {
-        fn(0, int64_t(0), n);
-        return;
-    }
-    std::vector<std::thread> th;
-    th.reserve(nt);
-    for (int t = 0; t < nt; ++t) {
-        const int64_t b = n * t / nt, e = n * (t + 1) / nt;
-        th.emplace_back([&fn, t, b, e] { fn(t, b, e); });
-    }
-    for (auto& x : th) x.join();
-}
 
 struct Csr {
     int64_t n = 0;

@@ -4,21 +4,15 @@
 #include "element.h"
 
 #include <algorithm>
-#include <thread>
+
+#include "host_threads.h"
 
 namespace qpat {
 namespace {
 
 template <typename F>
 void parallel(int64_t n, const F& fn) {
-    const int nt = n < 8192 ? 1 : int(std::max(1u, std::min(std::thread::hardware_concurrency(), 16u)));
-    if (nt == 1) {
-        fn(int64_t(0), n);
-        return;
-    }
-    std::vector<std::thread> th;
-    for (int t = 0; t < nt; ++t) th.emplace_back([&fn, n, t, nt] { fn(n * t / nt, n * (t + 1) / nt); });
-    for (auto& x : th) x.join();
+    parallel_ranges(n, n < 8192 ? 1 : host_threads(), [&](int, int64_t b, int64_t e) { fn(b, e); });
 }
 
 inline int64_t sell_at(const std::vector<int64_t>& ptr, int64_t row, int k) {
