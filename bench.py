@@ -714,7 +714,8 @@ def mg_roofline(kern, dom, f64_peak, hbm_peak, hbm_kind, sm_mhz, nsm, workload):
     out["launches"] = k["fine_launches"]
     out["hbm_peak_gbs"] = hbm_peak
     out["traffic"] = None
-    tf = os.path.join(ROOT, "profiles", f"k_cheb_{workload}_traffic.json")
+    # one file per kernel: the degree-1 cycle's residual is k_level, a higher degree's smoothing step k_cheb
+    tf = os.path.join(ROOT, "profiles", f"{k['kernel'].split('<')[0]}_{workload}_traffic.json")
     if os.path.exists(tf):
         try:
             tr = json.load(open(tf))
