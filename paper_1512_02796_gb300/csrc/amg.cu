@@ -750,16 +750,19 @@ __global__ void __launch_bounds__(256) k_cg_clear(int64_t n, const double* bb, d
 // Control words of a CG solve (int ctl[]): [0] status, [1] right-hand sides
 // still running, [2] iterations done, [3] 1 before the first direction,
 // [4] iteration cap, [5] right-hand sides with b = 0 and a residual (from a
-// guess); the per-RHS running flags follow at ctl + kCtlActive.
+// guess), [6] right-hand sides with a scale other than 1; the per-RHS running
+// flags follow at ctl + kCtlActive.
 constexpr int kCtlActive = 8;
 
 // bb = totals of b.b.  A right-hand side with b = 0 is solved by x = 0, and
 // one whose guess already meets the target by that guess: neither runs (a
 // residual of 0 would have no direction).  Q: quantities per right-hand side
-// in the partials (2: r.r behind b.b; 1: r = b).  scale: the power of two that
-// brings |r| to [1, 2); the FP32 cycle works on scale r, so that neither small
-// nor large right-hand sides leave FP32's range.  z, p and q then carry it too,
-// alpha its inverse, and beta and the iterates are the same to the bit.
+// in the partials (2: r.r behind b.b; 1: r = b).  scale: the FP32 cycle works on
+// scale r, so that neither small nor large right-hand sides leave FP32's range:
+// 1 where |r| lies in [2^-20, 2^60] (53 binary digits less at the end of a solve,
+// and as many again between entries, still lie above 2^-126), else the
+// power of two that brings |r| to [1, 2).  z, p and q then carry it too, alpha
+// its inverse, and beta and the iterates are the same to the bit.
 // stop: the |r|^2 at which the iteration leaves a right-hand side: the target
 // tol[0] |b|^2, or, in sweeps (tol[1] > 0), tol[1] times |r|^2 at the sweep's
 // start, but no less than two such sweeps from |b|^2 would leave.
@@ -773,7 +776,8 @@ __global__ void k_cg_start(const double* part, int G, const double* tol, double*
     const double rr = Q == 1 ? t : total_of(part, G, Q * R, (Q - 1) * R + r);
     if ((threadIdx.x & 31) == 0) {
         bb[r] = t;
-        scale[r] = rr > 0.0 && isfinite(rr) ? scalbn(1.0, -(ilogb(rr) >> 1)) : 1.0;
+        const int e = rr > 0.0 && isfinite(rr) ? ilogb(rr) >> 1 : 0;
+        scale[r] = e >= -20 && e < 60 ? 1.0 : scalbn(1.0, -e);
         stop[r] = tol[1] > 0.0 ? fmax(tol[1] * rr, tol[1] * tol[1] * t) : tol[0] * t;
         active[r] = t > 0.0 && rr > tol[0] * t ? 1 : 0;
         clear[r] = t == 0.0 && rr > 0.0 ? 1 : 0;
@@ -784,15 +788,17 @@ __global__ void k_cg_start(const double* part, int G, const double* tol, double*
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        int c = 0, z = 0;
+        int c = 0, z = 0, s = 0;
         for (int q = 0; q < R; ++q) {
             c += active[q];
             z += clear[q];
+            s += scale[q] != 1.0;
         }
         ctl[1] = c;
         ctl[2] = 0;
         ctl[3] = 1;
         ctl[5] = z;
+        ctl[6] = s;
     }
 }
 
@@ -958,13 +964,14 @@ __global__ void __launch_bounds__(256) k_cg_dir(int64_t n, const double* beta, c
     }
 }
 
-// x += alpha p, r -= alpha q (b32: and the FP32 copy of scale r), r.r.  The last
+// x += alpha p, r -= alpha q (b32: and the FP32 copy of r, SCALED: of scale r;
+// a multiplication by 1 for every entry would cost a fifth of this kernel), r.r.  The last
 // block checks: a right-hand side stops once |r|^2 <= stop; one more
 // iteration is done.  Inside a graph (use_graph) it also sets the loop's
 // condition: go on while some right-hand side runs, the status is clean and
 // the cap is not reached (reaching it with a running right-hand side is
 // QPAT_ENOCONV).
-template <int R>
+template <int R, bool SCALED>
 __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alpha, const double* __restrict__ p,
                                                    const double* __restrict__ q, double* __restrict__ x,
                                                    double* __restrict__ r, const double* scale,
@@ -978,7 +985,7 @@ __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alph
 #pragma unroll
     for (int t = 0; t < C; ++t) {
         al[t] = alpha[m.c0 + t];
-        sc[t] = scale[m.c0 + t];
+        if (SCALED) sc[t] = scale[m.c0 + t];
         dot[t] = 0.0;
     }
     FOR_FLAT(n, R) {
@@ -997,7 +1004,7 @@ __global__ void __launch_bounds__(256) k_cg_update(int64_t n, const double* alph
         stR<double, C>(r + o, rv);
         if (b32)
 #pragma unroll
-            for (int t = 0; t < C; ++t) b32[o + t] = float(sc[t] * rv[t]);
+            for (int t = 0; t < C; ++t) b32[o + t] = float(SCALED ? sc[t] * rv[t] : rv[t]);
     }
     m.template block_totals<1>(dot, part);
     if (!last_block_totals<R>(part, count, tot)) return;
@@ -1725,6 +1732,7 @@ struct CgSolve {
         zp = z;
     }
     const double* zp = nullptr;  // z where it is not C.z
+    bool scaled = false;         // some right-hand side goes into the FP32 cycle with a scale
 
     // one iteration on stream t; use_graph: the check sets the loop condition
     void body(cudaStream_t t, cudaGraphConditionalHandle cond, int use_graph) {
@@ -1736,8 +1744,13 @@ struct CgSolve {
         // K's rows hold 15 entries, M_delta's 7: one group per row, the lanes of its right-hand sides side by side
         k_cg_apply<R, NV, 1><<<full_grid(k_cg_apply<R, NV, 1>, G), 256, 0, t>>>(NV == 1 ? H.K : H.lv[0].A, st.v64[0], st.v64[1], C.p, C.q, C.part, C.count,
                                                C.rz, C.alpha, C.ctl);
-        k_cg_update<R><<<full_grid(k_cg_update<R>, G), 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, C.scale,
-                                         f32 ? static_cast<float*>(W.b[0]) : nullptr, C.part, C.count, C.stop, C.rr, C.ctl, cond, use_graph);
+        float* const b32 = f32 ? static_cast<float*>(W.b[0]) : nullptr;
+        auto update = [&](auto kernel) {
+            kernel<<<full_grid(kernel, G), 256, 0, t>>>(n, C.alpha, C.p, C.q, C.x, C.r, C.scale, b32, C.part, C.count, C.stop,
+                                                        C.rr, C.ctl, cond, use_graph);
+        };
+        if (scaled) update(k_cg_update<R, true>);
+        else update(k_cg_update<R, false>);
     }
 
     // With so.sweep_rtol the solve is a refinement: sweeps of the iteration,
@@ -1751,7 +1764,7 @@ struct CgSolve {
         int* hc = reinterpret_cast<int*>(M->host_scratch + 240);
         cudaError_t e = cudaSuccess;
         auto read_ctl = [&]() -> cudaError_t {
-            cudaError_t x = cudaMemcpyAsync(hc, C.ctl, 6 * sizeof(int), cudaMemcpyDeviceToHost, s);
+            cudaError_t x = cudaMemcpyAsync(hc, C.ctl, 7 * sizeof(int), cudaMemcpyDeviceToHost, s);
             if (x == cudaSuccess) x = cudaStreamSynchronize(s);
             return x;
         };
@@ -1786,17 +1799,19 @@ struct CgSolve {
                 break;
             }
             ++count->sweeps;
+            scaled = f32 && hc[6] > 0;
             if (f32) {
                 note_launch(1);
                 k_cg_cast<R><<<G, 256, 0, s>>>(n, C.scale, C.r, static_cast<float*>(W.b[0]));
             }
             if (!timer->on) {
-                auto g = V.graphs.find(key);
+                const std::string name = scaled ? key + "/scaled" : key;
+                auto g = V.graphs.find(name);
                 if (g == V.graphs.end()) {
                     AmgGraph fresh;
                     const int rc = capture(A, fresh);
                     if (rc != QPAT_OK) return rc;
-                    g = V.graphs.emplace(key, std::move(fresh)).first;
+                    g = V.graphs.emplace(name, std::move(fresh)).first;
                 }
                 if ((e = cudaGraphLaunch(g->second.exec, s)) != cudaSuccess) return cuda_fail(e, "multigrid graph");
                 if ((e = read_ctl()) != cudaSuccess) return cuda_fail(e, "multigrid cg");
