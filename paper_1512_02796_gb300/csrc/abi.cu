@@ -290,10 +290,11 @@ static bool prefers_multigrid(const qpat_mesh_s* M, const OpState& st, const Sol
     return R > 1 && N * R >= 350000;
 }
 
-// Iterations that the library's own attempt at multigrid may take: the most
-// that any mesh above needed is 85, and a system that takes several times as
-// many is not one for which this choice is the faster.
-constexpr int kAttemptIterations = 400;
+// Iterations that the library's own attempt at multigrid may take.  The meshes
+// above need 16 to 97 and, behind random points, 81 to 235, growing slowly with the
+// size; a system that takes several times as many is not one for which this
+// choice is the faster.
+constexpr int kAttemptIterations = 1000;
 // Sweeps of its refinement: two reach the target in the recursive residual, a
 // third takes off the rounding of their iterates.  What the FP64 residual is
 // above the target then, the FP64 solver that precision 1 falls back to (which
