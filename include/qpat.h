@@ -160,9 +160,11 @@ typedef struct {
                               (the CG iterates stay FP64 and take the flexible
                               beta = r.(z - z_old) / (r.z)_old); M_delta keeps the
                               FP64 cycle.
-                              The hierarchy's patterns are built on the host on the
-                              first such solve of a mesh (seconds at 2 M nodes),
-                              its values on the device once per prepared operator. */
+                              The hierarchy's patterns are built on the host in the
+                              first such solve of a mesh, named or chosen (0.2 s
+                              at 2 M nodes on 16 cores; mesh preparation takes
+                              12 s), its values on the device once per prepared
+                              operator. */
     int mg_degree;         /* Chebyshev degree of the fine level's multigrid
                               smoothing, 1..8 (default and 0: 1, i.e. one
                               damped-Jacobi step before and after the coarse

@@ -2,15 +2,15 @@
 // the FP64 conjugate-gradient solves of K (Eq. (7)) and of M_delta (Eq. (19))
 // selected by qpat_params.multigrid.
 //
-// The method is the textbook smoothed aggregation of Vanek, Mandel and
-// Brezina (Computing 56, 1996): aggregates of the matrix graph (here of 8
-// nodes, by three rounds of pairwise matching), a piecewise-constant tentative prolongator smoothed by one damped Jacobi step,
-// a damped Jacobi step along the couplings between graph neighbours, weighted
-// so that the constants are kept (which keeps the coarse rows at ~30 to 70
-// entries), Galerkin
-// coarse operators A_c = P^T A P, Chebyshev smoothing in D^-1 A on each level
-// and an exact solve on the coarsest level; applied as one symmetric V-cycle
-// per CG iteration.
+// The method is the smoothed aggregation of Vanek, Mandel and Brezina
+// (Computing 56, 1996): aggregates of the matrix graph (here of 8 nodes, by
+// three rounds of pairwise matching), a piecewise-constant tentative
+// prolongator smoothed by one damped Jacobi step, taken along the couplings
+// between graph neighbours only (which keeps the coarse rows at ~30 to 70
+// entries) and weighted so that the constants are kept, Galerkin coarse
+// operators A_c = P^T A P, smoothing by one damped Jacobi step on each level (on
+// the fine level by a Chebyshev polynomial in D^-1 A, if asked for) and an exact
+// solve on the coarsest level; applied as one symmetric V-cycle per CG iteration.
 //
 // Split of the work:
 //  * symbolic (host, once per mesh and matrix pattern, amg_setup.cpp): the

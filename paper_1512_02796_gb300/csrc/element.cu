@@ -8,7 +8,8 @@
 // are the same from run to run, with no atomics, no colours and no barriers.
 //
 // Bound: FP64 issue and the plan's bytes about equally.  At 128^3 (2.1 M
-// nodes, 12.3 M tets) K takes ~200 FP64 operations and ~900 bytes a node;
+// nodes, 12.3 M tets) K takes ~200 FP64 operations and ~1.5 KB a node (per tet
+// 144 bytes with the lists that name it, per edge 64, per entry 16);
 // the element-by-element form that this replaces recomputed the geometry of
 // every tet (some 150 FP64 operations, for each patch that lists it),
 // searched the row for every entry and waited at ~26 barriers a patch.

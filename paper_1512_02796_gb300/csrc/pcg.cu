@@ -784,7 +784,8 @@ constexpr int min_ctas() {
     return (OP == OP_CSR1 || OP == OP_CSR2) ? 4 : 1;
 }
 
-// FP64 on the assembled operators: three resident CTAs per SM (80 registers).
+// FP64 on the assembled operators: three resident CTAs per SM (80 registers;
+// at most 4 bytes spilled for K, 60 for the two-block Jacobi form of M_delta).
 template <typename T, int OP, bool kPoly>
 constexpr int pcg_ctas() {
     return sizeof(T) == 8 && (OP == OP_CSR1 || (OP == OP_CSR2 && !kPoly)) ? 3 : 1;
@@ -1480,8 +1481,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_pcg_ring(PcgArgs<T> a, RingLayo
 // [cta_begin[j], cta_begin[j+1]) solve problem j, and each problem's barriers
 // and reductions involve only its own CTAs.  FP64 multiply-adds bound a
 // problem with several patches per CTA, so padding its right-hand sides to
-// the batch's largest number would cost in proportion.  Three CTAs per SM (70
-// registers for Jacobi, no spills) instead of the two that 102 registers allow.
+// the batch's largest number would cost in proportion.  Three CTAs per SM (80
+// registers at most) instead of the two that 102 registers allow.  The forms for
+// up to 4 and 8 right-hand sides spill for it, 12 and 136 bytes with Jacobi, 72
+// and 216 with the polynomial; against two CTAs without spills and one width for
+// all (the form before), 12 cubes of 16 to 39 nodes a side: 21.6 -> 16.3 ms (Jacobi)
+// and 22.7 -> 18.9 (degree 2) with 4 right-hand sides each, 33.7 -> 30.9 and 35.4 ->
+// 35.0 with 8; 20 cubes of 30 to 33: 47.4 -> 32.1, 47.0 -> 37.0, 74.0 -> 60.3, 75.0 -> 69.7.
 template <typename T, int RM, int OP, bool kPoly = false>
 __global__ void __launch_bounds__(kThreads, 3) k_pcg_batch(const PcgArgs<T>* __restrict__ probs,
                                                         const int* __restrict__ cta_begin, int nprob) {
