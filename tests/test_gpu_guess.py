@@ -20,7 +20,7 @@ pytestmark = pytest.mark.gpu
 
 # the persistent solvers, the library's choice (multigrid at this size) and the multigrid CG by name
 SOLVERS = [dict(), dict(multigrid=1), dict(multigrid=2), dict(multigrid=1, mg_degree=2), dict(pcg_variant=1),
-           dict(precision=1, fp32_operator=1), dict(precision=1, fp32_operator=1, pcg_variant=1)]
+           dict(precision=1), dict(precision=1, fp32_operator=1), dict(precision=1, fp32_operator=1, pcg_variant=1)]
 
 
 @pytest.fixture(scope="module")
