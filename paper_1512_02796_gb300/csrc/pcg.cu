@@ -807,10 +807,14 @@ __global__ void __launch_bounds__(kThreads, 3) k_pcg_occ3(PcgArgs<T> a) {
 // The same solver with kWideThreads threads per CTA, for the launches whose
 // shared memory (the staged direction or the preconditioner's owned-row
 // vectors of many RHS on large patches) leaves room for one CTA per SM only:
-// twice the warps per SM to hide the shared-memory and FP64 latencies.
+// twice the warps per SM to hide the shared-memory and FP64 latencies.  Held to
+// 88 registers, which all forms reach without spills: free to take 106 to 112, the
+// compiler orders the FP64 forms' loads so that an iteration waits longer for them (64^3, 16
+// right-hand sides, Jacobi 69 -> 60 ms, degree 2 68 -> 66; 96^3 348 -> 301 and 350 -> 334;
+// 80 registers: 69, 66, 344 and 332).
 constexpr int kWideThreads = 2 * kThreads;
 template <typename T, int R, int OP, bool kPoly = false>
-__global__ void __launch_bounds__(kWideThreads) k_pcg_wide(PcgArgs<T> a) {
+__global__ void __maxnreg__(88) k_pcg_wide(PcgArgs<T> a) {
     pcg_body<T, R, OP, kPoly, kWideThreads>(a, blockIdx.x, gridDim.x);
 }
 
